@@ -47,7 +47,6 @@ NCU_TRAFFIC = {  # (kernel family, formulation or "any", far-rule points, band) 
     ("cheb", "juffer", 667788, 3.0): 16.04e6,
     ("tree32", "juffer", 667788, 3.0): 246.8e6,
     ("pair32acc", "juffer", 667788, 3.0): 496.5e6,
-    ("near_adj", "any", 667788, 3.0): 1372.1e6,  # mean of the edge-pair and vertex-pair launches
     ("near_band", "any", 667788, 3.0): 15203.8e6,
     ("near_coin", "any", 667788, 3.0): 233.9e6,
 }
@@ -273,7 +272,7 @@ def _kernels():
             pb.PB_KERNEL_PAIR32_ACCURATE: ("k_pair32x2 split-coordinate (FP32 far field, FP64 tile sums)",
                                            "pair32acc", "alu", FP32_LANES_PER_SM, "FP32 ops"),
             pb.PB_KERNEL_PAIR64: ("k_pair64 (FP64 far field)", "pair64", "alu", FP64_FLOPS_PER_SM, "FP64 flops"),
-            pb.PB_KERNEL_NEAR_ADJ: ("k_near_pairs (FP64 singular quadrature, edge/vertex pairs)", "near_adj", "alu",
+            pb.PB_KERNEL_NEAR_ADJ: ("k_adj_pairs (FP64 singular quadrature, edge/vertex pairs)", "near_adj", "alu",
                                     FP64_FLOPS_PER_SM, "FP64 flops"),
             pb.PB_KERNEL_NEAR_COIN: ("k_coin_pairs (FP64 singular quadrature, coincident pairs)", "near_coin", "alu",
                                      FP64_FLOPS_PER_SM, "FP64 flops"),

@@ -143,25 +143,30 @@ __global__ void k_ss_table(Gauss gq, int n, double* __restrict__ tab) {
     for (int c = 0; c < 8; ++c) tab[(5 + c) * n + e] = mono[c];
 }
 
-// Outer points of the edge (kind 1, 6 regions) and vertex (kind 2, 2 regions)
-// maps: one entry per (region, xi, eta1, eta2). In both maps the innermost
-// Gauss variable eta3 enters a single coordinate, the second one (t) of one
-// frame, and linearly, while the region Jacobian does not involve it; so
-// over the eta3 points of an entry x - y = D0 + eta3 D1 and every weighted
-// monomial is affine in eta3. A pair's kernel sums then take two partial sums
-// per kernel over eta3 (sum w3 g, sum w3 eta3 g) and expand them into the
-// nine moments once per entry. Per entry (array c at v[c * n + e]):
+// Points of the edge (kind 1, 6 regions) and vertex (kind 2, 2 regions) maps.
+// Three properties of both maps carry the pair sums (k_adj_pairs):
+//   - every frame coordinate is proportional to xi, so with both frames starting
+//     at the shared vertex x - y = xi d(eta) and r = xi |d|: the geometry is
+//     evaluated at xi = 1 only, once per (eta1, eta2, eta3);
+//   - the Laplace kernels are homogeneous in xi (G ~ 1/xi, K ~ 1/xi^2), so their
+//     xi sums are the constants mu_m = sum_i w_i xi_i^m; the Yukawa kernels need
+//     E_m(z) = sum_i w_i xi_i^m e^{-z xi_i}, z = kappa |d|, m = 1..4 (Radial);
+//   - eta3 enters a single coordinate, the second one (t) of one frame, and
+//     linearly, while the region Jacobian does not involve it; so over the eta3
+//     points of an entry d = D0 + eta3 D1 and every weighted monomial is affine
+//     in eta3: two sums per kernel (sum w3 g, sum w3 eta3 g), expanded into the
+//     nine moments once per entry.
+// One entry per (region, eta1, eta2), at xi = 1 (array c at v[c * n + e]):
 //   0..3  sa, ta, sa', ta': the frame coordinates at eta3 = 0 (x: s, t; y: s', t')
 //   4, 5  tb, tb': the slopes of t and t' in eta3 (one of them is zero)
 //   6..14 c0[3 alpha + beta] = W P_alpha Q_beta, P = (1, sa, ta), Q = (1, sa', ta'),
-//         W = the Gauss weights of xi, eta1, eta2 times the Jacobian
+//         W = the Gauss weights of eta1, eta2 times the Jacobian
 //   15..19 the eta3-slope coefficients of the moments that change with eta3:
 //         (0,2) W tb', (1,2) W sa tb', (2,0) W tb, (2,1) W tb sa', (2,2) W (ta tb' + tb ta')
-// followed by the eta3 Gauss nodes and weights (2 n doubles).
 // One table per class (edge or vertex), each with its own Gauss rule.
 struct SSOuter {
     const double* v;
-    int n;        // entries (regions x nss^3)
+    int n;        // entries (regions x nss^2)
     int nss;      // Gauss points per dimension
     int nreg;     // regions of the map: 6 (edge) or 2 (vertex)
 };
@@ -169,18 +174,15 @@ constexpr int SS_OUTER_ARRAYS = 20;
 
 __global__ void k_ss_outer(Gauss gq, int kind, int n, double* __restrict__ tab) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    const int q = gq.n, n3 = q * q * q;
-    if (e < 2 * q) {  // the eta3 rule after the entries
-        tab[SS_OUTER_ARRAYS * n + e] = e < q ? gq.x[e] : gq.w[e - q];
-    }
+    const int q = gq.n, n2 = q * q;
     if (e >= n) return;
-    const int reg = e / n3, r = e - reg * n3;
-    const int i0 = r / (q * q), i1 = (r / q) % q, i2 = r % q;
+    const int reg = e / n2, r = e - reg * n2;
+    const int i1 = r / q, i2 = r % q;
     double sx0, tx0, sy0, ty0, sx1, tx1, sy1, ty1;
-    const double jac = ss_map(kind, reg, gq.x[i0], gq.x[i1], gq.x[i2], 0.0, sx0, tx0, sy0, ty0);
-    const double jac1 = ss_map(kind, reg, gq.x[i0], gq.x[i1], gq.x[i2], 1.0, sx1, tx1, sy1, ty1);
+    const double jac = ss_map(kind, reg, 1.0, gq.x[i1], gq.x[i2], 0.0, sx0, tx0, sy0, ty0);
+    const double jac1 = ss_map(kind, reg, 1.0, gq.x[i1], gq.x[i2], 1.0, sx1, tx1, sy1, ty1);
     const double tb = tx1 - tx0, tb2 = ty1 - ty0;
-    const double W = gq.w[i0] * gq.w[i1] * gq.w[i2] * jac;
+    const double W = gq.w[i1] * gq.w[i2] * jac;
     // the structure the factorisation relies on: s, s' and the Jacobian free of eta3
     const bool ok = sx1 == sx0 && sy1 == sy0 && jac1 == jac;
     const double P[3] = {1.0, sx0, tx0}, Q[3] = {1.0, sy0, ty0};
@@ -193,6 +195,48 @@ __global__ void k_ss_outer(Gauss gq, int kind, int n, double* __restrict__ tab) 
     v[18] = W * tb * sy0;
     v[19] = W * (tx0 * tb2 + tb * ty0);
     for (int c = 0; c < SS_OUTER_ARRAYS; ++c) tab[c * n + e] = v[c];
+}
+
+// The xi rule of an adjacent pair's sums: mu_m and E_m(z), m = 1..4. For z up to
+// zlim[RAD_DEG] E_m is its Taylor polynomial, sum_k (-1)^k mu_{m+k} z^k / k!, of the
+// degree d whose first omitted term is below 2^-56 for z <= zlim[d] (its terms
+// alternate and fall); beyond, the exponentials themselves are summed. Passed
+// by value: the coefficients are then constant operands of the FMAs.
+constexpr int RAD_DEG = 13;
+struct Radial {
+    double c[4][RAD_DEG + 1];  // c[m - 1][k]
+    double mu[4];              // mu_1..mu_4
+    double x[12], w[12];       // the Gauss rule (xi and eta3)
+    double wx[4][12];          // w_i xi_i^m
+    float zlim[RAD_DEG + 1];
+    int n;
+};
+
+static Radial make_radial(const Gauss& g) {
+    Radial r;
+    r.n = g.n;
+    for (int i = 0; i < 12; ++i) {
+        r.x[i] = i < g.n ? g.x[i] : 0.0;
+        r.w[i] = i < g.n ? g.w[i] : 0.0;
+        double p = r.w[i];
+        for (int m = 0; m < 4; ++m) r.wx[m][i] = p *= r.x[i];
+    }
+    for (int m = 1; m <= 4; ++m) {
+        double f = 1.0;  // (-1)^k / k!
+        for (int k = 0; k <= RAD_DEG; ++k) {
+            double mu = 0.0;
+            for (int i = 0; i < g.n; ++i) mu += g.w[i] * std::pow(g.x[i], m + k);
+            r.c[m - 1][k] = f * mu;
+            f *= -1.0 / (k + 1);
+        }
+        r.mu[m - 1] = r.c[m - 1][0];
+    }
+    double fact = 1.0;
+    for (int d = 0; d <= RAD_DEG; ++d) {
+        fact *= d + 1;
+        r.zlim[d] = (float)std::pow(fact * std::ldexp(1.0, -56), 1.0 / (d + 1));
+    }
+    return r;
 }
 
 // Geometry of one triangle in the reordered frame of its singular map:
@@ -263,51 +307,10 @@ __device__ __forceinline__ double exp_nonpos(double x) {
     return x < -700.0 ? 0.0 : __longlong_as_double(bits);
 }
 
-// Accumulators: SL[9], SY[9], KL[9], KY[9], sum w G_L, sum w G_Y (38); with
-// the reversed pair also KTL[9], KTY[9] (56): the double-layer kernel with the
-// normal of the first triangle, which is the K block of the reversed pair.
-#define NACC_NEAR 38
+// Accumulators of a pair: SL[9], SY[9], KL[9], KY[9], sum w G_L, sum w G_Y, and
+// KTL[9], KTY[9]: the double-layer kernel with the normal of the first triangle,
+// which is the K block of the reversed pair.
 #define NACC_SYM 56
-
-template <bool SYM>
-__device__ __forceinline__ void accum_point(double* acc, double w, const double* x, const double* y,
-                                            const double* nx, const double* ny, const double* lx,
-                                            const double* ly, double kappa) {
-    const double d0 = x[0] - y[0], d1 = x[1] - y[1], d2 = x[2] - y[2];
-    const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-    const double rinv = rsqrt(r2);
-    const double r = r2 * rinv;
-    const double gl = rinv * 0.07957747154594767;  // 1 / (4 pi r)
-    const double ek = exp_nonpos(-kappa * r);
-    const double gy = ek * gl;
-    const double fl = gl * rinv * rinv;            // 1 / (4 pi r^3)
-    const double fy_over_fl = ek * (1.0 + kappa * r);
-    const double dn = d0 * ny[0] + d1 * ny[1] + d2 * ny[2];
-    const double kl = fl * dn;
-    const double ky = kl * fy_over_fl;
-    double ktl = 0.0, kty = 0.0;
-    if (SYM) {
-        const double dnx = -(d0 * nx[0] + d1 * nx[1] + d2 * nx[2]);  // (y - x).n_x
-        ktl = fl * dnx;
-        kty = ktl * fy_over_fl;
-    }
-    for (int a = 0; a < 3; ++a) {
-        const double wa = w * lx[a];
-        for (int b = 0; b < 3; ++b) {
-            const double ll = wa * ly[b];
-            acc[3 * a + b] += gl * ll;
-            acc[9 + 3 * a + b] += gy * ll;
-            acc[18 + 3 * a + b] += kl * ll;
-            acc[27 + 3 * a + b] += ky * ll;
-            if (SYM) {
-                acc[38 + 3 * a + b] += ktl * ll;
-                acc[47 + 3 * a + b] += kty * ll;
-            }
-        }
-    }
-    acc[36] += w * gl;
-    acc[37] += w * gy;
-}
 
 // Regularised rules in the frames' own coordinates. A point of a frame is
 // q0 + s e1 + t e2 and its corner basis values are mu = (1 - s, s - t, t) in the
@@ -315,85 +318,110 @@ __device__ __forceinline__ void accum_point(double* acc, double w, const double*
 // monomial bases (1, s, t) x (1, s', t') and turned into the corner blocks once
 // per pair (frame_to_corner). For an adjacent pair both frames start at the
 // shared vertex, and d = x - y is formed from the frame vectors directly.
-// mom[9 k + 3 alpha + beta], k = G_L, G_Y, K_L, K_Y (and with SYM the reversed
-// pair's double layers K^T_L, K^T_Y).
-// Kernel values at x - y = d for an adjacent pair: G_L, G_Y, the double layers
-// K_L, K_Y with the second triangle's normal and (SYM) the reversed pair's with
-// the first triangle's normal.
-template <bool SYM>
-__device__ __forceinline__ void adj_kernels(const double* d, const TriFrame& A, const TriFrame& B, double kappa,
-                                            double* g) {
-    const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    const double rinv = rsqrt(r2);
-    const double r = r2 * rinv;
-    const double gl = rinv * 0.07957747154594767;  // 1 / (4 pi r)
-    const double ek = exp_nonpos(-kappa * r);
-    const double fl = gl * rinv * rinv;  // 1 / (4 pi r^3)
-    const double fy_over_fl = ek * (1.0 + kappa * r);
-    const double kl = fl * (d[0] * B.n[0] + d[1] * B.n[1] + d[2] * B.n[2]);
-    g[0] = gl;
-    g[1] = ek * gl;
-    g[2] = kl;
-    g[3] = kl * fy_over_fl;
-    if (SYM) {
-        const double ktl = fl * -(d[0] * A.n[0] + d[1] * A.n[1] + d[2] * A.n[2]);  // (y - x).n_x
-        g[4] = ktl;
-        g[5] = ktl * fy_over_fl;
-    }
-}
 
-// One outer entry (region, xi, eta1, eta2) of an edge- or vertex-adjacent pair:
-// the NSS eta3 points summed per kernel into a0 = sum w3 g and a1 = sum w3 eta3 g,
-// then expanded into the moments (nine per kernel from a0, five from a1).
-// NSS = 0: the rule's size is read at run time.
-template <bool SYM, int NSS>
-__device__ __forceinline__ void accum_outer(double* mom, const SSOuter& tab, int e, const double* dq,
-                                            const TriFrame& A, const TriFrame& B, double kappa, const double* x3,
-                                            const double* w3) {
-    constexpr int NK = SYM ? 6 : 4;
+// The vectors of an adjacent pair that its lanes read by broadcast: the frames'
+// edges, and the normals' products with them: n_B . x = s al1 + t al2 is the
+// height of x over the second triangle's plane, so d . n_B needs no y, and
+// -d . n_A = s' be1 + t' be2 no x.
+struct AdjGeo {
+    double e1a[3], e2a[3], e1b[3], e2b[3];
+    double al1, al2, be1, be2;
+};
+
+// One entry (region, eta1, eta2) of an adjacent pair: the eta3 points' sums, then
+// the moments mom[9 k + 3 alpha + beta], k = G_L, G_Y, K_L, K_Y, K^T_L, K^T_Y (the
+// reversed pair's double layers), without the factor 1/(4 pi) and, for the Laplace
+// kernels, without the xi sums (mu). A moment of degree deg = [alpha > 0] +
+// [beta > 0] carries xi^deg: the Yukawa sums are kept per degree.
+template <int NSS>
+__device__ __forceinline__ void accum_entry(double* mom, const SSOuter& tab, const Radial& rad, int e,
+                                            const AdjGeo& P, double kappa, int deg) {
     const int n = tab.n;
-    const double sa = tab.v[e], ta = tab.v[n + e], sa2 = tab.v[2 * n + e], ta2 = tab.v[3 * n + e];
-    const double tb = tab.v[4 * n + e], tb2 = tab.v[5 * n + e];
-    double D0[3], D1[3];
+    const double ta = tab.v[n + e], ta2 = tab.v[3 * n + e], tb = tab.v[4 * n + e], tb2 = tab.v[5 * n + e];
+    double D0[3], D1[3], hb0, hb1, ha0, ha1;
+    {
+        const double sa = tab.v[e], sa2 = tab.v[2 * n + e];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            D0[k] = __fma_rn(-ta2, P.e2b[k], __fma_rn(-sa2, P.e1b[k], __fma_rn(ta, P.e2a[k], sa * P.e1a[k])));
+            D1[k] = __fma_rn(tb, P.e2a[k], -tb2 * P.e2b[k]);
+        }
+        hb0 = __fma_rn(ta, P.al2, sa * P.al1);
+        ha0 = __fma_rn(ta2, P.be2, sa2 * P.be1);
+    }
+    hb1 = tb * P.al2;
+    ha1 = tb2 * P.be2;
+    // Laplace: sums with w3 and w3 eta3; Yukawa: with w3 for degrees 0..2, with w3 eta3 for 1, 2
+    double l0[3] = {0, 0, 0}, l1[3] = {0, 0, 0}, y0[3][3], y1[3][2];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        D0[k] = __fma_rn(-ta2, B.e2[k], __fma_rn(-sa2, B.e1[k], __fma_rn(ta, A.e2[k], __fma_rn(sa, A.e1[k], dq[k]))));
-        D1[k] = __fma_rn(tb, A.e2[k], -tb2 * B.e2[k]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) y0[k][c] = 0.0;
+        y1[k][0] = y1[k][1] = 0.0;
     }
-    double a0[NK], a1[NK];
+    const int nss = NSS > 0 ? NSS : rad.n;
+#pragma unroll 1
+    for (int j = 0; j < nss; ++j) {
+        const double x3 = rad.x[j], w3 = rad.w[j];
+        double r2;
+        {
+            const double d0 = __fma_rn(x3, D1[0], D0[0]), d1 = __fma_rn(x3, D1[1], D0[1]),
+                         d2 = __fma_rn(x3, D1[2], D0[2]);
+            r2 = __fma_rn(d2, d2, __fma_rn(d1, d1, d0 * d0));
+        }
+        const double rinv = rsqrt(r2);
+        const double z = kappa * (r2 * rinv);
+        double E[4] = {0, 0, 0, 0};
+        if (deg <= RAD_DEG) {
 #pragma unroll
-    for (int k = 0; k < NK; ++k) a0[k] = a1[k] = 0.0;
-    const int nss = NSS > 0 ? NSS : tab.nss;
+            for (int k = RAD_DEG; k >= 0; --k)
+                if (k <= deg) {
 #pragma unroll
-    for (int j = 0; j < (NSS > 0 ? NSS : 12); ++j) {
-        if (NSS == 0 && j >= nss) break;
-        const double x = x3[j], w = w3[j], wx = w * x;
-        double d[3];
+                    for (int m = 0; m < 4; ++m) E[m] = __fma_rn(E[m], z, rad.c[m][k]);
+                }
+        } else {
+            for (int i = 0; i < nss; ++i) {
+                const double ex = exp_nonpos(-z * rad.x[i]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) d[k] = __fma_rn(x, D1[k], D0[k]);
-        double g[6];
-        adj_kernels<SYM>(d, A, B, kappa, g);
+                for (int m = 0; m < 4; ++m) E[m] = __fma_rn(rad.wx[m][i], ex, E[m]);
+            }
+        }
+        const double wr = w3 * rinv, fl = wr * (rinv * rinv);
+        // (1 + z xi) e^{-z xi}: the double layers' xi sums per degree
+        const double F[3] = {__fma_rn(z, E[1], E[0]), __fma_rn(z, E[2], E[1]), __fma_rn(z, E[3], E[2])};
+        const double g[3] = {wr, fl * __fma_rn(x3, hb1, hb0), fl * __fma_rn(x3, ha1, ha0)};
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            a0[k] = __fma_rn(w, g[k], a0[k]);
-            a1[k] = __fma_rn(wx, g[k], a1[k]);
+        for (int k = 0; k < 3; ++k) {
+            const double gx = g[k] * x3;
+            const double* W = k == 0 ? E + 1 : F;
+            l0[k] += g[k];
+            l1[k] += gx;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) y0[k][c] = __fma_rn(g[k], W[c], y0[k][c]);
+            y1[k][0] = __fma_rn(gx, W[1], y1[k][0]);
+            y1[k][1] = __fma_rn(gx, W[2], y1[k][1]);
         }
     }
-    double c0[9], c1[5];
 #pragma unroll
-    for (int c = 0; c < 9; ++c) c0[c] = tab.v[(6 + c) * n + e];
+    for (int c = 0; c < 9; ++c) {
+        const double c0 = tab.v[(6 + c) * n + e];
+        const int dg = (c >= 3) + (c % 3 > 0);
 #pragma unroll
-    for (int c = 0; c < 5; ++c) c1[c] = tab.v[(15 + c) * n + e];
+        for (int k = 0; k < 3; ++k) {
+            mom[18 * k + c] = __fma_rn(c0, l0[k], mom[18 * k + c]);
+            mom[18 * k + 9 + c] = __fma_rn(c0, y0[k][dg], mom[18 * k + 9 + c]);
+        }
+    }
+    constexpr int slot[5] = {2, 5, 6, 7, 8}, sdeg[5] = {1, 2, 1, 2, 2};
 #pragma unroll
-    for (int k = 0; k < NK; ++k) {
-        double* mk = mom + 9 * k;
+    for (int q = 0; q < 5; ++q) {
+        const double c1 = tab.v[(15 + q) * n + e];
+        const int c = slot[q];
 #pragma unroll
-        for (int c = 0; c < 9; ++c) mk[c] = __fma_rn(c0[c], a0[k], mk[c]);
-        mk[2] = __fma_rn(c1[0], a1[k], mk[2]);
-        mk[5] = __fma_rn(c1[1], a1[k], mk[5]);
-        mk[6] = __fma_rn(c1[2], a1[k], mk[6]);
-        mk[7] = __fma_rn(c1[3], a1[k], mk[7]);
-        mk[8] = __fma_rn(c1[4], a1[k], mk[8]);
+        for (int k = 0; k < 3; ++k) {
+            mom[18 * k + c] = __fma_rn(c1, l1[k], mom[18 * k + c]);
+            mom[18 * k + 9 + c] = __fma_rn(c1, y1[k][sdeg[q] - 1], mom[18 * k + 9 + c]);
+        }
     }
 }
 
@@ -483,16 +511,40 @@ __device__ __forceinline__ void warp_allsum(double* v, int lane, double* buf) {
     __syncwarp();  // the buffer is free again
 }
 
+// Sums of v[0..NV) over the groups of G lanes of a warp: a reduce-scatter over
+// the group's lane bits (N >= NV entries, those past NV being zero), after which lane
+// L of a group holds the totals of entries [L N/G, (L + 1) N/G) in v[0..N/G): N (1 -
+// 1/G) additions a lane, against NV log2(G) for a butterfly on every entry. Fixed
+// order: deterministic.
+template <int NV, int N, int G>
+__device__ __forceinline__ void group_sums(double* v, int lane) {
+    static_assert(N % G == 0 && NV <= N && 2 * NV >= N && (G == 4 || G == 8 || G == 32), "reduce-scatter size");
+    {
+        constexpr int h = N / 2;
+        const bool up = lane & (G / 2);
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double lo = v[i], hi = i + h < NV ? v[i + h] : 0.0;
+            v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, G / 2);
+        }
+    }
+    rs_level<N / 4>(v, lane, G / 4);
+    if (G >= 8) rs_level<N / 8>(v, lane, G / 8);
+    if (G >= 32) {
+        rs_level<N / 16>(v, lane, 2);
+        rs_level<N / 32>(v, lane, 1);
+    }
+}
 
 // Six 3x3 blocks (V_L, K_L, D_L, V_Y, K_Y, D_Y) of the pair (tau, sigma), or with
 // rev = true of the reversed pair (sigma, tau): every block transposed and the
 // double layer taken from the KT accumulators. Layout: out[6 (3a + b) + k] for
 // corner a of the test triangle, corner b of the trial one and operator k, so
 // that the six values one row-assembly lane reads are 48 contiguous bytes.
-__device__ void expand_blocks(const double* acc, const TriFrame& A, const TriFrame& B, const double* tgeoA,
-                              const double* tgeoB, double kappa, bool rev, double* out) {
-    double nn = A.n[0] * B.n[0] + A.n[1] * B.n[1] + A.n[2] * B.n[2];
-    double f = 1.0 / (4.0 * A.area * B.area);
+__device__ __forceinline__ void expand_blocks(const double* acc, const double* tgeoA, const double* tgeoB, double kappa,
+                                              bool rev, double* out) {
+    const double nn = tgeoA[0] * tgeoB[0] + tgeoA[1] * tgeoB[1] + tgeoA[2] * tgeoB[2];
+    const double f = 1.0 / (4.0 * tgeoA[3] * tgeoB[3]);
     const int kL = rev ? 38 : 18, kY = rev ? 47 : 27;
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) {
@@ -513,98 +565,153 @@ __device__ void expand_blocks(const double* acc, const TriFrame& A, const TriFra
 
 constexpr int NEAR_THREADS = 128;
 
-// FP64 flops per quadrature point pair by formula count (a fused multiply-add
-// counted as two). NEAR_FLOPS_SYM: one point pair with all six kernels and a
-// direct accumulation into the 3x3 blocks (the far-rule pairs of an adjacent
-// pair, accum_point). Kernel evaluation: d = x - y (24 when formed from frame
-// vectors); r^2 (5), rsqrt, r, 1/(4 pi r), kappa r, exp, the Yukawa single
-// layer (6), 1/r^3 (2), (1 + kappa r) and the Yukawa double-layer factor (3),
-// d.n_y (5) and both double layers (2): 47; with the reversed pair's double
-// layer, d.n_x (5) and its two kernels (2): 54. Accumulation: one FMA per
-// kernel and block entry, 2 x 6 x 9 (108). Coincident pairs (moments from the
-// rule's table of weighted monomials): d from (s - s', t - t') (11), r^2 to
-// the Yukawa single layer (11); 2 x 2 x 9 (36).
-constexpr double NEAR_FLOPS_SYM = 54 + 108;
+// FP64 flops by formula count (a fused multiply-add counted as two). An adjacent
+// pair's (eta1, eta2, eta3) point (k_adj_pairs): d and r^2 (6 FMA), rsqrt, r, z (3),
+// the four E_m at degree 10 (40 FMA), w rinv, w/r^3 (3), F (3 FMA), the heights and
+// kernels (2 FMA, 2), eta3 products (3), sums (6 + 15 FMA): 155; an entry: D0, D1 and
+// the heights (17 FMA, 7), the moments (6 x 14 FMA): 209. A coincident pair's point
+// (moments from the rule's table of weighted monomials): d from (s - s', t - t') (11),
+// r^2 to the Yukawa single layer (11), 2 x 2 x 9 (36).
+constexpr double NEAR_FLOPS_ADJ_POINT = 155;
+constexpr double NEAR_FLOPS_ADJ_ENTRY = 209;
 constexpr double NEAR_FLOPS_COIN = 22 + 36;
-// The factorised adjacent-pair sums (accum_outer): per quadrature point pair
-// the kernel evaluation with d = D0 + eta3 D1 (3 FMA instead of 12: 36) and the
-// two partial sums per kernel (2 x 6 FMA: 24); per outer entry D0 and D1
-// (12 FMA, 3 FMA and 3 products: 33) and the moments (6 kernels x 14 FMA: 168).
-constexpr double NEAR_FLOPS_ADJ_POINT = 36 + 24;
-constexpr double NEAR_FLOPS_ADJ_OUTER = 33 + 168;
 
-// One warp per listed pair. Writes ss[p][54] (regularised) and far[p][54] (far
-// rule, identical points excluded); with SYM also the blocks of the reversed
-// pair rev[p], whose rule is this one with the roles exchanged.
-template <int MINB, bool SYM, int NSS>
-__global__ void __launch_bounds__(NEAR_THREADS, MINB)
-k_near_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
-             const int4* __restrict__ pairs, const int32_t* __restrict__ list, int64_t nlist,
-             const int32_t* __restrict__ rev, SSOuter tab, Rule rule, double kappa,
-             double* __restrict__ ss_out, double* __restrict__ far_out) {
-    constexpr int NA = SYM ? NACC_SYM : NACC_NEAR;
-    constexpr int NM = SYM ? 54 : 36;  // frame moments
-    __shared__ TriFrame frames[NEAR_THREADS / 32][2];
-    __shared__ double red[NEAR_THREADS / 32][64];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t li = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (li >= nlist) return;  // whole warps leave together
-    const int64_t p = list[li];
+// Regularised blocks of the adjacent pairs of one class: G lanes per listed pair
+// (one of each two reversed ones) over the entries of the class's map, their
+// moments summed over the group by a reduce-scatter, turned into corner blocks in
+// shared memory by the group's lanes (a kernel each) and written for the pair and
+// for its reverse rev[p] (V and D transposed, K from the K^T moments).
+// Bound by the FP64 pipe (a warp instruction every 16 cycles of an SM). One xi
+// evaluation instead of n (the Laplace kernels' xi sums are constants, the Yukawa
+// kernels' polynomials of z) takes an (eta1, eta2, eta3) point from 4 x 59
+// instructions to about 95 at n = 4; small groups keep the per-pair work (sums over
+// lanes, corner blocks) to a few per cent: 8 lanes hold 12 of an edge pair's 96
+// entries each, 4 lanes 8 of a vertex pair's 32; G = 32 for few pairs (adj_group).
+// 38,720 triangles, n = 4: edge and vertex launches 34.0 -> 10.05 ms (with the far
+// rule in both); 2,000 triangles 1.91 -> 0.58 ms.
+template <int NSS, int G>
+__global__ void __launch_bounds__(NEAR_THREADS, 2)
+k_adj_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
+            const int4* __restrict__ pairs, const int32_t* __restrict__ list, int64_t nlist,
+            const int32_t* __restrict__ rev, SSOuter tab, const __grid_constant__ Radial rad, double kappa,
+            double* __restrict__ ss_out) {
+    constexpr int N = G == 32 ? 64 : 56, K = N / G;  // moments after padding, and of one lane after the reduction
+    struct Shared {
+        AdjGeo geo;
+        double mom[N];  // moments, then the corner blocks 9 k + 3 a + b
+        double cc[9];   // curl products of the corners
+        double sum[2];  // sums of w G_L and w G_Y
+        int inv[2][3];  // frame index of original corner a
+    };
+    __shared__ Shared sh[NEAR_THREADS / G];
+    const int lane = threadIdx.x & 31, gl = threadIdx.x % G;
+    const int64_t li = (blockIdx.x * (int64_t)NEAR_THREADS + threadIdx.x) / G;
+    const bool live = li < nlist;  // the last block's spare groups repeat the last pair and write nothing
+    const int64_t p = list[live ? li : nlist - 1];
     const int4 pr = pairs[p];
-    TriFrame& A = frames[wid][0];
-    TriFrame& B = frames[wid][1];
-    if (lane == 0) make_frame(verts, tris, tgeo, pr.x, pr.w & 63, A);
-    if (lane == 1) make_frame(verts, tris, tgeo, pr.y, (pr.w >> 6) & 63, B);
-    __syncwarp();
-    const int nreg = tab.nreg;  // every pair of the list has the table's class
-    const int e0 = 0;
-    const int n3 = tab.nss * tab.nss * tab.nss;
-    const double jac_ab = (2.0 * A.area) * (2.0 * B.area);
-    const double dq[3] = {A.q0[0] - B.q0[0], A.q0[1] - B.q0[1], A.q0[2] - B.q0[2]};  // 0: the shared vertex
-    // the eta3 rule, in registers for a fixed size
-    double x3[NSS > 0 ? NSS : 1], w3[NSS > 0 ? NSS : 1];
-    const double* rule3 = tab.v + (size_t)SS_OUTER_ARRAYS * tab.n;
-    if (NSS > 0) {
-#pragma unroll
-        for (int j = 0; j < (NSS > 0 ? NSS : 1); ++j) {
-            x3[j] = rule3[j];
-            w3[j] = rule3[tab.nss + j];
-        }
-    }
-    double acc[NA];
-    {
-        double mom[NM];
-        for (int k = 0; k < NM; ++k) mom[k] = 0.0;
-        for (int idx = lane; idx < nreg * n3; idx += 32)
-            accum_outer<SYM, NSS>(mom, tab, e0 + idx, dq, A, B, kappa, NSS > 0 ? x3 : rule3,
-                                  NSS > 0 ? w3 : rule3 + tab.nss);
-        warp_allsum<NM, 64>(mom, lane, red[wid]);
-        for (int k = 0; k < NM; ++k) mom[k] *= jac_ab;  // the pair's Jacobian, once
-        // corner blocks in the accumulator layout of accum_point
-        for (int k = 0; k < NM / 9; ++k) frame_to_corner(mom + 9 * k, A, B, acc + (k < 4 ? 9 * k : 38 + 9 * (k - 4)));
-        acc[36] = mom[0];  // sum w G_L: the (1, 1) moment
-        acc[37] = mom[9];
-    }
+    Shared& S = sh[threadIdx.x / G];
     const double* gA = tgeo + 16 * (int64_t)pr.x;
     const double* gB = tgeo + 16 * (int64_t)pr.y;
-    if (lane == 0) expand_blocks(acc, A, B, gA, gB, kappa, false, ss_out + 54 * p);
-    if (SYM && lane == 1) expand_blocks(acc, A, B, gA, gB, kappa, true, ss_out + 54 * (int64_t)rev[p]);
-    // far rule on the same pair (what the pair kernel adds for it)
-    for (int k = 0; k < NA; ++k) acc[k] = 0.0;
-    const int Q = rule.Q;
-    for (int idx = lane; idx < Q * Q; idx += 32) {
-        const int i = idx / Q, j = idx % Q;
-        double x[3], y[3];
-        for (int k = 0; k < 3; ++k) {
-            x[k] = rule.l[i][0] * corner(A, 0, k) + rule.l[i][1] * corner(A, 1, k) + rule.l[i][2] * corner(A, 2, k);
-            y[k] = rule.l[j][0] * corner(B, 0, k) + rule.l[j][1] * corner(B, 1, k) + rule.l[j][2] * corner(B, 2, k);
+    const double areaA = gA[3], areaB = gB[3];
+    if (gl < 3) {  // component gl of the frames' edges
+        const int k = gl;
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const int perm = pr.w >> (6 * f);
+            const int32_t* t = tris + 3 * (int64_t)(f ? pr.y : pr.x);
+            const double q0 = verts[3 * (int64_t)t[perm & 3] + k], q1 = verts[3 * (int64_t)t[(perm >> 2) & 3] + k],
+                         q2 = verts[3 * (int64_t)t[(perm >> 4) & 3] + k];
+            (f ? S.geo.e1b : S.geo.e1a)[k] = q1 - q0;
+            (f ? S.geo.e2b : S.geo.e2a)[k] = q2 - q1;
+            S.inv[f][(perm >> (2 * k)) & 3] = k;
         }
-        const double w = rule.w[i] * A.area * rule.w[j] * B.area;
-        accum_point<SYM>(acc, w, x, y, A.n, B.n, rule.l[i], rule.l[j], kappa);
     }
-    warp_allsum<NA, 64>(acc, lane, red[wid]);
-    if (lane == 0) expand_blocks(acc, A, B, gA, gB, kappa, false, far_out + 54 * p);
-    if (SYM && lane == 1) expand_blocks(acc, A, B, gA, gB, kappa, true, far_out + 54 * (int64_t)rev[p]);
+    __syncwarp();
+    if (gl < 4) {  // heights of the edges' ends over the other triangle's plane (a shared edge lies in both)
+        const double* e = gl == 0 ? S.geo.e1a : gl == 1 ? S.geo.e2a : gl == 2 ? S.geo.e1b : S.geo.e2b;
+        const double* n = gl < 2 ? gB : gA;
+        double h = e[0] * n[0] + e[1] * n[1] + e[2] * n[2];
+        if (pr.z == 1 && (gl & 1) == 0) h = 0.0;
+        (&S.geo.al1)[gl] = h;
+    }
+    const double fc = 1.0 / (4.0 * areaA * areaB);
+    for (int ab = gl; ab < 9; ab += G) {
+        const double *ea = gA + 4 + 3 * (ab / 3), *eb = gB + 4 + 3 * (ab % 3);
+        S.cc[ab] = fc * (ea[0] * eb[0] + ea[1] * eb[1] + ea[2] * eb[2]);
+    }
+    __syncwarp();
+    int deg = RAD_DEG + 1;
+    {   // |x - y| at xi = 1 is at most the sum of the triangles' longest distances from the shared vertex
+        float z = 0.f;
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const double *e1 = f ? S.geo.e1b : S.geo.e1a, *e2 = f ? S.geo.e2b : S.geo.e2a;
+            float u = 0.f, v = 0.f;
+            for (int k = 0; k < 3; ++k) {
+                const float c1 = (float)e1[k], c2 = (float)(e1[k] + e2[k]);
+                u = fmaf(c1, c1, u);
+                v = fmaf(c2, c2, v);
+            }
+            z += sqrtf(fmaxf(u, v));
+        }
+        z *= 1.0001f * (float)kappa;
+        for (int d = RAD_DEG; d >= 0; --d)
+            if (z <= rad.zlim[d]) deg = d;
+    }
+    deg = __reduce_max_sync(0xffffffffu, deg);
+    double mom[54];
+#pragma unroll
+    for (int k = 0; k < 54; ++k) mom[k] = 0.0;
+    for (int e = gl; e < tab.n; e += G) accum_entry<NSS>(mom, tab, rad, e, S.geo, kappa, deg);
+    __syncwarp();
+    group_sums<54, N, G>(mom, lane);
+#pragma unroll
+    for (int j = 0; j < K; ++j) S.mom[gl * K + j] = mom[j];
+    __syncwarp();
+    // the pair's Jacobian, 1/(4 pi) and the Laplace kernels' xi sums; frame moments -> corner blocks
+    const double scale = (2.0 * areaA) * (2.0 * areaB) * 0.07957747154594767;
+    for (int k = gl; k < 6; k += G) {
+        double m[9], R[3][3], U[3][3];
+        const int m0 = k == 0 ? 1 : 0;  // mu index of degree 0: G_L mu_2, K_L and K^T_L mu_1
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            const int dg = (c >= 3) + (c % 3 > 0);
+            m[c] = S.mom[9 * k + c] * (k & 1 ? scale : scale * rad.mu[m0 + dg]);
+        }
+        if (k < 2) S.sum[k] = m[0];  // the (1, 1) moment
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {  // mu_0 = 1 - s, mu_1 = s - t, mu_2 = t on the first frame
+            R[0][b] = m[b] - m[3 + b];
+            R[1][b] = m[3 + b] - m[6 + b];
+            R[2][b] = m[6 + b];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {  // and on the second
+            U[a][0] = R[a][0] - R[a][1];
+            U[a][1] = R[a][1] - R[a][2];
+            U[a][2] = R[a][2];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) S.mom[9 * k + 3 * a + b] = U[a][b];
+    }
+    __syncwarp();
+    if (!live) return;
+    const double knn = kappa * kappa * (gA[0] * gB[0] + gA[1] * gB[1] + gA[2] * gB[2]);
+    const int64_t pv = rev[p];
+    for (int idx = gl; idx < 108; idx += G) {
+        const bool r = idx >= 54;
+        const int i = r ? idx - 54 : idx, o = i / 6, k = i - 6 * o;
+        const int a = r ? o % 3 : o / 3, b = r ? o / 3 : o % 3;  // corners of the first and the second triangle
+        const int at = 3 * S.inv[0][a] + S.inv[1][b];
+        // kernels 0..5: G_L, G_Y, K_L, K_Y, K^T_L, K^T_Y; values V_L, K_L, D_L, V_Y, K_Y, D_Y
+        const int blk = (k >= 3) + (k % 3 == 1 ? (r ? 4 : 2) : 0);
+        double v = S.mom[9 * blk + at];
+        if (k == 2) v = S.cc[3 * a + b] * S.sum[0];
+        if (k == 5) v = __fma_rn(S.cc[3 * a + b], S.sum[1], knn * v);
+        ss_out[54 * (r ? pv : p) + i] = v;
+    }
 }
 
 // Coincident pairs (tau, tau). The double layer vanishes (x - y lies in the
@@ -713,6 +820,7 @@ k_coin_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
 // the single-layer blocks, the basis functions summing to one at every point.
 // The y points of both rules are staged in shared memory, per thread.
 constexpr int BAND_THREADS = 128;
+constexpr int ADJ_FAR_THREADS = 64;
 
 // FP64 flops of one band pair under a Q-point rule by formula count: per point
 // pair the kernel evaluation (33, as for the regularised pairs) and the partial
@@ -720,7 +828,7 @@ constexpr int BAND_THREADS = 128;
 // its weights (4) and the block updates (54 FMA).
 __host__ __device__ constexpr double band_flops(int Q) { return Q * Q * (33.0 + 36.0) + Q * (30.0 + 4.0 + 108.0); }
 
-template <int Q>
+template <int Q, int NT>
 __device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3], const double* ys,
                                           const double (*wl)[3], const Rule& R, double wscale, const double* na,
                                           const double* nb, double kappa) {
@@ -734,8 +842,8 @@ __device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3],
         for (int k = 0; k < 6; ++k) u[k][0] = u[k][1] = u[k][2] = 0.0;
 #pragma unroll 1
         for (int j = 0; j < Q; ++j) {
-            const double d0 = x[0] - ys[(3 * j) * BAND_THREADS], d1 = x[1] - ys[(3 * j + 1) * BAND_THREADS],
-                         d2 = x[2] - ys[(3 * j + 2) * BAND_THREADS];
+            const double d0 = x[0] - ys[(3 * j) * NT], d1 = x[1] - ys[(3 * j + 1) * NT],
+                         d2 = x[2] - ys[(3 * j + 2) * NT];
             const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
             const double rinv = rsqrt(r2);
             const double r = r2 * rinv;
@@ -764,6 +872,22 @@ __device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3],
             }
         }
     }
+}
+
+// the pair's blocks and its reverse's from the accumulators, the sums of w G_L and
+// w G_Y following from the single-layer blocks
+__device__ __forceinline__ void write_blocks(double* acc, const double* gA, const double* gB, double kappa,
+                                             double* out, double* out_rev) {
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        s0 += acc[k];
+        s1 += acc[9 + k];
+    }
+    acc[36] = s0;
+    acc[37] = s1;
+    expand_blocks(acc, gA, gB, kappa, false, out);
+    expand_blocks(acc, gA, gB, kappa, true, out_rev);
 }
 
 template <int QF, int QC>
@@ -823,25 +947,50 @@ k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
 #pragma unroll
     for (int k = 0; k < NACC_SYM; ++k) acc[k] = 0.0;
     const double area2 = gA[3] * gB[3];
-    band_pass<QF>(acc, pa, ysm + threadIdx.x, wl[0], fine, area2, na, nb, kappa);
-    band_pass<QC>(acc, pa, ysm + threadIdx.x + 3 * QF * BAND_THREADS, wl[1], coarse, -area2, na, nb, kappa);
-    double s0 = 0.0, s1 = 0.0;  // sums of w G_L and w G_Y over the pair
+    band_pass<QF, BAND_THREADS>(acc, pa, ysm + threadIdx.x, wl[0], fine, area2, na, nb, kappa);
+    band_pass<QC, BAND_THREADS>(acc, pa, ysm + threadIdx.x + 3 * QF * BAND_THREADS, wl[1], coarse, -area2, na, nb, kappa);
+    write_blocks(acc, gA, gB, kappa, ss_out + 54 * p, ss_out + 54 * pr_rev);
+}
+
+// The far rule's blocks of the adjacent pairs (what the pair kernel adds for them):
+// one thread per pair and its reverse, by the band pairs' sums. (As a lane's share of
+// a warp per pair, 9 or 36 point pairs left most lanes idle: 260 FP64 instructions of
+// a warp per pair, against 25 or 85 here. 3-point rule, 38,720 triangles: 0.44 ms.)
+template <int Q>
+__global__ void __launch_bounds__(ADJ_FAR_THREADS)
+k_adj_far(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
+          const int4* __restrict__ pairs, const int32_t* __restrict__ list, int64_t nlist,
+          const int32_t* __restrict__ rev, Rule rule, double kappa, double* __restrict__ far_out) {
+    __shared__ double ysm[Q * 3 * ADJ_FAR_THREADS];
+    __shared__ double wl[6][3];  // w_j l_b(y_j)
+    if (threadIdx.x < 3 * Q) wl[threadIdx.x / 3][threadIdx.x % 3] = rule.w[threadIdx.x / 3] * rule.l[threadIdx.x / 3][threadIdx.x % 3];
+    __syncthreads();
+    const int64_t li = blockIdx.x * (int64_t)ADJ_FAR_THREADS + threadIdx.x;
+    if (li >= nlist) return;  // no barrier follows
+    const int64_t p = list[li];
+    const int4 pr = pairs[p];
+    double pa[3][3], pb[3][3];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        s0 += acc[k];
-        s1 += acc[9 + k];
-    }
-    acc[36] = s0;
-    acc[37] = s1;
-    TriFrame A, B;  // expand_blocks reads the normals and areas only
-    for (int k = 0; k < 3; ++k) {
-        A.n[k] = na[k];
-        B.n[k] = nb[k];
-    }
-    A.area = gA[3];
-    B.area = gB[3];
-    expand_blocks(acc, A, B, gA, gB, kappa, false, ss_out + 54 * p);
-    expand_blocks(acc, A, B, gA, gB, kappa, true, ss_out + 54 * pr_rev);
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            pa[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)pr.x + a] + k];
+            pb[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)pr.y + a] + k];
+        }
+#pragma unroll
+    for (int j = 0; j < Q; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            ysm[(3 * j + k) * ADJ_FAR_THREADS + threadIdx.x] =
+                rule.l[j][0] * pb[0][k] + rule.l[j][1] * pb[1][k] + rule.l[j][2] * pb[2][k];
+    const double* gA = tgeo + 16 * (int64_t)pr.x;
+    const double* gB = tgeo + 16 * (int64_t)pr.y;
+    const double na[3] = {gA[0], gA[1], gA[2]}, nb[3] = {gB[0], gB[1], gB[2]};
+    double acc[NACC_SYM];
+#pragma unroll
+    for (int k = 0; k < NACC_SYM; ++k) acc[k] = 0.0;
+    band_pass<Q, ADJ_FAR_THREADS>(acc, pa, ysm + threadIdx.x, wl, rule, gA[3] * gB[3], na, nb, kappa);
+    write_blocks(acc, gA, gB, kappa, far_out + 54 * p, far_out + 54 * (int64_t)rev[p]);
 }
 
 // One warp per row i. The warp walks the contributions of the row in a fixed
@@ -996,6 +1145,36 @@ static void free_near(pb_near* nf) {
     nf->mrow_ptr = nullptr;
 }
 
+// Lanes per adjacent pair: 8 for edge pairs and 4 for vertex pairs, or a whole warp for
+// few pairs, where small groups leave the last of one or two waves of CTAs nearly empty
+// and a pair's entries in sequence set the time. Edge and vertex launches together, us,
+// small groups | whole warps, by triangles: 320: 385 | 142, 1,280: 523 | 459, 2,000: 721 |
+// 628 (582 with whole warps for the edge pairs alone), 5,120: 1,558 | 1,574 (1,449),
+// 8,000: 2,192 | 2,436. Lines: 16 warps per SM for edge pairs, 6 for vertex pairs.
+static int adj_group(int64_t nlist, int cls, int num_sms) {
+    const int g = cls == 0 ? 8 : 4, warps_per_sm = cls == 0 ? 16 : 6;
+    return nlist * g < (int64_t)32 * warps_per_sm * num_sms ? 32 : g;
+}
+
+template <int G>
+static void launch_adj_g(const pb_mesh* m, const int32_t* list, int64_t nlist, const SSOuter& ot, const Radial& rad,
+                         double kappa, double* ss, cudaStream_t s) {
+    const unsigned b = (unsigned)((nlist * G + NEAR_THREADS - 1) / NEAR_THREADS);
+    if (ot.nss == 4)
+        k_adj_pairs<4, G><<<b, NEAR_THREADS, 0, s>>>(m->verts, m->tris, m->tgeo, m->pairs, list, nlist, m->pair_rev, ot,
+                                                     rad, kappa, ss);
+    else
+        k_adj_pairs<0, G><<<b, NEAR_THREADS, 0, s>>>(m->verts, m->tris, m->tgeo, m->pairs, list, nlist, m->pair_rev, ot,
+                                                     rad, kappa, ss);
+}
+
+static void launch_adj(int group, const pb_mesh* m, const int32_t* list, int64_t nlist, const SSOuter& ot,
+                       const Radial& rad, double kappa, double* ss, cudaStream_t s) {
+    if (group == 32) launch_adj_g<32>(m, list, nlist, ot, rad, kappa, ss, s);
+    else if (group == 8) launch_adj_g<8>(m, list, nlist, ot, rad, kappa, ss, s);
+    else launch_adj_g<4>(m, list, nlist, ot, rad, kappa, ss, s);
+}
+
 static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaStream_t s) {
     nf->mesh = m;
     nf->kappa = kappa;
@@ -1010,10 +1189,10 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         const Gauss gq = gauss01(nc);
         const int n4i = nc * nc * nc * nc, ntab = 3 * n4i;
         // edge and vertex pairs: the outer entries of their maps, each with its own rule
-        const int nout_e = 6 * ne * ne * ne, nout_v = 2 * nvx * nvx * nvx;
+        const int nout_e = 6 * ne * ne, nout_v = 2 * nvx * nvx;
         const size_t bt = sizeof(double) * SS_TABLE_ARRAYS * ntab;
-        const size_t be = sizeof(double) * ((size_t)SS_OUTER_ARRAYS * nout_e + 2 * ne);
-        const size_t bv = sizeof(double) * ((size_t)SS_OUTER_ARRAYS * nout_v + 2 * nvx);
+        const size_t be = sizeof(double) * (size_t)SS_OUTER_ARRAYS * nout_e;
+        const size_t bv = sizeof(double) * (size_t)SS_OUTER_ARRAYS * nout_v;
         double* tabm = nullptr;
         rc = dev_alloc((void**)&tabm, bt + be + bv);
         if (rc != PB_OK) {
@@ -1024,8 +1203,9 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         double* tabe = tabm + bt / sizeof(double);
         double* tabv = tabe + be / sizeof(double);
         k_ss_table<<<(ntab + 127) / 128, 128, 0, s>>>(gq, ntab, tabm);
-        k_ss_outer<<<(std::max(nout_e, 2 * ne) + 127) / 128, 128, 0, s>>>(gauss01(ne), 1, nout_e, tabe);
-        k_ss_outer<<<(std::max(nout_v, 2 * nvx) + 127) / 128, 128, 0, s>>>(gauss01(nvx), 2, nout_v, tabv);
+        const Gauss gauss_e = gauss01(ne), gauss_v = gauss01(nvx);
+        k_ss_outer<<<(nout_e + 127) / 128, 128, 0, s>>>(gauss_e, 1, nout_e, tabe);
+        k_ss_outer<<<(nout_v + 127) / 128, 128, 0, s>>>(gauss_v, 2, nout_v, tabv);
         ::pb::count_launch(3);
         SSTable tab = {tabm, tabm + ntab, tabm + 2 * ntab, tabm + 3 * ntab, tabm + 4 * ntab, tabm + 5 * ntab, ntab};
         const SSOuter outer_e = {tabe, nout_e, ne, 6}, outer_v = {tabv, nout_v, nvx, 2};
@@ -1048,18 +1228,25 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
             if (nlist == 0) continue;
             const int32_t* list = m->pair_prim + (cls == 0 ? 0 : m->n_prim_edge);
             const SSOuter& ot = cls == 0 ? outer_e : outer_v;
-            const unsigned bp = (unsigned)((nlist * 32 + threads - 1) / threads);
-            const double outer_pts = (double)nlist * ot.n;
-            const double reg = outer_pts * ot.nss, farp = (double)nlist * Q * Q;
-            const double flops = reg * NEAR_FLOPS_ADJ_POINT + outer_pts * NEAR_FLOPS_ADJ_OUTER + farp * NEAR_FLOPS_SYM;
-            Timer tm(ctx, PB_KERNEL_NEAR_ADJ, s, reg + farp, flops / (reg + farp));
-#define PB_NEAR_ARGS m->verts, m->tris, m->tgeo, m->pairs, list, nlist, m->pair_rev, ot, mesh_rule(m), kappa, ss, far
-            if (ot.nss == 4) k_near_pairs<2, true, 4><<<bp, threads, 0, s>>>(PB_NEAR_ARGS);
-            else if (ot.nss == 3) k_near_pairs<2, true, 3><<<bp, threads, 0, s>>>(PB_NEAR_ARGS);
-            else k_near_pairs<2, true, 0><<<bp, threads, 0, s>>>(PB_NEAR_ARGS);
-#undef PB_NEAR_ARGS
+            const Radial rad = make_radial(cls == 0 ? gauss_e : gauss_v);
+            const double entries = (double)nlist * ot.n, points = entries * ot.nss;
+            {
+                Timer tm(ctx, PB_KERNEL_NEAR_ADJ, s, points,
+                         (points * NEAR_FLOPS_ADJ_POINT + entries * NEAR_FLOPS_ADJ_ENTRY) / points);
+                launch_adj(adj_group(nlist, cls, ctx->num_sms), m, list, nlist, ot, rad, kappa, ss, s);
+                ::pb::count_launch();
+                tm.stop();
+            }
+        }
+        if (m->n_prim) {
+            const Rule rule = mesh_rule(m);
+            const unsigned gf = (unsigned)((m->n_prim + ADJ_FAR_THREADS - 1) / ADJ_FAR_THREADS);
+#define PB_FAR_ARGS m->verts, m->tris, m->tgeo, m->pairs, m->pair_prim, m->n_prim, m->pair_rev, rule, kappa, far
+            if (m->Q == 6) k_adj_far<6><<<gf, ADJ_FAR_THREADS, 0, s>>>(PB_FAR_ARGS);
+            else if (m->Q == 3) k_adj_far<3><<<gf, ADJ_FAR_THREADS, 0, s>>>(PB_FAR_ARGS);
+            else k_adj_far<1><<<gf, ADJ_FAR_THREADS, 0, s>>>(PB_FAR_ARGS);
+#undef PB_FAR_ARGS
             ::pb::count_launch();
-            tm.stop();
         }
         if (m->n_band) {
             Rule fine = mesh_ref_rule(m), coarse = mesh_rule(m);

@@ -1,0 +1,51 @@
+"""Near field of adjacent pairs against the oracle over what selects its code path: the lanes per pair (few or many
+pairs), the degree of the Yukawa polynomials (kappa times the triangles' size, past their range the exponentials), the
+singular order and the far rule. One FP64 application per operator; tolerance as the operator parity tests (1e-12)."""
+import numpy as np
+import pytest
+
+import oracle
+from .gpu_common import OPS, rel
+from oracle import oracle as O
+from synth import icosphere
+from synth.icosphere import uv_ellipsoid
+
+pytestmark = pytest.mark.gpu
+
+
+def check(v, t, kappa, plan):
+    import torch
+
+    import paper_2108_10481_gb300 as pb
+    ref = oracle.assemble(v, t, kappa, O.Plan(**plan))
+    ctx = pb.pb_init(0)
+    m = pb.pb_mesh_load(ctx, v, t, **plan)
+    nf = pb.pb_near_build(ctx, m, kappa)
+    x = np.random.default_rng(5).standard_normal(v.shape[0])
+    dx = torch.as_tensor(x, device="cuda")
+    for name in ("VL", "KL", "DL", "VY", "KY", "TY", "DY"):
+        op, kern = OPS[name]
+        y = pb.pb_op_apply(ctx, m, nf, op, kern, pb.PB_F64, dx).cpu().numpy()
+        assert rel(y, getattr(ref, name) @ x) < 1e-12, (name, kappa, plan)
+    nf.free()
+    m.free()
+
+
+@pytest.mark.parametrize("kappa", [0.0, 0.01, 0.125, 0.3, 2.0])
+def test_yukawa_sums_at_every_degree(kappa):
+    v, t = icosphere(2, 2.0)
+    check(v, t, kappa, {"far_q": 6, "n_ss": 4})
+
+
+@pytest.mark.parametrize("plan", [{"far_q": 3, "n_ss": 3}, {"far_q": 1, "n_ss": 2}, {"far_q": 6, "n_ss": 5},
+                                  {"far_q": 3, "n_ss": 4, "n_ss_coin": 1, "n_ss_edge": 3, "n_ss_vert": 6}])
+def test_orders_and_far_rules(plan):
+    v, t = uv_ellipsoid(9, 8, (2.0, 1.6, 1.3), center=(0.3, -0.2, 0.1), twist=0.15)
+    check(v, t, 0.125, plan)
+
+
+@pytest.mark.parametrize("n_lon,n_lat,length", [(31, 29, 2.3), (20, 190, 14.0)])
+def test_many_pairs(n_lon, n_lat, length):
+    """1,736 triangles (4 lanes per vertex pair, a warp per edge pair) and 7,560 (4 and 8 lanes)."""
+    v, t = uv_ellipsoid(n_lon, n_lat, (1.5, 1.4, length), twist=0.05)
+    check(v, t, 0.125, {"far_q": 3, "n_ss": 4})

@@ -37,45 +37,63 @@ constexpr int REC32 = 16;  // floats per FP32 source record
 constexpr double INV4PI = 0.07957747154594767;  // 1 / (4 pi)
 
 // ------------------------------------------------------------ sources (a4 i)
+// One thread per point (a triangle's coefficients and curl are formed by each of its
+// points' threads: the kernel is a few microseconds of launch and dependent loads; with
+// a thread per triangle and its points in sequence it took 12 us at any size below 10,000
+// triangles, now 5.)
+struct SourceValues {
+    double s, p[3], c[3];
+};
+__device__ __forceinline__ SourceValues source_values(int64_t i, int Q, const Rule& rule,
+                                                      const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
+                                                      const double* __restrict__ pts64, const double* __restrict__ u,
+                                                      const double* __restrict__ v, int need_u, int need_v) {
+    const int64_t t = i / Q;
+    const int q = (int)(i - t * Q);
+    const double* g = tgeo + 16 * t;
+    const int32_t i0 = tris[3 * t], i1 = tris[3 * t + 1], i2 = tris[3 * t + 2];
+    double ua[3] = {0, 0, 0}, va[3] = {0, 0, 0};
+    if (need_u) { ua[0] = u[i0]; ua[1] = u[i1]; ua[2] = u[i2]; }
+    if (need_v) { va[0] = v[i0]; va[1] = v[i1]; va[2] = v[i2]; }
+    const double inv2a = -1.0 / (2.0 * g[3]);
+    const double w = pts64[4 * i + 3] * INV4PI;
+    const double uq = rule.l[q][0] * ua[0] + rule.l[q][1] * ua[1] + rule.l[q][2] * ua[2];
+    const double vq = rule.l[q][0] * va[0] + rule.l[q][1] * va[1] + rule.l[q][2] * va[2];
+    SourceValues r;
+    r.s = w * vq;
+    for (int k = 0; k < 3; ++k) {
+        r.p[k] = w * uq * g[k];
+        r.c[k] = w * (inv2a * (ua[0] * g[4 + k] + ua[1] * g[7 + k] + ua[2] * g[10 + k]));
+    }
+    return r;
+}
+
 template <typename T, int REC>
-__global__ void k_sources(int64_t nt, int Q, Rule rule, const int32_t* __restrict__ tris,
+__global__ void k_sources(int64_t np, int Q, Rule rule, const int32_t* __restrict__ tris,
                           const double* __restrict__ tgeo, const double* __restrict__ pts64,
                           const float* __restrict__ pts32, const float* __restrict__ pts32lo,
                           const double* __restrict__ u, const double* __restrict__ v, int need_u,
                           int need_v, T* __restrict__ rec) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nt) return;
-    const double* g = tgeo + 16 * t;
-    int32_t i0 = tris[3 * t], i1 = tris[3 * t + 1], i2 = tris[3 * t + 2];
-    double ua[3] = {0, 0, 0}, va[3] = {0, 0, 0};
-    if (need_u) { ua[0] = u[i0]; ua[1] = u[i1]; ua[2] = u[i2]; }
-    if (need_v) { va[0] = v[i0]; va[1] = v[i1]; va[2] = v[i2]; }
-    double inv2a = -1.0 / (2.0 * g[3]);
-    double cu[3];
-    for (int k = 0; k < 3; ++k) cu[k] = inv2a * (ua[0] * g[4 + k] + ua[1] * g[7 + k] + ua[2] * g[10 + k]);
-    for (int q = 0; q < Q; ++q) {
-        int64_t i = t * Q + q;
-        double w = pts64[4 * i + 3] * INV4PI;
-        double uq = rule.l[q][0] * ua[0] + rule.l[q][1] * ua[1] + rule.l[q][2] * ua[2];
-        double vq = rule.l[q][0] * va[0] + rule.l[q][1] * va[1] + rule.l[q][2] * va[2];
-        T* r = rec + REC * i;
-        if (REC == REC64) {
-            for (int k = 0; k < 3; ++k) r[k] = (T)pts64[4 * i + k];
-        } else {
-            for (int k = 0; k < 3; ++k) {
-                r[k] = (T)pts32[4 * i + k];
-                r[12 + k] = (T)pts32lo[4 * i + k];
-            }
-            r[15] = (T)0;
-        }
-        r[3] = (T)(w * vq);
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    const SourceValues sv = source_values(i, Q, rule, tris, tgeo, pts64, u, v, need_u, need_v);
+    T* r = rec + REC * i;
+    if (REC == REC64) {
+        for (int k = 0; k < 3; ++k) r[k] = (T)pts64[4 * i + k];
+    } else {
         for (int k = 0; k < 3; ++k) {
-            r[4 + k] = (T)(w * uq * g[k]);
-            r[7 + k] = (T)(w * cu[k]);
+            r[k] = (T)pts32[4 * i + k];
+            r[12 + k] = (T)pts32lo[4 * i + k];
         }
-        if (REC == REC64) { r[10] = (T)0; r[11] = (T)0; }
-        else { r[10] = (T)0; r[11] = (T)0; }
+        r[15] = (T)0;
     }
+    r[3] = (T)sv.s;
+    for (int k = 0; k < 3; ++k) {
+        r[4 + k] = (T)sv.p[k];
+        r[7 + k] = (T)sv.c[k];
+    }
+    r[10] = (T)0;
+    r[11] = (T)0;
 }
 
 // ------------------------------------------------------- FP64 pair kernel (a3)
@@ -486,34 +504,20 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 }
 __device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
 
-template <typename T>
-__global__ void k_sources2(int64_t nt, int Q, Rule rule, const int32_t* __restrict__ tris,
+__global__ void k_sources2(int64_t np, int Q, Rule rule, const int32_t* __restrict__ tris,
                            const double* __restrict__ tgeo, const double* __restrict__ pts64,
                            const float* __restrict__ pts32, const float* __restrict__ pts32lo,
                            const double* __restrict__ u, const double* __restrict__ v, int need_u, int need_v,
                            float* __restrict__ rec) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nt) return;
-    const double* g = tgeo + 16 * t;
-    int32_t i0 = tris[3 * t], i1 = tris[3 * t + 1], i2 = tris[3 * t + 2];
-    double ua[3] = {0, 0, 0}, va[3] = {0, 0, 0};
-    if (need_u) { ua[0] = u[i0]; ua[1] = u[i1]; ua[2] = u[i2]; }
-    if (need_v) { va[0] = v[i0]; va[1] = v[i1]; va[2] = v[i2]; }
-    double inv2a = -1.0 / (2.0 * g[3]);
-    double cu[3];
-    for (int k = 0; k < 3; ++k) cu[k] = inv2a * (ua[0] * g[4 + k] + ua[1] * g[7 + k] + ua[2] * g[10 + k]);
-    for (int q = 0; q < Q; ++q) {
-        int64_t i = t * Q + q;
-        double w = pts64[4 * i + 3] * INV4PI;
-        double uq = rule.l[q][0] * ua[0] + rule.l[q][1] * ua[1] + rule.l[q][2] * ua[2];
-        double vq = rule.l[q][0] * va[0] + rule.l[q][1] * va[1] + rule.l[q][2] * va[2];
-        float val[16] = {pts32[4 * i], pts32[4 * i + 1], pts32[4 * i + 2], (float)(w * vq),
-                         (float)(w * uq * g[0]), (float)(w * uq * g[1]), (float)(w * uq * g[2]),
-                         (float)(w * cu[0]), (float)(w * cu[1]), (float)(w * cu[2]),
-                         pts32lo[4 * i], pts32lo[4 * i + 1], pts32lo[4 * i + 2], 0.f, 0.f, 0.f};
-        float4* r = reinterpret_cast<float4*>(rec + REC2 * i);
-        for (int k = 0; k < 8; ++k) r[k] = make_float4(val[2 * k], val[2 * k], val[2 * k + 1], val[2 * k + 1]);
-    }
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    const SourceValues sv = source_values(i, Q, rule, tris, tgeo, pts64, u, v, need_u, need_v);
+    const float val[16] = {pts32[4 * i], pts32[4 * i + 1], pts32[4 * i + 2], (float)sv.s,
+                           (float)sv.p[0], (float)sv.p[1], (float)sv.p[2],
+                           (float)sv.c[0], (float)sv.c[1], (float)sv.c[2],
+                           pts32lo[4 * i], pts32lo[4 * i + 1], pts32lo[4 * i + 2], 0.f, 0.f, 0.f};
+    float4* r = reinterpret_cast<float4*>(rec + REC2 * i);
+    for (int k = 0; k < 8; ++k) r[k] = make_float4(val[2 * k], val[2 * k], val[2 * k + 1], val[2 * k + 1]);
 }
 
 struct Coef2 {
@@ -884,48 +888,114 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2_queue(const PairJob* __restri
 }
 
 // --------------------------------------------- point sums -> test functions (a4 ii)
-template <typename P>
-__global__ void k_tri_reduce(int64_t nt, int64_t np, Rule rule, int nsplit, int mode, FarPlan fp,
-                             const double* __restrict__ tgeo, const double* __restrict__ pts64,
-                             const P* __restrict__ part, double* __restrict__ tri_out) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nt) return;
+// SPL threads per point add the splits' partial sums (each every SPL-th split, all
+// accumulators' loads of a split in flight at once, coalesced over the points) and
+// the first forms the point's scalars; the triangles' six sums are then taken from
+// shared memory. A block's points are whole triangles for every rule. Latency-bound
+// at small sizes, where a thread per triangle walking its points and their splits
+// took 37 us (1,920 points in 30 splits, V/K rows; now 8) and 107 us (7,680 points
+// in 25, V/K + D/T rows; now 12); FP64-bound at large ones (661,500 points in one
+// split, V/K + D/T rows: 72 us before, now 48).
+constexpr int RED_POINTS = 192;  // points per block (half with SPL = 4)
+
+template <typename P, int MODE, int SPL>
+__global__ void __launch_bounds__(SPL == 1 ? RED_POINTS : 2 * RED_POINTS)
+k_tri_reduce(int64_t np, Rule rule, int nsplit, int row0, double kb,  // kappa^2 x the coefficient of D_Y
+             const double* __restrict__ tgeo, const double* __restrict__ pts64, const P* __restrict__ part,
+             double* __restrict__ tri_out) {
+    constexpr int NACC = MODE == 0 ? 2 : 10, NV = MODE == 0 ? 2 : 5;
+    constexpr int RP = SPL == 1 ? RED_POINTS : RED_POINTS / 2;
+    __shared__ double val[NV][RP];  // w x the rows' sums; then w x the curl part's vector
+    __shared__ double other[SPL - 1 > 0 ? SPL - 1 : 1][SPL - 1 > 0 ? NACC : 1][SPL - 1 > 0 ? RP : 1];
     const int Q = rule.Q;
-    const int NACC = mode == 0 ? 2 : 10;
-    const double* g = tgeo + 16 * t;
-    double out[2][3] = {{0, 0, 0}, {0, 0, 0}};
-    double ctot[3] = {0, 0, 0};
-    for (int q = 0; q < Q; ++q) {
-        int64_t i = t * Q + q;
-        double w = pts64[4 * i + 3];
-        double a[10];
-        for (int k = 0; k < NACC; ++k) {
-            double s = 0.0;
-            for (int sp = 0; sp < nsplit; ++sp) s += (double)part[((int64_t)sp * NACC + k) * np + i];
-            a[k] = s;
+    const int lp = SPL == 1 ? threadIdx.x : threadIdx.x % RP, grp = SPL == 1 ? 0 : threadIdx.x / RP;
+    const int64_t i = blockIdx.x * (int64_t)RP + lp;
+    double a[NACC];
+#pragma unroll
+    for (int k = 0; k < NACC; ++k) a[k] = 0.0;
+    if (i < np && grp < nsplit) {
+        const P* p0 = part + (int64_t)grp * NACC * np + i;
+#pragma unroll
+        for (int k = 0; k < NACC; ++k) a[k] = (double)p0[(int64_t)k * np];
+#pragma unroll 2
+        for (int sp = grp + SPL; sp < nsplit; sp += SPL) {
+            const P* p = part + (int64_t)sp * NACC * np + i;
+#pragma unroll
+            for (int k = 0; k < NACC; ++k) a[k] += (double)p[(int64_t)k * np];
         }
-        // kernel row 0: phi-row
-        for (int b = 0; b < 3; ++b) out[0][b] += w * rule.l[q][b] * a[0];
-        if (mode == 0) {
-            for (int b = 0; b < 3; ++b) out[1][b] += w * rule.l[q][b] * a[1];
+    }
+    if (SPL > 1) {
+        if (grp > 0)
+#pragma unroll
+            for (int k = 0; k < NACC; ++k) other[grp - 1][k][lp] = a[k];
+        __syncthreads();
+        if (grp == 0)
+#pragma unroll
+            for (int g = 0; g < SPL - 1; ++g)
+#pragma unroll
+                for (int k = 0; k < NACC; ++k) a[k] += other[g][k][lp];
+    }
+    if (grp == 0) {
+        double v[NV];
+        if (i < np) {
+            const double w = pts64[4 * i + 3];
+            v[0] = w * a[0];
+            if (MODE == 0) {
+                v[1] = w * a[1];
+            } else {
+                const double* g = tgeo + 16 * (i / Q);
+                v[1] = w * (g[0] * (kb * a[7] - a[1]) + g[1] * (kb * a[8] - a[2]) + g[2] * (kb * a[9] - a[3]));
+#pragma unroll
+                for (int k = 0; k < 3; ++k) v[2 + k] = w * a[4 + k];
+            }
         } else {
-            double nT = g[0] * a[1] + g[1] * a[2] + g[2] * a[3];
-            double nB = g[0] * a[7] + g[1] * a[8] + g[2] * a[9];
-            double sc = -nT + fp.kappa * fp.kappa * fp.k[1][1] * nB;
-            for (int b = 0; b < 3; ++b) out[1][b] += w * rule.l[q][b] * sc;
-            for (int k = 0; k < 3; ++k) ctot[k] += w * a[4 + k];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) v[k] = 0.0;
         }
+#pragma unroll
+        for (int k = 0; k < NV; ++k) val[k][lp] = v[k];
     }
-    if (mode == 1) {
-        double inv2a = -1.0 / (2.0 * g[3]);
-        for (int b = 0; b < 3; ++b) {
-            const double* e = g + 4 + 3 * b;
-            out[1][b] += inv2a * (e[0] * ctot[0] + e[1] * ctot[1] + e[2] * ctot[2]);
+    __syncthreads();
+    const int64_t t0 = blockIdx.x * (int64_t)(RP / Q);
+    const int ntri = (int)min((int64_t)(RP / Q), np / Q - t0);
+    for (int k = threadIdx.x; k < 2 * ntri; k += blockDim.x) {  // a row's three sums of a triangle
+        const int r = k >= ntri, t = r ? k - ntri : k;
+        double out[3] = {0, 0, 0};
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) out[b] += rule.l[q][b] * val[r][t * Q + q];
+        if (MODE == 1 && r == 1) {
+            double c[3] = {0, 0, 0};
+            for (int q = 0; q < Q; ++q)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) c[d] += val[2 + d][t * Q + q];
+            const double* g = tgeo + 16 * (t0 + t);
+            const double inv2a = -1.0 / (2.0 * g[3]);
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                out[b] += inv2a * (g[4 + 3 * b] * c[0] + g[5 + 3 * b] * c[1] + g[6 + 3 * b] * c[2]);
         }
+        double* o = tri_out + 6 * (t0 + t) + 3 * (r == 0 ? row0 : 1 - row0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) o[b] = out[b];
     }
-    double* o = tri_out + 6 * t;
-    for (int r = 0; r < 2; ++r)
-        for (int b = 0; b < 3; ++b) o[3 * fp.out_row[r] + b] = out[r][b];
+}
+
+template <typename P>
+static void tri_reduce(const pb_mesh* m, const FarPlan& fp, int nsplit, const P* part, double* tri, cudaStream_t s) {
+    const double kb = fp.kappa * fp.kappa * fp.k[1][1];
+#define PB_RED_ARGS m->np, mesh_rule(m), nsplit, fp.out_row[0], kb, m->tgeo, m->pts64, part, tri
+    if (nsplit < 4) {  // four threads a point need a split each
+        const unsigned b = (unsigned)((m->np + RED_POINTS - 1) / RED_POINTS);
+        if (fp.mode == 0) k_tri_reduce<P, 0, 1><<<b, RED_POINTS, 0, s>>>(PB_RED_ARGS);
+        else k_tri_reduce<P, 1, 1><<<b, RED_POINTS, 0, s>>>(PB_RED_ARGS);
+    } else {
+        const unsigned b = (unsigned)((m->np + RED_POINTS / 2 - 1) / (RED_POINTS / 2));
+        if (fp.mode == 0) k_tri_reduce<P, 0, 4><<<b, 2 * RED_POINTS, 0, s>>>(PB_RED_ARGS);
+        else k_tri_reduce<P, 1, 4><<<b, 2 * RED_POINTS, 0, s>>>(PB_RED_ARGS);
+    }
+#undef PB_RED_ARGS
+    ::pb::count_launch();
 }
 
 // ------------------------------------- gather + near-field SpMV (a4 ii + a5)
@@ -1151,10 +1221,10 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             }
         const int nacc = fp.mode == 0 ? 2 : 10;
         Rule rule = mesh_rule(m);
-        unsigned tb = (unsigned)((nt + 127) / 128);
+        const unsigned sb = (unsigned)((np + 127) / 128);
         if (prec == PB_F64) {
             double* rec = (double*)m->ws_src.ptr;
-            k_sources<double, REC64><<<tb, 128, 0, s>>>(nt, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32,
+            k_sources<double, REC64><<<sb, 128, 0, s>>>(np, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32,
                                                         m->pts32lo, x, x + nv, need_u, need_v, rec); ::pb::count_launch();
             Coef cf;
             const Pair64Kernel kern = pair64_kernel(fp, &cf);
@@ -1168,19 +1238,17 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             kern<<<grid, TPB64, 0, s>>>(np, m->pts64, rec, cf, chunk, part);
             ::pb::count_launch();
             tm.stop();
-            k_tri_reduce<double><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64, part, tri);
-            ::pb::count_launch();
+            tri_reduce<double>(m, fp, S, part, tri, s);
         } else if (prec == PB_F32 && m->ctx->tree_enable && np >= m->ctx->tree_min_points && np > 256) {
             // treecode far field (inner iterations)
             float* part = nullptr;
             int S = 1;
             PB_TRY(tree_far(m, fp, x, need_u, need_v, &part, &S, s));
-            k_tri_reduce<float><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64, part, tri);
-            ::pb::count_launch();
+            tri_reduce<float>(m, fp, S, part, tri, s);
         } else if (tuned(m->ctx, np, fp.mode, prec == PB_F32_ACCURATE).kernel == 2 ||
                    (tuned(m->ctx, np, fp.mode, prec == PB_F32_ACCURATE).kernel == 0 && m->ctx->pair_kernel == 2)) {
             float* rec = (float*)m->ws_src.ptr;
-            k_sources2<float><<<tb, 128, 0, s>>>(nt, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32, m->pts32lo, x,
+            k_sources2<<<sb, 128, 0, s>>>(np, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32, m->pts32lo, x,
                                                  x + nv, need_u, need_v, rec);
             ::pb::count_launch();
             bool acc = prec == PB_F32_ACCURATE;
@@ -1207,15 +1275,12 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             ::pb::count_launch();
             tm.stop();
             if (acc)
-                k_tri_reduce<double><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64,
-                                                        (const double*)part, tri);
+                tri_reduce<double>(m, fp, S, (const double*)part, tri, s);
             else
-                k_tri_reduce<float><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64,
-                                                       (const float*)part, tri);
-            ::pb::count_launch();
+                tri_reduce<float>(m, fp, S, (const float*)part, tri, s);
         } else {
             float* rec = (float*)m->ws_src.ptr;
-            k_sources<float, REC32><<<tb, 128, 0, s>>>(nt, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32,
+            k_sources<float, REC32><<<sb, 128, 0, s>>>(np, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32,
                                                        m->pts32lo, x, x + nv, need_u, need_v, rec);
             ::pb::count_launch();
             CUtensorMap map;
@@ -1247,12 +1312,9 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             ::pb::count_launch();
             tm.stop();
             if (acc)
-                k_tri_reduce<double><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64,
-                                                        (const double*)part, tri);
+                tri_reduce<double>(m, fp, S, (const double*)part, tri, s);
             else
-                k_tri_reduce<float><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64,
-                                                       (const float*)part, tri);
-            ::pb::count_launch();
+                tri_reduce<float>(m, fp, S, (const float*)part, tri, s);
         }
     }
     unsigned gb = (unsigned)((nv * 8 + 255) / 256);
@@ -1336,8 +1398,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
             continue;
         }
         float* rec = (float*)m->ws_src.ptr;
-        unsigned tb = (unsigned)((nt + 127) / 128);
-        k_sources2<float><<<tb, 128, 0, js>>>(nt, m->Q, mesh_rule(m), m->tris, m->tgeo, m->pts64, m->pts32,
+        k_sources2<<<(unsigned)((np + 127) / 128), 128, 0, js>>>(np, m->Q, mesh_rule(m), m->tris, m->tgeo, m->pts64, m->pts32,
                                               m->pts32lo, J.x, J.x + m->nv, need_u, need_v, rec);
         ::pb::count_launch();
         if (np_pad > np) PB_CUDA(cudaMemsetAsync(rec + REC2 * np, 0, sizeof(float) * REC2 * (np_pad - np), js));
@@ -1441,14 +1502,8 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         const Prep& P = prep[k];
         cudaStream_t js = J.s ? J.s : s;
         if (P.fp.any) {
-            unsigned tb = (unsigned)((m->nt + 127) / 128);
-            if (acc)
-                k_tri_reduce<double><<<tb, 128, 0, js>>>(m->nt, m->np, mesh_rule(m), P.S, P.fp.mode, P.fp, m->tgeo,
-                                                         m->pts64, (const double*)m->ws_part.ptr, P.tri);
-            else
-                k_tri_reduce<float><<<tb, 128, 0, js>>>(m->nt, m->np, mesh_rule(m), P.S, P.fp.mode, P.fp, m->tgeo,
-                                                        m->pts64, (const float*)m->ws_part.ptr, P.tri);
-            ::pb::count_launch();
+            if (acc) tri_reduce<double>(m, P.fp, P.S, (const double*)m->ws_part.ptr, P.tri, js);
+            else tri_reduce<float>(m, P.fp, P.S, (const float*)m->ws_part.ptr, P.tri, js);
         }
         unsigned gb = (unsigned)((m->nv * 8 + 255) / 256);
         if (prec == PB_F32)
@@ -1572,8 +1627,8 @@ extern "C" int pb_system_apply_noalloc(pb_ctx* ctx, const pb_mesh* m, const pb_n
                 need_v = need_v || B.c[R][1][o] != 0.0;
             }
         Rule rule = mesh_rule(m);
-        unsigned tb = (unsigned)((nt + 127) / 128);
-        k_sources<float, REC32><<<tb, 128, 0, s>>>(nt, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32, m->pts32lo,
+        const unsigned sb = (unsigned)((np + 127) / 128);
+        k_sources<float, REC32><<<sb, 128, 0, s>>>(np, m->Q, rule, m->tris, m->tgeo, m->pts64, m->pts32, m->pts32lo,
                                                    x, x + nv, need_u, need_v, rec);
         ::pb::count_launch();
         CUtensorMap map;
@@ -1593,8 +1648,7 @@ extern "C" int pb_system_apply_noalloc(pb_ctx* ctx, const pb_mesh* m, const pb_n
         else
             k_pair32<1, false><<<grid, TPB32, 0, s>>>(map, np, m->pts32, m->pts32lo, cf, chunk, part, m->status);
         ::pb::count_launch();
-        k_tri_reduce<float><<<tb, 128, 0, s>>>(nt, np, rule, S, fp.mode, fp, m->tgeo, m->pts64, part, tri);
-        ::pb::count_launch();
+        tri_reduce<float>(m, fp, S, part, tri, s);
     }
     (void)nacc;
     unsigned gb = (unsigned)((nv * 8 + 255) / 256);

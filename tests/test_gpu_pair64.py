@@ -1,6 +1,6 @@
-"""FP64 pair kernel: every kind of row pair it has its own loop for (V/K rows with and without a Yukawa term; V/K + D/T
-rows with any coefficients, without a Yukawa term, with both kernels everywhere), at point counts around its 128-target
-blocks and 64-source tiles and at strong screening, against the oracle's dense operators. Tolerance as the FP64 operator
+"""FP64 pair kernels (both directions of a pair at once up to 65,536 points, else one): every kind of row pair they have their own loop for (V/K rows with and without a Yukawa term; V/K + D/T
+rows with any coefficients, without a Yukawa term, with both kernels everywhere), at point counts around the
+kernels' blocks and chunks and at strong screening, against the oracle's dense operators. Tolerance as the FP64 operator
 parity tests (1e-12 of the result, for the system forms of its largest block's result)."""
 import numpy as np
 import pytest
@@ -21,12 +21,13 @@ def load(v, t, kappa, **plan):
     return pb, ctx, m, pb.pb_near_build(ctx, m, kappa)
 
 
-# 6, 64, 128, 132, 126 and 420 points
-@pytest.mark.parametrize("n_lon,n_lat,far_q", [(3, 2, 1), (4, 9, 1), (8, 9, 1), (11, 7, 1), (7, 4, 3), (5, 8, 6)])
+# 6, 64, 128, 132, 126, 420, 1,980, 8,976, 17,460 and 45,360 points (the last two: blocks of 512 and 1,024)
+@pytest.mark.parametrize("n_lon,n_lat,far_q", [(3, 2, 1), (4, 9, 1), (8, 9, 1), (11, 7, 1), (7, 4, 3), (5, 8, 6),
+                                               (11, 31, 3), (22, 35, 6), (30, 98, 3), (20, 190, 6)])
 @pytest.mark.parametrize("form", ["direct_int", "juffer", "cfie_ext"])
 def test_forms_at_ragged_sizes(n_lon, n_lat, far_q, form):
     import torch
-    v, t = uv_ellipsoid(n_lon, n_lat, (2.0, 1.6, 1.3), twist=0.1)
+    v, t = uv_ellipsoid(n_lon, n_lat, (2.0, 1.6, 1.3 * n_lat / n_lon), twist=0.1)
     pb, ctx, m, nf = load(v, t, PHYS.kappa, far_q=far_q, n_ss=3)
     ops = oracle.assemble(v, t, PHYS.kappa, O.Plan(far_q, 3))
     z = np.zeros(v.shape[0])
@@ -50,3 +51,18 @@ def test_single_operators_and_screening(kappa):
         op, kern = OPS[name]
         y = pb.pb_op_apply(ctx, m, nf, op, kern, pb.PB_F64, torch.as_tensor(x, device="cuda")).cpu().numpy()
         assert rel(y, getattr(ops, name) @ x) < 1e-12, name
+
+
+def test_one_direction_at_a_time_beyond_the_symmetric_kernel():
+    """75,600 points (more than 64 blocks of 1,024): V and T rows against the oracle's at a few vertices."""
+    import torch
+    v, t = uv_ellipsoid(20, 316, (2.0, 1.6, 20.0), twist=0.05)
+    pb, ctx, m, nf = load(v, t, PHYS.kappa, far_q=6, n_ss=3)
+    assert m.info()["n_points"] > 65536
+    rows = np.array([0, 7, 1500, 6000, v.shape[0] - 1])
+    ops = oracle.assemble_rows(v, t, rows, PHYS.kappa, O.Plan(6, 3))
+    x = np.random.default_rng(3).standard_normal(v.shape[0])
+    for name in ("VL", "KY", "DY"):
+        op, kern = OPS[name]
+        y = pb.pb_op_apply(ctx, m, nf, op, kern, pb.PB_F64, torch.as_tensor(x, device="cuda")).cpu().numpy()
+        assert rel(y[rows], ops[name] @ x) < 1e-12, name

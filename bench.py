@@ -44,7 +44,6 @@ L2_FLUSH_BYTES = 256 << 20
 NCU_TRAFFIC = {  # (kernel family, formulation or "any", far-rule points, band) -> dram read + write per launch
     # 5,000-atom molecule (667,788 far-rule points, band of 3 radii), ncu dram__bytes_{read,write}.sum
     ("spmv", "juffer", 667788, 3.0): 337.5e6,
-    ("cheb", "juffer", 667788, 3.0): 16.04e6,
     ("tree32", "juffer", 667788, 3.0): 246.8e6,
     ("pair32acc", "juffer", 667788, 3.0): 496.5e6,
     ("near_band", "any", 667788, 3.0): 15203.8e6,

@@ -297,9 +297,10 @@ int far_splits_estimate(pb_ctx* ctx, int64_t np);
 TuneEntry tuned(const pb_ctx* ctx, int64_t np, int mode, bool acc);
 int tune_bucket(int64_t np);
 
-// Chebyshev solve with the mass matrix: y = M^-1 x on both halves of a 2 nv vector
+// Chebyshev solve with the mass matrix: y = M^-1 x on both halves of a 2 nv vector, the halves then
+// scaled (work: 3 x 2 nv doubles)
 int mass_solve(const pb_mesh* m, const pb_near* nf, const double* x, double* y, double* work,
-               int iters, cudaStream_t s);
+               int iters, cudaStream_t s, double scale0 = 1.0, double scale1 = 1.0);
 
 // CUDA events around one launch on its stream, when the context profiles.
 // Host worker pool, created on first use and kept for the life of the process:

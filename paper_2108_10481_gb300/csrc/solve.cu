@@ -25,10 +25,6 @@ __global__ void k_copy(int64_t n, const double* __restrict__ x, double* __restri
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) y[i] = x[i];
 }
-__global__ void k_scale_halves(int64_t nv, double a, double b, double* __restrict__ y) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < 2 * nv) y[i] *= (i < nv) ? a : b;
-}
 __global__ void k_sub(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
                       double* __restrict__ y) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -83,6 +79,18 @@ __global__ void k_block_diag_apply(int64_t nv, const double* __restrict__ inv, c
 // interval. Chebyshev iteration on that interval needs no inner products.
 constexpr double CH_LO = 0.5, CH_HI = 2.0;
 
+// The steps depend on one another and each is a few microseconds of work at most, so
+// latency bounds the solve. Two forms, the same sums in the same order:
+//   - up to CHEB_CLUSTER_ROWS vertices one cluster of eight CTAs runs the whole solve
+//     (k_cheb_cluster): rows and vectors in registers, the neighbours' d read from the
+//     owning CTA's shared memory, a cluster barrier between steps;
+//   - beyond that a kernel per step over the whole GPU (k_cheb_step), launched with
+//     programmatic dependent launch: what does not depend on the step before (the row, its
+//     values, the reciprocal of the diagonal) is loaded before the wait for it.
+// 34 steps of both halves, us, cluster | kernel per step, by vertices: 252: 31 | 73, 1,002:
+// 45 | 79, 1,962: 77 | 83, 2,562: 97 | 82 (eight SMs' FP64 pipes bound the cluster there);
+// 10,242: 104. Before, with three dependent loads, a divide and a plain launch per step:
+// 220 at 252 and at 10,242 vertices.
 __global__ void k_cheb_init(int64_t nv, const double* __restrict__ mdiag, const double* __restrict__ b,
                             double* __restrict__ x, double* __restrict__ r, double* __restrict__ d, double theta) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -92,33 +100,129 @@ __global__ void k_cheb_init(int64_t nv, const double* __restrict__ mdiag, const 
     x[i] = 0.0;
     d[i] = b[i] / (theta * mdiag[row]);
 }
-// one thread per vertex: row i of both halves (they share the pattern and values)
+
+// One thread per vertex and half (grid y). last: x receives its final value, the last
+// direction added and scaled (scale0, scale1 of the halves).
+constexpr int CHEB_PRE = 8;  // row entries loaded ahead (a vertex of a closed surface has seven on average)
 __global__ void k_cheb_step(int64_t nv, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                            const double* __restrict__ mval, const double* __restrict__ mdiag,
-                            const double* __restrict__ d, double* __restrict__ dn, double* __restrict__ x,
-                            double* __restrict__ r, double c_d, double c_r) {
+                            const double* __restrict__ mval, const double* __restrict__ mdiag, const double* d,
+                            double* dn, double* x, double* r, double c_d, double c_r, int last, double scale0,
+                            double scale1) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nv) return;
-    double md0 = 0.0, md1 = 0.0;
-    for (int32_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
-        const double mv = mval[k];
-        const int32_t c = col[k];
-        md0 += mv * d[c];
-        md1 += mv * d[nv + c];
+    const bool live = i < nv;
+    int32_t k0 = 0, k1 = 0, cp[CHEB_PRE];
+    double vp[CHEB_PRE], inv = 0.0;
+    if (live) {
+        k0 = row_ptr[i];
+        k1 = row_ptr[i + 1];
+        inv = c_r / mdiag[i];
     }
-    const double md[2] = {md0, md1};
-    const double inv = mdiag[i];
-    for (int h = 0; h < 2; ++h) {
-        const int64_t ii = i + h * nv;
-        const double rn = r[ii] - md[h];
-        x[ii] += d[ii];
-        r[ii] = rn;
-        dn[ii] = c_d * d[ii] + c_r * rn / inv;
+#pragma unroll
+    for (int q = 0; q < CHEB_PRE; ++q) {
+        const bool in = k0 + q < k1;
+        cp[q] = in ? col[k0 + q] : 0;
+        vp[q] = in ? mval[k0 + q] : 0.0;
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!live) return;
+    // written by the step before, which may have started on this SM: read past L1
+    const int64_t o = blockIdx.y * nv, ii = i + o;
+    const double di = __ldcg(d + ii), ri = __ldcg(r + ii), xi = __ldcg(x + ii);
+    double md = 0.0, dv[CHEB_PRE];
+#pragma unroll
+    for (int q = 0; q < CHEB_PRE; ++q) dv[q] = k0 + q < k1 ? __ldcg(d + o + cp[q]) : 0.0;
+#pragma unroll
+    for (int q = 0; q < CHEB_PRE; ++q) md += vp[q] * dv[q];
+    for (int32_t k = k0 + CHEB_PRE; k < k1; ++k) md += mval[k] * __ldcg(d + o + col[k]);
+    const double rn = ri - md, dnew = c_d * di + inv * rn;
+    double xn = xi + di;
+    if (last) xn = (xn + dnew) * (blockIdx.y ? scale1 : scale0);
+    x[ii] = xn;
+    r[ii] = rn;
+    dn[ii] = dnew;
+}
+
+constexpr int CHEB_CLUSTER = 8;          // CTAs (the portable cluster size)
+constexpr int CHEB_CLUSTER_ROWS = 2048;
+constexpr int CHEB_CLUSTER_N = CHEB_CLUSTER_ROWS / CHEB_CLUSTER;  // rows of a CTA at most
+
+// address of a shared-memory word in the cluster's CTA `rank`
+__device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
+    uint32_t ra;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    return ra;
+}
+__device__ __forceinline__ double ld_cluster(uint32_t addr) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+struct ChebCoef {  // c_d and c_r of every step
+    double cd[64], cr[64];
+};
+
+// n rows per CTA (CTA c: rows [c n, (c + 1) n)), a thread per row and half, which keeps its
+// row's first entries, r, x and its own d in registers; d is read by the neighbours from
+// shared memory, in two buffers, so that a step needs one barrier.
+__global__ void __launch_bounds__(2 * CHEB_CLUSTER_N)
+k_cheb_cluster(int nv, int n, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+               const double* __restrict__ mval, const double* __restrict__ mdiag, const double* __restrict__ b,
+               double* __restrict__ x, double theta, int iters, const __grid_constant__ ChebCoef cc, double scale0,
+               double scale1) {
+    __shared__ double dsh[2][2][CHEB_CLUSTER_N];
+    const int h = threadIdx.x >= n, i = threadIdx.x - h * n;  // half and row of this CTA
+    const int64_t row = (int64_t)blockIdx.x * n + i;
+    const bool live = i < n && row < nv;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(&dsh[0][h][0]);
+    constexpr uint32_t FLIP = 2 * CHEB_CLUSTER_N * sizeof(double);  // from one buffer to the other
+    int32_t k0 = 0, k1 = 0;
+    double inv = 0.0, r = 0.0, xs = 0.0, d = 0.0;
+    if (live) {
+        k0 = row_ptr[row];
+        k1 = row_ptr[row + 1];
+        const double m = mdiag[row];
+        r = b[(int64_t)h * nv + row];
+        inv = 1.0 / m;
+        d = r / (theta * m);
+        dsh[0][h][i] = d;
+    }
+    auto where = [&](int32_t c) { return map_cluster(base + 8u * ((uint32_t)c % (uint32_t)n), (uint32_t)c / (uint32_t)n); };
+    uint32_t at[CHEB_PRE];
+    double val[CHEB_PRE];
+#pragma unroll
+    for (int q = 0; q < CHEB_PRE; ++q) {  // past the row's end: its own d, times zero
+        const bool in = k0 + q < k1;
+        at[q] = where(in ? col[k0 + q] : (int32_t)(live ? row : 0));
+        val[q] = in ? mval[k0 + q] : 0.0;
+    }
+    cluster_sync();
+    for (int s = 0; s < iters; ++s) {
+        const uint32_t cur = (s & 1) ? FLIP : 0u;
+        if (live) {
+            double dv[CHEB_PRE];
+#pragma unroll
+            for (int q = 0; q < CHEB_PRE; ++q) dv[q] = ld_cluster(at[q] + cur);
+            double md = 0.0;
+#pragma unroll
+            for (int q = 0; q < CHEB_PRE; ++q) md += val[q] * dv[q];
+            for (int32_t k = k0 + CHEB_PRE; k < k1; ++k) md += mval[k] * ld_cluster(where(col[k]) + cur);
+            r -= md;
+            xs += d;
+            d = cc.cd[s] * d + cc.cr[s] * inv * r;
+            dsh[(s & 1) ^ 1][h][i] = d;
+        }
+        cluster_sync();
+    }
+    if (live) x[(int64_t)h * nv + row] = (xs + d) * (h ? scale1 : scale0);
 }
 
 int mass_solve(const pb_mesh* m, const pb_near* nf, const double* b, double* x, double* work, int iters,
-               cudaStream_t s) {
+               cudaStream_t s, double scale0, double scale1) {
     const int64_t nv = m->nv, n2 = 2 * nv;
     double* r = work;
     double* d0 = work + n2;
@@ -126,27 +230,59 @@ int mass_solve(const pb_mesh* m, const pb_near* nf, const double* b, double* x, 
     const double theta = 0.5 * (CH_HI + CH_LO), delta = 0.5 * (CH_HI - CH_LO), sigma = theta / delta;
     const double* mval = nf->mval;  // the mass matrix on its own pattern
     const double* mdiag = nf->diag + N_M * nv;
-    unsigned blocks = (unsigned)((n2 + 255) / 256);
-    k_cheb_init<<<blocks, 256, 0, s>>>(nv, mdiag, b, x, r, d0, theta); ::pb::count_launch();
     // algorithmic bytes of one step: the mass pattern once (row pointers, columns and
     // values; nv + 3 nt entries on a closed surface) and its diagonal, d read, the
     // next d written, x and r read and written (2 nv doubles each)
     const double mnnz = (double)nv + 3.0 * (double)m->nt;
     const double step_bytes = 4.0 * (double)(nv + 1) + 12.0 * mnnz + 8.0 * (double)nv + 6.0 * 8.0 * (double)n2;
     double rho = 1.0 / sigma;
+    if (nv <= CHEB_CLUSTER_ROWS && iters <= 64) {
+        ChebCoef cc;
+        for (int k = 0; k < iters; ++k) {
+            const double rho_n = 1.0 / (2.0 * sigma - rho);
+            cc.cd[k] = rho_n * rho;
+            cc.cr[k] = 2.0 * rho_n / delta;
+            rho = rho_n;
+        }
+        const int n = (int)((nv + CHEB_CLUSTER - 1) / CHEB_CLUSTER);
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = CHEB_CLUSTER;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(CHEB_CLUSTER);
+        cfg.blockDim = dim3((unsigned)((2 * n + 31) / 32 * 32));
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        Timer tm(m->ctx, PB_KERNEL_CHEB, s, step_bytes * iters, 1.0);
+        PB_CUDA(cudaLaunchKernelEx(&cfg, k_cheb_cluster, (int)nv, n, (const int32_t*)nf->mrow_ptr,
+                                   (const int32_t*)nf->mcol, mval, mdiag, b, x, theta, iters, cc, scale0, scale1));
+        ::pb::count_launch();
+        tm.stop();
+        return PB_OK;
+    }
+    k_cheb_init<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(nv, mdiag, b, x, r, d0, theta); ::pb::count_launch();
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((nv + 127) / 128), 2);
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = m->ctx->profile ? 0 : 1;  // profiled: events lie between the steps
     for (int k = 0; k < iters; ++k) {
-        double rho_n = 1.0 / (2.0 * sigma - rho);
+        const double rho_n = 1.0 / (2.0 * sigma - rho);
         Timer tm(m->ctx, PB_KERNEL_CHEB, s, step_bytes, 1.0);
-        k_cheb_step<<<(unsigned)((nv + 255) / 256), 256, 0, s>>>(nv, nf->mrow_ptr, nf->mcol, mval, mdiag, d0, d1, x,
-                                                                  r, rho_n * rho, 2.0 * rho_n / delta);
+        PB_CUDA(cudaLaunchKernelEx(&cfg, k_cheb_step, nv, (const int32_t*)nf->mrow_ptr, (const int32_t*)nf->mcol, mval,
+                                   mdiag, (const double*)d0, d1, x, r, rho_n * rho, 2.0 * rho_n / delta,
+                                   (int)(k + 1 == iters), scale0, scale1));
         ::pb::count_launch();
         tm.stop();
         rho = rho_n;
-        double* t = d0;
-        d0 = d1;
-        d1 = t;
+        std::swap(d0, d1);
     }
-    k_add_inplace<<<blocks, 256, 0, s>>>(n2, d0, x); ::pb::count_launch();
     PB_CUDA(cudaGetLastError());
     return PB_OK;
 }
@@ -348,8 +484,8 @@ int apply_prec(Solver& S, int prec, const double* x, double* y) {
             break;
         case PB_PC_MASS:
         case PB_PC_SCALED_MASS:
-            PB_TRY(mass_solve(m, S.nf, x, y, S.cheb, ci, S.s));
-            break;
+            PB_TRY(mass_solve(m, S.nf, x, y, S.cheb, ci, S.s, 1.0 / S.sa, 1.0 / S.sb));
+            return PB_OK;
         default:  // Calderon: M^-1 C M^-1
             PB_TRY(mass_solve(m, S.nf, x, S.t1, S.cheb, ci, S.s));
             {
@@ -358,12 +494,8 @@ int apply_prec(Solver& S, int prec, const double* x, double* y) {
                 PB_TRY(apply_blockop(S.mc, S.nc, S.C, prec, S.t1, S.t2, S.s, cc));
             }
             S.applies++;
-            PB_TRY(mass_solve(m, S.nf, S.t2, y, S.cheb, ci, S.s));
-            break;
-    }
-    if (S.sa != 1.0 || S.sb != 1.0) {
-        k_scale_halves<<<nb(n2), 256, 0, S.s>>>(nv, 1.0 / S.sa, 1.0 / S.sb, y);
-        ::pb::count_launch();
+            PB_TRY(mass_solve(m, S.nf, S.t2, y, S.cheb, ci, S.s, 1.0 / S.sa, 1.0 / S.sb));
+            return PB_OK;
     }
     PB_CUDA(cudaGetLastError());
     return PB_OK;
@@ -652,13 +784,7 @@ int calderon_pre(Solver& S, int prec, const double* x) {
 }
 
 int calderon_post(Solver& S, int prec, double* y) {
-    PB_TRY(mass_solve(S.m, S.nf, S.t2, y, S.cheb, cheb_count(S, prec), S.s));
-    if (S.sa != 1.0 || S.sb != 1.0) {
-        k_scale_halves<<<nb(2 * S.m->nv), 256, 0, S.s>>>(S.m->nv, 1.0 / S.sa, 1.0 / S.sb, y);
-        ::pb::count_launch();
-    }
-    PB_CUDA(cudaGetLastError());
-    return PB_OK;
+    return mass_solve(S.m, S.nf, S.t2, y, S.cheb, cheb_count(S, prec), S.s, 1.0 / S.sa, 1.0 / S.sb);
 }
 
 void vec_sub(int64_t n, const double* a, const double* b, double* y, cudaStream_t s) {

@@ -200,6 +200,9 @@ struct pb_mesh {
     int* status = nullptr;          // device status word of bounded waits (0 = fine)
     // workspaces (grown on demand)
     pb::Workspace ws_src, ws_part, ws_tri, ws_vec, ws_comb, ws_tree;
+    // pb_energy's point values and partial sums: in use only during the call, held by no graph
+    pb::Workspace ws_energy;
+    uint64_t ws_energy_gen = 0;
     uint64_t ws_gen = 0;  // bumped when one of the workspaces above moves or is freed
     pb::PbTree* tree = nullptr;  // built on the first treecode application
     size_t device_bytes = 0;

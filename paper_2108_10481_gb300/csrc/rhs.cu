@@ -7,6 +7,7 @@
 // Delta G = 1/2 sum_j q_j phi_reac(x_j).
 #include <math.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "internal.h"
@@ -31,21 +32,44 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
     return __fma_rn(0.5 * y, e, y);
 }
 
-// per point: phi_D and phi_N of all charges, then per triangle the tested sums
-// (templated on the rule's point count, so that the per-point sums stay in registers)
-template <int Q>
-__global__ void k_rhs_points(int64_t nt, Rule rule, const double* __restrict__ pts64, const double* __restrict__ tgeo,
-                             const double* __restrict__ xq, const double* __restrict__ q, int64_t nq, double eps_int,
-                             double* __restrict__ tri_out) {
+// One thread per point of the reference rule: phi_D and phi_N of all charges there, the
+// charges staged in shared memory; the triangles' tested sums are then taken from the
+// block's points (192: whole triangles for every rule). Bound by the FP64 (FP32) pipe;
+// with a thread per triangle 38,720 of them were eight warps an SM, too few to cover a
+// pair's chain: 484 charges in FP32 147 -> 115 us.
+constexpr int RHS_POINTS = 192;
+
+// the triangles' sums of a block from its points' values times their weights
+__device__ __forceinline__ void test_points(const double (&val)[2][RHS_POINTS], const Rule& rule, int64_t np,
+                                            double* __restrict__ tri_out) {
+    const int Q = rule.Q;
+    const int64_t t0 = blockIdx.x * (int64_t)(RHS_POINTS / Q);
+    const int ntri = (int)min((int64_t)(RHS_POINTS / Q), np / Q - t0);
+    for (int k = threadIdx.x; k < 6 * ntri; k += RHS_POINTS) {
+        const int t = k / 6, r = (k - 6 * t) / 3, c = k % 3;
+        double o = 0.0;
+        for (int q = 0; q < Q; ++q) o += rule.l[q][c] * val[r][t * Q + q];
+        tri_out[6 * t0 + k] = o;
+    }
+}
+
+__global__ void __launch_bounds__(RHS_POINTS)
+k_rhs_points(int64_t np, Rule rule, const double* __restrict__ pts64, const double* __restrict__ tgeo,
+             const double* __restrict__ xq, const double* __restrict__ q, int64_t nq, double eps_int,
+             double* __restrict__ tri_out) {
     __shared__ double sq[QTILE * 4];
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    bool live = t < nt;
-    double pd[6] = {0, 0, 0, 0, 0, 0}, pn[6] = {0, 0, 0, 0, 0, 0};
-    double nx = 0, ny = 0, nz = 0;
-    if (live) { nx = tgeo[16 * t]; ny = tgeo[16 * t + 1]; nz = tgeo[16 * t + 2]; }
+    __shared__ double val[2][RHS_POINTS];
+    const int64_t i = blockIdx.x * (int64_t)RHS_POINTS + threadIdx.x;
+    const bool live = i < np;
+    double x0 = 0, x1 = 0, x2 = 0, w = 0, nx = 0, ny = 0, nz = 0, pd = 0, pn = 0;
+    if (live) {
+        const double* g = tgeo + 16 * (i / rule.Q);
+        x0 = pts64[4 * i]; x1 = pts64[4 * i + 1]; x2 = pts64[4 * i + 2]; w = pts64[4 * i + 3];
+        nx = g[0]; ny = g[1]; nz = g[2];
+    }
     for (int64_t j0 = 0; j0 < nq; j0 += QTILE) {
-        int cnt = (int)min((int64_t)QTILE, nq - j0);
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
+        const int cnt = (int)min((int64_t)QTILE, nq - j0);
+        for (int k = threadIdx.x; k < cnt; k += RHS_POINTS) {
             sq[4 * k] = xq[3 * (j0 + k)];
             sq[4 * k + 1] = xq[3 * (j0 + k) + 1];
             sq[4 * k + 2] = xq[3 * (j0 + k) + 2];
@@ -53,32 +77,22 @@ __global__ void k_rhs_points(int64_t nt, Rule rule, const double* __restrict__ p
         }
         __syncthreads();
         if (live)
-#pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                const double* x = pts64 + 4 * (t * Q + k);
-                for (int j = 0; j < cnt; ++j) {
-                    double d0 = x[0] - sq[4 * j], d1 = x[1] - sq[4 * j + 1], d2 = x[2] - sq[4 * j + 2];
-                    double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-                    double rinv = rsqrt_nr(r2);
-                    double c = sq[4 * j + 3] * rinv;
-                    pd[k] += c;
-                    pn[k] -= c * rinv * rinv * (d0 * nx + d1 * ny + d2 * nz);
-                }
+#pragma unroll 2
+            for (int j = 0; j < cnt; ++j) {
+                const double d0 = x0 - sq[4 * j], d1 = x1 - sq[4 * j + 1], d2 = x2 - sq[4 * j + 2];
+                const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
+                const double rinv = rsqrt_nr(r2);
+                const double c = sq[4 * j + 3] * rinv;
+                pd += c;
+                pn -= c * rinv * rinv * (d0 * nx + d1 * ny + d2 * nz);
             }
         __syncthreads();
     }
-    if (!live) return;
-    const double f = 1.0 / (4.0 * M_PI * eps_int);
-    double out[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        double w = pts64[4 * (t * Q + k) + 3] * f;
-        for (int a = 0; a < 3; ++a) {
-            out[a] += w * rule.l[k][a] * pd[k];
-            out[3 + a] += w * rule.l[k][a] * pn[k];
-        }
-    }
-    for (int k = 0; k < 6; ++k) tri_out[6 * t + k] = out[k];
+    const double f = w / (4.0 * M_PI * eps_int);
+    val[0][threadIdx.x] = f * pd;
+    val[1][threadIdx.x] = f * pn;
+    __syncthreads();
+    test_points(val, rule, np, tri_out);
 }
 
 // FP32 pair arithmetic on split coordinates (PB_F32_ACCURATE): every position
@@ -105,32 +119,27 @@ struct Ctr {
 
 // the right-hand side's point sums (k_rhs_points) in FP32 on split coordinates:
 // per charge tile the sums in FP32, added into FP64 sums per tile
-template <int Q>
-__global__ void k_rhs_points32(int64_t nt, Rule rule, const double* __restrict__ pts64,
-                               const double* __restrict__ tgeo, const double* __restrict__ xq,
-                               const double* __restrict__ q, int64_t nq, double eps_int, Ctr ctr,
-                               double* __restrict__ tri_out) {
+__global__ void __launch_bounds__(RHS_POINTS)
+k_rhs_points32(int64_t np, Rule rule, const double* __restrict__ pts64, const double* __restrict__ tgeo,
+               const double* __restrict__ xq, const double* __restrict__ q, int64_t nq, double eps_int, Ctr ctr,
+               double* __restrict__ tri_out) {
     __shared__ float4 sh[QTILE], sl[QTILE];
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool live = t < nt;
-    float xh[Q][3], xl[Q][3];
-    float nx = 0.f, ny = 0.f, nz = 0.f;
+    __shared__ double val[2][RHS_POINTS];
+    const int64_t i = blockIdx.x * (int64_t)RHS_POINTS + threadIdx.x;
+    const bool live = i < np;
+    float xh[3] = {0.f, 0.f, 0.f}, xl[3] = {0.f, 0.f, 0.f}, nx = 0.f, ny = 0.f, nz = 0.f;
+    double w = 0.0, pd = 0.0, pn = 0.0;
     if (live) {
-        nx = (float)tgeo[16 * t];
-        ny = (float)tgeo[16 * t + 1];
-        nz = (float)tgeo[16 * t + 2];
+        const double* g = tgeo + 16 * (i / rule.Q);
+        split3(pts64 + 4 * i, ctr.c, xh, xl);
+        w = pts64[4 * i + 3];
+        nx = (float)g[0];
+        ny = (float)g[1];
+        nz = (float)g[2];
     }
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        if (live) split3(pts64 + 4 * (t * Q + k), ctr.c, xh[k], xl[k]);
-        else xh[k][0] = xh[k][1] = xh[k][2] = xl[k][0] = xl[k][1] = xl[k][2] = 0.f;
-    }
-    double pd[Q], pn[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k) pd[k] = pn[k] = 0.0;
     for (int64_t j0 = 0; j0 < nq; j0 += QTILE) {
         const int cnt = (int)min((int64_t)QTILE, nq - j0);
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
+        for (int k = threadIdx.x; k < cnt; k += RHS_POINTS) {
             float h[3], l[3];
             split3(xq + 3 * (j0 + k), ctr.c, h, l);
             sh[k] = make_float4(h[0], h[1], h[2], (float)q[j0 + k]);
@@ -138,43 +147,29 @@ __global__ void k_rhs_points32(int64_t nt, Rule rule, const double* __restrict__
         }
         __syncthreads();
         if (live) {
-            float fd[Q], fn[Q];
-#pragma unroll
-            for (int k = 0; k < Q; ++k) fd[k] = fn[k] = 0.f;
+            float fd = 0.f, fn = 0.f;
+#pragma unroll 4
             for (int j = 0; j < cnt; ++j) {
                 const float4 a = sh[j], b = sl[j];
-#pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    const float d0 = (xh[k][0] - a.x) + (xl[k][0] - b.x);
-                    const float d1 = (xh[k][1] - a.y) + (xl[k][1] - b.y);
-                    const float d2 = (xh[k][2] - a.z) + (xl[k][2] - b.z);
-                    const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-                    const float rinv = rsqrt_f32(r2);
-                    const float c = a.w * rinv;
-                    fd[k] += c;
-                    fn[k] = fmaf(-c * rinv * rinv, fmaf(d0, nx, fmaf(d1, ny, d2 * nz)), fn[k]);
-                }
+                const float d0 = (xh[0] - a.x) + (xl[0] - b.x);
+                const float d1 = (xh[1] - a.y) + (xl[1] - b.y);
+                const float d2 = (xh[2] - a.z) + (xl[2] - b.z);
+                const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
+                const float rinv = rsqrt_f32(r2);
+                const float c = a.w * rinv;
+                fd += c;
+                fn = fmaf(-c * rinv * rinv, fmaf(d0, nx, fmaf(d1, ny, d2 * nz)), fn);
             }
-#pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                pd[k] += (double)fd[k];
-                pn[k] += (double)fn[k];
-            }
+            pd += (double)fd;
+            pn += (double)fn;
         }
         __syncthreads();
     }
-    if (!live) return;
-    const double f = 1.0 / (4.0 * M_PI * eps_int);
-    double out[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        double w = pts64[4 * (t * Q + k) + 3] * f;
-        for (int a = 0; a < 3; ++a) {
-            out[a] += w * rule.l[k][a] * pd[k];
-            out[3 + a] += w * rule.l[k][a] * pn[k];
-        }
-    }
-    for (int k = 0; k < 6; ++k) tri_out[6 * t + k] = out[k];
+    const double f = w / (4.0 * M_PI * eps_int);
+    val[0][threadIdx.x] = f * pd;
+    val[1][threadIdx.x] = f * pn;
+    __syncthreads();
+    test_points(val, rule, np, tri_out);
 }
 
 __global__ void k_rhs_gather(int64_t nv, const int32_t* __restrict__ v2t_ptr, const int32_t* __restrict__ v2t,
@@ -252,11 +247,21 @@ __global__ void k_energy_part(int64_t np, const double* __restrict__ pv, const d
 }
 
 // the energy's pair sums in FP32 on split coordinates: the point values once
-// as (hi, w v), (lo, 0), (w u n, 0) floats, then a thread per charge over a
-// chunk of points staged in shared memory, FP32 sums per tile added in FP64
-constexpr int EN32_THREADS = 128;  // charges per block
+// as (hi, w v), (lo, 0), (w u n, 0) floats, then a block per 32 charges and chunk of
+// points staged in shared memory: a lane per charge, the four warps taking every
+// fourth point of a tile, FP32 sums per tile added in FP64, the warps' at the end in
+// warp order. (With a thread per charge and chunks of 4,096 points, 484 charges were six
+// warps an SM, and 20 left most lanes of a block idle: 484 charges, 232,320 points 207 ->
+// 120 us.)
+constexpr int EN32_CHARGES = 32;  // per block
+constexpr int EN32_WARPS = 4;
+constexpr int EN32_THREADS = 32 * EN32_WARPS;
 constexpr int EN32_TILE = 256;     // points per staged tile
-constexpr int EN32_CHUNK = 4096;   // points per block
+// points per block: 1,024, or more (whole tiles) where that would be over 512 chunks
+static int64_t en32_chunk(int64_t np) {
+    const int64_t c = (np + 511) / 512;
+    return std::max<int64_t>(1024, (c + EN32_TILE - 1) / EN32_TILE * EN32_TILE);
+}
 
 __global__ void k_energy_points32(int64_t nt, Rule rule, const int32_t* __restrict__ tris,
                                   const double* __restrict__ tgeo, const double* __restrict__ pts64,
@@ -279,15 +284,17 @@ __global__ void k_energy_points32(int64_t nt, Rule rule, const int32_t* __restri
     pv[3 * i + 2] = make_float4((float)(y[3] * u * g[0]), (float)(y[3] * u * g[1]), (float)(y[3] * u * g[2]), 0.f);
 }
 
-__global__ void __launch_bounds__(EN32_THREADS) k_energy_part32(int64_t np, const float4* __restrict__ pv,
+__global__ void __launch_bounds__(EN32_THREADS) k_energy_part32(int64_t np, int64_t chunk, const float4* __restrict__ pv,
                                                                 const double* __restrict__ xq, int64_t nq, Ctr ctr,
                                                                 double* __restrict__ part, int nchunk) {
     __shared__ float4 tile[3 * EN32_TILE];
-    const int64_t j = blockIdx.y * (int64_t)EN32_THREADS + threadIdx.x;
+    __shared__ double red[EN32_WARPS][EN32_CHARGES];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t j = blockIdx.y * (int64_t)EN32_CHARGES + lane;
     const bool live = j < nq;
     float qh[3] = {0.f, 0.f, 0.f}, ql[3] = {0.f, 0.f, 0.f};
     if (live) split3(xq + 3 * j, ctr.c, qh, ql);
-    const int64_t i0 = (int64_t)blockIdx.x * EN32_CHUNK, i1 = min(np, i0 + EN32_CHUNK);
+    const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = min(np, i0 + chunk);
     double s = 0.0;
     for (int64_t b0 = i0; b0 < i1; b0 += EN32_TILE) {
         const int cnt = (int)min((int64_t)EN32_TILE, i1 - b0);
@@ -295,7 +302,8 @@ __global__ void __launch_bounds__(EN32_THREADS) k_energy_part32(int64_t np, cons
         for (int k = threadIdx.x; k < 3 * cnt; k += EN32_THREADS) tile[k] = pv[3 * b0 + k];
         __syncthreads();
         float f = 0.f;
-        for (int p = 0; p < cnt; ++p) {
+#pragma unroll 4
+        for (int p = w; p < cnt; p += EN32_WARPS) {
             const float4 a = tile[3 * p], b = tile[3 * p + 1], c = tile[3 * p + 2];
             const float d0 = (qh[0] - a.x) + (ql[0] - b.x);
             const float d1 = (qh[1] - a.y) + (ql[1] - b.y);
@@ -307,27 +315,43 @@ __global__ void __launch_bounds__(EN32_THREADS) k_energy_part32(int64_t np, cons
         }
         s += (double)f;
     }
-    if (live) part[j * nchunk + blockIdx.x] = s;
+    red[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && live) {
+        for (int k = 1; k < EN32_WARPS; ++k) s += red[k][lane];
+        part[j * nchunk + blockIdx.x] = s;
+    }
 }
 
-// phi_reac(x_j) per charge (its chunks in order), then Delta G by one thread
-// over the charges in order: the summation order is fixed.
-__global__ void k_energy_rows(int64_t nq, int nchunk, const double* __restrict__ part, double* __restrict__ phi) {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= nq) return;
+// phi_reac(x_j), a warp per charge over its chunks' sums, then Delta G by one block over
+// the charges: the summation order is fixed. (One thread over 484 charges took 53 us.)
+__global__ void k_energy_rows(int64_t nq, int nchunk, const double* __restrict__ part, double* __restrict__ phi_all,
+                              double* __restrict__ phi) {
+    const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (j >= nq) return;  // whole warps
     double p = 0.0;
-    for (int c = 0; c < nchunk; ++c) p += part[j * nchunk + c];
-    phi[j] = p * (1.0 / (4.0 * M_PI));
-}
-__global__ void k_energy_final(int64_t nq, const double* __restrict__ phi_all, const double* __restrict__ q,
-                               double* __restrict__ phi, double* __restrict__ dG) {
-    double e = 0.0;
-    for (int64_t j = 0; j < nq; ++j) {
-        const double p = phi_all[j];
+    for (int c = lane; c < nchunk; c += 32) p += part[j * nchunk + c];
+    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+    if (lane == 0) {
+        p *= 1.0 / (4.0 * M_PI);
+        phi_all[j] = p;
         if (phi) phi[j] = p;
-        e += q[j] * p;
     }
-    dG[0] = 0.5 * e;
+}
+constexpr int EN_FINAL_THREADS = 256;
+__global__ void __launch_bounds__(EN_FINAL_THREADS)
+k_energy_final(int64_t nq, const double* __restrict__ phi_all, const double* __restrict__ q, double* __restrict__ dG) {
+    __shared__ double red[EN_FINAL_THREADS / 32];
+    double e = 0.0;
+    for (int64_t j = threadIdx.x; j < nq; j += EN_FINAL_THREADS) e += q[j] * phi_all[j];
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < EN_FINAL_THREADS / 32; ++w) e += red[w];
+        dG[0] = 0.5 * e;
+    }
 }
 
 }  // namespace pb
@@ -348,19 +372,12 @@ extern "C" int pb_rhs_charges(pb_ctx* ctx, const pb_mesh* m, const double* xq, c
     double* tri = (double*)m->ws_tri.ptr;
     // the plan's reference rule (the band rule when the plan has a band)
     const Rule rr = mesh_ref_rule(m);
-    const unsigned nbk = (unsigned)((m->nt + 127) / 128);
+    const unsigned nbk = (unsigned)((m->np_ref + RHS_POINTS - 1) / RHS_POINTS);
     if (prec == PB_F64) {
-        if (rr.Q == 6) k_rhs_points<6><<<nbk, 128, 0, s>>>(m->nt, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, tri);
-        else if (rr.Q == 3) k_rhs_points<3><<<nbk, 128, 0, s>>>(m->nt, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, tri);
-        else k_rhs_points<1><<<nbk, 128, 0, s>>>(m->nt, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, tri);
+        k_rhs_points<<<nbk, RHS_POINTS, 0, s>>>(m->np_ref, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, tri);
     } else {
         const Ctr c = {{m->ctr[0], m->ctr[1], m->ctr[2]}};
-        if (rr.Q == 6)
-            k_rhs_points32<6><<<nbk, 128, 0, s>>>(m->nt, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, c, tri);
-        else if (rr.Q == 3)
-            k_rhs_points32<3><<<nbk, 128, 0, s>>>(m->nt, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, c, tri);
-        else
-            k_rhs_points32<1><<<nbk, 128, 0, s>>>(m->nt, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, c, tri);
+        k_rhs_points32<<<nbk, RHS_POINTS, 0, s>>>(m->np_ref, rr, m->pts_ref, m->tgeo, xq, q, n_q, prm->eps_int, c, tri);
     }
     ::pb::count_launch();
     k_rhs_gather<<<(unsigned)((m->nv + 255) / 256), 256, 0, s>>>(m->nv, m->v2t_ptr, m->v2t, tri, d[0], d[1], n[0],
@@ -381,11 +398,14 @@ extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int for
     // exterior unknowns -> interior traces: u_int = u_ext, v_int = (eps_ext/eps_int) v_ext
     double vscale = form_is_exterior(form) ? prm->eps_ext / prm->eps_int : 1.0;
     const bool f32 = prec == PB_F32_ACCURATE;
-    const int nchunk = (int)((m->np_ref + (f32 ? EN32_CHUNK : EN_CHUNK) - 1) / (f32 ? EN32_CHUNK : EN_CHUNK));
-    double* part = nullptr;
-    // partial sums, phi per charge, Delta G, then the point values (32-byte aligned)
-    const size_t n_part = (size_t)n_q * nchunk, n_head = (n_part + 2 * (size_t)n_q + 1 + 3) / 4 * 4;
-    PB_TRY(dev_alloc((void**)&part, sizeof(double) * (n_head + 8 * (size_t)m->np_ref)));
+    const int64_t chunk = f32 ? en32_chunk(m->np_ref) : EN_CHUNK;
+    const int nchunk = (int)((m->np_ref + chunk - 1) / chunk);
+    // partial sums, phi per charge, Delta G, then the point values (32-byte aligned); a workspace of
+    // its own, free again when the call returns (the call waits for its work)
+    const size_t n_part = (size_t)n_q * nchunk, n_head = (n_part + (size_t)n_q + 1 + 3) / 4 * 4;
+    pb_mesh* mm = const_cast<pb_mesh*>(m);
+    PB_TRY(ws_reserve(mm->ws_energy, sizeof(double) * (n_head + (f32 ? 6 : 8) * (size_t)m->np_ref)));
+    double* part = (double*)mm->ws_energy.ptr;
     double* phi_all = part + n_part;
     double* dG = phi_all + n_q;
     double* pv = part + n_head;
@@ -395,21 +415,20 @@ extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int for
         const Ctr c = {{m->ctr[0], m->ctr[1], m->ctr[2]}};
         k_energy_points32<<<pb_, 256, 0, s>>>(m->nt, rr, m->tris, m->tgeo, m->pts_ref, x, m->nv, vscale, c,
                                               reinterpret_cast<float4*>(pv));
-        const dim3 grid(nchunk, (unsigned)((n_q + EN32_THREADS - 1) / EN32_THREADS));
-        k_energy_part32<<<grid, EN32_THREADS, 0, s>>>(m->np_ref, reinterpret_cast<const float4*>(pv), xq, n_q, c, part,
-                                                      nchunk);
+        const dim3 grid(nchunk, (unsigned)((n_q + EN32_CHARGES - 1) / EN32_CHARGES));
+        k_energy_part32<<<grid, EN32_THREADS, 0, s>>>(m->np_ref, chunk, reinterpret_cast<const float4*>(pv), xq, n_q, c,
+                                                      part, nchunk);
     } else {
         k_energy_points<<<pb_, 256, 0, s>>>(m->nt, rr, m->tris, m->tgeo, m->pts_ref, x, m->nv, vscale, pv);
         const dim3 grid(nchunk, (unsigned)n_q);
         k_energy_part<<<grid, EN_THREADS, 0, s>>>(m->np_ref, pv, xq, part, nchunk);
     }
-    k_energy_rows<<<(unsigned)((n_q + 127) / 128), 128, 0, s>>>(n_q, nchunk, part, phi_all);
-    k_energy_final<<<1, 1, 0, s>>>(n_q, phi_all, q, phi, dG);
+    k_energy_rows<<<(unsigned)((n_q * 32 + 127) / 128), 128, 0, s>>>(n_q, nchunk, part, phi_all, phi);
+    k_energy_final<<<1, EN_FINAL_THREADS, 0, s>>>(n_q, phi_all, q, dG);
     ::pb::count_launch(4);
     double h = 0.0;
     cudaError_t e = cudaMemcpyAsync(&h, dG, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(part);
     if (e != cudaSuccess) return set_error(PB_ECUDA, "pb_energy: %s", cudaGetErrorString(e));
     if (dG_paper) *dG_paper = h;
     if (dG_kcal) *dG_kcal = h * 4.0 * M_PI * 332.0636;

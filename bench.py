@@ -46,7 +46,6 @@ NCU_TRAFFIC = {  # (kernel family, formulation or "any", far-rule points, band) 
     ("spmv", "juffer", 667788, 3.0): 337.5e6,
     ("tree32", "juffer", 667788, 3.0): 246.8e6,
     ("pair32acc", "juffer", 667788, 3.0): 496.5e6,
-    ("near_band", "any", 667788, 3.0): 15203.8e6,
     ("near_coin", "any", 667788, 3.0): 233.9e6,
 }
 

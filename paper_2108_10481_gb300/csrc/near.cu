@@ -14,6 +14,7 @@
 #include <cmath>
 #include <cstdlib>
 
+#include "exp64.cuh"
 #include "internal.h"
 
 namespace pb {
@@ -812,63 +813,104 @@ k_coin_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
 // combinations of the corners, in the corners' original order. Band pair q is
 // stored at n_adj + q.
 //
-// Both rules are products of one triangle rule on each triangle, so every block
-// entry factors as sum_i w_i l_a(x_i) [sum_j w_j l_b(y_j) g(x_i, y_j)]: for each
-// x point the thread first sums the six kernels against the y points' three
-// basis values (18 FMA per point pair), then adds those partial sums into the
-// 3x3 blocks (54 FMA per x point). The sums of w G over the pair follow from
-// the single-layer blocks, the basis functions summing to one at every point.
-// The y points of both rules are staged in shared memory, per thread.
+// Bound by the FP64 pipe, so by the instructions of a point pair:
+//   - both rules are products of one triangle rule on each triangle, so every block
+//     entry factors as sum_i w_i l_a(x_i) [sum_j w_j l_b(y_j) g(x_i, y_j)]: for each x
+//     point the kernels are first summed over the y points, then added into the blocks;
+//   - the points come in orbits of three with l_b(y_j) = a + (1 - 3 a) [b = j mod 3], so
+//     the inner sums take two FMAs per kernel: one sum over the orbit and one per corner;
+//   - (x - y) . n_y is the height of x over the plane of y's triangle, whatever y: it
+//     multiplies the inner sums; (y - x) . n_x, the height of y, goes into y's weights.
+// 39 instructions a point pair (27 the kernels) and 92 an x point; 60 and 95 with the
+// normal products per point pair and three FMAs per kernel. 38,720 triangles, band of 3
+// radii, 6- and 3-point rules: 17.7 -> 9.9 ms (with full lanes, below). The y points of both rules are staged in
+// shared memory, per thread.
 constexpr int BAND_THREADS = 128;
 constexpr int ADJ_FAR_THREADS = 64;
+constexpr int BAND_Y = 5;  // doubles staged per y point: position, and a w and (1 - 3 a) w times its height
 
 // FP64 flops of one band pair under a Q-point rule by formula count: per point
-// pair the kernel evaluation (33, as for the regularised pairs) and the partial
-// sums (18 FMA); per point of either triangle its position (15); per x point
-// its weights (4) and the block updates (54 FMA).
-__host__ __device__ constexpr double band_flops(int Q) { return Q * Q * (33.0 + 36.0) + Q * (30.0 + 4.0 + 108.0); }
+// pair the kernels (d 3, r^2 5, rsqrt, r, exp and its argument 17, 1/r^2, the four
+// kernels 6: 33) and the sums (12 FMA); per point of either triangle its position (15) and
+// height (5); per x point its weights (6), the sums' ends (18) and the block updates (54 FMA).
+__host__ __device__ constexpr double band_flops(int Q) { return Q * Q * (33.0 + 24.0) + Q * (40.0 + 24.0 + 108.0); }
 
+// the Q points of a triangle with corners pb into ys (BAND_Y x Q slots, NT apart), their
+// heights over the plane through a0 with normal n
 template <int Q, int NT>
-__device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3], const double* ys,
-                                          const double (*wl)[3], const Rule& R, double wscale, const double* na,
-                                          const double* nb, double kappa) {
+__device__ __forceinline__ void stage_points(double* ys, const double (&pb)[3][3], const Rule& R, const double* a0,
+                                             const double* n) {
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+        double y[3], h = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            y[k] = R.l[j][0] * pb[0][k] + R.l[j][1] * pb[1][k] + R.l[j][2] * pb[2][k];
+            h += (y[k] - a0[k]) * n[k];
+            ys[(BAND_Y * j + k) * NT] = y[k];
+        }
+        const double a = R.l[j][Q == 1 ? 0 : (j + 1) % 3];
+        ys[(BAND_Y * j + 3) * NT] = R.w[j] * a * h;
+        ys[(BAND_Y * j + 4) * NT] = R.w[j] * (1.0 - 3.0 * a) * h;
+    }
+}
+
+// blocks: V_L, V_Y, K_L, K_Y at 0, 9, 18, 27; the reversed pair's K_L, K_Y at 38, 47 (without 1/(4 pi))
+template <int Q, int NT>
+__device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3], const double* ys, const Rule& R,
+                                          double wscale, const double* b0, const double* nb, double kappa, double t64) {
+    constexpr int ORB = Q == 1 ? 1 : 3;
 #pragma unroll 1
     for (int i = 0; i < Q; ++i) {
-        double x[3];
+        double x[3], hx = 0.0;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) x[k] = R.l[i][0] * pa[0][k] + R.l[i][1] * pa[1][k] + R.l[i][2] * pa[2][k];
-        double u[6][3];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) u[k][0] = u[k][1] = u[k][2] = 0.0;
-#pragma unroll 1
-        for (int j = 0; j < Q; ++j) {
-            const double d0 = x[0] - ys[(3 * j) * NT], d1 = x[1] - ys[(3 * j + 1) * NT],
-                         d2 = x[2] - ys[(3 * j + 2) * NT];
-            const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-            const double rinv = rsqrt(r2);
-            const double r = r2 * rinv;
-            const double gl = rinv * 0.07957747154594767;  // 1 / (4 pi r)
-            const double ek = exp_nonpos(-kappa * r);
-            const double fl = gl * rinv * rinv;  // 1 / (4 pi r^3)
-            const double fy_over_fl = ek * (1.0 + kappa * r);
-            const double kl = fl * (d0 * nb[0] + d1 * nb[1] + d2 * nb[2]);
-            const double ktl = fl * -(d0 * na[0] + d1 * na[1] + d2 * na[2]);  // (y - x).n_x
-            const double g[6] = {gl, ek * gl, kl, kl * fy_over_fl, ktl, ktl * fy_over_fl};
-#pragma unroll
-            for (int k = 0; k < 6; ++k)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) u[k][c] += g[k] * wl[j][c];
+        for (int k = 0; k < 3; ++k) {
+            x[k] = R.l[i][0] * pa[0][k] + R.l[i][1] * pa[1][k] + R.l[i][2] * pa[2][k];
+            hx += (x[k] - b0[k]) * nb[k];
         }
-        // blocks: V_L, V_Y, K_L, K_Y at 0, 9, 18, 27; the reversed pair's K_L, K_Y at 38, 47
+        double T[6], U[6][3];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) T[k] = U[k][0] = U[k][1] = U[k][2] = 0.0;
+#pragma unroll 1
+        for (int o = 0; o < Q; o += ORB) {
+            const double a = R.l[o][Q == 1 ? 0 : 1], al = R.w[o] * a, be = R.w[o] * (1.0 - 3.0 * a);
+            const double* yo = ys + BAND_Y * o * NT;
+#pragma unroll
+            for (int c = 0; c < ORB; ++c) {  // the orbit's point whose own corner is c
+                const double* y = yo + BAND_Y * c * NT;
+                const double d0 = x[0] - y[0], d1 = x[1] - y[NT], d2 = x[2] - y[2 * NT];
+                const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
+                const double rinv = rsqrt(r2);
+                const double e = exp2_64th((r2 * rinv) * t64);
+                const double ri2 = rinv * rinv, g = e * rinv;
+                const double v[4] = {rinv, g, rinv * ri2, __fma_rn(kappa, e, g) * ri2};
+                const double ah = y[3 * NT], bh = y[4 * NT];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    T[k] = __fma_rn(al, v[k], T[k]);
+                    U[k][c] = __fma_rn(be, v[k], U[k][c]);
+                }
+#pragma unroll
+                for (int k = 4; k < 6; ++k) {
+                    T[k] = __fma_rn(ah, v[k - 2], T[k]);
+                    U[k][c] = __fma_rn(bh, v[k - 2], U[k][c]);
+                }
+            }
+        }
         const double wi = wscale * R.w[i];
 #pragma unroll
+        for (int k = 0; k < 6; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) U[k][c] += T[k];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const double wa = wi * R.l[i][a];
+            const double wa = wi * R.l[i][a], wh = wa * hx;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const int base = k < 4 ? 9 * k : 38 + 9 * (k - 4);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) acc[base + 3 * a + c] += wa * u[k][c];
+                for (int c = 0; c < 3; ++c)
+                    acc[base + 3 * a + c] = __fma_rn(k == 2 || k == 3 ? wh : wa, U[k][c], acc[base + 3 * a + c]);
             }
         }
     }
@@ -891,23 +933,13 @@ __device__ __forceinline__ void write_blocks(double* acc, const double* gA, cons
 }
 
 template <int QF, int QC>
-__global__ void __launch_bounds__(BAND_THREADS, 2)
-k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
-             const int32_t* __restrict__ band_ptr, const int32_t* __restrict__ band_s,
-             const int32_t* __restrict__ band_t, int64_t n_band, int64_t n_adj, Rule fine, Rule coarse, double kappa,
-             double* __restrict__ ss_out, int* __restrict__ status) {
-    __shared__ double ysm[(QF + QC) * 3 * BAND_THREADS];
-    __shared__ double wl[2][6][3];  // w_j l_b(y_j) of the fine and the coarse rule
-    if (threadIdx.x < 36) {
-        const int r = threadIdx.x / 18, j = (threadIdx.x / 3) % 6, c = threadIdx.x % 3;
-        const Rule& R = r == 0 ? fine : coarse;
-        wl[r][j][c] = R.w[j] * R.l[j][c];
-    }
-    __syncthreads();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= n_band) return;  // no barrier follows
+__device__ __forceinline__ void band_pair(int64_t q, double* ys, const double* __restrict__ verts,
+                                          const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
+                                          const int32_t* __restrict__ band_ptr, const int32_t* __restrict__ band_s,
+                                          const int32_t* __restrict__ band_t, int64_t n_adj, const Rule& fine,
+                                          const Rule& coarse, double kappa, double* __restrict__ ss_out,
+                                          int* __restrict__ status) {
     const int32_t pt = band_t[q], ps = band_s[q];
-    if (pt > ps) return;  // the reverse of a pair handled by its other thread
     // the reversed pair: t among the partners of s (sorted)
     int32_t lo = band_ptr[ps], hi = band_ptr[ps + 1];
     while (lo < hi) {
@@ -920,7 +952,9 @@ k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
         return;
     }
     const int64_t p = n_adj + q, pr_rev = n_adj + lo;
-    double pa[3][3];
+    const double* gA = tgeo + 16 * (int64_t)pt;
+    const double* gB = tgeo + 16 * (int64_t)ps;
+    double pa[3][3], b0[3];
     {
         double pb[3][3];
 #pragma unroll
@@ -930,28 +964,56 @@ k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
                 pa[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)pt + a] + k];
                 pb[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)ps + a] + k];
             }
-        double* ys = ysm + threadIdx.x;
+        const double na[3] = {gA[0], gA[1], gA[2]};
+        stage_points<QF, BAND_THREADS>(ys, pb, fine, pa[0], na);
+        stage_points<QC, BAND_THREADS>(ys + BAND_Y * QF * BAND_THREADS, pb, coarse, pa[0], na);
 #pragma unroll
-        for (int j = 0; j < QF + QC; ++j) {
-            const Rule& R = j < QF ? fine : coarse;
-            const int jj = j < QF ? j : j - QF;
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-                ys[(3 * j + k) * BAND_THREADS] = R.l[jj][0] * pb[0][k] + R.l[jj][1] * pb[1][k] + R.l[jj][2] * pb[2][k];
-        }
+        for (int k = 0; k < 3; ++k) b0[k] = pb[0][k];
     }
-    const double* gA = tgeo + 16 * (int64_t)pt;
-    const double* gB = tgeo + 16 * (int64_t)ps;
-    const double na[3] = {gA[0], gA[1], gA[2]}, nb[3] = {gB[0], gB[1], gB[2]};
+    const double nb[3] = {gB[0], gB[1], gB[2]};
     double acc[NACC_SYM];
 #pragma unroll
     for (int k = 0; k < NACC_SYM; ++k) acc[k] = 0.0;
-    const double area2 = gA[3] * gB[3];
-    band_pass<QF, BAND_THREADS>(acc, pa, ysm + threadIdx.x, wl[0], fine, area2, na, nb, kappa);
-    band_pass<QC, BAND_THREADS>(acc, pa, ysm + threadIdx.x + 3 * QF * BAND_THREADS, wl[1], coarse, -area2, na, nb, kappa);
+    const double area2 = gA[3] * gB[3] * 0.07957747154594767, t64 = -kappa * EXP64_PER_UNIT;  // 1 / (4 pi)
+    band_pass<QF, BAND_THREADS>(acc, pa, ys, fine, area2, b0, nb, kappa, t64);
+    band_pass<QC, BAND_THREADS>(acc, pa, ys + BAND_Y * QF * BAND_THREADS, coarse, -area2, b0, nb, kappa, t64);
     write_blocks(acc, gA, gB, kappa, ss_out + 54 * p, ss_out + 54 * pr_rev);
 }
 
+// A block takes `span` consecutive entries of the band list, of which those with t < s are
+// integrated: it lists them first, so that its lanes stay full (with a thread per entry
+// about a third of the lanes of an active warp had nothing to do).
+constexpr int BAND_SPAN = 1024;
+template <int QF, int QC>
+__global__ void __launch_bounds__(BAND_THREADS, 2)
+k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
+             const int32_t* __restrict__ band_ptr, const int32_t* __restrict__ band_s,
+             const int32_t* __restrict__ band_t, int64_t n_band, int span, int64_t n_adj, Rule fine, Rule coarse,
+             double kappa, double* __restrict__ ss_out, int* __restrict__ status) {
+    __shared__ double ysm[(QF + QC) * BAND_Y * BAND_THREADS];
+    __shared__ uint16_t todo[BAND_SPAN];  // the block's entries with t < s, in order
+    __shared__ int wcnt[BAND_THREADS / 32];
+    const int64_t q0 = blockIdx.x * (int64_t)span;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int total = 0;
+    for (int k0 = 0; k0 < span; k0 += BAND_THREADS) {
+        const int64_t q = q0 + k0 + threadIdx.x;
+        const bool mine = q < n_band && band_t[q] < band_s[q];
+        const unsigned m = __ballot_sync(0xffffffffu, mine);
+        if (lane == 0) wcnt[wid] = __popc(m);
+        __syncthreads();
+        int at = total + __popc(m & ((1u << lane) - 1u));
+        for (int w = 0; w < BAND_THREADS / 32; ++w) {
+            if (w < wid) at += wcnt[w];
+            total += wcnt[w];
+        }
+        if (mine) todo[at] = (uint16_t)(k0 + threadIdx.x);
+        __syncthreads();
+    }
+    for (int k = threadIdx.x; k < total; k += BAND_THREADS)
+        band_pair<QF, QC>(q0 + todo[k], ysm + threadIdx.x, verts, tris, tgeo, band_ptr, band_s, band_t, n_adj, fine,
+                          coarse, kappa, ss_out, status);
+}
 // The far rule's blocks of the adjacent pairs (what the pair kernel adds for them):
 // one thread per pair and its reverse, by the band pairs' sums. (As a lane's share of
 // a warp per pair, 9 or 36 point pairs left most lanes idle: 260 FP64 instructions of
@@ -961,12 +1023,9 @@ __global__ void __launch_bounds__(ADJ_FAR_THREADS)
 k_adj_far(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
           const int4* __restrict__ pairs, const int32_t* __restrict__ list, int64_t nlist,
           const int32_t* __restrict__ rev, Rule rule, double kappa, double* __restrict__ far_out) {
-    __shared__ double ysm[Q * 3 * ADJ_FAR_THREADS];
-    __shared__ double wl[6][3];  // w_j l_b(y_j)
-    if (threadIdx.x < 3 * Q) wl[threadIdx.x / 3][threadIdx.x % 3] = rule.w[threadIdx.x / 3] * rule.l[threadIdx.x / 3][threadIdx.x % 3];
-    __syncthreads();
+    __shared__ double ysm[Q * BAND_Y * ADJ_FAR_THREADS];
     const int64_t li = blockIdx.x * (int64_t)ADJ_FAR_THREADS + threadIdx.x;
-    if (li >= nlist) return;  // no barrier follows
+    if (li >= nlist) return;
     const int64_t p = list[li];
     const int4 pr = pairs[p];
     double pa[3][3], pb[3][3];
@@ -977,19 +1036,15 @@ k_adj_far(const double* __restrict__ verts, const int32_t* __restrict__ tris, co
             pa[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)pr.x + a] + k];
             pb[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)pr.y + a] + k];
         }
-#pragma unroll
-    for (int j = 0; j < Q; ++j)
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            ysm[(3 * j + k) * ADJ_FAR_THREADS + threadIdx.x] =
-                rule.l[j][0] * pb[0][k] + rule.l[j][1] * pb[1][k] + rule.l[j][2] * pb[2][k];
     const double* gA = tgeo + 16 * (int64_t)pr.x;
     const double* gB = tgeo + 16 * (int64_t)pr.y;
     const double na[3] = {gA[0], gA[1], gA[2]}, nb[3] = {gB[0], gB[1], gB[2]};
+    stage_points<Q, ADJ_FAR_THREADS>(ysm + threadIdx.x, pb, rule, pa[0], na);
     double acc[NACC_SYM];
 #pragma unroll
     for (int k = 0; k < NACC_SYM; ++k) acc[k] = 0.0;
-    band_pass<Q, ADJ_FAR_THREADS>(acc, pa, ysm + threadIdx.x, wl, rule, gA[3] * gB[3], na, nb, kappa);
+    band_pass<Q, ADJ_FAR_THREADS>(acc, pa, ysm + threadIdx.x, rule, gA[3] * gB[3] * 0.07957747154594767, pb[0], nb,
+                                  kappa, -kappa * EXP64_PER_UNIT);
     write_blocks(acc, gA, gB, kappa, far_out + 54 * p, far_out + 54 * (int64_t)rev[p]);
 }
 
@@ -1253,8 +1308,11 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
             const double ppairs = 0.5 * m->n_band * (Qb * Qb + Q * Q);
             Timer tm(ctx, PB_KERNEL_NEAR_BAND, s, ppairs,
                      0.5 * m->n_band * (band_flops(m->Qr) + band_flops(m->Q)) / ppairs);
-            const unsigned gb = (unsigned)((m->n_band + BAND_THREADS - 1) / BAND_THREADS);
-#define PB_BAND_ARGS m->verts, m->tris, m->tgeo, m->band_ptr, m->band_s, m->band_t, m->n_band, m->n_adj, fine, \
+            // few entries: smaller shares, so that every SM has some
+            int span = BAND_SPAN;
+            while (span > 2 * BAND_THREADS && m->n_band < (int64_t)4 * ctx->num_sms * span) span /= 2;
+            const unsigned gb = (unsigned)((m->n_band + span - 1) / span);
+#define PB_BAND_ARGS m->verts, m->tris, m->tgeo, m->band_ptr, m->band_s, m->band_t, m->n_band, span, m->n_adj, fine, \
                      coarse, kappa, ss, m->status
             if (m->Qr == 6 && m->Q == 3) k_band_pairs<6, 3><<<gb, BAND_THREADS, 0, s>>>(PB_BAND_ARGS);
             else if (m->Qr == 6 && m->Q == 1) k_band_pairs<6, 1><<<gb, BAND_THREADS, 0, s>>>(PB_BAND_ARGS);

@@ -1,6 +1,6 @@
-"""Near field of adjacent pairs against the oracle over what selects its code path: the lanes per pair (few or many
+"""Near field of adjacent and band pairs against the oracle over what selects its code path: the lanes per pair (few or many
 pairs), the degree of the Yukawa polynomials (kappa times the triangles' size, past their range the exponentials), the
-singular order and the far rule. One FP64 application per operator; tolerance as the operator parity tests (1e-12)."""
+singular order, the far rule and the band's rules. One FP64 application per operator; tolerance as the operator parity tests (1e-12)."""
 import numpy as np
 import pytest
 
@@ -42,6 +42,13 @@ def test_yukawa_sums_at_every_degree(kappa):
 def test_orders_and_far_rules(plan):
     v, t = uv_ellipsoid(9, 8, (2.0, 1.6, 1.3), center=(0.3, -0.2, 0.1), twist=0.15)
     check(v, t, 0.125, plan)
+
+
+@pytest.mark.parametrize("far_q,band_q,eta", [(3, 6, 2.0), (1, 6, 1.5), (1, 3, 6.0)])
+@pytest.mark.parametrize("n_lon,n_lat", [(9, 8), (31, 29)])
+def test_band_rules(n_lon, n_lat, far_q, band_q, eta):
+    v, t = uv_ellipsoid(n_lon, n_lat, (2.0, 1.6, 1.3), center=(0.3, -0.2, 0.1), twist=0.15)
+    check(v, t, 0.125, {"far_q": far_q, "n_ss": 3, "band_eta": eta, "band_q": band_q})
 
 
 @pytest.mark.parametrize("n_lon,n_lat,length", [(31, 29, 2.3), (20, 190, 14.0)])

@@ -46,7 +46,6 @@ NCU_TRAFFIC = {  # (kernel family, formulation or "any", far-rule points, band) 
     ("spmv", "juffer", 667788, 3.0): 337.5e6,
     ("tree32", "juffer", 667788, 3.0): 246.8e6,
     ("pair32acc", "juffer", 667788, 3.0): 496.5e6,
-    ("near_coin", "any", 667788, 3.0): 233.9e6,
 }
 
 
@@ -272,7 +271,7 @@ def _kernels():
             pb.PB_KERNEL_PAIR64: ("k_pair64 (FP64 far field)", "pair64", "alu", FP64_FLOPS_PER_SM, "FP64 flops"),
             pb.PB_KERNEL_NEAR_ADJ: ("k_adj_pairs (FP64 singular quadrature, edge/vertex pairs)", "near_adj", "alu",
                                     FP64_FLOPS_PER_SM, "FP64 flops"),
-            pb.PB_KERNEL_NEAR_COIN: ("k_coin_pairs (FP64 singular quadrature, coincident pairs)", "near_coin", "alu",
+            pb.PB_KERNEL_NEAR_COIN: ("k_coin_poly (FP64 singular quadrature, coincident pairs)", "near_coin", "alu",
                                      FP64_FLOPS_PER_SM, "FP64 flops"),
             pb.PB_KERNEL_NEAR_BAND: ("k_band_pairs (FP64 band-rule corrections)", "near_band", "alu",
                                      FP64_FLOPS_PER_SM, "FP64 flops"),

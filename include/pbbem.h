@@ -437,9 +437,10 @@ int pb_autotune_plan(pb_ctx* ctx, const double* verts, int64_t n_verts, const in
 #define PB_KERNEL_COUNT 10
 /* For the pair kernels, "pairs" are target-source point pairs and "ops" FP32
  * (FP64 for PB_KERNEL_PAIR64) operations by the kernel's formula count; for
- * the near-field kernels, "pairs" are quadrature point pairs (kernel
- * evaluations) and "ops" FP64 flops by formula count (kernel evaluation and
- * accumulation into the local blocks, a fused multiply-add counted as two).
+ * the near-field kernels, "pairs" are quadrature point pairs of the rules (the
+ * kernels evaluate fewer: some of the sums are taken in closed form) and "ops"
+ * FP64 flops by formula count (kernel evaluation and accumulation into the local
+ * blocks, a fused multiply-add counted as two).
  * For the memory-bound families (SPMV, CHEB, KRYLOV) "pairs" and "ops" are
  * both the algorithmic bytes of the launches: every array element the launch
  * must read or write, counted once. */
@@ -457,8 +458,9 @@ int pb_profile_read(pb_ctx* ctx, int kernel, int64_t* launches, double* total_ms
  * *status_out receives the status word the kernel wrote (PB_ETIMEOUT when the
  * wait ran out). The kernel returns normally and the context stays usable. */
 int pb_selftest_wait(pb_ctx* ctx, int64_t polls, int* status_out);
-/* Self-test of the exponential the FP64 near-field kernels use for the Yukawa
- * factor e^{-kappa r} (a table-driven e^x for x <= 0 after Tang, ACM TOMS
+/* Self-test of the exponential of the adjacent triangle pairs' Yukawa factor
+ * e^{-kappa r} where kappa times the triangles' size is too large for their
+ * polynomials (a table-driven e^x for x <= 0 after Tang, ACM TOMS
  * 15(2), 1989): y[i] = e^{x[i]} for the n device doubles x (each <= 0; 0 is
  * returned below -700), on `stream` (NULL: the default stream), synchronised
  * before return. x and y are caller-owned device buffers of n doubles. */

@@ -457,7 +457,7 @@ static int load(pb_ctx* ctx, const double* verts_in, int64_t nv, const int32_t* 
         }
     double diag2 = 0.0;
     for (int k = 0; k < 3; ++k) diag2 += (hi[k] - lo[k]) * (hi[k] - lo[k]);
-    double vol6 = 0.0;
+    double vol6 = 0.0, edge2 = 0.0;  // edge2: the longest edge, squared
     for (int64_t t = 0; t < nt; ++t) {
         const int32_t* f = &T[3 * t];
         for (int a = 0; a < 3; ++a)
@@ -475,9 +475,17 @@ static int load(pb_ctx* ctx, const double* verts_in, int64_t nv, const int32_t* 
         double a2 = c0 * c0 + c1 * c1 + c2 * c2;
         if (!(a2 > 1e-24 * diag2 * diag2))
             return set_error(PB_EMESH, "triangle %lld has (near) zero area", (long long)t);
+        double e0 = 0.0, e1 = 0.0, e2 = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            e0 += u[k] * u[k];
+            e1 += w[k] * w[k];
+            e2 += (u[k] - w[k]) * (u[k] - w[k]);
+        }
+        edge2 = std::max(edge2, std::max(e0, std::max(e1, e2)));
         vol6 += p0[0] * (p1[1] * p2[2] - p1[2] * p2[1]) - p0[1] * (p1[0] * p2[2] - p1[2] * p2[0]) +
                 p0[2] * (p1[0] * p2[1] - p1[1] * p2[0]);
     }
+    m->max_edge = std::sqrt(edge2);
     tr.lap("validate");
 
     // ---- vertex -> triangle map

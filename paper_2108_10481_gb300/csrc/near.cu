@@ -572,10 +572,12 @@ constexpr int NEAR_THREADS = 128;
 // kernels (2 FMA, 2), eta3 products (3), sums (6 + 15 FMA): 155; an entry: D0, D1 and
 // the heights (17 FMA, 7), the moments (6 x 14 FMA): 209. A coincident pair's point
 // (moments from the rule's table of weighted monomials): d from (s - s', t - t') (11),
-// r^2 to the Yukawa single layer (11), 2 x 2 x 9 (36).
+// r^2 to the Yukawa single layer (11), 2 x 2 x 9 (36); by the polynomials (k_coin_poly), per
+// direction: v and r^2 (24), rsqrt, r, z (3), the Yukawa moments (18 a degree), both kernels' (36).
 constexpr double NEAR_FLOPS_ADJ_POINT = 155;
 constexpr double NEAR_FLOPS_ADJ_ENTRY = 209;
 constexpr double NEAR_FLOPS_COIN = 22 + 36;
+static double coin_dir_flops(int deg) { return 63.0 + 18.0 * deg; }
 
 // Regularised blocks of the adjacent pairs of one class: G lanes per listed pair
 // (one of each two reversed ones) over the entries of the class's map, their
@@ -740,9 +742,9 @@ __device__ __forceinline__ void accum_v(double* acc, double w, const double* x, 
     acc[19] += w * gy;
 }
 
-__device__ void expand_coin(const double* acc, const TriFrame& A, const double* tgeoA, double kappa, double* out) {
-    const double nn = A.n[0] * A.n[0] + A.n[1] * A.n[1] + A.n[2] * A.n[2];
-    const double f = 1.0 / (4.0 * A.area * A.area);
+__device__ __forceinline__ void expand_coin(const double* acc, const double* tgeoA, double kappa, double* out) {
+    const double nn = tgeoA[0] * tgeoA[0] + tgeoA[1] * tgeoA[1] + tgeoA[2] * tgeoA[2];
+    const double f = 1.0 / (4.0 * tgeoA[3] * tgeoA[3]);
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) {
             const double* ea = tgeoA + 4 + 3 * a;
@@ -789,7 +791,7 @@ k_coin_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
         acc[19] = mom[9];
     }
     const double* gA = tgeo + 16 * (int64_t)pr.x;
-    if (lane == 0) expand_coin(acc, A, gA, kappa, ss_out + 54 * p);
+    if (lane == 0) expand_coin(acc, gA, kappa, ss_out + 54 * p);
     for (int k = 0; k < 20; ++k) acc[k] = 0.0;
     const int Q = rule.Q;
     for (int idx = lane; idx < Q * Q; idx += 32) {
@@ -804,7 +806,146 @@ k_coin_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
         accum_v(acc, w, x, y, rule.l[i], rule.l[j], kappa);
     }
     warp_allsum<20, 32>(acc, lane, red[wid]);
-    if (lane == 0) expand_coin(acc, A, gA, kappa, far_out + 54 * p);
+    if (lane == 0) expand_coin(acc, gA, kappa, far_out + 54 * p);
+}
+
+// The same by the structure of the coincident map: in regions 0..2 x - y = rho v(eta3) with
+// rho = xi eta1 eta2, so r = rho |v| takes 3 n directions per triangle, the Laplace moments
+// over (xi, eta1, eta2) are constants over |v|, and the Yukawa ones polynomials of z =
+// kappa |v| (as the adjacent pairs' E_m, RAD_DEG). Four lanes per triangle share the
+// directions and the far rule's point pairs. Table entry
+// (direction q = region n + j, moment c, k), at tab[(q (RAD_DEG + 1) + k) 9 + c]: the rule's sum
+// of w mono_c rho^{k - 1} (-1)^k / k!; then 3 n pairs (s - s', t - t') of v.
+// n = 4, 38,720 triangles: 1.70 -> 0.23 ms; 2,000: 223 -> 72 us. Used while kappa times the
+// longest edge is within the polynomials' range; beyond, k_coin_pairs.
+constexpr int COIN_STRIDE = 9 * (RAD_DEG + 1);
+static_assert(sizeof(double) * 36 * (COIN_STRIDE + 2) <= (48u << 10), "the table at n = 12 in shared memory");
+
+// a warp per (direction, moment), its lanes over the points (xi, eta1, eta2)
+__global__ void k_coin_table(Gauss gq, double* __restrict__ tab) {
+    const int n = gq.n, e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (e >= 3 * n * 9) return;  // whole warps
+    const int q = e / 9, c = e % 9, reg = q / n, j = q % n;
+    double v[RAD_DEG + 1], sx, tx, sy, ty;
+#pragma unroll
+    for (int k = 0; k <= RAD_DEG; ++k) v[k] = 0.0;
+    for (int i = lane; i < n * n * n; i += 32) {
+        const int i0 = i / (n * n), i1 = (i / n) % n, i2 = i % n;
+        const double jac = ss_map(0, reg, gq.x[i0], gq.x[i1], gq.x[i2], gq.x[j], sx, tx, sy, ty);
+        const double rho = gq.x[i0] * gq.x[i1] * gq.x[i2];
+        const double px = c < 3 ? 1.0 : c < 6 ? sx : tx, py = c % 3 == 0 ? 1.0 : c % 3 == 1 ? sy : ty;
+        double t = gq.w[i0] * gq.w[i1] * gq.w[i2] * gq.w[j] * jac * px * py / rho;
+#pragma unroll
+        for (int k = 0; k <= RAD_DEG; ++k) {
+            v[k] += t;
+            t *= rho * (-1.0 / (k + 1));
+        }
+    }
+#pragma unroll
+    for (int k = 0; k <= RAD_DEG; ++k)
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane > 0) return;
+#pragma unroll
+    for (int k = 0; k <= RAD_DEG; ++k) tab[q * COIN_STRIDE + 9 * k + c] = v[k];
+    if (c == 0) {
+        ss_map(0, reg, 1.0, 1.0, 1.0, gq.x[j], sx, tx, sy, ty);
+        tab[3 * n * COIN_STRIDE + 2 * q] = sx - sy;
+        tab[3 * n * COIN_STRIDE + 2 * q + 1] = tx - ty;
+    }
+}
+
+constexpr int COIN_THREADS = 128;
+constexpr int COIN_LANES = 4;  // per triangle
+
+__global__ void __launch_bounds__(COIN_THREADS)
+k_coin_poly(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
+            const int4* __restrict__ pairs, const int32_t* __restrict__ list, int64_t nlist, int n, int deg,
+            const double* __restrict__ table, Rule rule, double kappa, double* __restrict__ ss_out,
+            double* __restrict__ far_out) {
+    extern __shared__ double tab[];
+    for (int k = threadIdx.x; k < 3 * n * (COIN_STRIDE + 2); k += COIN_THREADS) tab[k] = table[k];
+    __syncthreads();
+    const int gl = threadIdx.x % COIN_LANES;
+    const int64_t li = (blockIdx.x * (int64_t)COIN_THREADS + threadIdx.x) / COIN_LANES;
+    const bool live = li < nlist;  // the last block's spare lanes repeat the last triangle and write nothing
+    const int64_t p = list[live ? li : nlist - 1];
+    const int32_t t = pairs[p].x;
+    const double* g = tgeo + 16 * (int64_t)t;
+    double c[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) c[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)t + a] + k];
+    double mom[18];
+#pragma unroll
+    for (int k = 0; k < 18; ++k) mom[k] = 0.0;
+    const double* dir = tab + 3 * n * COIN_STRIDE;
+    for (int q = gl; q < 3 * n; q += COIN_LANES) {
+        const double ds = dir[2 * q], dt = dir[2 * q + 1];
+        double r2 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {  // v = ds e1 + dt e2, e1 = c1 - c0, e2 = c2 - c1
+            const double v = __fma_rn(dt, c[2][k] - c[1][k], ds * (c[1][k] - c[0][k]));
+            r2 = __fma_rn(v, v, r2);
+        }
+        const double rinv = rsqrt(r2), z = kappa * (r2 * rinv);
+        const double* tq = tab + q * COIN_STRIDE;
+        double y[9];
+#pragma unroll
+        for (int m = 0; m < 9; ++m) y[m] = tq[9 * deg + m];
+        for (int k = deg - 1; k >= 0; --k)
+#pragma unroll
+            for (int m = 0; m < 9; ++m) y[m] = __fma_rn(y[m], z, tq[9 * k + m]);
+#pragma unroll
+        for (int m = 0; m < 9; ++m) {
+            mom[m] = __fma_rn(rinv, tq[m], mom[m]);
+            mom[9 + m] = __fma_rn(rinv, y[m], mom[9 + m]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 18; ++k)
+        for (int o = COIN_LANES / 2; o > 0; o >>= 1) mom[k] += __shfl_xor_sync(0xffffffffu, mom[k], o);
+    double acc[20];  // the far rule's point pairs i < j
+#pragma unroll
+    for (int k = 0; k < 20; ++k) acc[k] = 0.0;
+    int ij = 0;
+    for (int i = 0; i < rule.Q; ++i)
+        for (int j = i + 1; j < rule.Q; ++j, ++ij) {
+            if (ij % COIN_LANES != gl) continue;
+            double x[3], y[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                x[k] = rule.l[i][0] * c[0][k] + rule.l[i][1] * c[1][k] + rule.l[i][2] * c[2][k];
+                y[k] = rule.l[j][0] * c[0][k] + rule.l[j][1] * c[1][k] + rule.l[j][2] * c[2][k];
+            }
+            accum_v(acc, rule.w[i] * g[3] * rule.w[j] * g[3], x, y, rule.l[i], rule.l[j], kappa);
+        }
+#pragma unroll
+    for (int k = 0; k < 20; ++k)
+        for (int o = COIN_LANES / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    // lane 0 writes the regularised blocks, lane 1 the far rule's
+    const double scale = 4.0 * g[3] * g[3] * 0.07957747154594767;  // the Jacobians and 1/(4 pi)
+    if (gl == 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            double R[3][3];
+            const double* mh = mom + 9 * h;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                R[0][b] = mh[b] - mh[3 + b];
+                R[1][b] = mh[3 + b] - mh[6 + b];
+                R[2][b] = mh[6 + b];
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                acc[9 * h + 3 * a] = scale * (R[a][0] - R[a][1]);
+                acc[9 * h + 3 * a + 1] = scale * (R[a][1] - R[a][2]);
+                acc[9 * h + 3 * a + 2] = scale * R[a][2];
+            }
+            acc[18 + h] = scale * mh[0];
+        }
+    }
+    if (live && gl < 2) expand_coin(acc, g, kappa, (gl ? far_out : ss_out) + 54 * p);
 }
 
 // Band pairs (share no vertex, closer than the plan's band): the blocks of the
@@ -1014,6 +1155,7 @@ k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
         band_pair<QF, QC>(q0 + todo[k], ysm + threadIdx.x, verts, tris, tgeo, band_ptr, band_s, band_t, n_adj, fine,
                           coarse, kappa, ss_out, status);
 }
+
 // The far rule's blocks of the adjacent pairs (what the pair kernel adds for them):
 // one thread per pair and its reverse, by the band pairs' sums. (As a lane's share of
 // a warp per pair, 9 or 36 point pairs left most lanes idle: 260 FP64 instructions of
@@ -1050,15 +1192,19 @@ k_adj_far(const double* __restrict__ verts, const int32_t* __restrict__ tris, co
 
 // One warp per row i. The warp walks the contributions of the row in a fixed
 // order (the triangles t of i; each one's adjacent pairs, then its band pairs;
-// the trial corner b), 32 at a time: each lane finds its contribution's
-// column position (binary search in the row's sorted columns) and stages its
-// values; then the lane that owns a position (position mod 32) adds the
-// staged values for it in slot order. Every entry therefore sums its
-// contributions in the walk's order, whatever the scheduling. Adjacent pairs
-// (p < n_adj) hold the regularised blocks in ss and the far rule's in far;
-// band pairs hold the difference in ss. The row's accumulators (6 operators
-// and M) live in shared memory, maxrow entries per warp.
-constexpr int ROW_STAGE = 13;  // near[6], full[6] (kept for the diagonal), mass; positions apart (ints)
+// the trial corner b), BATCH (128) at a time: each lane finds its contributions'
+// column positions (binary search in the row's sorted columns) and stages their
+// six values; then the two lanes that own a position (position mod 16; three
+// operators each) add the staged values for it in slot order. Every entry
+// therefore sums its contributions in the walk's order, whatever the scheduling.
+// Adjacent pairs (p < n_adj) hold the regularised blocks in ss and the far rule's in
+// far; band pairs hold the difference in ss. The row's accumulators (6 operators and
+// M) live in shared memory, maxrow entries per warp. Bound by the FP64 additions of
+// the busiest lane of a batch: with 32 slots a batch, seven values and a lane per
+// position, its busiest lane had nearly four times the average (38,720 triangles, band
+// of 3 radii: 3.28 -> 2.00 ms).
+// Batches of 32 are for rows so long that a warp's shared memory holds no more.
+constexpr int ROW_OWNERS = 16;
 
 __device__ __forceinline__ int row_lower_bound(const int32_t* c, int n, int32_t v) {
     int lo = 0, hi = n;
@@ -1070,11 +1216,14 @@ __device__ __forceinline__ int row_lower_bound(const int32_t* c, int n, int32_t 
     return lo;
 }
 
-// shared memory of one warp, in doubles
-__host__ __device__ inline size_t row_warp_doubles(int maxrow) {
-    return 32 * ROW_STAGE + 16 + 7 * (size_t)maxrow + ((size_t)maxrow + 1) / 2;
+// shared memory of one warp, in doubles: the staged values, positions and adjacent pairs of
+// a batch; seven accumulators and the column of every entry (even: values are staged by
+// 16-byte stores)
+__host__ __device__ inline size_t row_warp_doubles(int batch, int maxrow) {
+    return (7 * (size_t)batch + 7 * (size_t)maxrow + ((size_t)maxrow + 1) / 2 + 1) / 2 * 2;
 }
 
+template <int BATCH>
 __global__ void k_near_rows(int64_t nv, int64_t nnz, int maxrow, int warps, const int32_t* __restrict__ row_ptr,
                             const int32_t* __restrict__ col, const int32_t* __restrict__ v2t_ptr,
                             const int32_t* __restrict__ v2t, const int32_t* __restrict__ tris,
@@ -1082,93 +1231,119 @@ __global__ void k_near_rows(int64_t nv, int64_t nnz, int maxrow, int warps, cons
                             const int32_t* __restrict__ band_ptr, const int32_t* __restrict__ band_s, int64_t n_adj,
                             const double* __restrict__ tgeo, const double* __restrict__ ss,
                             const double* __restrict__ far, double* __restrict__ val, double* __restrict__ diag) {
-    extern __shared__ double rsm[];
+    static_assert(BATCH == 32 || BATCH == 128, "the owned slots are kept in two 64-bit words");
+    extern __shared__ __align__(16) double rsm[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * warps + w;
     if (i >= nv) return;  // whole warps
-    double* stage = rsm + (size_t)w * row_warp_doubles(maxrow);
-    int32_t* spos = (int32_t*)(stage + 32 * ROW_STAGE);  // 32 ints
-    double* acc = stage + 32 * ROW_STAGE + 16;
-    int32_t* scol = (int32_t*)(acc + 7 * (size_t)maxrow);
+    double* stage = rsm + (size_t)w * row_warp_doubles(BATCH, maxrow);
+    int32_t* spos = (int32_t*)(stage + BATCH * 6);  // BATCH positions
+    int32_t* sadj = spos + BATCH;                   // the adjacent pair of a slot on the diagonal, or -1
+    double* acc = stage + BATCH * 7;
+    double* accm = acc + 6 * (size_t)maxrow;
+    int32_t* scol = (int32_t*)(accm + maxrow);
     const int32_t r0 = row_ptr[i];
     const int n = row_ptr[i + 1] - r0;  // <= maxrow
-    for (int k = lane; k < n; k += 32) scol[k] = col[r0 + k];
-    for (int k = lane; k < 7 * n; k += 32) acc[k] = 0.0;
+    for (int k = lane; k < n; k += 32) {
+        scol[k] = col[r0 + k];
+        accm[k] = 0.0;
+    }
+    for (int k = lane; k < 6 * n; k += 32) acc[k] = 0.0;
     __syncwarp();
     const int diag_pos = row_lower_bound(scol, n, (int32_t)i);
-    double dfull[6] = {0, 0, 0, 0, 0, 0};  // the diagonal entry's full values (kept by its owner lane)
+    const int owner = lane & (ROW_OWNERS - 1), half = lane / ROW_OWNERS;
+    double dfull[3] = {0, 0, 0};  // the diagonal entry's full values (kept by its owner lanes)
     for (int32_t k = v2t_ptr[i]; k < v2t_ptr[i + 1]; ++k) {
         const int32_t t = v2t[k] / 3, a = v2t[k] % 3;
         const int32_t p0 = adj_ptr[t], L1 = adj_ptr[t + 1] - p0;
         const int32_t q0 = band_ptr ? band_ptr[t] : 0, L2 = band_ptr ? band_ptr[t + 1] - q0 : 0;
         const int total = 3 * (L1 + L2);
-        for (int c0 = 0; c0 < total; c0 += 32) {
-            const int c = c0 + lane;
-            if (c < total) {
-                double* my = stage + lane * ROW_STAGE;
-                const int idx = c / 3, b = c - 3 * idx, ab = 3 * a + b;
-                if (idx < L1) {
-                    const int64_t pp = p0 + idx;
-                    const int4 pr = pairs[pp];
-                    const int32_t j = tris[3 * (int64_t)pr.y + b];
-                    spos[lane] = row_lower_bound(scol, n, j);
-                    const double2* s2 = reinterpret_cast<const double2*>(ss + 54 * pp + 6 * ab);
-                    const double2* f2 = reinterpret_cast<const double2*>(far + 54 * pp + 6 * ab);
+        // the triangle's own mass entries
+        if (lane < 3) {
+            const int pos = row_lower_bound(scol, n, tris[3 * (int64_t)t + lane]);
+            accm[pos] += tgeo[16 * (int64_t)t + 3] / 12.0 * (lane == a ? 2.0 : 1.0);
+        }
+        for (int c0 = 0; c0 < total; c0 += BATCH) {
+            const int m = min(BATCH, total - c0);
+            unsigned own[BATCH / 32];
 #pragma unroll
-                    for (int h = 0; h < 3; ++h) {
-                        const double2 sv = s2[h], fv = f2[h];
-                        my[2 * h] = sv.x - fv.x;
-                        my[2 * h + 1] = sv.y - fv.y;
-                        my[6 + 2 * h] = sv.x;
-                        my[7 + 2 * h] = sv.y;
-                    }
-                    my[12] = pr.z == 0 ? tgeo[16 * (int64_t)pr.x + 3] / 12.0 * ((ab % 4 == 0) ? 2.0 : 1.0) : 0.0;
-                } else {
-                    const int32_t q = q0 + idx - L1;
-                    const int64_t pp = n_adj + q;
-                    const int32_t j = tris[3 * (int64_t)band_s[q] + b];
-                    spos[lane] = row_lower_bound(scol, n, j);
-                    const double2* s2 = reinterpret_cast<const double2*>(ss + 54 * pp + 6 * ab);
+            for (int g = 0; g < BATCH / 32; ++g) {
+                const int sl = 32 * g + lane, c = c0 + sl;
+                int pos = -1;
+                if (sl < m) {
+                    double2* my = reinterpret_cast<double2*>(stage + 6 * sl);
+                    const int idx = c / 3, b = c - 3 * idx, ab = 3 * a + b;
+                    int at = -1;
+                    if (idx < L1) {
+                        const int64_t pp = p0 + idx;
+                        const int32_t j = tris[3 * (int64_t)pairs[pp].y + b];
+                        pos = row_lower_bound(scol, n, j);
+                        if (pos == diag_pos) at = (int32_t)pp;
+                        const double2* s2 = reinterpret_cast<const double2*>(ss + 54 * pp + 6 * ab);
+                        const double2* f2 = reinterpret_cast<const double2*>(far + 54 * pp + 6 * ab);
 #pragma unroll
-                    for (int h = 0; h < 3; ++h) {
-                        const double2 sv = s2[h];
-                        my[2 * h] = sv.x;
-                        my[2 * h + 1] = sv.y;
+                        for (int h = 0; h < 3; ++h) {
+                            const double2 sv = s2[h], fv = f2[h];
+                            my[h] = make_double2(sv.x - fv.x, sv.y - fv.y);
+                        }
+                    } else {
+                        const int32_t q = q0 + idx - L1;
+                        const double2* s2 = reinterpret_cast<const double2*>(ss + 54 * (n_adj + q) + 6 * ab);
+                        const double2 v0 = s2[0], v1 = s2[1], v2 = s2[2];
+                        pos = row_lower_bound(scol, n, tris[3 * (int64_t)band_s[q] + b]);
+                        my[0] = v0;
+                        my[1] = v1;
+                        my[2] = v2;
                     }
-                    for (int o = 0; o < 6; ++o) my[6 + o] = 0.0;  // band pairs never touch the diagonal
-                    my[12] = 0.0;
+                    spos[sl] = pos;
+                    sadj[sl] = at;
+                }
+                // the slots whose position this lane owns
+                const int o = pos < 0 ? -1 : pos & (ROW_OWNERS - 1);
+                own[g] = 0;
+#pragma unroll
+                for (int q = 0; q < ROW_OWNERS; ++q) {
+                    const unsigned b = __ballot_sync(0xffffffffu, o == q);
+                    if (q == owner) own[g] = b;
                 }
             }
             __syncwarp();
-            // the slots this lane owns, then their values in slot order (lanes in parallel)
-            const int m = min(32, total - c0);
-            unsigned own = 0;
-            for (int sl = 0; sl < m; ++sl)
-                if ((spos[sl] & 31) == lane) own |= 1u << sl;
-            while (own) {
-                const int sl = __ffs(own) - 1;
-                own &= own - 1;
-                const double* st = stage + sl * ROW_STAGE;
-                const int pos = spos[sl];
-                double* e = acc + 7 * (size_t)pos;
-                for (int o = 0; o < 6; ++o) e[o] += st[o];
-                e[6] += st[12];
-                if (pos == diag_pos)
-                    for (int o = 0; o < 6; ++o) dfull[o] += st[6 + o];
+            unsigned long long lo = own[0], hi = 0;
+            if (BATCH == 128) {
+                lo |= (unsigned long long)own[BATCH / 32 > 1 ? 1 : 0] << 32;
+                hi = own[BATCH / 32 > 2 ? 2 : 0] | (unsigned long long)own[BATCH / 32 > 3 ? 3 : 0] << 32;
+            }
+            while (lo | hi) {  // in slot order
+                int sl;
+                if (lo) {
+                    sl = __ffsll((long long)lo) - 1;
+                    lo &= lo - 1;
+                } else {
+                    sl = 63 + __ffsll((long long)hi);
+                    hi &= hi - 1;
+                }
+                const double* st = stage + 6 * sl + 3 * half;
+                double* e = acc + 6 * (size_t)spos[sl] + 3 * half;
+                const int32_t at = sadj[sl];
+#pragma unroll
+                for (int o = 0; o < 3; ++o) e[o] += st[o];
+                if (at >= 0)
+#pragma unroll
+                    for (int o = 0; o < 3; ++o)
+                        dfull[o] += ss[54 * (int64_t)at + 6 * (3 * a + (c0 + sl) % 3) + 3 * half + o];
             }
             __syncwarp();
         }
     }
     const int map[6] = {N_VL, N_KL, N_DL, N_VY, N_KY, N_DY};
-    for (int k = lane; k < n; k += 32) {
-        const double* e = acc + 7 * (size_t)k;
-        for (int o = 0; o < 6; ++o) val[map[o] * nnz + r0 + k] = e[o];
-        val[N_M * nnz + r0 + k] = e[6];
-        if (k == diag_pos) {
-            for (int o = 0; o < 6; ++o) diag[map[o] * nv + i] = dfull[o];
-            diag[N_M * nv + i] = e[6];
-        }
-    }
+#pragma unroll
+    for (int o = 0; o < 6; ++o)
+        for (int k = lane; k < n; k += 32) val[map[o] * nnz + r0 + k] = acc[6 * (size_t)k + o];
+    for (int k = lane; k < n; k += 32) val[N_M * nnz + r0 + k] = accm[k];
+    if (owner == (diag_pos & (ROW_OWNERS - 1)))
+#pragma unroll
+        for (int o = 0; o < 3; ++o) diag[(half ? map[3 + o] : map[o]) * nv + i] = dfull[o];
+    if (lane == 0) diag[N_M * nv + i] = accm[diag_pos];
 }
 
 // The mass matrix on its own pattern: the entries of each row whose mass value
@@ -1245,7 +1420,17 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         const int n4i = nc * nc * nc * nc, ntab = 3 * n4i;
         // edge and vertex pairs: the outer entries of their maps, each with its own rule
         const int nout_e = 6 * ne * ne, nout_v = 2 * nvx * nvx;
-        const size_t bt = sizeof(double) * SS_TABLE_ARRAYS * ntab;
+        // the coincident pairs' polynomials, where kappa times the longest edge is within their range
+        int coin_deg = RAD_DEG + 1;
+        {
+            const Radial lim = make_radial(gq);
+            const float z = 1.0001f * (float)(kappa * m->max_edge);
+            for (int d = RAD_DEG; d >= 0; --d)
+                if (z <= lim.zlim[d]) coin_deg = d;
+        }
+        const bool poly = coin_deg <= RAD_DEG;
+        const size_t coin_bytes = sizeof(double) * 3 * nc * (COIN_STRIDE + 2);
+        const size_t bt = poly ? coin_bytes : sizeof(double) * SS_TABLE_ARRAYS * ntab;
         const size_t be = sizeof(double) * (size_t)SS_OUTER_ARRAYS * nout_e;
         const size_t bv = sizeof(double) * (size_t)SS_OUTER_ARRAYS * nout_v;
         double* tabm = nullptr;
@@ -1257,7 +1442,8 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         }
         double* tabe = tabm + bt / sizeof(double);
         double* tabv = tabe + be / sizeof(double);
-        k_ss_table<<<(ntab + 127) / 128, 128, 0, s>>>(gq, ntab, tabm);
+        if (poly) k_coin_table<<<(27 * nc + 3) / 4, 128, 0, s>>>(gq, tabm);
+        else k_ss_table<<<(ntab + 127) / 128, 128, 0, s>>>(gq, ntab, tabm);
         const Gauss gauss_e = gauss01(ne), gauss_v = gauss01(nvx);
         k_ss_outer<<<(nout_e + 127) / 128, 128, 0, s>>>(gauss_e, 1, nout_e, tabe);
         k_ss_outer<<<(nout_v + 127) / 128, 128, 0, s>>>(gauss_v, 2, nout_v, tabv);
@@ -1267,10 +1453,18 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         int threads = NEAR_THREADS;  // one warp per pair
         // coincident pairs, then one of each pair of reversed pairs (which also writes the other)
         unsigned bc = (unsigned)((m->n_coin * 32 + threads - 1) / threads);
-        // quadrature point pairs of each kernel, for the profile (formula flop counts per pair in
+        // quadrature point pairs of each kernel's rule, for the profile (formula flop counts in
         // NEAR_FLOPS_*: kernel evaluation and accumulation, a fused multiply-add counted as two)
         const double n4 = (double)n4i, Q = m->Q, Qb = m->Qr;
-        if (bc) {
+        if (bc && poly) {
+            const double rule_pairs = 3.0 * n4 + Q * (Q - 1) / 2;
+            Timer tm(ctx, PB_KERNEL_NEAR_COIN, s, m->n_coin * rule_pairs,
+                     (3.0 * nc * coin_dir_flops(coin_deg) + Q * (Q - 1) / 2 * NEAR_FLOPS_COIN) / rule_pairs);
+            k_coin_poly<<<(unsigned)((m->n_coin * COIN_LANES + COIN_THREADS - 1) / COIN_THREADS), COIN_THREADS, coin_bytes, s>>>(
+                m->verts, m->tris, m->tgeo, m->pairs, m->pair_coin, m->n_coin, nc, coin_deg, tabm, mesh_rule(m), kappa,
+                ss, far);
+            tm.stop();
+        } else if (bc) {
             Timer tm(ctx, PB_KERNEL_NEAR_COIN, s, m->n_coin * (3.0 * n4 + Q * (Q - 1) / 2), NEAR_FLOPS_COIN);
             k_coin_pairs<<<bc, threads, 0, s>>>(m->verts, m->tris, m->tgeo, m->pairs, m->pair_coin, m->n_coin, tab,
                                                 n4i, mesh_rule(m), kappa, ss, far);
@@ -1286,8 +1480,9 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
             const Radial rad = make_radial(cls == 0 ? gauss_e : gauss_v);
             const double entries = (double)nlist * ot.n, points = entries * ot.nss;
             {
-                Timer tm(ctx, PB_KERNEL_NEAR_ADJ, s, points,
-                         (points * NEAR_FLOPS_ADJ_POINT + entries * NEAR_FLOPS_ADJ_ENTRY) / points);
+                const double rule_pairs = points * ot.nss;  // the xi points are not evaluated one by one
+                Timer tm(ctx, PB_KERNEL_NEAR_ADJ, s, rule_pairs,
+                         (points * NEAR_FLOPS_ADJ_POINT + entries * NEAR_FLOPS_ADJ_ENTRY) / rule_pairs);
                 launch_adj(adj_group(nlist, cls, ctx->num_sms), m, list, nlist, ot, rad, kappa, ss, s);
                 ::pb::count_launch();
                 tm.stop();
@@ -1324,17 +1519,19 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         }
         cudaMemsetAsync(nf->diag, 0, sizeof(double) * N_VALS * m->nv, s);
         {
-            const size_t per_warp = sizeof(double) * row_warp_doubles(m->max_row);
+            const int batch = sizeof(double) * row_warp_doubles(128, m->max_row) <= (227u << 10) ? 128 : 32;
+            const size_t per_warp = sizeof(double) * row_warp_doubles(batch, m->max_row);
             const int warps = (int)std::max<size_t>(1, std::min<size_t>(8, (200u << 10) / per_warp));
             const size_t sm = per_warp * warps;
             if (sm > (227u << 10)) {
                 rc = set_error(PB_EINVAL, "near pattern rows too long (%d entries) for one warp's shared memory",
                                m->max_row);
             } else {
+                const auto rows = batch == 128 ? k_near_rows<128> : k_near_rows<32>;
                 // the largest allowed (227 KB), not this launch's sm: builds on other host threads
                 // set the same value, so none lowers it under another's launch
-                cudaFuncSetAttribute(k_near_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
-                k_near_rows<<<(unsigned)((m->nv + warps - 1) / warps), 32 * warps, sm, s>>>(
+                cudaFuncSetAttribute((const void*)rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
+                rows<<<(unsigned)((m->nv + warps - 1) / warps), 32 * warps, sm, s>>>(
                     m->nv, m->nnz, m->max_row, warps, m->row_ptr, m->col, m->v2t_ptr, m->v2t, m->tris, m->adj_ptr,
                     m->pairs, m->n_band ? m->band_ptr : nullptr, m->band_s, m->n_adj, m->tgeo, ss, far, nf->val,
                     nf->diag);

@@ -31,7 +31,7 @@ def check(v, t, kappa, plan):
     m.free()
 
 
-@pytest.mark.parametrize("kappa", [0.0, 0.01, 0.125, 0.3, 2.0])
+@pytest.mark.parametrize("kappa", [0.0, 0.01, 0.125, 0.3, 0.45, 2.0])
 def test_yukawa_sums_at_every_degree(kappa):
     v, t = icosphere(2, 2.0)
     check(v, t, kappa, {"far_q": 6, "n_ss": 4})
@@ -56,3 +56,23 @@ def test_many_pairs(n_lon, n_lat, length):
     """1,736 triangles (4 lanes per vertex pair, a warp per edge pair) and 7,560 (4 and 8 lanes)."""
     v, t = uv_ellipsoid(n_lon, n_lat, (1.5, 1.4, length), twist=0.05)
     check(v, t, 0.125, {"far_q": 3, "n_ss": 4})
+
+
+def test_rows_too_long_for_a_full_batch():
+    """3,762 vertices, every pair of triangles in the band: rows of 3,762 entries, which leave room for 32 staged
+    contributions a warp only. Rows of M, V_L and D_Y against the oracle's."""
+    import torch
+
+    import paper_2108_10481_gb300 as pb
+    v, t = uv_ellipsoid(80, 48, (2.0, 1.6, 1.3), twist=0.02)
+    plan = {"far_q": 1, "n_ss": 2, "band_eta": 64.0, "band_q": 3}
+    rows = np.array([0, 5, 1900, v.shape[0] - 1])
+    ref = oracle.assemble_rows(v, t, rows, 0.125, O.Plan(**plan))
+    ctx = pb.pb_init(0)
+    m = pb.pb_mesh_load(ctx, v, t, **plan)
+    nf = pb.pb_near_build(ctx, m, 0.125)
+    x = np.random.default_rng(6).standard_normal(v.shape[0])
+    for name in ("M", "VL", "DY"):
+        op, kern = OPS[name]
+        y = pb.pb_op_apply(ctx, m, nf, op, kern, pb.PB_F64, torch.as_tensor(x, device="cuda")).cpu().numpy()
+        assert rel(y[rows], ref[name] @ x) < 1e-12, name

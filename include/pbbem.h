@@ -66,7 +66,8 @@ extern "C" {
 #define PB_F64 0          /* FP64 everywhere */
 #define PB_F32 1          /* FP32 pair sums and FP32 near field (inner solves) */
 #define PB_F32_ACCURATE 2 /* FP32 pair arithmetic on split (hi+lo) coordinates with
-                             FP64 accumulation per source tile, FP64 near field */
+                             the tiles' sums accumulated in two FP32 words (about 48
+                             bits), FP64 near field */
 #define PB_MIXED 3        /* (pb_solve_opts.precision) FP32 inner GMRES inside FP64
                              iterative refinement */
 
@@ -384,7 +385,7 @@ typedef struct {
     int tile_records;       /* source records per TMA tile of the chosen launch */
     int stages;             /* its pipeline stages */
     int targets_per_thread; /* its targets per thread */
-    int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into FP64 at a time */
+    int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide sums at a time */
     double split_scale;     /* chosen multiplier of the wave-filling split count */
     double best_ms;         /* one FP32 system application with the choice */
     double default_ms;      /* ... with the untuned default (packed, shape 0, x1) */
@@ -397,7 +398,7 @@ typedef struct {
  * on this mesh (fast and split-coordinate variants; the scalar kernel and the
  * packed kernel in each of its launch shapes - records per TMA tile 32, 64
  * or 128, 2 or 4 pipeline stages, 2 or 4 targets per thread, for the
- * split-coordinate variant 1, 2 or 4 tiles per FP64 addition - each with the
+ * split-coordinate variant 1, 2 or 4 tiles per addition to the wide sums - each with the
  * wave-filling split count x0.5, x1 and x2) and keep the fastest of each
  * variant in ctx for meshes of this size (same power-of-two bucket of
  * quadrature points). Later applications, solves and the server use it. out

@@ -542,9 +542,38 @@ __device__ __forceinline__ float ex2_approx(float x) {
 
 struct Coef32 {
     float k[2][4];
+    float rho[4];  // kind 2: Yukawa over Laplace coefficient of V, K, D, T
     float kappa;
     float mk2;  // -kappa * log2(e)
+    int kind;   // loop of the packed kernel (far_kind)
 };
+
+// The packed kernels' loop for a plan's coefficients, as the FP64 kernel's: 1 no Yukawa term
+// (V/K + D/T rows), 2 V, K, D and T all with a Laplace coefficient (V/K + D/T rows), 0 otherwise.
+static int far_kind(const FarPlan& fp) {
+    if (fp.mode == 0) return 0;
+    bool yukawa = false, all_laplace = true;
+    for (int R = 0; R < 2; ++R)
+        for (int j = 0; j < 4; ++j) {
+            if (j & 1) yukawa = yukawa || fp.k[R][j] != 0.0;
+            else all_laplace = all_laplace && fp.k[R][j] != 0.0;
+        }
+    return !yukawa ? 1 : all_laplace ? 2 : 0;
+}
+
+static Coef32 coef32(const FarPlan& fp) {
+    Coef32 cf;
+    cf.kind = far_kind(fp);
+    for (int R = 0; R < 2; ++R)
+        for (int j = 0; j < 4; ++j) cf.k[R][j] = (float)fp.k[R][j];
+    for (int q = 0; q < 4; ++q) {
+        const double* k = fp.k[q / 2] + 2 * (q % 2);
+        cf.rho[q] = cf.kind == 2 ? (float)(k[1] / k[0]) : 0.0f;
+    }
+    cf.kappa = (float)fp.kappa;
+    cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);
+    return cf;
+}
 
 template <int MODE, bool ACC>
 __global__ void __launch_bounds__(TPB32) k_pair32(const __grid_constant__ CUtensorMap tmap, int64_t np,
@@ -721,13 +750,69 @@ __global__ void k_sources2(int64_t np, int Q, Rule rule, const int32_t* __restri
 
 struct Coef2 {
     float2 c[2][4];
+    float2 rho[4];
     float2 kap, mk2;
 };
+__device__ __forceinline__ Coef2 coef2(const Coef32& c32) {
+    Coef2 cf;
+    for (int R = 0; R < 2; ++R)
+        for (int k = 0; k < 4; ++k) cf.c[R][k] = splat(c32.k[R][k]);
+    for (int k = 0; k < 4; ++k) cf.rho[k] = splat(c32.rho[k]);
+    cf.kap = splat(c32.kappa);
+    cf.mk2 = splat(c32.mk2);
+    return cf;
+}
 
-template <int MODE, bool ACC, int NPK, bool GUARD, int TS>
+// Raw sums of a target (far_raw) and its outputs from them (x2_out): MODE 0 the four sums
+// s/r, d.p/r^3 and their Yukawa forms, which both rows combine; MODE 1 V and K apart, T, C and
+// B (KIND 0: V + K together, the coefficients already in the kernels).
+__host__ __device__ constexpr int far_raw(int mode, int kind) { return mode == 0 ? 4 : kind == 0 ? 10 : kind == 1 ? 8 : 11; }
+
+template <int MODE, int KIND>
+__device__ __forceinline__ void x2_out(const Coef2& cf, const float2* v, float2* out) {
+    if (MODE == 0) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            out[r] = fma2(cf.c[r][0], v[0], fma2(cf.c[r][2], v[1], fma2(cf.c[r][1], v[2], mul2(cf.c[r][3], v[3]))));
+    } else if (KIND == 0) {
+#pragma unroll
+        for (int a = 0; a < 10; ++a) out[a] = v[a];
+    } else {
+        out[0] = fma2(cf.c[0][0], v[0], mul2(cf.c[0][2], v[1]));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            out[1 + a] = mul2(cf.c[1][2], v[2 + a]);
+            out[4 + a] = mul2(cf.c[1][0], v[5 + a]);
+            out[7 + a] = KIND == 1 ? make_float2(0.f, 0.f) : v[8 + a];
+        }
+    }
+}
+
+// Wide sums of the split-coordinate variant: two FP32 words per sum (hi + lo, about 48 bits),
+// a tile's FP32 sum added exactly (Knuth's two-sum, the rounding error into lo). Seven packed
+// operations a value; FP64 additions and the conversions to it, at the GB300's FP64 rate, took
+// a third of the kernel's time when every tile of 64 sources was added (61,440 points, V/K +
+// D/T rows: 5.89 -> 4.98 ms; tiles of 128 sources would take 4.58, but their FP32 sums raise the
+// PMCHWT forms' error against the FP64 application from 4.0e-8 to 5.5e-8).
+struct Wide2 {
+    float2 hi, lo;
+};
+__device__ __forceinline__ void wide_add(Wide2& w, float2 b) {
+    const float2 s = add2(w.hi, b), bb = sub2(s, w.hi);
+    w.lo = add2(w.lo, add2(sub2(w.hi, sub2(s, bb)), sub2(b, bb)));
+    w.hi = s;
+}
+
+// The tile's sums. FP32 operations per pair, with the packed pipe the limit: MODE 0 19; MODE 1
+// KIND 0 36, KIND 1 20 (no exponential), KIND 2 32; split coordinates 6 more (25 and 36 with the
+// coefficients applied to every pair): e^{-kappa r}(1 + kappa r)/r is g + kappa e with g = e/r,
+// and a kernel with both Green's functions takes one FMA on their ratio. 30,720 points, V/K +
+// D/T rows: 1,064 -> 983 us, 0.79 of the packed pipe's measured rate.
+template <int MODE, bool ACC, int NPK, bool GUARD, int TS, int KIND>
 __device__ __forceinline__ void tile_x2(const float* __restrict__ tile, const float2 (&X)[NPK][3],
-                                        const float2 (&XL)[NPK][3], float2 (&acc)[NPK][MODE == 0 ? 2 : 10],
+                                        const float2 (&XL)[NPK][3], float2 (&acc)[NPK][far_raw(MODE, KIND)],
                                         const Coef2& cf) {
+    constexpr bool YUK = KIND != 1;
 #pragma unroll 2
     for (int j = 0; j < TS; ++j) {
         const float* r = tile + REC2 * j;
@@ -758,31 +843,48 @@ __device__ __forceinline__ void tile_x2(const float* __restrict__ tile, const fl
                 rinv.x = r2.x > 0.0f ? rinv.x : 0.0f;
                 rinv.y = r2.y > 0.0f ? rinv.y : 0.0f;
             }
-            const float2 rr = mul2(r2, rinv);
-            const float2 arg = mul2(rr, cf.mk2);
-            const float2 e = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
-            const float2 ek = fma2(e, mul2(rr, cf.kap), e);
-            const float2 rinv3 = mul2(mul2(rinv, rinv), rinv);
-            const float2 dp = fma2(d0, Px, fma2(d1, Py, mul2(d2, Pz)));
-            const float2 rs = mul2(rinv, Ss), r3dp = mul2(rinv3, dp);
-            acc[p][0] = fma2(fma2(cf.c[0][1], e, cf.c[0][0]), rs, acc[p][0]);
-            acc[p][0] = fma2(fma2(cf.c[0][3], ek, cf.c[0][2]), r3dp, acc[p][0]);
+            float2 g = make_float2(0.f, 0.f), gw = g;
+            if (YUK) {
+                const float2 arg = mul2(mul2(r2, rinv), cf.mk2);
+                const float2 e = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
+                g = mul2(e, rinv);
+                gw = fma2(cf.kap, e, g);
+            }
+            const float2 ri2 = mul2(rinv, rinv);
+            const float2 dp = mul2(ri2, fma2(d0, Px, fma2(d1, Py, mul2(d2, Pz))));
             if (MODE == 0) {
-                acc[p][1] = fma2(fma2(cf.c[1][1], e, cf.c[1][0]), rs, acc[p][1]);
-                acc[p][1] = fma2(fma2(cf.c[1][3], ek, cf.c[1][2]), r3dp, acc[p][1]);
+                acc[p][0] = fma2(rinv, Ss, acc[p][0]);
+                acc[p][1] = fma2(rinv, dp, acc[p][1]);
+                acc[p][2] = fma2(g, Ss, acc[p][2]);
+                acc[p][3] = fma2(gw, dp, acc[p][3]);
             } else {
-                const float2 ts = mul2(fma2(cf.c[1][3], ek, cf.c[1][2]), mul2(rinv3, Ss));
-                acc[p][1] = fma2(ts, d0, acc[p][1]);
-                acc[p][2] = fma2(ts, d1, acc[p][2]);
-                acc[p][3] = fma2(ts, d2, acc[p][3]);
-                const float2 gc = mul2(fma2(cf.c[1][1], e, cf.c[1][0]), rinv);
-                acc[p][4] = fma2(gc, make_float2(q3.z, q3.w), acc[p][4]);
-                acc[p][5] = fma2(gc, make_float2(q4.x, q4.y), acc[p][5]);
-                acc[p][6] = fma2(gc, make_float2(q4.z, q4.w), acc[p][6]);
-                const float2 gb = mul2(e, rinv);
-                acc[p][7] = fma2(gb, Px, acc[p][7]);
-                acc[p][8] = fma2(gb, Py, acc[p][8]);
-                acc[p][9] = fma2(gb, Pz, acc[p][9]);
+                float2 kv = rinv, kk = rinv, kd = rinv, kt = rinv;
+                if (KIND == 0) {
+                    kv = fma2(cf.c[0][1], g, mul2(cf.c[0][0], rinv));
+                    kk = fma2(cf.c[0][3], gw, mul2(cf.c[0][2], rinv));
+                    kd = fma2(cf.c[1][1], g, mul2(cf.c[1][0], rinv));
+                    kt = fma2(cf.c[1][3], gw, mul2(cf.c[1][2], rinv));
+                } else if (KIND == 2) {
+                    kv = fma2(cf.rho[0], g, rinv);
+                    kk = fma2(cf.rho[1], gw, rinv);
+                    kd = fma2(cf.rho[2], g, rinv);
+                    kt = fma2(cf.rho[3], gw, rinv);
+                }
+                constexpr int VK = KIND == 0 ? 0 : 1, T = VK + 1;  // V and K summed apart unless KIND 0
+                const float2 ts = mul2(kt, mul2(ri2, Ss));
+                acc[p][0] = fma2(kv, Ss, acc[p][0]);
+                acc[p][VK] = fma2(kk, dp, acc[p][VK]);
+                acc[p][T] = fma2(ts, d0, acc[p][T]);
+                acc[p][T + 1] = fma2(ts, d1, acc[p][T + 1]);
+                acc[p][T + 2] = fma2(ts, d2, acc[p][T + 2]);
+                acc[p][T + 3] = fma2(kd, make_float2(q3.z, q3.w), acc[p][T + 3]);
+                acc[p][T + 4] = fma2(kd, make_float2(q4.x, q4.y), acc[p][T + 4]);
+                acc[p][T + 5] = fma2(kd, make_float2(q4.z, q4.w), acc[p][T + 5]);
+                if (YUK) {
+                    acc[p][far_raw(MODE, KIND) - 3] = fma2(g, Px, acc[p][far_raw(MODE, KIND) - 3]);
+                    acc[p][far_raw(MODE, KIND) - 2] = fma2(g, Py, acc[p][far_raw(MODE, KIND) - 2]);
+                    acc[p][far_raw(MODE, KIND) - 1] = fma2(g, Pz, acc[p][far_raw(MODE, KIND) - 1]);
+                }
             }
         }
     }
@@ -790,16 +892,15 @@ __device__ __forceinline__ void tile_x2(const float* __restrict__ tile, const fl
 
 // Templated on its launch shape: source records per TMA tile (TS), pipeline
 // stages (ST), packed target pairs per thread (NPK) and, for the
-// split-coordinate variant, the tiles whose FP32 sums are added into the FP64
-// sums at a time (PROMO: each FP64 addition takes about as much of the GB300's
-// FP64 pipe as 64 FP32 operations take of the FMA pipe); the autotuner picks
-// the shape per mesh-size bucket.
-template <int MODE, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
+// split-coordinate variant, the tiles whose FP32 sums are added into the wide
+// sums at a time (PROMO); the autotuner picks the shape per mesh-size bucket.
+template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
 __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUtensorMap tmap, int64_t np,
                                                    const float* __restrict__ pts32, const float* __restrict__ pts32lo,
                                                    Coef32 c32, int64_t chunk, void* __restrict__ part_out,
                                                    int* __restrict__ status) {
     constexpr int NACC = MODE == 0 ? 2 : 10;
+    constexpr int NRAW = far_raw(MODE, KIND);
     constexpr int TGT = 2 * NPK;
     __shared__ __align__(128) float sh[ST][TS * REC2];
     __shared__ __align__(8) uint64_t bar[ST];
@@ -820,11 +921,7 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
             tma_load_2d(sh[s], &tmap, 0, (int)(j0 + (int64_t)s * TS), &bar[s]);
         }
     }
-    Coef2 cf;
-    for (int R = 0; R < 2; ++R)
-        for (int k = 0; k < 4; ++k) cf.c[R][k] = splat(c32.k[R][k]);
-    cf.kap = splat(c32.kappa);
-    cf.mk2 = splat(c32.mk2);
+    const Coef2 cf = coef2(c32);
     float2 X[NPK][3], XL[NPK][3];
     int64_t tg[TGT];
     for (int t = 0; t < TGT; ++t) tg[t] = blk0 + t * TPB2 + threadIdx.x;
@@ -836,12 +933,12 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
             XL[p][k] = ACC ? make_float2(pts32lo[4 * a + k], pts32lo[4 * b + k]) : make_float2(0.f, 0.f);
         }
     }
-    float2 acc[NPK][NACC];
-    double accd[TGT][ACC ? NACC : 1];
-    for (int p = 0; p < NPK; ++p)
-        for (int a = 0; a < NACC; ++a) acc[p][a] = make_float2(0.f, 0.f);
-    for (int t = 0; t < TGT; ++t)
-        for (int a = 0; a < (ACC ? NACC : 1); ++a) accd[t][a] = 0.0;
+    float2 acc[NPK][NRAW];
+    Wide2 wide[NPK][ACC ? NACC : 1];
+    for (int p = 0; p < NPK; ++p) {
+        for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
+        for (int a = 0; a < (ACC ? NACC : 1); ++a) wide[p][a].hi = wide[p][a].lo = make_float2(0.f, 0.f);
+    }
     int failed_at = -1;
     for (int it = 0; it < ntiles; ++it) {
         const int st = it % ST;
@@ -849,15 +946,15 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
         if (!cta_wait(&bar[st], phase, status)) { failed_at = it; break; }
         const int64_t jt = j0 + (int64_t)it * TS;
         const bool guard = (jt < blk1 && jt + TS > blk0) || jt + TS > np;
-        if (guard) tile_x2<MODE, ACC, NPK, true, TS>(sh[st], X, XL, acc, cf);
-        else tile_x2<MODE, ACC, NPK, false, TS>(sh[st], X, XL, acc, cf);
+        if (guard) tile_x2<MODE, ACC, NPK, true, TS, KIND>(sh[st], X, XL, acc, cf);
+        else tile_x2<MODE, ACC, NPK, false, TS, KIND>(sh[st], X, XL, acc, cf);
         if (ACC && ((it + 1) % PROMO == 0 || it + 1 == ntiles)) {
-            for (int p = 0; p < NPK; ++p)
-                for (int a = 0; a < NACC; ++a) {
-                    accd[2 * p][a] += (double)acc[p][a].x;
-                    accd[2 * p + 1][a] += (double)acc[p][a].y;
-                    acc[p][a] = make_float2(0.f, 0.f);
-                }
+            for (int p = 0; p < NPK; ++p) {
+                float2 out[NACC];
+                x2_out<MODE, KIND>(cf, acc[p], out);
+                for (int a = 0; a < NACC; ++a) wide_add(wide[p][a], out[a]);
+                for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
+            }
         }
         __syncthreads();  // every thread is done with this stage
         if (threadIdx.x == 0 && it + ST < ntiles) {
@@ -870,13 +967,19 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
         cta_drain(bar, ST, failed_at, ntiles);
         return;
     }
-    for (int t = 0; t < TGT; ++t) {
-        if (tg[t] >= np) continue;
-        const int p = t >> 1, h = t & 1;
-        for (int a = 0; a < NACC; ++a) {
-            int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
-            if (ACC) static_cast<double*>(part_out)[o] = accd[t][a];
-            else static_cast<float*>(part_out)[o] = h ? acc[p][a].y : acc[p][a].x;
+    for (int p = 0; p < NPK; ++p) {
+        float2 out[NACC];
+        if (!ACC) x2_out<MODE, KIND>(cf, acc[p], out);
+        for (int h = 0; h < 2; ++h) {
+            const int t = 2 * p + h;
+            if (tg[t] >= np) continue;
+            for (int a = 0; a < NACC; ++a) {
+                int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
+                if (ACC)
+                    static_cast<double*>(part_out)[o] = h ? (double)wide[p][a].hi.y + (double)wide[p][a].lo.y
+                                                          : (double)wide[p][a].hi.x + (double)wide[p][a].lo.x;
+                else static_cast<float*>(part_out)[o] = h ? out[a].y : out[a].x;
+            }
         }
     }
 }
@@ -884,7 +987,7 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
 // Launch shapes of the packed kernel, one table per row mode and variant; the
 // autotuner picks one per mesh-size bucket (shape 0: the default).
 // Shapes: (records per tile, stages, packed target pairs per thread, tiles per
-// FP64 addition of the split-coordinate variant).
+// addition to the wide sums of the split-coordinate variant).
 typedef void (*X2Launch)(dim3, cudaStream_t, const CUtensorMap&, int64_t, const float*, const float*, Coef32,
                          int64_t, void*, int*);
 struct X2Entry {
@@ -894,37 +997,39 @@ struct X2Entry {
 };
 constexpr int X2_SHAPES = 4;
 
-template <int MODE, bool ACC, int TS, int ST, int NPK, int PROMO>
+template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO>
 static void x2_launch(dim3 g, cudaStream_t s, const CUtensorMap& map, int64_t np, const float* p32,
                       const float* plo, Coef32 cf, int64_t chunk, void* part, int* status) {
-    k_pair32x2<MODE, ACC, TS, ST, NPK, PROMO><<<g, TPB2, 0, s>>>(map, np, p32, plo, cf, chunk, part, status);
+    k_pair32x2<MODE, KIND, ACC, TS, ST, NPK, PROMO><<<g, TPB2, 0, s>>>(map, np, p32, plo, cf, chunk, part, status);
 }
-template <int MODE, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
+template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
 static X2Entry x2_entry() {
-    return {TS, ST, NPK, PROMO, (const void*)k_pair32x2<MODE, ACC, TS, ST, NPK, PROMO>,
-            x2_launch<MODE, ACC, TS, ST, NPK, PROMO>};
+    return {TS, ST, NPK, PROMO, (const void*)k_pair32x2<MODE, KIND, ACC, TS, ST, NPK, PROMO>,
+            x2_launch<MODE, KIND, ACC, TS, ST, NPK, PROMO>};
 }
-template <int MODE>
+template <int MODE, int KIND>
 static void x2_row(X2Entry (&fast)[X2_SHAPES], X2Entry (&acc)[X2_SHAPES]) {
-    fast[0] = x2_entry<MODE, false, 64, 4, 2>();
-    fast[1] = x2_entry<MODE, false, 32, 4, 2>();
-    fast[2] = x2_entry<MODE, false, 128, 2, 2>();
-    fast[3] = x2_entry<MODE, false, 64, 4, 1>();
-    acc[0] = x2_entry<MODE, true, 64, 4, 1>();
-    acc[1] = x2_entry<MODE, true, 128, 2, 1>();
-    acc[2] = x2_entry<MODE, true, 128, 2, 1, 2>();
-    acc[3] = x2_entry<MODE, true, 64, 4, 1, 4>();
+    fast[0] = x2_entry<MODE, KIND, false, 64, 4, 2>();
+    fast[1] = x2_entry<MODE, KIND, false, 32, 4, 2>();
+    fast[2] = x2_entry<MODE, KIND, false, 128, 2, 2>();
+    fast[3] = x2_entry<MODE, KIND, false, 64, 4, 1>();
+    acc[0] = x2_entry<MODE, KIND, true, 64, 4, 1>();
+    acc[1] = x2_entry<MODE, KIND, true, 128, 2, 1>();
+    acc[2] = x2_entry<MODE, KIND, true, 128, 2, 1, 2>();
+    acc[3] = x2_entry<MODE, KIND, true, 64, 4, 1, 4>();
 }
-static const X2Entry& x2_kernel(int mode, bool acc, int shape) {
+static const X2Entry& x2_kernel(int mode, int kind, bool acc, int shape) {
     struct Table {
-        X2Entry e[2][2][X2_SHAPES];
+        X2Entry e[4][2][X2_SHAPES];  // V/K rows; V/K + D/T rows of kinds 0, 1, 2
         Table() {
-            x2_row<0>(e[0][0], e[0][1]);
-            x2_row<1>(e[1][0], e[1][1]);
+            x2_row<0, 0>(e[0][0], e[0][1]);
+            x2_row<1, 0>(e[1][0], e[1][1]);
+            x2_row<1, 1>(e[2][0], e[2][1]);
+            x2_row<1, 2>(e[3][0], e[3][1]);
         }
     };
     static const Table t;
-    return t.e[mode ? 1 : 0][acc ? 1 : 0][(shape >= 0 && shape < X2_SHAPES) ? shape : 0];
+    return t.e[mode ? 1 + kind : 0][acc ? 1 : 0][(shape >= 0 && shape < X2_SHAPES) ? shape : 0];
 }
 
 // ------------------------- batched FP32 pair kernel: many meshes in one launch
@@ -968,18 +1073,106 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 // as its scratch). The staging pipeline of the pair items runs on across
 // items: g counts the tiles a CTA has consumed, so tile it of the current item
 // sits on stage (g + it) % ST2 with phase parity ((g + it) / ST2) & 1.
+// One pair item on the CTA: g tiles consumed before it; false when a wait ran out.
+template <int MODE, bool ACC, int KIND>
+__device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, float (&sh)[ST2][TS2 * REC2], uint64_t* bar,
+                                          uint32_t& g, int* status) {
+    constexpr int NACC = MODE == 0 ? 2 : 10, NRAW = far_raw(MODE, KIND);
+    constexpr int NPK = ACC ? 1 : 2;
+    constexpr int TGT = 2 * NPK;
+    const uint32_t tile_bytes = TS2 * REC2 * sizeof(float);
+    const int64_t np = J.np;
+    const int64_t j0 = split * J.chunk;
+    const int64_t j1 = min(np, j0 + J.chunk);
+    const int ntiles = (int)((j1 - j0 + TS2 - 1) / TS2);
+    const int64_t blk0 = (int64_t)tb * (TPB2 * TGT), blk1 = blk0 + TPB2 * TGT;
+    if (threadIdx.x == 0) {
+        // the stages were last read through the generic proxy
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int k = 0; k < ST2 && k < ntiles; ++k) {
+            const int st = (int)((g + k) % ST2);
+            mbar_expect_tx(&bar[st], tile_bytes);
+            bulk_load(sh[st], J.rec + (j0 + (int64_t)k * TS2) * REC2, tile_bytes, &bar[st]);
+        }
+    }
+    const Coef2 cf = coef2(J.cf);
+    float2 X[NPK][3], XL[NPK][3];
+    int64_t tg[TGT];
+    for (int t = 0; t < TGT; ++t) tg[t] = blk0 + t * TPB2 + threadIdx.x;
+    for (int p = 0; p < NPK; ++p) {
+        int64_t a = tg[2 * p] < np ? tg[2 * p] : np - 1;
+        int64_t b = tg[2 * p + 1] < np ? tg[2 * p + 1] : np - 1;
+        for (int k = 0; k < 3; ++k) {
+            X[p][k] = make_float2(J.pts32[4 * a + k], J.pts32[4 * b + k]);
+            XL[p][k] = ACC ? make_float2(J.pts32lo[4 * a + k], J.pts32lo[4 * b + k]) : make_float2(0.f, 0.f);
+        }
+    }
+    float2 acc[NPK][NRAW];
+    Wide2 wide[NPK][ACC ? NACC : 1];
+    for (int p = 0; p < NPK; ++p) {
+        for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
+        for (int a = 0; a < (ACC ? NACC : 1); ++a) wide[p][a].hi = wide[p][a].lo = make_float2(0.f, 0.f);
+    }
+    int failed_at = -1;
+    for (int it = 0; it < ntiles; ++it) {
+        const int st = (int)((g + it) % ST2);
+        const uint32_t phase = (uint32_t)(((g + it) / ST2) & 1);
+        if (!cta_wait(&bar[st], phase, status)) { failed_at = it; break; }
+        const int64_t jt = j0 + (int64_t)it * TS2;
+        const bool guard = (jt < blk1 && jt + TS2 > blk0) || jt + TS2 > np;
+        if (guard) tile_x2<MODE, ACC, NPK, true, TS2, KIND>(sh[st], X, XL, acc, cf);
+        else tile_x2<MODE, ACC, NPK, false, TS2, KIND>(sh[st], X, XL, acc, cf);
+        if (ACC) {
+            for (int p = 0; p < NPK; ++p) {
+                float2 out[NACC];
+                x2_out<MODE, KIND>(cf, acc[p], out);
+                for (int a = 0; a < NACC; ++a) wide_add(wide[p][a], out[a]);
+                for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && it + ST2 < ntiles) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_expect_tx(&bar[st], tile_bytes);
+            bulk_load(sh[st], J.rec + (j0 + (int64_t)(it + ST2) * TS2) * REC2, tile_bytes, &bar[st]);
+        }
+    }
+    if (failed_at >= 0) {
+        // the copies still in flight (tiles failed_at .. failed_at + ST2 - 1), then leave
+        if (threadIdx.x == 0)
+            for (int k = failed_at; k < ntiles && k < failed_at + ST2; ++k)
+                for (int i = 0; i < (1 << 20); ++i)
+                    if (mbar_try_wait(&bar[(g + k) % ST2], (uint32_t)(((g + k) / ST2) & 1))) break;
+        __syncthreads();
+        return false;
+    }
+    for (int p = 0; p < NPK; ++p) {
+        float2 out[NACC];
+        if (!ACC) x2_out<MODE, KIND>(cf, acc[p], out);
+        for (int h = 0; h < 2; ++h) {
+            const int t = 2 * p + h;
+            if (tg[t] >= np) continue;
+            for (int a = 0; a < NACC; ++a) {
+                int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
+                if (ACC)
+                    static_cast<double*>(J.part)[o] = h ? (double)wide[p][a].hi.y + (double)wide[p][a].lo.y
+                                                        : (double)wide[p][a].hi.x + (double)wide[p][a].lo.x;
+                else static_cast<float*>(J.part)[o] = h ? out[a].y : out[a].x;
+            }
+        }
+    }
+    g += (uint32_t)ntiles;
+    return true;
+}
+
 template <int MODE, bool ACC>
-__global__ void __launch_bounds__(TPB2) k_pair32x2_queue(const PairJob* __restrict__ jobs,
+__global__ void __launch_bounds__(TPB2, 2) k_pair32x2_queue(const PairJob* __restrict__ jobs,
                                                          const TreeJob* __restrict__ tjobs,
                                                          const PairItem* __restrict__ items, int n_items,
                                                          int* __restrict__ counter, int* __restrict__ status) {
-    constexpr int NACC = MODE == 0 ? 2 : 10;
-    constexpr int NPK = ACC ? 1 : 2;
-    constexpr int TGT = 2 * NPK;
     __shared__ __align__(128) float sh[ST2][TS2 * REC2];
     __shared__ __align__(8) uint64_t bar[ST2];
     __shared__ int s_item;
-    const uint32_t tile_bytes = TS2 * REC2 * sizeof(float);
     if (threadIdx.x == 0) {
         for (int st = 0; st < ST2; ++st) mbar_init(&bar[st], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -998,91 +1191,25 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2_queue(const PairJob* __restri
                 static_assert(ST2 * TS2 * REC2 >= TREE_EVAL_TILE * (2 * TREE_REC + TREE_DUP) &&
                               ST2 * TS2 * REC2 >= 3 * (MODE == 0 ? 2 : 10) * TREE_LEAF, "tree scratch");
                 static_assert(TPB2 == 4 * (TREE_LEAF / 2), "tree groups");
-                tree_leaf_body<MODE, 4>(tjobs[it0.job], it0.tb, it0.split, &sh[0][0]);
+                const TreeJob& T = tjobs[it0.job];
+                if (MODE == 0) {
+                    if (T.cf.kind == 3) tree_leaf_body<0, 3, 4>(T, it0.tb, it0.split, &sh[0][0]);
+                    else tree_leaf_body<0, 0, 4>(T, it0.tb, it0.split, &sh[0][0]);
+                } else {
+                    if (T.cf.kind == 2) tree_leaf_body<1, 2, 4>(T, it0.tb, it0.split, &sh[0][0]);
+                    else if (T.cf.kind == 1) tree_leaf_body<1, 1, 4>(T, it0.tb, it0.split, &sh[0][0]);
+                    else tree_leaf_body<1, 0, 4>(T, it0.tb, it0.split, &sh[0][0]);
+                }
             }
             continue;
         }
         const PairJob& J = jobs[it0.job];
-        const int64_t np = J.np;
-        const int split = it0.split;
-        const int64_t j0 = split * J.chunk;
-        const int64_t j1 = min(np, j0 + J.chunk);
-        const int ntiles = (int)((j1 - j0 + TS2 - 1) / TS2);
-        const int64_t blk0 = (int64_t)it0.tb * (TPB2 * TGT), blk1 = blk0 + TPB2 * TGT;
-        if (threadIdx.x == 0) {
-            // the stages were last read through the generic proxy
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            for (int k = 0; k < ST2 && k < ntiles; ++k) {
-                const int st = (int)((g + k) % ST2);
-                mbar_expect_tx(&bar[st], tile_bytes);
-                bulk_load(sh[st], J.rec + (j0 + (int64_t)k * TS2) * REC2, tile_bytes, &bar[st]);
-            }
-        }
-        Coef2 cf;
-        for (int R = 0; R < 2; ++R)
-            for (int k = 0; k < 4; ++k) cf.c[R][k] = splat(J.cf.k[R][k]);
-        cf.kap = splat(J.cf.kappa);
-        cf.mk2 = splat(J.cf.mk2);
-        float2 X[NPK][3], XL[NPK][3];
-        int64_t tg[TGT];
-        for (int t = 0; t < TGT; ++t) tg[t] = blk0 + t * TPB2 + threadIdx.x;
-        for (int p = 0; p < NPK; ++p) {
-            int64_t a = tg[2 * p] < np ? tg[2 * p] : np - 1;
-            int64_t b = tg[2 * p + 1] < np ? tg[2 * p + 1] : np - 1;
-            for (int k = 0; k < 3; ++k) {
-                X[p][k] = make_float2(J.pts32[4 * a + k], J.pts32[4 * b + k]);
-                XL[p][k] = ACC ? make_float2(J.pts32lo[4 * a + k], J.pts32lo[4 * b + k]) : make_float2(0.f, 0.f);
-            }
-        }
-        float2 acc[NPK][NACC];
-        double accd[TGT][ACC ? NACC : 1];
-        for (int p = 0; p < NPK; ++p)
-            for (int a = 0; a < NACC; ++a) acc[p][a] = make_float2(0.f, 0.f);
-        for (int t = 0; t < TGT; ++t)
-            for (int a = 0; a < (ACC ? NACC : 1); ++a) accd[t][a] = 0.0;
-        int failed_at = -1;
-        for (int it = 0; it < ntiles; ++it) {
-            const int st = (int)((g + it) % ST2);
-            const uint32_t phase = (uint32_t)(((g + it) / ST2) & 1);
-            if (!cta_wait(&bar[st], phase, status)) { failed_at = it; break; }
-            const int64_t jt = j0 + (int64_t)it * TS2;
-            const bool guard = (jt < blk1 && jt + TS2 > blk0) || jt + TS2 > np;
-            if (guard) tile_x2<MODE, ACC, NPK, true, TS2>(sh[st], X, XL, acc, cf);
-            else tile_x2<MODE, ACC, NPK, false, TS2>(sh[st], X, XL, acc, cf);
-            if (ACC) {
-                for (int p = 0; p < NPK; ++p)
-                    for (int a = 0; a < NACC; ++a) {
-                        accd[2 * p][a] += (double)acc[p][a].x;
-                        accd[2 * p + 1][a] += (double)acc[p][a].y;
-                        acc[p][a] = make_float2(0.f, 0.f);
-                    }
-            }
-            __syncthreads();
-            if (threadIdx.x == 0 && it + ST2 < ntiles) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_expect_tx(&bar[st], tile_bytes);
-                bulk_load(sh[st], J.rec + (j0 + (int64_t)(it + ST2) * TS2) * REC2, tile_bytes, &bar[st]);
-            }
-        }
-        if (failed_at >= 0) {
-            // the copies still in flight (tiles failed_at .. failed_at + ST2 - 1), then leave
-            if (threadIdx.x == 0)
-                for (int k = failed_at; k < ntiles && k < failed_at + ST2; ++k)
-                    for (int i = 0; i < (1 << 20); ++i)
-                        if (mbar_try_wait(&bar[(g + k) % ST2], (uint32_t)(((g + k) / ST2) & 1))) break;
-            __syncthreads();
-            return;
-        }
-        for (int t = 0; t < TGT; ++t) {
-            if (tg[t] >= np) continue;
-            const int p = t >> 1, h = t & 1;
-            for (int a = 0; a < NACC; ++a) {
-                int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
-                if (ACC) static_cast<double*>(J.part)[o] = accd[t][a];
-                else static_cast<float*>(J.part)[o] = h ? acc[p][a].y : acc[p][a].x;
-            }
-        }
-        g += (uint32_t)ntiles;
+        bool ok;
+        if (MODE == 0) ok = pair_item<0, ACC, 0>(J, it0.tb, it0.split, sh, bar, g, status);
+        else if (J.cf.kind == 2) ok = pair_item<1, ACC, 2>(J, it0.tb, it0.split, sh, bar, g, status);
+        else if (J.cf.kind == 1) ok = pair_item<1, ACC, 1>(J, it0.tb, it0.split, sh, bar, g, status);
+        else ok = pair_item<1, ACC, 0>(J, it0.tb, it0.split, sh, bar, g, status);
+        if (!ok) return;
     }
 }
 
@@ -1375,8 +1502,13 @@ static int make_tmap(const pb_mesh* m, const float* rec, CUtensorMap* map, int r
 
 // FP32-pipe operations per point pair by the formula count of the kernels
 // above (FADD, FMUL and FFMA each one; the two MUFU operations not counted):
-// shared geometry 17, a phi-row 4, a DT-row 15, split coordinates +6.
-constexpr double OPS_VK2 = 25.0, OPS_VKDT = 36.0, OPS_SPLIT = 6.0;
+// V/K rows 19; V/K + D/T rows 36, 20 or 32 by kind; split coordinates +6. (The
+// scalar kernel and the one-direction FP64 kernel by the same counts.)
+constexpr double OPS_SPLIT = 6.0;
+static double pair_ops(const FarPlan& fp) {
+    static const double vkdt[3] = {36.0, 20.0, 32.0};
+    return fp.mode == 0 ? 19.0 : vkdt[far_kind(fp)];
+}
 
 
 
@@ -1437,7 +1569,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             }
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, sizeof(double) * (size_t)S * nacc * np));
             double* part = (double*)m->ws_part.ptr;
-            Timer tm(m->ctx, PB_KERNEL_PAIR64, s, (double)np * (double)np, fp.mode == 0 ? OPS_VK2 : OPS_VKDT);
+            Timer tm(m->ctx, PB_KERNEL_PAIR64, s, (double)np * (double)np, pair_ops(fp));
             if (sy.nblock) {
                 const size_t smem = sizeof(double) * 32 * (10 + (size_t)kern.sums * sy.warps * (1 + sy.sub));
                 // the largest any shape takes, whatever this one does: other host threads set the same
@@ -1465,7 +1597,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             ::pb::count_launch();
             bool acc = prec == PB_F32_ACCURATE;
             const TuneEntry te = tuned(m->ctx, np, fp.mode, acc);
-            const X2Entry& xk = x2_kernel(fp.mode, acc, te.shape);
+            const X2Entry& xk = x2_kernel(fp.mode, far_kind(fp), acc, te.shape);
             CUtensorMap map;
             PB_TRY(make_tmap(m, rec, &map, REC2, xk.ts));
             const int tpc = TPB2 * 2 * xk.npk;
@@ -1473,15 +1605,11 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             S = scaled_splits(S, te.split_scale, np, xk.ts);
             int64_t chunk = ((np + S - 1) / S + xk.ts - 1) / xk.ts * xk.ts;
             S = (int)((np + chunk - 1) / chunk);
-            Coef32 cf;
-            for (int R = 0; R < 2; ++R)
-                for (int j = 0; j < 4; ++j) cf.k[R][j] = (float)fp.k[R][j];
-            cf.kappa = (float)fp.kappa;
-            cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);
+            const Coef32 cf = coef32(fp);
             dim3 grid((unsigned)((np + tpc - 1) / tpc), (unsigned)S);
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)S * nacc * np));
             void* part = m->ws_part.ptr;
-            double ops = (fp.mode == 0 ? OPS_VK2 : OPS_VKDT) + (acc ? OPS_SPLIT : 0.0);
+            double ops = pair_ops(fp) + (acc ? OPS_SPLIT : 0.0);
             Timer tm(m->ctx, acc ? PB_KERNEL_PAIR32_ACCURATE : PB_KERNEL_PAIR32, s, (double)np * (double)np, ops);
             xk.launch(grid, s, map, np, m->pts32, m->pts32lo, cf, chunk, part, status);
             ::pb::count_launch();
@@ -1504,15 +1632,11 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             S = scaled_splits(S, tuned(m->ctx, np, fp.mode, acc).split_scale, np, TS32);
             int64_t chunk = ((np + S - 1) / S + TS32 - 1) / TS32 * TS32;
             S = (int)((np + chunk - 1) / chunk);
-            Coef32 cf;
-            for (int R = 0; R < 2; ++R)
-                for (int j = 0; j < 4; ++j) cf.k[R][j] = (float)fp.k[R][j];
-            cf.kappa = (float)fp.kappa;
-            cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);
+            const Coef32 cf = coef32(fp);
             dim3 grid((unsigned)((np + TPB32 * TGT32 - 1) / (TPB32 * TGT32)), (unsigned)S);
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)S * nacc * np));
             void* part = m->ws_part.ptr;
-            double ops = (fp.mode == 0 ? OPS_VK2 : OPS_VKDT) + (acc ? OPS_SPLIT : 0.0);
+            double ops = pair_ops(fp) + (acc ? OPS_SPLIT : 0.0);
             Timer tm(m->ctx, acc ? PB_KERNEL_PAIR32_ACCURATE : PB_KERNEL_PAIR32, s, (double)np * (double)np, ops);
             if (fp.mode == 0) {
                 if (acc) k_pair32<0, true><<<grid, TPB32, 0, s>>>(map, np, m->pts32, m->pts32lo, cf, chunk, part, status);
@@ -1615,7 +1739,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         ::pb::count_launch();
         if (np_pad > np) PB_CUDA(cudaMemsetAsync(rec + REC2 * np, 0, sizeof(float) * REC2 * (np_pad - np), js));
         // the single-mesh decomposition (same kernel occupancy as that path)
-        const void* kern = x2_kernel(P.fp.mode, acc, 0).fn;  // the default shape's occupancy (the batched kernel's)
+        const void* kern = x2_kernel(P.fp.mode, 0, acc, 0).fn;  // the default shape's occupancy (the batched kernel's)
         int S = choose_splits(np, tpc, TS2, occupancy_slots(m, kern, TPB2));
         S = scaled_splits(S, tuned(m->ctx, np, P.fp.mode, acc).split_scale, np, TS2);
         P.chunk = ((np + S - 1) / S + TS2 - 1) / TS2 * TS2;
@@ -1629,10 +1753,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         pj.part = m->ws_part.ptr;
         pj.np = np;
         pj.chunk = P.chunk;
-        for (int R = 0; R < 2; ++R)
-            for (int j = 0; j < 4; ++j) pj.cf.k[R][j] = (float)P.fp.k[R][j];
-        pj.cf.kappa = (float)P.fp.kappa;
-        pj.cf.mk2 = (float)(-P.fp.kappa * 1.4426950408889634);
+        pj.cf = coef32(P.fp);
         pj.nsplit = P.S;
         pj.pad = 0;
         hjobs[P.fp.mode].push_back(pj);
@@ -1740,7 +1861,7 @@ void batch_scratch_free(BatchScratch& bs) {
 
 int far_splits_estimate(pb_ctx* ctx, int64_t np) {
     int best = 1;
-    const void* kerns[2] = {x2_kernel(1, true, 0).fn, x2_kernel(1, false, 0).fn};
+    const void* kerns[2] = {x2_kernel(1, 0, true, 0).fn, x2_kernel(1, 0, false, 0).fn};
     const int tpcs[2] = {TPB2 * 2, TPB2 * 4};
     for (int k = 0; k < 2; ++k) {
         int per_sm = 1;
@@ -1849,11 +1970,7 @@ extern "C" int pb_system_apply_noalloc(pb_ctx* ctx, const pb_mesh* m, const pb_n
         int S = std::min(NOALLOC_MAX_SPLITS, choose_splits(np, TPB32 * TGT32, TS32, occupancy_slots(m, kern, TPB32)));
         int64_t chunk = ((np + S - 1) / S + TS32 - 1) / TS32 * TS32;
         S = (int)((np + chunk - 1) / chunk);
-        Coef32 cf;
-        for (int R = 0; R < 2; ++R)
-            for (int j = 0; j < 4; ++j) cf.k[R][j] = (float)fp.k[R][j];
-        cf.kappa = (float)fp.kappa;
-        cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);
+        const Coef32 cf = coef32(fp);
         dim3 grid((unsigned)((np + TPB32 * TGT32 - 1) / (TPB32 * TGT32)), (unsigned)S);
         if (fp.mode == 0)
             k_pair32<0, false><<<grid, TPB32, 0, s>>>(map, np, m->pts32, m->pts32lo, cf, chunk, part, m->status);
@@ -1952,7 +2069,7 @@ extern "C" int pb_autotune(pb_ctx* ctx, const pb_mesh* m, const pb_near* nf, con
             pb_tune_choice& o = acc ? out->accurate : out->fast;
             o.kernel = best_e.kernel;
             o.shape = best_e.shape;
-            const X2Entry& xk = x2_kernel(fp.mode, acc != 0, best_e.shape);
+            const X2Entry& xk = x2_kernel(fp.mode, far_kind(fp), acc != 0, best_e.shape);
             o.tile_records = best_e.kernel == 2 ? xk.ts : (int)TS32;
             o.stages = best_e.kernel == 2 ? xk.st : (int)ST32;
             o.targets_per_thread = best_e.kernel == 2 ? 2 * xk.npk : (int)TGT32;

@@ -503,12 +503,12 @@ k_proxy_charges(const int32_t* __restrict__ slots, const int32_t* __restrict__ s
 // The treecode's own launch: one CTA per leaf of targets and split, TREE_LEAF
 // threads in two groups (tree_leaf_body with NQ = 2); the linear block index
 // walks the leaves longest first, a leaf's splits side by side.
-template <int MODE>
+template <int MODE, int KIND>
 __global__ void __launch_bounds__(TREE_LEAF, 7) k_tree_eval(TreeJob job) {
     __shared__ __align__(16) float tile[TREE_EVAL_TILE * (2 * TREE_REC + TREE_DUP)];
     static_assert((MODE == 0 ? 2 : 10) * TREE_LEAF <= TREE_EVAL_TILE * (2 * TREE_REC + TREE_DUP), "reduction buffer");
     const int sp = (int)(blockIdx.x % (unsigned)job.nsplit);
-    tree_leaf_body<MODE, 2>(job, job.leaf_order[blockIdx.x / (unsigned)job.nsplit], sp, tile);
+    tree_leaf_body<MODE, KIND, 2>(job, job.leaf_order[blockIdx.x / (unsigned)job.nsplit], sp, tile);
 }
 
 // y-part of the far field by the treecode: per-target partial sums in the
@@ -551,6 +551,24 @@ int tree_prepare(const pb_mesh* mc, const FarPlan& fp, const double* x, bool nee
     TreeJob& J = *job;
     for (int R = 0; R < 2; ++R)
         for (int j = 0; j < 4; ++j) J.cf.k[R][j] = (float)fp.k[R][j];
+    {   // the loops for these coefficients (TreeCoef)
+        bool yukawa = false, all_laplace = true;
+        for (int R = 0; R < 2; ++R)
+            for (int j = 0; j < 4; j += 2) {
+                yukawa = yukawa || fp.k[R][j + 1] != 0.0;
+                all_laplace = all_laplace && fp.k[R][j] != 0.0;
+            }
+        auto only = [&](int R, int j) { return fp.k[R][1 - j] == 0.0 && fp.k[R][3 - j] == 0.0; };
+        J.cf.lrow = only(0, 0) ? 0 : 1;  // only(R, j): row R has terms of kernel j (0 Laplace, 1 Yukawa) alone
+        if (fp.mode == 0) J.cf.kind = only(J.cf.lrow, 0) && only(1 - J.cf.lrow, 1) ? 3 : 0;
+        else J.cf.kind = fp.k[0][2] == 0.0 ? 0 : !yukawa ? 1 : all_laplace ? 2 : 0;
+        for (int q = 0; q < 3; ++q) J.cf.rho[q] = 0.f;
+        if (J.cf.kind == 2) {
+            J.cf.rho[0] = (float)(fp.k[0][3] / fp.k[0][2]);
+            J.cf.rho[1] = (float)(fp.k[1][1] / fp.k[1][0]);
+            J.cf.rho[2] = (float)(fp.k[1][3] / fp.k[1][2]);
+        }
+    }
     J.cf.kappa = (float)fp.kappa;
     J.cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);
     // splits of each leaf's lists, so that the grid holds about eight CTAs per SM
@@ -585,14 +603,21 @@ int tree_far(const pb_mesh* m, const FarPlan& fp, const double* x, bool need_u, 
     const PbTree* t = m->tree;
     const unsigned grid = (unsigned)(t->nleaf * job.nsplit);
     // FP32 operations per interaction as the evaluation does them (f32x2 lanes counted singly; the two
-    // MUFU operations, rsqrt and ex2, not counted): a direct pair 24 (V/K rows) or 35 (V/K + D/T
-    // rows), a proxy 12 or 29 (its charges come combined with the kernel coefficients)
-    const double ops_near = fp.mode == 0 ? 24.0 : 35.0, ops_far = fp.mode == 0 ? 12.0 : 29.0;
+    // MUFU operations, rsqrt and ex2, not counted), by kind
+    static const double near1[3] = {36.0, 20.0, 32.0}, far1[3] = {29.0, 16.0, 26.0};
+    const int kind = job.cf.kind;
+    const double ops_near = fp.mode == 0 ? 19.0 : near1[kind], ops_far = fp.mode == 0 ? (kind == 3 ? 11.0 : 12.0) : far1[kind];
     const double inter = (double)(t->direct_pairs + t->proxy_pairs);
     const double ops = ((double)t->direct_pairs * ops_near + (double)t->proxy_pairs * ops_far) / std::max(1.0, inter);
     Timer tm(m->ctx, PB_KERNEL_TREE32, s, inter, ops);
-    if (fp.mode == 0) k_tree_eval<0><<<grid, TREE_LEAF, 0, s>>>(job);
-    else k_tree_eval<1><<<grid, TREE_LEAF, 0, s>>>(job);
+    if (fp.mode == 0) {
+        if (kind == 3) k_tree_eval<0, 3><<<grid, TREE_LEAF, 0, s>>>(job);
+        else k_tree_eval<0, 0><<<grid, TREE_LEAF, 0, s>>>(job);
+    } else {
+        if (kind == 2) k_tree_eval<1, 2><<<grid, TREE_LEAF, 0, s>>>(job);
+        else if (kind == 1) k_tree_eval<1, 1><<<grid, TREE_LEAF, 0, s>>>(job);
+        else k_tree_eval<1, 0><<<grid, TREE_LEAF, 0, s>>>(job);
+    }
     ::pb::count_launch();
     tm.stop();
     PB_CUDA(cudaGetLastError());

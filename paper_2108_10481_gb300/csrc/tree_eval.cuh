@@ -12,10 +12,16 @@ constexpr int TREE_DUP = 24;       // floats per record as summed from shared me
                                    // so that one load gives both halves of a packed f32x2 operand
 constexpr int TREE_EVAL_TILE = 128;  // sources staged per round
 
+// kind: the loops of the evaluation. V/K rows: 3 one row without a Yukawa and the other
+// without a Laplace term (the direct forms), 0 otherwise; V/K + D/T rows: 1 no Yukawa term,
+// 2 V, K, D and T all with a Laplace coefficient, 0 otherwise.
 struct TreeCoef {
     float k[2][4];
+    float rho[3];  // kind 2: Yukawa over Laplace coefficient of K, D, T
     float kappa;
     float mk2;  // -kappa log2(e)
+    int kind;
+    int lrow;   // kind 3: the row without a Yukawa term
 };
 
 __device__ __forceinline__ float t_rsqrt(float x) {
@@ -128,9 +134,18 @@ struct TreeTiles {
 // `tile` holds at least TREE_EVAL_TILE x (2 TREE_REC + TREE_DUP) floats and
 // (NQ - 1) x NACC x TREE_LEAF floats. Every thread of the group calls it (it
 // synchronises the CTA) and returns with no copy in flight.
-template <int MODE, int NQ>
+//
+// FP32 operations per interaction (the packed pipe is the limit), proxy and direct: V/K rows
+// 11 (kind 3) or 12, and 19; V/K + D/T rows 26 and 32 (kind 2), 16 and 20 (kind 1), 29 and 36
+// (kind 0); 12, 24, 29 and 35 before with one loop for all coefficients. Sums kept per target
+// (NS): V/K rows the two rows' proxy sums (kind 3: the Laplace and the Yukawa one), then the four
+// sums of the direct pairs; V/K + D/T rows phi, T, C, B, scaled at the end by kind. 116,160
+// points, direct form: 1,122 -> 940 us; 661,500 points, Juffer form: 12.57 -> 11.9 ms.
+template <int MODE, int KIND, int NQ>
 __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int sp, float* tile) {
     constexpr int NACC = MODE == 0 ? 2 : 10;
+    constexpr int NS = MODE == 0 ? 6 : 10;
+    constexpr bool YUK = KIND != 1;
     constexpr int TILE = TREE_EVAL_TILE;
     constexpr int HALF = TREE_LEAF / 2;
     constexpr int NTH = HALF * NQ;
@@ -158,12 +173,15 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
         X2.y = rec[TREE_REC * (int64_t)ti1 + 2];
     }
     const TreeCoef& cf = T.cf;
-    const float2 c00 = t_splat(cf.k[0][0]), c01 = t_splat(cf.k[0][1]), c02 = t_splat(cf.k[0][2]),
-                 c03 = t_splat(cf.k[0][3]), c10 = t_splat(cf.k[1][0]), c11 = t_splat(cf.k[1][1]),
-                 c12 = t_splat(cf.k[1][2]), c13 = t_splat(cf.k[1][3]), kap = t_splat(cf.kappa),
-                 mk2 = t_splat(cf.mk2);
-    float2 acc[NACC];
-    for (int k = 0; k < NACC; ++k) acc[k] = t_splat(0.f);
+    const float2 c02 = t_splat(cf.k[0][2]), c03 = t_splat(cf.k[0][3]), c10 = t_splat(cf.k[1][0]),
+                 c11 = t_splat(cf.k[1][1]), c12 = t_splat(cf.k[1][2]), c13 = t_splat(cf.k[1][3]),
+                 kap = t_splat(cf.kappa), mk2 = t_splat(cf.mk2), rhoK = t_splat(cf.rho[0]),
+                 rhoD = t_splat(cf.rho[1]), rhoT = t_splat(cf.rho[2]);
+    // charges of a staged record: the phi row's coefficients (kind 3: of the row each kernel belongs to)
+    const int rl = KIND == 3 ? cf.lrow : 0, ry = KIND == 3 ? 1 - cf.lrow : 0;
+    const float pscale = KIND == 1 || KIND == 2 ? cf.k[0][2] : 1.0f;  // K's Laplace coefficient, carried by p (and N)
+    float2 acc[NS];
+    for (int k = 0; k < NS; ++k) acc[k] = t_splat(0.f);
     const bool any = live0;  // the first target of a thread is live whenever the second is
     TreeTiles it = {fb, fe, qb, qe, 0};
     const float* src = nullptr;
@@ -195,23 +213,23 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
             const float s_ = v[3];
             if (far) {
                 const float q_ = v[4];  // proxy: x, S, Q, C, N
-                if (MODE == 0) {        // x, (a, b) of both rows
-                    v[3] = fmaf(cf.k[0][2], q_, cf.k[0][0] * s_);
-                    v[4] = fmaf(cf.k[0][3], q_, cf.k[0][1] * s_);
+                if (MODE == 0) {        // x, a and b (kind 3), or (a, b) of both rows
+                    const float a0 = fmaf(cf.k[rl][2], q_, cf.k[rl][0] * s_), b0 = fmaf(cf.k[ry][3], q_, cf.k[ry][1] * s_);
+                    v[3] = a0;
+                    v[4] = b0;
                     v[5] = fmaf(cf.k[1][2], q_, cf.k[1][0] * s_);
                     v[6] = fmaf(cf.k[1][3], q_, cf.k[1][1] * s_);
                 } else {  // x, S, (a, b) of the phi row, C, N
 #pragma unroll
-                    for (int k = TREE_REC - 1; k >= 6; --k) v[k] = v[k - 1];
+                    for (int k = TREE_REC - 1; k >= 9; --k) v[k] = pscale * v[k - 1];
+#pragma unroll
+                    for (int k = 8; k >= 6; --k) v[k] = v[k - 1];
                     v[4] = fmaf(cf.k[0][2], q_, cf.k[0][0] * s_);
                     v[5] = fmaf(cf.k[0][3], q_, cf.k[0][1] * s_);
                 }
-            } else if (MODE == 0) {  // source: x, s, p, (a, b) of both rows' single layers
-                v[7] = cf.k[0][0] * s_;
-                v[8] = cf.k[0][1] * s_;
-                v[9] = cf.k[1][0] * s_;
-                v[10] = cf.k[1][1] * s_;
-            } else {  // x, s, p, c, (a, b) of the phi row's single layer
+            } else if (MODE == 1) {  // x, s, p, c, (a, b) of the phi row's single layer
+#pragma unroll
+                for (int k = 4; k < 7; ++k) v[k] *= pscale;
                 v[10] = cf.k[0][0] * s_;
                 v[11] = cf.k[0][1] * s_;
             }
@@ -231,70 +249,105 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
                              d2 = t_sub2(X2, make_float2(b.x, b.y));
                 const float2 r2 = t_fma2(d0, d0, t_fma2(d1, d1, t_mul2(d2, d2)));
                 const float2 rinv = make_float2(t_rsqrt(r2.x), t_rsqrt(r2.y));
-                const float2 rr = t_mul2(r2, rinv);
-                const float2 arg = t_mul2(rr, mk2);
-                const float2 e = make_float2(t_ex2(arg.x), t_ex2(arg.y));
+                float2 e = t_splat(0.f), g = e;
+                if (YUK) {
+                    const float2 arg = t_mul2(t_mul2(r2, rinv), mk2);
+                    e = make_float2(t_ex2(arg.x), t_ex2(arg.y));
+                }
                 if (MODE == 0) {
-                    const float4 dd = z4[3];
-                    acc[0] = t_fma2(rinv, t_fma2(e, make_float2(c.x, c.y), make_float2(b.z, b.w)), acc[0]);
-                    acc[1] = t_fma2(rinv, t_fma2(e, make_float2(dd.x, dd.y), make_float2(c.z, c.w)), acc[1]);
+                    if (KIND == 3) {
+                        acc[0] = t_fma2(rinv, make_float2(b.z, b.w), acc[0]);
+                        acc[1] = t_fma2(t_mul2(e, rinv), make_float2(c.x, c.y), acc[1]);
+                    } else {
+                        const float4 dd = z4[3];
+                        acc[0] = t_fma2(rinv, t_fma2(e, make_float2(c.x, c.y), make_float2(b.z, b.w)), acc[0]);
+                        acc[1] = t_fma2(rinv, t_fma2(e, make_float2(dd.x, dd.y), make_float2(c.z, c.w)), acc[1]);
+                    }
                 } else {
-                    acc[0] = t_fma2(rinv, t_fma2(e, make_float2(c.z, c.w), make_float2(c.x, c.y)), acc[0]);
-                    const float2 ek = t_fma2(e, t_mul2(rr, kap), e);
-                    const float2 ts = t_mul2(t_fma2(c13, ek, c12),
-                                             t_mul2(t_mul2(rinv, rinv), t_mul2(rinv, make_float2(b.z, b.w))));
+                    const float2 ri2 = t_mul2(rinv, rinv);
+                    float2 kt = rinv, kd = rinv;
+                    acc[0] = t_fma2(rinv, make_float2(c.x, c.y), acc[0]);
+                    if (YUK) {
+                        g = t_mul2(e, rinv);
+                        acc[0] = t_fma2(g, make_float2(c.z, c.w), acc[0]);
+                        const float2 gw = t_fma2(kap, e, g);
+                        if (KIND == 2) {
+                            kt = t_fma2(rhoT, gw, rinv);
+                            kd = t_fma2(rhoD, g, rinv);
+                        } else {
+                            kt = t_fma2(c13, gw, t_mul2(c12, rinv));
+                            kd = t_fma2(c11, g, t_mul2(c10, rinv));
+                        }
+                    }
+                    const float2 ts = t_mul2(kt, t_mul2(ri2, make_float2(b.z, b.w)));
                     acc[1] = t_fma2(ts, d0, acc[1]);
                     acc[2] = t_fma2(ts, d1, acc[2]);
                     acc[3] = t_fma2(ts, d2, acc[3]);
                     const float4 dd = z4[3], ee = z4[4], ff = z4[5];
-                    const float2 gc = t_mul2(t_fma2(c11, e, c10), rinv);
-                    acc[4] = t_fma2(gc, make_float2(dd.x, dd.y), acc[4]);
-                    acc[5] = t_fma2(gc, make_float2(dd.z, dd.w), acc[5]);
-                    acc[6] = t_fma2(gc, make_float2(ee.x, ee.y), acc[6]);
-                    const float2 gb = t_mul2(e, rinv);
-                    acc[7] = t_fma2(gb, make_float2(ee.z, ee.w), acc[7]);
-                    acc[8] = t_fma2(gb, make_float2(ff.x, ff.y), acc[8]);
-                    acc[9] = t_fma2(gb, make_float2(ff.z, ff.w), acc[9]);
+                    acc[4] = t_fma2(kd, make_float2(dd.x, dd.y), acc[4]);
+                    acc[5] = t_fma2(kd, make_float2(dd.z, dd.w), acc[5]);
+                    acc[6] = t_fma2(kd, make_float2(ee.x, ee.y), acc[6]);
+                    if (YUK) {
+                        acc[7] = t_fma2(g, make_float2(ee.z, ee.w), acc[7]);
+                        acc[8] = t_fma2(g, make_float2(ff.x, ff.y), acc[8]);
+                        acc[9] = t_fma2(g, make_float2(ff.z, ff.w), acc[9]);
+                    }
                 }
             }
         } else if (any) {
 #pragma unroll 2
             for (int j = grp; j < cnt; j += NQ) {
                 const float4* y4 = reinterpret_cast<const float4*>(cur + TREE_DUP * j);
-                const float4 a = y4[0], b = y4[1], c = y4[2], dd = y4[3], ee = y4[4], ff = y4[5];
+                const float4 a = y4[0], b = y4[1], c = y4[2], dd = y4[3];
                 const float2 y3 = make_float2(b.z, b.w), p0 = make_float2(c.x, c.y), p1 = make_float2(c.z, c.w),
                              p2 = make_float2(dd.x, dd.y);
                 const float2 d0 = t_sub2(X0, make_float2(a.x, a.y)), d1 = t_sub2(X1, make_float2(a.z, a.w)),
                              d2 = t_sub2(X2, make_float2(b.x, b.y));
                 const float2 r2 = t_fma2(d0, d0, t_fma2(d1, d1, t_mul2(d2, d2)));
                 const float2 rinv = make_float2(r2.x > 0.f ? t_rsqrt(r2.x) : 0.f, r2.y > 0.f ? t_rsqrt(r2.y) : 0.f);
-                const float2 rr = t_mul2(r2, rinv);
-                const float2 arg = t_mul2(rr, mk2);
-                const float2 e = make_float2(t_ex2(arg.x), t_ex2(arg.y));
-                const float2 ek = t_fma2(e, t_mul2(rr, kap), e);
-                const float2 rinv3 = t_mul2(t_mul2(rinv, rinv), rinv);
-                const float2 dp = t_fma2(d0, p0, t_fma2(d1, p1, t_mul2(d2, p2)));
-                const float2 r3dp = t_mul2(rinv3, dp);
+                float2 g = t_splat(0.f), gw = g;
+                if (YUK) {
+                    const float2 arg = t_mul2(t_mul2(r2, rinv), mk2);
+                    const float2 e = make_float2(t_ex2(arg.x), t_ex2(arg.y));
+                    g = t_mul2(e, rinv);
+                    gw = t_fma2(kap, e, g);
+                }
+                const float2 ri2 = t_mul2(rinv, rinv);
+                const float2 dp = t_mul2(ri2, t_fma2(d0, p0, t_fma2(d1, p1, t_mul2(d2, p2))));
                 if (MODE == 0) {
-                    acc[0] = t_fma2(rinv, t_fma2(e, make_float2(ee.x, ee.y), make_float2(dd.z, dd.w)), acc[0]);
-                    acc[0] = t_fma2(t_fma2(c03, ek, c02), r3dp, acc[0]);
-                    acc[1] = t_fma2(rinv, t_fma2(e, make_float2(ff.x, ff.y), make_float2(ee.z, ee.w)), acc[1]);
-                    acc[1] = t_fma2(t_fma2(c13, ek, c12), r3dp, acc[1]);
+                    acc[2] = t_fma2(rinv, y3, acc[2]);
+                    acc[3] = t_fma2(rinv, dp, acc[3]);
+                    acc[4] = t_fma2(g, y3, acc[4]);
+                    acc[5] = t_fma2(gw, dp, acc[5]);
                 } else {
-                    acc[0] = t_fma2(rinv, t_fma2(e, make_float2(ff.z, ff.w), make_float2(ff.x, ff.y)), acc[0]);
-                    acc[0] = t_fma2(t_fma2(c03, ek, c02), r3dp, acc[0]);
-                    const float2 ts = t_mul2(t_fma2(c13, ek, c12), t_mul2(rinv3, y3));
+                    const float4 ee = y4[4], ff = y4[5];
+                    float2 kk = rinv, kt = rinv, kd = rinv;
+                    acc[0] = t_fma2(rinv, make_float2(ff.x, ff.y), acc[0]);
+                    if (YUK) {
+                        acc[0] = t_fma2(g, make_float2(ff.z, ff.w), acc[0]);
+                        if (KIND == 2) {
+                            kk = t_fma2(rhoK, gw, rinv);
+                            kt = t_fma2(rhoT, gw, rinv);
+                            kd = t_fma2(rhoD, g, rinv);
+                        } else {
+                            kk = t_fma2(c03, gw, t_mul2(c02, rinv));
+                            kt = t_fma2(c13, gw, t_mul2(c12, rinv));
+                            kd = t_fma2(c11, g, t_mul2(c10, rinv));
+                        }
+                    }
+                    acc[0] = t_fma2(kk, dp, acc[0]);
+                    const float2 ts = t_mul2(kt, t_mul2(ri2, y3));
                     acc[1] = t_fma2(ts, d0, acc[1]);
                     acc[2] = t_fma2(ts, d1, acc[2]);
                     acc[3] = t_fma2(ts, d2, acc[3]);
-                    const float2 gc = t_mul2(t_fma2(c11, e, c10), rinv);
-                    acc[4] = t_fma2(gc, make_float2(dd.z, dd.w), acc[4]);
-                    acc[5] = t_fma2(gc, make_float2(ee.x, ee.y), acc[5]);
-                    acc[6] = t_fma2(gc, make_float2(ee.z, ee.w), acc[6]);
-                    const float2 gb = t_mul2(e, rinv);
-                    acc[7] = t_fma2(gb, p0, acc[7]);
-                    acc[8] = t_fma2(gb, p1, acc[8]);
-                    acc[9] = t_fma2(gb, p2, acc[9]);
+                    acc[4] = t_fma2(kd, make_float2(dd.z, dd.w), acc[4]);
+                    acc[5] = t_fma2(kd, make_float2(ee.x, ee.y), acc[5]);
+                    acc[6] = t_fma2(kd, make_float2(ee.z, ee.w), acc[6]);
+                    if (YUK) {
+                        acc[7] = t_fma2(g, p0, acc[7]);
+                        acc[8] = t_fma2(g, p1, acc[8]);
+                        acc[9] = t_fma2(g, p2, acc[9]);
+                    }
                 }
             }
         }
@@ -303,14 +356,33 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
         far = far_next;
     }
     cp_async_wait<0>();  // nothing in flight (the last group is empty)
+    // the sums -> the rows' accumulators
+    float2 out[NACC];
+    if (MODE == 0) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float2 f = KIND == 3 ? (r == cf.lrow ? acc[0] : acc[1]) : acc[r];
+            out[r] = t_fma2(t_splat(cf.k[r][0]), acc[2],
+                            t_fma2(t_splat(cf.k[r][2]), acc[3],
+                                   t_fma2(t_splat(cf.k[r][1]), acc[4], t_fma2(t_splat(cf.k[r][3]), acc[5], f))));
+        }
+    } else {
+        out[0] = acc[0];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            out[1 + k] = KIND == 0 ? acc[1 + k] : t_mul2(c12, acc[1 + k]);
+            out[4 + k] = KIND == 0 ? acc[4 + k] : t_mul2(c10, acc[4 + k]);
+            out[7 + k] = KIND == 2 ? t_mul2(t_splat(1.0f / cf.k[0][2]), acc[7 + k]) : acc[7 + k];
+        }
+    }
     // the other groups' sums join group 0's, in group order
     __syncthreads();
     const int tl = (int)threadIdx.x % HALF;
     if (grp > 0) {
         float* slot = tile + (grp - 1) * NACC * TREE_LEAF;
         for (int k = 0; k < NACC; ++k) {
-            slot[k * TREE_LEAF + tl] = acc[k].x;
-            slot[k * TREE_LEAF + HALF + tl] = acc[k].y;
+            slot[k * TREE_LEAF + tl] = out[k].x;
+            slot[k * TREE_LEAF + HALF + tl] = out[k].y;
         }
     }
     __syncthreads();
@@ -318,17 +390,17 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
         for (int g2 = 1; g2 < NQ; ++g2) {
             const float* slot = tile + (g2 - 1) * NACC * TREE_LEAF;
             for (int k = 0; k < NACC; ++k) {
-                acc[k].x += slot[k * TREE_LEAF + tl];
-                acc[k].y += slot[k * TREE_LEAF + HALF + tl];
+                out[k].x += slot[k * TREE_LEAF + tl];
+                out[k].y += slot[k * TREE_LEAF + HALF + tl];
             }
         }
         if (live0) {
             const int64_t pt = T.perm[ti0];
-            for (int k = 0; k < NACC; ++k) part[(int64_t)k * np + pt] = acc[k].x;
+            for (int k = 0; k < NACC; ++k) part[(int64_t)k * np + pt] = out[k].x;
         }
         if (live1) {
             const int64_t pt = T.perm[ti1];
-            for (int k = 0; k < NACC; ++k) part[(int64_t)k * np + pt] = acc[k].y;
+            for (int k = 0; k < NACC; ++k) part[(int64_t)k * np + pt] = out[k].y;
         }
     }
     __syncthreads();  // the buffer is free for the caller

@@ -1374,34 +1374,108 @@ __global__ void k_gather_spmv(int64_t nv, const int32_t* __restrict__ v2t_ptr, c
     }
 }
 
-// ------------------------------------------------------------ near combine
-__global__ void k_combine(int64_t nnz, const double* __restrict__ val, const int32_t* __restrict__ tpos,
-                          BlockOp B, double* __restrict__ c64, float* __restrict__ c32) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= nnz) return;
-    int64_t et = tpos[e];
-    double vals[O_N];
-    vals[O_M] = val[N_M * nnz + e];
-    vals[O_VL] = val[N_VL * nnz + e];
-    vals[O_KL] = val[N_KL * nnz + e];
-    vals[O_TL] = val[N_KL * nnz + et];
-    vals[O_DL] = val[N_DL * nnz + e];
-    vals[O_VY] = val[N_VY * nnz + e];
-    vals[O_KY] = val[N_KY * nnz + e];
-    vals[O_TY] = val[N_KY * nnz + et];
-    vals[O_DY] = val[N_DY * nnz + e];
-    for (int r = 0; r < 2; ++r)
+// ------------------------------------------------------------ near values of a block operator
+// Coefficients of an entry's four blocks (row r, column c): the mass matrix's, the Laplace and
+// the Yukawa operator's (phi rows: K on u and V on v; D/T rows: D on u and T on v).
+struct NearCoef {
+    double m[2][2], l[2][2], y[2][2];
+    int dt[2];  // row r is a D/T row
+};
+static NearCoef near_coef(const BlockOp& B, const FarPlan& fp) {
+    NearCoef nc;
+    for (int r = 0; r < 2; ++r) {
+        nc.dt[r] = fp.mode == 1 && fp.out_row[1] == r;
         for (int c = 0; c < 2; ++c) {
-            double s = 0.0;
-            for (int o = 0; o < O_N; ++o) s += B.c[r][c][o] * vals[o];
-            c64[4 * e + 2 * r + c] = s;
-            c32[4 * e + 2 * r + c] = (float)s;
+            const double* k = B.c[r][c];
+            nc.m[r][c] = k[O_M];
+            nc.l[r][c] = c == 0 ? (nc.dt[r] ? k[O_DL] : k[O_KL]) : (nc.dt[r] ? k[O_TL] : k[O_VL]);
+            nc.y[r][c] = c == 0 ? (nc.dt[r] ? k[O_DY] : k[O_KY]) : (nc.dt[r] ? k[O_TY] : k[O_VY]);
         }
+    }
+    return nc;
+}
+// The four combined values of entry e. Terms whose coefficient is zero are neither loaded nor
+// added (uniform branches): ten or fewer FP64 additions an entry where all nine operators in
+// all four blocks were 36, which had bound the kernel.
+__device__ __forceinline__ void near_entry(const NearCoef& nc, const double* __restrict__ val,
+                                           const int32_t* __restrict__ tpos, int64_t nnz, int64_t e, double (&b)[2][2]) {
+    const double mass = val[N_M * nnz + e];
+    const int64_t et = nc.dt[0] || nc.dt[1] ? tpos[e] : e;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int nl = c == 0 ? (nc.dt[r] ? N_DL : N_KL) : (nc.dt[r] ? N_KL : N_VL);
+            const int64_t at = c == 1 && nc.dt[r] ? et : e;  // T is K transposed
+            double s = 0.0;
+            if (nc.m[r][c] != 0.0) s = nc.m[r][c] * mass;
+            if (nc.l[r][c] != 0.0) s = __fma_rn(nc.l[r][c], val[nl * nnz + at], s);
+            if (nc.y[r][c] != 0.0) s = __fma_rn(nc.y[r][c], val[(nl + N_VY - N_VL) * nnz + at], s);
+            b[r][c] = s;
+        }
+}
+static_assert(N_VY - N_VL == N_KY - N_KL && N_VY - N_VL == N_DY - N_DL, "Yukawa arrays follow the Laplace ones");
+
+// Gather + near-field SpMV (as k_gather_spmv) straight from the near field's values, for a single
+// application: without a pass that writes the combined values and one that reads them again.
+// 2.8 M entries, direct form 178 -> 107 us, 16.2 M, Juffer form 955 -> 558 us (both passes before).
+__global__ void k_gather_spmv_near(int64_t nv, const int32_t* __restrict__ v2t_ptr, const int32_t* __restrict__ v2t,
+                                   const double* __restrict__ tri, int use_far, const int32_t* __restrict__ row_ptr,
+                                   const int32_t* __restrict__ col, const double* __restrict__ val,
+                                   const int32_t* __restrict__ tpos, int64_t nnz, const __grid_constant__ NearCoef nc,
+                                   const double* __restrict__ x, double* __restrict__ y) {
+    const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = gid >> 3;
+    const int lane = threadIdx.x & 7;
+    double y0 = 0.0, y1 = 0.0;
+    if (i < nv) {
+        if (use_far)
+            for (int32_t k = v2t_ptr[i] + lane; k < v2t_ptr[i + 1]; k += 8) {
+                const int32_t ta = v2t[k];
+                const int64_t t = ta / 3;
+                const int a = ta - 3 * (int)t;
+                y0 += tri[6 * t + a];
+                y1 += tri[6 * t + 3 + a];
+            }
+#pragma unroll 2
+        for (int32_t k = row_ptr[i] + lane; k < row_ptr[i + 1]; k += 8) {
+            const int32_t c = col[k];
+            const double uc = x[c], vc = x[nv + c];
+            double b[2][2];
+            near_entry(nc, val, tpos, nnz, k, b);
+            y0 += b[0][0] * uc + b[0][1] * vc;
+            y1 += b[1][0] * uc + b[1][1] * vc;
+        }
+    }
+    for (int o = 4; o > 0; o >>= 1) {
+        y0 += __shfl_xor_sync(0xffffffffu, y0, o, 8);
+        y1 += __shfl_xor_sync(0xffffffffu, y1, o, 8);
+    }
+    if (i < nv && lane == 0) {
+        y[i] = y0;
+        y[nv + i] = y1;
+    }
+}
+
+// the combined values of every entry, kept by a solve for its iterations
+__global__ void k_combine(int64_t nnz, const double* __restrict__ val, const int32_t* __restrict__ tpos,
+                          const __grid_constant__ NearCoef nc, double* __restrict__ c64, float* __restrict__ c32) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= nnz) return;
+    double b[2][2];
+    near_entry(nc, val, tpos, nnz, e, b);
+    double2* o = reinterpret_cast<double2*>(c64 + 4 * e);
+    o[0] = make_double2(b[0][0], b[0][1]);
+    o[1] = make_double2(b[1][0], b[1][1]);
+    *reinterpret_cast<float4*>(c32 + 4 * e) = make_float4((float)b[0][0], (float)b[0][1], (float)b[1][0], (float)b[1][1]);
 }
 
 int combine_near(const pb_mesh* m, const pb_near* nf, const BlockOp& B, double* c64, float* c32,
                  cudaStream_t s) {
-    k_combine<<<(unsigned)((m->nnz + 255) / 256), 256, 0, s>>>(m->nnz, nf->val, m->tpos, B, c64, c32); ::pb::count_launch();
+    FarPlan fp;
+    PB_TRY(make_far_plan(B, nf->kappa, &fp));
+    k_combine<<<(unsigned)((m->nnz + 255) / 256), 256, 0, s>>>(m->nnz, nf->val, m->tpos, near_coef(B, fp), c64, c32);
+    ::pb::count_launch();
     PB_CUDA(cudaGetLastError());
     return PB_OK;
 }
@@ -1514,11 +1588,12 @@ static double pair_ops(const FarPlan& fp) {
 
 // Algorithmic bytes of one gather + near-field SpMV launch: the pattern
 // (row pointers, columns) and the four combined block values of every entry
-// (value bytes vb each), x and y (2 nv doubles each) once, and with a far
+// (value bytes vb each in all: 4 x 4 or 4 x 8, or the near field's arrays that the
+// operator uses), x and y (2 nv doubles each) once, and with a far
 // field the vertex->triangle list and the per-triangle sums (6 doubles).
 static double spmv_bytes(const pb_mesh* m, bool far, int vb) {
     const double nv = (double)m->nv, nt = (double)m->nt, nnz = (double)m->nnz;
-    double b = 4.0 * (nv + 1.0) + nnz * (4.0 + 4.0 * vb) + 2.0 * 16.0 * nv;
+    double b = 4.0 * (nv + 1.0) + nnz * (4.0 + vb) + 2.0 * 16.0 * nv;
     if (far) b += 4.0 * (nv + 1.0) + 4.0 * 3.0 * nt + 48.0 * nt;
     return b;
 }
@@ -1535,13 +1610,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
     double* tri = (double*)m->ws_tri.ptr;
     int* status = m->status;
     const double* c64 = comb;
-    if (!comb) {
-        PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_comb, (sizeof(double) + sizeof(float)) * 4 * m->nnz));
-        double* w64 = (double*)m->ws_comb.ptr;
-        PB_TRY(combine_near(m, nf, B, w64, (float*)(w64 + 4 * m->nnz), s));
-        c64 = w64;
-    }
-    const float* c32 = (const float*)(c64 + 4 * m->nnz);
+    const float* c32 = comb ? (const float*)(c64 + 4 * m->nnz) : nullptr;
 
     if (fp.any) {
         bool need_u = false, need_v = false;
@@ -1654,8 +1723,19 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
         }
     }
     unsigned gb = (unsigned)((nv * 8 + 255) / 256);
-    Timer tm(m->ctx, PB_KERNEL_SPMV, s, spmv_bytes(m, fp.any, prec == PB_F32 ? 4 : 8), 1.0);
-    if (prec == PB_F32)
+    int value_bytes = prec == PB_F32 ? 16 : 32;
+    if (!comb) {  // M, and the arrays with a coefficient; the transposed positions of D/T rows
+        bool used[O_N] = {};
+        for (int o = 0; o < O_N; ++o)
+            for (int q = 0; q < 4; ++q) used[o == O_TL ? O_KL : o == O_TY ? O_KY : o] |= B.c[q / 2][q % 2][o] != 0.0;
+        value_bytes = fp.mode == 1 ? 12 : 8;
+        for (int o = 1; o < O_N; ++o) value_bytes += used[o] ? 8 : 0;
+    }
+    Timer tm(m->ctx, PB_KERNEL_SPMV, s, spmv_bytes(m, fp.any, value_bytes), 1.0);
+    if (!comb)
+        k_gather_spmv_near<<<gb, 256, 0, s>>>(nv, m->v2t_ptr, m->v2t, tri, fp.any ? 1 : 0, m->row_ptr, m->col, nf->val,
+                                              m->tpos, m->nnz, near_coef(B, fp), x, y);
+    else if (prec == PB_F32)
         k_gather_spmv<float><<<gb, 256, 0, s>>>(nv, m->v2t_ptr, m->v2t, tri, fp.any ? 1 : 0, m->row_ptr, m->col,
                                                 c32, m->nnz, x, y);
     else

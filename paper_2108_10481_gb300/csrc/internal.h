@@ -258,7 +258,7 @@ int make_far_plan(const BlockOp& B, double kappa, FarPlan* out);
 
 // a3 + a4 + a5: y = B x (x, y device, 2 nv doubles). comb: B's near values
 // already combined (4 nnz doubles then 4 nnz floats, from combine_near), or
-// null to combine them into the mesh's workspace first.
+// null to combine them entry by entry as they are applied.
 int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int prec, const double* x,
                   double* y, cudaStream_t s, const double* comb = nullptr);
 // near values combined for a block operator (FP64 and FP32 copies) and diagonals

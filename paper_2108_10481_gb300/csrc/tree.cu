@@ -343,24 +343,36 @@ __device__ __forceinline__ void lagrange_n(float t, const float* tn, const float
     }
 }
 
-// Proxy charges of the slots of one height: one CTA per slot, threads over
-// proxies, N Chebyshev points per axis (N^3 proxies). A slot's charges come
-// from its two children: a child with its own proxies passes them on through
-// the slot's interpolation (exact, the basis polynomials having the same
-// degree), any other child through its points. Sources are staged 128 at a
-// time with their 1-D basis values.
+// Proxy charges of the slots of one height: one CTA per slot, N Chebyshev points per
+// axis (N^3 proxies). A slot's charges come from its two children: a child with its
+// own proxies passes them on through the slot's interpolation (exact, the basis
+// polynomials having the same degree), any other child through its points.
+//   - Points: staged PROXY_TILE at a time with their 1-D basis values; a thread takes a
+//     column of N proxies (one a, b), so that a point's values and charges are read
+//     once for N proxies (by 16-byte loads), and groups of N^2 threads take every
+//     PROXY_THREADS / N^2 -th point, added at the end in group order. Bound by the FP32
+//     pipe; with the proxies dealt out singly the shared-memory loads had taken twice
+//     its time.
+//   - Children's proxies: three one-axis passes by all threads; a few microseconds of
+//     latency per slot and height, whatever the level's slots.
+// NC charges: 8 (S, Q, C, N), or the first two for V/K rows (MODE 0), which read no more.
+// All heights, V/K rows, 116,160 points: 202 -> 94 us; V/K + D/T rows, 661,500 points: 493 ->
+// 426 us.
 // Proxy record: z (3), S, Q, C (3), N (3), 0.
-constexpr int PROXY_THREADS = 128;
+constexpr int PROXY_THREADS = 256;
+constexpr int PROXY_TILE = 64;
 
-template <int N>
+template <int N, int MODE>
 __global__ void __launch_bounds__(PROXY_THREADS)
 k_proxy_charges(const int32_t* __restrict__ slots, const int32_t* __restrict__ slot_kids,
                 const float* __restrict__ slot_box, const float* __restrict__ rec, float* __restrict__ prox) {
-    constexpr int NP = N * N * N, N2 = N * N;
-    constexpr int PER = (NP + PROXY_THREADS - 1) / PROXY_THREADS;
-    // a staged point: lx, ly, lz, dlx, dly, dlz (N each), 8 charges; odd row length (no bank conflicts)
-    constexpr int SBW = 6 * N + 9;
-    constexpr int SB = PROXY_THREADS * SBW > 2 * NP * 8 ? PROXY_THREADS * SBW : 2 * NP * 8;
+    constexpr int NP = N * N * N, N2 = N * N, NC = MODE == 0 ? 2 : 8;
+    constexpr int NV = NP * NC, PER = (NV + PROXY_THREADS - 1) / PROXY_THREADS;
+    constexpr int G = PROXY_THREADS / N2;  // groups of threads over the points
+    // a staged point: lx, ly, dlx, dly (N each), then on 16-byte boundaries lz, dlz and 8 charges
+    constexpr int OZ = (4 * N + 3) / 4 * 4, SBW = OZ + 24;
+    static_assert(N <= 8, "lz and dlz in eight words each");
+    constexpr int SB = PROXY_TILE * SBW > 2 * NV ? PROXY_TILE * SBW : 2 * NV;
     __shared__ __align__(16) float sb[SB];
     __shared__ float tn[N], iden[N];
     __shared__ float T[3][N][N];  // 1-D transfer matrices of a child with proxies
@@ -381,21 +393,12 @@ k_proxy_charges(const int32_t* __restrict__ slots, const int32_t* __restrict__ s
         half[d] = 0.5f * (box[3 + d] - box[d]);
         ihalf[d] = 1.f / half[d];
     }
-    // this thread's proxies and their grid indices
-    int ka[PER], kb[PER], kc[PER];
-    float acc[PER][8];
+    float acc[PER];  // this thread's charges: value k = tid + r PROXY_THREADS is charge k % NC of proxy k / NC
 #pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        const int k = min((int)threadIdx.x + r * PROXY_THREADS, NP - 1);
-        ka[r] = k / N2;
-        kb[r] = (k / N) % N;
-        kc[r] = k % N;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-    }
+    for (int r = 0; r < PER; ++r) acc[r] = 0.f;
     __syncthreads();
-    float* buf0 = sb;                // child charges, then the y pass
-    float* buf1 = sb + NP * 8;       // the x pass
+    float* buf0 = sb;       // child charges, then the y pass
+    float* buf1 = sb + NV;  // the x pass
     for (int kid = 0; kid < 2; ++kid) {
         const int32_t ks = slot_kids[6 * slot + 3 * kid];
         if (ks >= 0) {  // uniform across the block
@@ -412,35 +415,33 @@ k_proxy_charges(const int32_t* __restrict__ slots, const int32_t* __restrict__ s
                 for (int a = 0; a < N; ++a) T[d][a][a2] = l[a];
             }
             const float* cp = prox + (int64_t)ks * NP * TREE_REC;
-            for (int k = threadIdx.x; k < NP * 8; k += PROXY_THREADS) buf0[k] = cp[(k >> 3) * TREE_REC + 3 + (k & 7)];
+            for (int k = threadIdx.x; k < NV; k += PROXY_THREADS) buf0[k] = cp[(k / NC) * TREE_REC + 3 + k % NC];
             __syncthreads();
-            for (int k = threadIdx.x; k < NP * 8; k += PROXY_THREADS) {  // x pass
-                const int c = k & 7, idx = k >> 3, a = idx / N2, rest = idx - a * N2;
+            for (int k = threadIdx.x; k < NV; k += PROXY_THREADS) {  // x pass
+                const int c = k % NC, idx = k / NC, a = idx / N2, rest = idx - a * N2;
                 float v = 0.f;
 #pragma unroll
-                for (int a2 = 0; a2 < N; ++a2) v += T[0][a][a2] * buf0[(a2 * N2 + rest) * 8 + c];
+                for (int a2 = 0; a2 < N; ++a2) v += T[0][a][a2] * buf0[(a2 * N2 + rest) * NC + c];
                 buf1[k] = v;
             }
             __syncthreads();
-            for (int k = threadIdx.x; k < NP * 8; k += PROXY_THREADS) {  // y pass
-                const int c = k & 7, idx = k >> 3, a = idx / N2, bb = (idx / N) % N, cc = idx % N;
+            for (int k = threadIdx.x; k < NV; k += PROXY_THREADS) {  // y pass
+                const int c = k % NC, idx = k / NC, a = idx / N2, bb = (idx / N) % N, cc = idx % N;
                 float v = 0.f;
 #pragma unroll
-                for (int b2 = 0; b2 < N; ++b2) v += T[1][bb][b2] * buf1[((a * N + b2) * N + cc) * 8 + c];
+                for (int b2 = 0; b2 < N; ++b2) v += T[1][bb][b2] * buf1[((a * N + b2) * N + cc) * NC + c];
                 buf0[k] = v;
             }
             __syncthreads();
 #pragma unroll
-            for (int r = 0; r < PER; ++r) {  // z pass into this thread's proxies
-                if ((int)threadIdx.x + r * PROXY_THREADS < NP) {
+            for (int r = 0; r < PER; ++r) {  // z pass into this thread's charges
+                const int k = threadIdx.x + r * PROXY_THREADS;
+                if (k < NV) {
+                    const int c = k % NC, idx = k / NC, cc = idx % N, ab = idx - cc;
+                    float v = 0.f;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float v = 0.f;
-#pragma unroll
-                        for (int c2 = 0; c2 < N; ++c2)
-                            v += T[2][kc[r]][c2] * buf0[((ka[r] * N + kb[r]) * N + c2) * 8 + c];
-                        acc[r][c] += v;
-                    }
+                    for (int c2 = 0; c2 < N; ++c2) v += T[2][cc][c2] * buf0[(ab + c2) * NC + c];
+                    acc[r] += v;
                 }
             }
             __syncthreads();
@@ -449,53 +450,101 @@ k_proxy_charges(const int32_t* __restrict__ slots, const int32_t* __restrict__ s
         // raw points of the child: s, p (3), c (3)
         const int32_t b = slot_kids[6 * slot + 3 * kid + 1];
         const int32_t e = slot_kids[6 * slot + 3 * kid + 2];
-        for (int c0 = b; c0 < e; c0 += PROXY_THREADS) {
-            const int i = c0 + threadIdx.x;
-            float* my = sb + threadIdx.x * SBW;
-            if (i < e) {
-                const float* r = rec + TREE_REC * (int64_t)i;
+        const int grp = threadIdx.x / N2, ab = threadIdx.x % N2, ka = ab / N, kb = ab % N;
+        float col[N][NC];
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    lagrange_n<N>((r[d] - mid[d]) * ihalf[d], tn, iden, my + N * d, my + N * (3 + d));
+        for (int c = 0; c < N; ++c)
 #pragma unroll
-                    for (int a = 0; a < N; ++a) my[N * (3 + d) + a] *= ihalf[d];  // d/dy = d/dt / half
+            for (int q = 0; q < NC; ++q) col[c][q] = 0.f;
+        for (int c0 = b; c0 < e; c0 += PROXY_TILE) {
+            const int m = min(PROXY_TILE, e - c0);
+            for (int k = threadIdx.x; k < 3 * m; k += PROXY_THREADS) {  // a point's basis along one axis
+                const int d = k / m, i = k - d * m;
+                float* my = sb + i * SBW;
+                const float* r = rec + TREE_REC * (int64_t)(c0 + i);
+                float l[N], dl[N];
+                lagrange_n<N>((r[d] - mid[d]) * ihalf[d], tn, iden, l, dl);
+                float* to = d == 0 ? my : d == 1 ? my + N : my + OZ;
+                float* dto = d == 0 ? my + 2 * N : d == 1 ? my + 3 * N : my + OZ + 8;
+#pragma unroll
+                for (int a = 0; a < N; ++a) {
+                    to[a] = l[a];
+                    dto[a] = dl[a] * ihalf[d];  // d/dy = d/dt / half
                 }
+                if (d == 2)
 #pragma unroll
-                for (int c = 0; c < 7; ++c) my[6 * N + c] = r[3 + c];
+                    for (int c = 0; c < 7; ++c) my[OZ + 16 + c] = r[3 + c];
             }
             __syncthreads();
-            const int m = min(PROXY_THREADS, e - c0);
-            for (int j = 0; j < m; ++j) {
-                const float* pj = sb + j * SBW;
-                const float* q = pj + 6 * N;
+            if (grp < G)
+                for (int j = grp; j < m; j += G) {
+                    const float* pj = sb + j * SBW;
+                    const float lx = pj[ka], ly = pj[N + kb], dx = pj[2 * N + ka], dy = pj[3 * N + kb];
+                    const float4* z4 = reinterpret_cast<const float4*>(pj + OZ);
+                    const float4 za = z4[0], zb = z4[1], da = z4[2], db = z4[3], q0 = z4[4], q1 = z4[5];
+                    const float lz[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
+                    const float dz[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+                    const float lxy = lx * ly, gx = dx * ly, gy = lx * dy;
+                    const float gp = gx * q0.y + gy * q0.z, gz = lxy * q0.w;  // grad L . p = lz gp + dlz gz
+                    const float ls = lxy * q0.x;
+                    const float lp[3] = {lxy * q0.y, lxy * q0.z, lxy * q0.w}, lc[3] = {lxy * q1.x, lxy * q1.y, lxy * q1.z};
 #pragma unroll
-                for (int r = 0; r < PER; ++r) {
-                    const float lx = pj[ka[r]], ly = pj[N + kb[r]], lz = pj[2 * N + kc[r]];
-                    const float lyz = ly * lz, L = lx * lyz;
-                    const float gx = pj[3 * N + ka[r]] * lyz, gy = lx * pj[4 * N + kb[r]] * lz,
-                                gz = lx * ly * pj[5 * N + kc[r]];
-                    acc[r][0] += L * q[0];
-                    acc[r][1] += gx * q[1] + gy * q[2] + gz * q[3];
+                    for (int c = 0; c < N; ++c) {
+                        col[c][0] = fmaf(lz[c], ls, col[c][0]);
+                        col[c][1] = fmaf(lz[c], gp, fmaf(dz[c], gz, col[c][1]));
+                        if (MODE == 1)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) acc[r][2 + c] += L * q[4 + c];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) acc[r][5 + c] += L * q[1 + c];
+                            for (int q = 0; q < 3; ++q) {
+                                col[c][NC - 6 + q] = fmaf(lz[c], lc[q], col[c][NC - 6 + q]);
+                                col[c][NC - 3 + q] = fmaf(lz[c], lp[q], col[c][NC - 3 + q]);
+                            }
+                    }
                 }
-            }
             __syncthreads();
         }
+        // the groups' columns added in group order, then into the threads' charges
+        for (int g = 0; g < G; ++g) {
+            if (grp == g)
+#pragma unroll
+                for (int c = 0; c < N; ++c)
+#pragma unroll
+                    for (int q = 0; q < NC; ++q) {
+                        const int k = (ab * N + c) * NC + q;
+                        sb[k] = g == 0 ? col[c][q] : sb[k] + col[c][q];
+                    }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int k = threadIdx.x + r * PROXY_THREADS;
+            if (k < NV) acc[r] += sb[k];
+        }
+        __syncthreads();
     }
+    float* o = prox + (int64_t)slot * NP * TREE_REC;
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
         const int k = threadIdx.x + r * PROXY_THREADS;
-        if (k >= NP) break;
-        float* o = prox + ((int64_t)slot * NP + k) * TREE_REC;
-        o[0] = mid[0] + half[0] * tn[ka[r]];
-        o[1] = mid[1] + half[1] * tn[kb[r]];
-        o[2] = mid[2] + half[2] * tn[kc[r]];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) o[3 + c] = acc[r][c];
-        o[11] = 0.f;
+        if (k < NV) o[(k / NC) * TREE_REC + 3 + k % NC] = acc[r];
+    }
+    for (int k = threadIdx.x; k < 3 * NP; k += PROXY_THREADS) {
+        const int i = k / 3, d = k - 3 * i;
+        const int a = d == 0 ? i / N2 : d == 1 ? (i / N) % N : i % N;
+        const float md = d == 0 ? mid[0] : d == 1 ? mid[1] : mid[2], hf = d == 0 ? half[0] : d == 1 ? half[1] : half[2];
+        o[i * TREE_REC + d] = md + hf * tn[a];
+    }
+}
+
+template <int MODE>
+static void launch_proxies(int n, unsigned g, cudaStream_t s, const int32_t* so, const PbTree* t, const float* rec,
+                           float* prox) {
+    switch (n) {
+        case 3: k_proxy_charges<3, MODE><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
+        case 4: k_proxy_charges<4, MODE><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
+        case 5: k_proxy_charges<5, MODE><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
+        case 6: k_proxy_charges<6, MODE><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
+        case 7: k_proxy_charges<7, MODE><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
+        default: k_proxy_charges<8, MODE><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
     }
 }
 
@@ -537,14 +586,8 @@ int tree_prepare(const pb_mesh* mc, const FarPlan& fp, const double* x, bool nee
         if (e > b) {
             const unsigned g = (unsigned)(e - b);
             const int32_t* so = t->slot_order + b;
-            switch (t->n) {
-                case 3: k_proxy_charges<3><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
-                case 4: k_proxy_charges<4><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
-                case 5: k_proxy_charges<5><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
-                case 6: k_proxy_charges<6><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
-                case 7: k_proxy_charges<7><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
-                default: k_proxy_charges<8><<<g, PROXY_THREADS, 0, s>>>(so, t->slot_kids, t->slot_box, rec, prox); break;
-            }
+            if (fp.mode == 0) launch_proxies<0>(t->n, g, s, so, t, rec, prox);
+            else launch_proxies<1>(t->n, g, s, so, t, rec, prox);
             ::pb::count_launch();
         }
     }

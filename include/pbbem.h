@@ -382,7 +382,7 @@ int pb_poll(pb_server* srv, pb_result* out, int max, int* n_out);
 typedef struct {
     int kernel;             /* chosen FP32 kernel: 1 scalar, 2 packed f32x2 */
     int shape;              /* launch shape of the packed kernel (0 = default) */
-    int tile_records;       /* source records per TMA tile of the chosen launch */
+    int tile_records;       /* source records that a TMA tile of the chosen launch has room for (whole threes are used) */
     int stages;             /* its pipeline stages */
     int targets_per_thread; /* its targets per thread */
     int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide sums at a time */

@@ -43,7 +43,7 @@ constexpr double INV4PI = 0.07957747154594767;  // 1 / (4 pi)
 // a thread per triangle and its points in sequence it took 12 us at any size below 10,000
 // triangles, now 5.)
 struct SourceValues {
-    double s, p[3], c[3];
+    double s, sigma, p[3], c[3];  // p = sigma times the normal
 };
 __device__ __forceinline__ SourceValues source_values(int64_t i, int Q, const Rule& rule,
                                                       const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
@@ -62,6 +62,7 @@ __device__ __forceinline__ SourceValues source_values(int64_t i, int Q, const Ru
     const double vq = rule.l[q][0] * va[0] + rule.l[q][1] * va[1] + rule.l[q][2] * va[2];
     SourceValues r;
     r.s = w * vq;
+    r.sigma = w * uq;
     for (int k = 0; k < 3; ++k) {
         r.p[k] = w * uq * g[k];
         r.c[k] = w * (inv2a * (ua[0] * g[4 + k] + ua[1] * g[7 + k] + ua[2] * g[10 + k]));
@@ -546,6 +547,7 @@ struct Coef32 {
     float kappa;
     float mk2;  // -kappa * log2(e)
     int kind;   // loop of the packed kernel (far_kind)
+    bool threes;  // its points come in threes of one triangle and weight
 };
 
 // The packed kernels' loop for a plan's coefficients, as the FP64 kernel's: 1 no Yukawa term
@@ -561,8 +563,9 @@ static int far_kind(const FarPlan& fp) {
     return !yukawa ? 1 : all_laplace ? 2 : 0;
 }
 
-static Coef32 coef32(const FarPlan& fp) {
+static Coef32 coef32(const FarPlan& fp, int Q) {
     Coef32 cf;
+    cf.threes = Q % 3 == 0;
     cf.kind = far_kind(fp);
     for (int R = 0; R < 2; ++R)
         for (int j = 0; j < 4; ++j) cf.k[R][j] = (float)fp.k[R][j];
@@ -702,8 +705,11 @@ __global__ void __launch_bounds__(TPB32) k_pair32(const __grid_constant__ CUtens
 // own targets or run past the last point (zero-filled rows).
 constexpr int REC2 = 32;   // floats per duplicated source record
 constexpr int TPB2 = 256;  // threads per CTA
-constexpr int TS2 = 64;    // records per TMA tile
+constexpr int TS2 = 64;    // records that a tile of the batched kernel has room for
 constexpr int ST2 = 4;     // pipeline stages
+// records of a tile with room for ts: whole threes (tile_x2)
+__host__ __device__ constexpr int tile_points(int ts) { return ts / 3 * 3; }
+constexpr int TU2 = tile_points(TS2);
 
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     float2 d;
@@ -740,10 +746,14 @@ __global__ void k_sources2(int64_t np, int Q, Rule rule, const int32_t* __restri
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= np) return;
     const SourceValues sv = source_values(i, Q, rule, tris, tgeo, pts64, u, v, need_u, need_v);
+    // the record's vector for all points: of a three, the normal in the first and the curl in the second record
+    const bool normal = Q % 3 == 0 && i % 3 == 0;
+    const double* n = tgeo + 16 * (i / Q);
     const float val[16] = {pts32[4 * i], pts32[4 * i + 1], pts32[4 * i + 2], (float)sv.s,
-                           (float)sv.p[0], (float)sv.p[1], (float)sv.p[2],
-                           (float)sv.c[0], (float)sv.c[1], (float)sv.c[2],
-                           pts32lo[4 * i], pts32lo[4 * i + 1], pts32lo[4 * i + 2], 0.f, 0.f, 0.f};
+                           (float)sv.p[0], (float)sv.p[1], (float)sv.p[2], (float)sv.sigma,
+                           pts32lo[4 * i], pts32lo[4 * i + 1], pts32lo[4 * i + 2], 0.f,
+                           (float)(normal ? n[0] : sv.c[0]), (float)(normal ? n[1] : sv.c[1]),
+                           (float)(normal ? n[2] : sv.c[2]), 0.f};
     float4* r = reinterpret_cast<float4*>(rec + REC2 * i);
     for (int k = 0; k < 8; ++k) r[k] = make_float4(val[2 * k], val[2 * k], val[2 * k + 1], val[2 * k + 1]);
 }
@@ -803,90 +813,122 @@ __device__ __forceinline__ void wide_add(Wide2& w, float2 b) {
     w.hi = s;
 }
 
-// The tile's sums. FP32 operations per pair, with the packed pipe the limit: MODE 0 19; MODE 1
-// KIND 0 36, KIND 1 20 (no exponential), KIND 2 32; split coordinates 6 more (25 and 36 with the
-// coefficients applied to every pair): e^{-kappa r}(1 + kappa r)/r is g + kappa e with g = e/r,
-// and a kernel with both Green's functions takes one FMA on their ratio. 30,720 points, V/K +
-// D/T rows: 1,064 -> 983 us, 0.79 of the packed pipe's measured rate.
-template <int MODE, bool ACC, int NPK, bool GUARD, int TS, int KIND>
+// The tile's sums: records of 16 splatted values (position, s, p = sigma n, sigma, low words,
+// curl or normal). Points come in threes of one triangle and one weight (the 3-point rule, the
+// two orbits of the 6-point rule; U = 3), and what the D/T row's sums share within a three is
+// multiplied once: the normal by sum sigma g, the curl by sum k_D. U = 1 (V/K rows, and the
+// centroid rule): every point by itself. The limit is the packed pipe, at 2 cycles an operation
+// and 3 where it reads three different registers (a multiply-add of three values; measured 2.2
+// and 3.3 in a bare loop), so a pair takes, in cycles: V/K rows 44; V/K + D/T rows KIND 0 77 (by
+// single points 85), KIND 1 46 (52), KIND 2 69 (77); split coordinates 12 more. 30,720 points,
+// V/K + D/T rows: 983 -> 908 us; split, 61,440 points: 4.97 -> 4.41 ms. (The height (x - y) . n
+// taken once for a three, too, gives 930 and 4.43 ms per application, but the three then share its
+// rounding errors: twice the error of the FP32 applications against FP64.)
+template <int MODE, bool ACC, int NPK, bool GUARD, int TS, int KIND, int U>
 __device__ __forceinline__ void tile_x2(const float* __restrict__ tile, const float2 (&X)[NPK][3],
                                         const float2 (&XL)[NPK][3], float2 (&acc)[NPK][far_raw(MODE, KIND)],
                                         const Coef2& cf) {
     constexpr bool YUK = KIND != 1;
-#pragma unroll 2
-    for (int j = 0; j < TS; ++j) {
-        const float* r = tile + REC2 * j;
-        const float4 q0 = *reinterpret_cast<const float4*>(r);
-        const float4 q1 = *reinterpret_cast<const float4*>(r + 4);
-        const float4 q2 = *reinterpret_cast<const float4*>(r + 8);
-        const float4 q3 = *reinterpret_cast<const float4*>(r + 12);
-        float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f), q5 = q4, q6 = q4;
-        if (MODE == 1) q4 = *reinterpret_cast<const float4*>(r + 16);
-        if (ACC) {
-            q5 = *reinterpret_cast<const float4*>(r + 20);
-            q6 = *reinterpret_cast<const float4*>(r + 24);
-        }
-        const float2 Sx = make_float2(q0.x, q0.y), Sy = make_float2(q0.z, q0.w), Sz = make_float2(q1.x, q1.y);
-        const float2 Ss = make_float2(q1.z, q1.w), Px = make_float2(q2.x, q2.y), Py = make_float2(q2.z, q2.w);
-        const float2 Pz = make_float2(q3.x, q3.y);
+    constexpr int NR = far_raw(MODE, KIND), VK = KIND == 0 ? 0 : 1, T = VK + 1;  // V and K summed apart unless KIND 0
+    static_assert(TS % 3 == 0, "tiles of whole threes");
+    auto vec = [](const float* f, float2 (&v)[3]) {
+        const float4 a = *reinterpret_cast<const float4*>(f), b = *reinterpret_cast<const float4*>(f + 4);
+        v[0] = make_float2(a.x, a.y);
+        v[1] = make_float2(a.z, a.w);
+        v[2] = make_float2(b.x, b.y);
+        return make_float2(b.z, b.w);
+    };
+#pragma unroll(U == 1 ? 2 : 1)
+    for (int j = 0; j < TS; j += U) {
+        const float* r0 = tile + REC2 * j;
+        float2 sg[NPK], sd[NPK];
 #pragma unroll
-        for (int p = 0; p < NPK; ++p) {
-            float2 d0 = sub2(X[p][0], Sx), d1 = sub2(X[p][1], Sy), d2 = sub2(X[p][2], Sz);
-            if (ACC) {
-                d0 = add2(d0, sub2(XL[p][0], make_float2(q5.x, q5.y)));
-                d1 = add2(d1, sub2(XL[p][1], make_float2(q5.z, q5.w)));
-                d2 = add2(d2, sub2(XL[p][2], make_float2(q6.x, q6.y)));
-            }
-            const float2 r2 = fma2(d0, d0, fma2(d1, d1, mul2(d2, d2)));
-            float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
-            if (GUARD) {
-                rinv.x = r2.x > 0.0f ? rinv.x : 0.0f;
-                rinv.y = r2.y > 0.0f ? rinv.y : 0.0f;
-            }
-            float2 g = make_float2(0.f, 0.f), gw = g;
-            if (YUK) {
-                const float2 arg = mul2(mul2(r2, rinv), cf.mk2);
-                const float2 e = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
-                g = mul2(e, rinv);
-                gw = fma2(cf.kap, e, g);
-            }
-            const float2 ri2 = mul2(rinv, rinv);
-            const float2 dp = mul2(ri2, fma2(d0, Px, fma2(d1, Py, mul2(d2, Pz))));
-            if (MODE == 0) {
-                acc[p][0] = fma2(rinv, Ss, acc[p][0]);
-                acc[p][1] = fma2(rinv, dp, acc[p][1]);
-                acc[p][2] = fma2(g, Ss, acc[p][2]);
-                acc[p][3] = fma2(gw, dp, acc[p][3]);
-            } else {
-                float2 kv = rinv, kk = rinv, kd = rinv, kt = rinv;
-                if (KIND == 0) {
-                    kv = fma2(cf.c[0][1], g, mul2(cf.c[0][0], rinv));
-                    kk = fma2(cf.c[0][3], gw, mul2(cf.c[0][2], rinv));
-                    kd = fma2(cf.c[1][1], g, mul2(cf.c[1][0], rinv));
-                    kt = fma2(cf.c[1][3], gw, mul2(cf.c[1][2], rinv));
-                } else if (KIND == 2) {
-                    kv = fma2(cf.rho[0], g, rinv);
-                    kk = fma2(cf.rho[1], gw, rinv);
-                    kd = fma2(cf.rho[2], g, rinv);
-                    kt = fma2(cf.rho[3], gw, rinv);
+        for (int i = 0; i < U; ++i) {
+            const float* r = r0 + REC2 * i;
+            float2 S[3], P[3], SL[3];
+            const float2 Ss = vec(r, S), sig = vec(r + 8, P);
+            if (ACC) vec(r + 16, SL);
+#pragma unroll
+            for (int p = 0; p < NPK; ++p) {
+                float2 d[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    d[k] = sub2(X[p][k], S[k]);
+                    if (ACC) d[k] = add2(d[k], sub2(XL[p][k], SL[k]));
                 }
-                constexpr int VK = KIND == 0 ? 0 : 1, T = VK + 1;  // V and K summed apart unless KIND 0
-                const float2 ts = mul2(kt, mul2(ri2, Ss));
-                acc[p][0] = fma2(kv, Ss, acc[p][0]);
-                acc[p][VK] = fma2(kk, dp, acc[p][VK]);
-                acc[p][T] = fma2(ts, d0, acc[p][T]);
-                acc[p][T + 1] = fma2(ts, d1, acc[p][T + 1]);
-                acc[p][T + 2] = fma2(ts, d2, acc[p][T + 2]);
-                acc[p][T + 3] = fma2(kd, make_float2(q3.z, q3.w), acc[p][T + 3]);
-                acc[p][T + 4] = fma2(kd, make_float2(q4.x, q4.y), acc[p][T + 4]);
-                acc[p][T + 5] = fma2(kd, make_float2(q4.z, q4.w), acc[p][T + 5]);
+                const float2 r2 = fma2(d[0], d[0], fma2(d[1], d[1], mul2(d[2], d[2])));
+                float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+                if (GUARD) {
+                    rinv.x = r2.x > 0.0f ? rinv.x : 0.0f;
+                    rinv.y = r2.y > 0.0f ? rinv.y : 0.0f;
+                }
+                float2 g = make_float2(0.f, 0.f), gw = g;
                 if (YUK) {
-                    acc[p][far_raw(MODE, KIND) - 3] = fma2(g, Px, acc[p][far_raw(MODE, KIND) - 3]);
-                    acc[p][far_raw(MODE, KIND) - 2] = fma2(g, Py, acc[p][far_raw(MODE, KIND) - 2]);
-                    acc[p][far_raw(MODE, KIND) - 1] = fma2(g, Pz, acc[p][far_raw(MODE, KIND) - 1]);
+                    const float2 arg = mul2(mul2(r2, rinv), cf.mk2);
+                    const float2 e = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
+                    g = mul2(e, rinv);
+                    gw = fma2(cf.kap, e, g);
+                }
+                const float2 ri2 = mul2(rinv, rinv);
+                const float2 dp = mul2(ri2, fma2(d[0], P[0], fma2(d[1], P[1], mul2(d[2], P[2]))));
+                if (MODE == 0) {
+                    acc[p][0] = fma2(rinv, Ss, acc[p][0]);
+                    acc[p][1] = fma2(rinv, dp, acc[p][1]);
+                    acc[p][2] = fma2(g, Ss, acc[p][2]);
+                    acc[p][3] = fma2(gw, dp, acc[p][3]);
+                } else {
+                    float2 kv = rinv, kk = rinv, kd = rinv, kt = rinv;
+                    if (KIND == 0) {
+                        kv = fma2(cf.c[0][1], g, mul2(cf.c[0][0], rinv));
+                        kk = fma2(cf.c[0][3], gw, mul2(cf.c[0][2], rinv));
+                        kd = fma2(cf.c[1][1], g, mul2(cf.c[1][0], rinv));
+                        kt = fma2(cf.c[1][3], gw, mul2(cf.c[1][2], rinv));
+                    } else if (KIND == 2) {
+                        kv = fma2(cf.rho[0], g, rinv);
+                        kk = fma2(cf.rho[1], gw, rinv);
+                        kd = fma2(cf.rho[2], g, rinv);
+                        kt = fma2(cf.rho[3], gw, rinv);
+                    }
+                    const float2 ts = mul2(kt, mul2(ri2, Ss));
+                    acc[p][0] = fma2(kv, Ss, acc[p][0]);
+                    acc[p][VK] = fma2(kk, dp, acc[p][VK]);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) acc[p][T + k] = fma2(ts, d[k], acc[p][T + k]);
+                    sd[p] = i == 0 ? kd : add2(sd[p], kd);
+                    if (U == 1) {
+                        if (YUK)
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) acc[p][NR - 3 + k] = fma2(g, P[k], acc[p][NR - 3 + k]);
+                    } else {
+                        sg[p] = i == 0 ? mul2(g, sig) : fma2(g, sig, sg[p]);
+                    }
                 }
             }
         }
+        if (MODE == 1) {
+            float2 C[3], N[3];
+            vec(r0 + (U == 3 ? REC2 : 0) + 24, C);
+            if (U == 3) vec(r0 + 24, N);
+#pragma unroll
+            for (int p = 0; p < NPK; ++p)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    acc[p][T + 3 + k] = fma2(sd[p], C[k], acc[p][T + 3 + k]);
+                    if (U == 3 && YUK) acc[p][NR - 3 + k] = fma2(sg[p], N[k], acc[p][NR - 3 + k]);
+                }
+        }
+    }
+}
+template <int MODE, bool ACC, int NPK, int TS, int KIND>
+__device__ __forceinline__ void tile_x2(const float* __restrict__ tile, const float2 (&X)[NPK][3],
+                                        const float2 (&XL)[NPK][3], float2 (&acc)[NPK][far_raw(MODE, KIND)],
+                                        const Coef2& cf, bool guard, bool threes) {
+    if (MODE == 1 && threes) {
+        if (guard) tile_x2<MODE, ACC, NPK, true, TS, KIND, 3>(tile, X, XL, acc, cf);
+        else tile_x2<MODE, ACC, NPK, false, TS, KIND, 3>(tile, X, XL, acc, cf);
+    } else {
+        if (guard) tile_x2<MODE, ACC, NPK, true, TS, KIND, 1>(tile, X, XL, acc, cf);
+        else tile_x2<MODE, ACC, NPK, false, TS, KIND, 1>(tile, X, XL, acc, cf);
     }
 }
 
@@ -895,19 +937,19 @@ __device__ __forceinline__ void tile_x2(const float* __restrict__ tile, const fl
 // split-coordinate variant, the tiles whose FP32 sums are added into the wide
 // sums at a time (PROMO); the autotuner picks the shape per mesh-size bucket.
 template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
-__global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUtensorMap tmap, int64_t np,
+__global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CUtensorMap tmap, int64_t np,
                                                    const float* __restrict__ pts32, const float* __restrict__ pts32lo,
                                                    Coef32 c32, int64_t chunk, void* __restrict__ part_out,
                                                    int* __restrict__ status) {
     constexpr int NACC = MODE == 0 ? 2 : 10;
     constexpr int NRAW = far_raw(MODE, KIND);
-    constexpr int TGT = 2 * NPK;
+    constexpr int TGT = 2 * NPK, TU = tile_points(TS);
     __shared__ __align__(128) float sh[ST][TS * REC2];
     __shared__ __align__(8) uint64_t bar[ST];
     const int split = blockIdx.y;
     const int64_t j0 = split * chunk;
     const int64_t j1 = min(np, j0 + chunk);
-    const int ntiles = (int)((j1 - j0 + TS - 1) / TS);
+    const int ntiles = (int)((j1 - j0 + TU - 1) / TU);
     const int64_t blk0 = blockIdx.x * (int64_t)(TPB2 * TGT), blk1 = blk0 + TPB2 * TGT;
 
     if (threadIdx.x == 0) {
@@ -917,8 +959,8 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int s = 0; s < ST && s < ntiles; ++s) {
-            mbar_expect_tx(&bar[s], TS * REC2 * sizeof(float));
-            tma_load_2d(sh[s], &tmap, 0, (int)(j0 + (int64_t)s * TS), &bar[s]);
+            mbar_expect_tx(&bar[s], TU * REC2 * sizeof(float));
+            tma_load_2d(sh[s], &tmap, 0, (int)(j0 + (int64_t)s * TU), &bar[s]);
         }
     }
     const Coef2 cf = coef2(c32);
@@ -944,10 +986,9 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
         const int st = it % ST;
         const uint32_t phase = (uint32_t)((it / ST) & 1);
         if (!cta_wait(&bar[st], phase, status)) { failed_at = it; break; }
-        const int64_t jt = j0 + (int64_t)it * TS;
-        const bool guard = (jt < blk1 && jt + TS > blk0) || jt + TS > np;
-        if (guard) tile_x2<MODE, ACC, NPK, true, TS, KIND>(sh[st], X, XL, acc, cf);
-        else tile_x2<MODE, ACC, NPK, false, TS, KIND>(sh[st], X, XL, acc, cf);
+        const int64_t jt = j0 + (int64_t)it * TU;
+        const bool guard = (jt < blk1 && jt + TU > blk0) || jt + TU > np;
+        tile_x2<MODE, ACC, NPK, TU, KIND>(sh[st], X, XL, acc, cf, guard, c32.threes);
         if (ACC && ((it + 1) % PROMO == 0 || it + 1 == ntiles)) {
             for (int p = 0; p < NPK; ++p) {
                 float2 out[NACC];
@@ -959,8 +1000,8 @@ __global__ void __launch_bounds__(TPB2) k_pair32x2(const __grid_constant__ CUten
         __syncthreads();  // every thread is done with this stage
         if (threadIdx.x == 0 && it + ST < ntiles) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_expect_tx(&bar[st], TS * REC2 * sizeof(float));
-            tma_load_2d(sh[st], &tmap, 0, (int)(j0 + (int64_t)(it + ST) * TS), &bar[st]);
+            mbar_expect_tx(&bar[st], TU * REC2 * sizeof(float));
+            tma_load_2d(sh[st], &tmap, 0, (int)(j0 + (int64_t)(it + ST) * TU), &bar[st]);
         }
     }
     if (failed_at >= 0) {
@@ -1080,11 +1121,11 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
     constexpr int NACC = MODE == 0 ? 2 : 10, NRAW = far_raw(MODE, KIND);
     constexpr int NPK = ACC ? 1 : 2;
     constexpr int TGT = 2 * NPK;
-    const uint32_t tile_bytes = TS2 * REC2 * sizeof(float);
+    const uint32_t tile_bytes = TU2 * REC2 * sizeof(float);
     const int64_t np = J.np;
     const int64_t j0 = split * J.chunk;
     const int64_t j1 = min(np, j0 + J.chunk);
-    const int ntiles = (int)((j1 - j0 + TS2 - 1) / TS2);
+    const int ntiles = (int)((j1 - j0 + TU2 - 1) / TU2);
     const int64_t blk0 = (int64_t)tb * (TPB2 * TGT), blk1 = blk0 + TPB2 * TGT;
     if (threadIdx.x == 0) {
         // the stages were last read through the generic proxy
@@ -1092,7 +1133,7 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
         for (int k = 0; k < ST2 && k < ntiles; ++k) {
             const int st = (int)((g + k) % ST2);
             mbar_expect_tx(&bar[st], tile_bytes);
-            bulk_load(sh[st], J.rec + (j0 + (int64_t)k * TS2) * REC2, tile_bytes, &bar[st]);
+            bulk_load(sh[st], J.rec + (j0 + (int64_t)k * TU2) * REC2, tile_bytes, &bar[st]);
         }
     }
     const Coef2 cf = coef2(J.cf);
@@ -1118,10 +1159,9 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
         const int st = (int)((g + it) % ST2);
         const uint32_t phase = (uint32_t)(((g + it) / ST2) & 1);
         if (!cta_wait(&bar[st], phase, status)) { failed_at = it; break; }
-        const int64_t jt = j0 + (int64_t)it * TS2;
-        const bool guard = (jt < blk1 && jt + TS2 > blk0) || jt + TS2 > np;
-        if (guard) tile_x2<MODE, ACC, NPK, true, TS2, KIND>(sh[st], X, XL, acc, cf);
-        else tile_x2<MODE, ACC, NPK, false, TS2, KIND>(sh[st], X, XL, acc, cf);
+        const int64_t jt = j0 + (int64_t)it * TU2;
+        const bool guard = (jt < blk1 && jt + TU2 > blk0) || jt + TU2 > np;
+        tile_x2<MODE, ACC, NPK, TU2, KIND>(sh[st], X, XL, acc, cf, guard, J.cf.threes);
         if (ACC) {
             for (int p = 0; p < NPK; ++p) {
                 float2 out[NACC];
@@ -1134,7 +1174,7 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
         if (threadIdx.x == 0 && it + ST2 < ntiles) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_expect_tx(&bar[st], tile_bytes);
-            bulk_load(sh[st], J.rec + (j0 + (int64_t)(it + ST2) * TS2) * REC2, tile_bytes, &bar[st]);
+            bulk_load(sh[st], J.rec + (j0 + (int64_t)(it + ST2) * TU2) * REC2, tile_bytes, &bar[st]);
         }
     }
     if (failed_at >= 0) {
@@ -1534,6 +1574,23 @@ static int choose_splits(int64_t np, int tpc, int tile, int slots) {
     return best;
 }
 
+// Split count of the packed kernel: an SM's pair rate hardly depends on how many CTAs share it (one
+// alone 5 % less, measured), so the time goes with the most CTAs that one SM gets times their
+// tiles; more slices cost the reduction, 0.2 % each. (By whole waves of resident CTAs, with 1 % a
+// slice, a part of the SMs had stood idle: 58,080 points, V/K + D/T rows 3,750 -> 3,510 us, split V/K
+// rows 3,050 -> 2,810 us at the counts chosen here.)
+static int x2_splits(int64_t np, int tpc, int tile, int num_sms) {
+    const int64_t nb = (np + tpc - 1) / tpc, ntiles = (np + tile - 1) / tile;
+    int best = 1;
+    double best_cost = 1e300;
+    for (int S = 1; S <= 32 && S <= ntiles; ++S) {
+        const int64_t deep = (nb * S + num_sms - 1) / num_sms, per = (ntiles + S - 1) / S;
+        const double cost = (double)(deep * per) * (1.0 + 0.05 / (double)deep) * (1.0 + 0.002 * S);
+        if (cost < best_cost) { best_cost = cost; best = S; }
+    }
+    return best;
+}
+
 int tune_bucket(int64_t np) {
     int b = 0;
     while (b + 1 < TUNE_BUCKETS && ((int64_t)1 << (b + 1)) <= np) ++b;
@@ -1577,14 +1634,13 @@ static int make_tmap(const pb_mesh* m, const float* rec, CUtensorMap* map, int r
 // FP32-pipe operations per point pair by the formula count of the kernels
 // above (FADD, FMUL and FFMA each one; the two MUFU operations not counted):
 // V/K rows 19; V/K + D/T rows 36, 20 or 32 by kind; split coordinates +6. (The
-// scalar kernel and the one-direction FP64 kernel by the same counts.)
-constexpr double OPS_SPLIT = 6.0;
-static double pair_ops(const FarPlan& fp) {
-    static const double vkdt[3] = {36.0, 20.0, 32.0};
-    return fp.mode == 0 ? 19.0 : vkdt[far_kind(fp)];
+// scalar kernel and the one-direction FP64 kernel by the same counts.) The packed
+// kernel's V/K + D/T rows on points in threes: 34, 18 or 30.
+static double pair_ops(const FarPlan& fp, bool threes = false) {
+    static const double vkdt[2][3] = {{36.0, 20.0, 32.0}, {34.0, 18.667, 29.667}};
+    return fp.mode == 0 ? 19.0 : vkdt[threes ? 1 : 0][far_kind(fp)];
 }
-
-
+constexpr double OPS_SPLIT = 6.0;
 
 // Algorithmic bytes of one gather + near-field SpMV launch: the pattern
 // (row pointers, columns) and the four combined block values of every entry
@@ -1667,18 +1723,19 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             bool acc = prec == PB_F32_ACCURATE;
             const TuneEntry te = tuned(m->ctx, np, fp.mode, acc);
             const X2Entry& xk = x2_kernel(fp.mode, far_kind(fp), acc, te.shape);
+            const int tu = tile_points(xk.ts);
             CUtensorMap map;
-            PB_TRY(make_tmap(m, rec, &map, REC2, xk.ts));
+            PB_TRY(make_tmap(m, rec, &map, REC2, tu));
             const int tpc = TPB2 * 2 * xk.npk;
-            int S = choose_splits(np, tpc, xk.ts, occupancy_slots(m, xk.fn, TPB2));
-            S = scaled_splits(S, te.split_scale, np, xk.ts);
-            int64_t chunk = ((np + S - 1) / S + xk.ts - 1) / xk.ts * xk.ts;
+            int S = x2_splits(np, tpc, tu, m->ctx->num_sms);
+            S = scaled_splits(S, te.split_scale, np, tu);
+            int64_t chunk = ((np + S - 1) / S + tu - 1) / tu * tu;
             S = (int)((np + chunk - 1) / chunk);
-            const Coef32 cf = coef32(fp);
+            const Coef32 cf = coef32(fp, m->Q);
             dim3 grid((unsigned)((np + tpc - 1) / tpc), (unsigned)S);
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)S * nacc * np));
             void* part = m->ws_part.ptr;
-            double ops = pair_ops(fp) + (acc ? OPS_SPLIT : 0.0);
+            double ops = pair_ops(fp, cf.threes) + (acc ? OPS_SPLIT : 0.0);
             Timer tm(m->ctx, acc ? PB_KERNEL_PAIR32_ACCURATE : PB_KERNEL_PAIR32, s, (double)np * (double)np, ops);
             xk.launch(grid, s, map, np, m->pts32, m->pts32lo, cf, chunk, part, status);
             ::pb::count_launch();
@@ -1701,7 +1758,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             S = scaled_splits(S, tuned(m->ctx, np, fp.mode, acc).split_scale, np, TS32);
             int64_t chunk = ((np + S - 1) / S + TS32 - 1) / TS32 * TS32;
             S = (int)((np + chunk - 1) / chunk);
-            const Coef32 cf = coef32(fp);
+            const Coef32 cf = coef32(fp, m->Q);
             dim3 grid((unsigned)((np + TPB32 * TGT32 - 1) / (TPB32 * TGT32)), (unsigned)S);
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)S * nacc * np));
             void* part = m->ws_part.ptr;
@@ -1785,7 +1842,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         cudaStream_t js = J.s ? J.s : s;
         PB_TRY(make_far_plan(J.B, J.nf->kappa, &P.fp));
         const int64_t nt = m->nt, np = m->np;
-        const int64_t np_pad = (np + TS2 - 1) / TS2 * TS2;
+        const int64_t np_pad = (np + TU2 - 1) / TU2 * TU2;
         PB_TRY(ws_reserve(m->ws_src, sizeof(float) * REC2 * np_pad + 256));
         PB_TRY(ws_reserve(m->ws_tri, sizeof(double) * 6 * nt));
         P.tri = (double*)m->ws_tri.ptr;
@@ -1818,11 +1875,9 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
                                               m->pts32lo, J.x, J.x + m->nv, need_u, need_v, rec);
         ::pb::count_launch();
         if (np_pad > np) PB_CUDA(cudaMemsetAsync(rec + REC2 * np, 0, sizeof(float) * REC2 * (np_pad - np), js));
-        // the single-mesh decomposition (same kernel occupancy as that path)
-        const void* kern = x2_kernel(P.fp.mode, 0, acc, 0).fn;  // the default shape's occupancy (the batched kernel's)
-        int S = choose_splits(np, tpc, TS2, occupancy_slots(m, kern, TPB2));
-        S = scaled_splits(S, tuned(m->ctx, np, P.fp.mode, acc).split_scale, np, TS2);
-        P.chunk = ((np + S - 1) / S + TS2 - 1) / TS2 * TS2;
+        int S = x2_splits(np, tpc, TU2, m->ctx->num_sms);  // the single-mesh decomposition
+        S = scaled_splits(S, tuned(m->ctx, np, P.fp.mode, acc).split_scale, np, TU2);
+        P.chunk = ((np + S - 1) / S + TU2 - 1) / TU2 * TU2;
         P.S = (int)((np + P.chunk - 1) / P.chunk);
         const int nacc = P.fp.mode == 0 ? 2 : 10;
         PB_TRY(ws_reserve(m->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)P.S * nacc * np));
@@ -1833,7 +1888,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         pj.part = m->ws_part.ptr;
         pj.np = np;
         pj.chunk = P.chunk;
-        pj.cf = coef32(P.fp);
+        pj.cf = coef32(P.fp, m->Q);
         pj.nsplit = P.S;
         pj.pad = 0;
         hjobs[P.fp.mode].push_back(pj);
@@ -1856,7 +1911,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
             const int ntb = (int)((pj.np + tpc - 1) / tpc);
             for (int sp = 0; sp < pj.nsplit; ++sp) {
                 const int64_t j0 = sp * pj.chunk, j1 = std::min(pj.np, j0 + pj.chunk);
-                const double cost = (double)tpc * (double)((j1 - j0 + TS2 - 1) / TS2 * TS2);
+                const double cost = (double)tpc * (double)((j1 - j0 + TU2 - 1) / TU2 * TU2);
                 for (int tb = 0; tb < ntb; ++tb) costed.push_back({cost, {(int)q, tb, sp, 0}});
             }
         }
@@ -1940,21 +1995,7 @@ void batch_scratch_free(BatchScratch& bs) {
 }
 
 int far_splits_estimate(pb_ctx* ctx, int64_t np) {
-    int best = 1;
-    const void* kerns[2] = {x2_kernel(1, 0, true, 0).fn, x2_kernel(1, 0, false, 0).fn};
-    const int tpcs[2] = {TPB2 * 2, TPB2 * 4};
-    for (int k = 0; k < 2; ++k) {
-        int per_sm = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kerns[k], TPB2, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 1;
-        cudaGetLastError();
-        best = std::max(best, choose_splits(np, tpcs[k], TS2, per_sm * ctx->num_sms));
-    }
-    return best;
-}
-
-int far_splits(const pb_mesh* m, int tpc, int ctas_per_sm) {
-    return choose_splits(m->np, tpc, TS32, ctas_per_sm * m->ctx->num_sms);
+    return std::max(x2_splits(np, TPB2 * 2, TU2, ctx->num_sms), x2_splits(np, TPB2 * 4, TU2, ctx->num_sms));
 }
 
 }  // namespace pb
@@ -2050,7 +2091,7 @@ extern "C" int pb_system_apply_noalloc(pb_ctx* ctx, const pb_mesh* m, const pb_n
         int S = std::min(NOALLOC_MAX_SPLITS, choose_splits(np, TPB32 * TGT32, TS32, occupancy_slots(m, kern, TPB32)));
         int64_t chunk = ((np + S - 1) / S + TS32 - 1) / TS32 * TS32;
         S = (int)((np + chunk - 1) / chunk);
-        const Coef32 cf = coef32(fp);
+        const Coef32 cf = coef32(fp, m->Q);
         dim3 grid((unsigned)((np + TPB32 * TGT32 - 1) / (TPB32 * TGT32)), (unsigned)S);
         if (fp.mode == 0)
             k_pair32<0, false><<<grid, TPB32, 0, s>>>(map, np, m->pts32, m->pts32lo, cf, chunk, part, m->status);

@@ -293,8 +293,6 @@ int tree_far(const pb_mesh* m, const FarPlan& fp, const double* x, bool need_u, 
 void tree_free(PbTree* t);
 int tree_info(const pb_mesh* m, int64_t out[6]);
 
-// far-field split count for the pair kernels
-int far_splits(const pb_mesh* m, int targets_per_cta, int ctas_per_sm);
 // largest split count the packed kernels use for np points (workspace estimates)
 int far_splits_estimate(pb_ctx* ctx, int64_t np);
 // the tuned entry that applies to np points (kernel 0 when none)

@@ -34,3 +34,9 @@ def test_row_kinds(form, alpha, beta, n_lon, n_lat, far_q):
         pb.pb_set_treecode(ctx, tree, 6, 0.7, 0)
         y = apply(prec)
         assert float((y - ref).norm() / ref.norm()) < tol, (prec, tree)
+
+
+@pytest.mark.parametrize("form,alpha,beta", FORMS)
+def test_centroid_rule(form, alpha, beta):
+    """One point per triangle: the packed kernel's loop over single points (966 of them)."""
+    test_row_kinds(form, alpha, beta, 21, 24, 1)

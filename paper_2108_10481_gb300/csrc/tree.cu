@@ -553,7 +553,7 @@ static void launch_proxies(int n, unsigned g, cudaStream_t s, const int32_t* so,
 // threads in two groups (tree_leaf_body with NQ = 2); the linear block index
 // walks the leaves longest first, a leaf's splits side by side.
 template <int MODE, int KIND>
-__global__ void __launch_bounds__(TREE_LEAF, 7) k_tree_eval(TreeJob job) {
+__global__ void __launch_bounds__(TREE_LEAF, MODE == 0 ? 7 : 5) k_tree_eval(TreeJob job) {
     __shared__ __align__(16) float tile[TREE_EVAL_TILE * (2 * TREE_REC + TREE_DUP)];
     static_assert((MODE == 0 ? 2 : 10) * TREE_LEAF <= TREE_EVAL_TILE * (2 * TREE_REC + TREE_DUP), "reduction buffer");
     const int sp = (int)(blockIdx.x % (unsigned)job.nsplit);
@@ -614,12 +614,14 @@ int tree_prepare(const pb_mesh* mc, const FarPlan& fp, const double* x, bool nee
     }
     J.cf.kappa = (float)fp.kappa;
     J.cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);
-    // splits of each leaf's lists, so that the grid holds about eight CTAs per SM
+    // splits of each leaf's lists, so that the grid holds at least 24 CTAs per SM, of which 5 to 7 are resident
+    // (216,000 points, V/K + D/T rows: 3.79 ms with 8, 3.61 with 16, 3.58 with 24 or 40; V/K rows 2.04 -> 1.91 ms)
     const int nacc = fp.mode == 0 ? 2 : 10;
     const int S = (int)std::min<int64_t>(
-        TREE_MAX_SPLITS, std::max<int64_t>(1, (8LL * std::max(1, ctx->num_sms) + t->nleaf - 1) / t->nleaf));
+        TREE_MAX_SPLITS, std::max<int64_t>(1, (24LL * std::max(1, ctx->num_sms) + t->nleaf - 1) / t->nleaf));
     PB_TRY(ws_reserve(m->ws_part, sizeof(float) * (size_t)S * nacc * np));
     J.np = np;
+    J.n = t->n;
     J.nprox = t->nprox;
     J.nsplit = S;
     J.perm = t->perm;
@@ -647,9 +649,10 @@ int tree_far(const pb_mesh* m, const FarPlan& fp, const double* x, bool need_u, 
     const unsigned grid = (unsigned)(t->nleaf * job.nsplit);
     // FP32 operations per interaction as the evaluation does them (f32x2 lanes counted singly; the two
     // MUFU operations, rsqrt and ex2, not counted), by kind
-    static const double near1[3] = {36.0, 20.0, 32.0}, far1[3] = {29.0, 16.0, 26.0};
+    static const double near1[3] = {36.0, 20.0, 32.0}, far1[3] = {23.0, 11.0, 21.0};
     const int kind = job.cf.kind;
-    const double ops_near = fp.mode == 0 ? 19.0 : near1[kind], ops_far = fp.mode == 0 ? (kind == 3 ? 11.0 : 12.0) : far1[kind];
+    const double ops_near = fp.mode == 0 ? 19.0 : near1[kind];
+    const double ops_far = (fp.mode == 0 ? (kind == 3 ? 7.0 : 8.0) : far1[kind]) + (fp.mode == 0 ? 4.0 : 6.0) / (double)t->n;
     const double inter = (double)(t->direct_pairs + t->proxy_pairs);
     const double ops = ((double)t->direct_pairs * ops_near + (double)t->proxy_pairs * ops_far) / std::max(1.0, inter);
     Timer tm(m->ctx, PB_KERNEL_TREE32, s, inter, ops);

@@ -41,6 +41,12 @@ __device__ __forceinline__ float2 t_sub2(float2 a, float2 b) {
         " mov.b64 {%0, %1}, rd;\n}\n" : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
 }
+__device__ __forceinline__ float2 t_add2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n .reg .b64 ra, rb, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n add.rn.f32x2 rd, ra, rb;\n"
+        " mov.b64 {%0, %1}, rd;\n}\n" : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 __device__ __forceinline__ float2 t_mul2(float2 a, float2 b) {
     float2 d;
     asm("{\n .reg .b64 ra, rb, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n mul.rn.f32x2 rd, ra, rb;\n"
@@ -61,7 +67,7 @@ __device__ __forceinline__ float2 t_splat(float v) { return make_float2(v, v); }
 // tree order, the kernel coefficients and the partial-sum slices.
 struct TreeJob {
     int64_t np;
-    int nprox;
+    int n, nprox;               // proxies per axis and cluster: n^3
     int nsplit;                 // slices of partial sums (the leaves' lists are cut into nsplit shares)
     const int32_t* perm;        // tree index -> point index
     const int32_t* leaf_rng;    // 2 per leaf
@@ -97,9 +103,9 @@ struct TreeTiles {
         constexpr int TILE = TREE_EVAL_TILE;
         if (f < fe) {
             *src = T.prox + ((int64_t)T.far_idx[f] * T.nprox + off) * TREE_REC;
-            *cnt = min(TILE, T.nprox - off);
+            *cnt = min(TILE / T.n * T.n, T.nprox - off);  // whole columns
             *far = true;
-            off += TILE;
+            off += *cnt;
             if (off >= T.nprox) { ++f; off = 0; }
             return true;
         }
@@ -116,6 +122,83 @@ struct TreeTiles {
         return false;
     }
 };
+
+// The proxies of a cluster are a tensor grid: a column of N has one x and one y, so that two of
+// the three differences and their squares are taken once for it, and its T sums' x and y parts by
+// one multiply-add of the column's sum. `cols` columns of staged records, those from g0 on in
+// steps of NQ, onto the sums acc of two targets X. A staged record, every value twice: z, the
+// charges (V/K rows: a, b of kind 3's two kernels or of both rows; V/K + D/T rows: S, a, b of the
+// phi row, C, N), and at 20 x, y.
+struct TreeConst {
+    float2 kap, mk2, rhoD, rhoT, c10, c11, c12, c13;
+};
+template <int MODE, int KIND, int NQ, int N, int NS>
+__device__ __forceinline__ void far_columns(const float* cur, int cols, int g0, const float2& X0, const float2& X1,
+                                            const float2& X2, const TreeConst& k, float2 (&acc)[NS]) {
+    constexpr bool YUK = KIND != 1;
+    for (int c = g0; c < cols; c += NQ) {
+        const float* col = cur + TREE_DUP * N * c;
+        const float4 xy = *reinterpret_cast<const float4*>(col + 20);
+        const float2 d0 = t_sub2(X0, make_float2(xy.x, xy.y)), d1 = t_sub2(X1, make_float2(xy.z, xy.w));
+        const float2 rho2 = t_fma2(d0, d0, t_mul2(d1, d1));
+        float2 st = t_splat(0.f);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float4* z4 = reinterpret_cast<const float4*>(col + TREE_DUP * i);
+            const float4 a = z4[0], b = z4[1];
+            const float2 d2 = t_sub2(X2, make_float2(a.x, a.y));
+            const float2 r2 = t_fma2(d2, d2, rho2);
+            const float2 rinv = make_float2(t_rsqrt(r2.x), t_rsqrt(r2.y));
+            float2 e = t_splat(0.f), g = e;
+            if (YUK) {
+                const float2 arg = t_mul2(t_mul2(r2, rinv), k.mk2);
+                e = make_float2(t_ex2(arg.x), t_ex2(arg.y));
+            }
+            if (MODE == 0) {
+                if (KIND == 3) {
+                    acc[0] = t_fma2(rinv, make_float2(a.z, a.w), acc[0]);
+                    acc[1] = t_fma2(t_mul2(e, rinv), make_float2(b.x, b.y), acc[1]);
+                } else {
+                    const float4 dd = z4[2];
+                    acc[0] = t_fma2(rinv, t_fma2(e, make_float2(b.x, b.y), make_float2(a.z, a.w)), acc[0]);
+                    acc[1] = t_fma2(rinv, t_fma2(e, make_float2(dd.x, dd.y), make_float2(b.z, b.w)), acc[1]);
+                }
+            } else {
+                const float4 cc = z4[2], dd = z4[3], ee = z4[4];
+                const float2 ri2 = t_mul2(rinv, rinv);
+                float2 kt = rinv, kd = rinv;
+                acc[0] = t_fma2(rinv, make_float2(b.x, b.y), acc[0]);
+                if (YUK) {
+                    g = t_mul2(e, rinv);
+                    acc[0] = t_fma2(g, make_float2(b.z, b.w), acc[0]);
+                    const float2 gw = t_fma2(k.kap, e, g);
+                    if (KIND == 2) {
+                        kt = t_fma2(k.rhoT, gw, rinv);
+                        kd = t_fma2(k.rhoD, g, rinv);
+                    } else {
+                        kt = t_fma2(k.c13, gw, t_mul2(k.c12, rinv));
+                        kd = t_fma2(k.c11, g, t_mul2(k.c10, rinv));
+                    }
+                }
+                const float2 ts = t_mul2(kt, t_mul2(ri2, make_float2(a.z, a.w)));
+                st = i == 0 ? ts : t_add2(st, ts);
+                acc[3] = t_fma2(ts, d2, acc[3]);
+                acc[4] = t_fma2(kd, make_float2(cc.x, cc.y), acc[4]);
+                acc[5] = t_fma2(kd, make_float2(cc.z, cc.w), acc[5]);
+                acc[6] = t_fma2(kd, make_float2(dd.x, dd.y), acc[6]);
+                if (YUK) {
+                    acc[7] = t_fma2(g, make_float2(dd.z, dd.w), acc[7]);
+                    acc[8] = t_fma2(g, make_float2(ee.x, ee.y), acc[8]);
+                    acc[9] = t_fma2(g, make_float2(ee.z, ee.w), acc[9]);
+                }
+            }
+        }
+        if (MODE == 1) {
+            acc[1] = t_fma2(st, d0, acc[1]);
+            acc[2] = t_fma2(st, d1, acc[2]);
+        }
+    }
+}
 
 // One leaf of targets and one split of its lists, on 64 NQ threads: a thread
 // holds two targets (the leaf's i-th and (i + 64)-th points) in packed f32x2
@@ -135,12 +218,13 @@ struct TreeTiles {
 // (NQ - 1) x NACC x TREE_LEAF floats. Every thread of the group calls it (it
 // synchronises the CTA) and returns with no copy in flight.
 //
-// FP32 operations per interaction (the packed pipe is the limit), proxy and direct: V/K rows
-// 11 (kind 3) or 12, and 19; V/K + D/T rows 26 and 32 (kind 2), 16 and 20 (kind 1), 29 and 36
-// (kind 0); 12, 24, 29 and 35 before with one loop for all coefficients. Sums kept per target
-// (NS): V/K rows the two rows' proxy sums (kind 3: the Laplace and the Yukawa one), then the four
-// sums of the direct pairs; V/K + D/T rows phi, T, C, B, scaled at the end by kind. 116,160
-// points, direct form: 1,122 -> 940 us; 661,500 points, Juffer form: 12.57 -> 11.9 ms.
+// FP32 operations per interaction (the packed pipe is the limit, with the loads of the splatted
+// records close behind), proxy and direct: V/K rows 7 (kind 3) or 8, and 19; V/K + D/T rows 21 and 32
+// (kind 2), 11 and 20 (kind 1), 23 and 36 (kind 0), with 4 or 6 more a column of proxies (every
+// proxy by itself: 11, 12; 26, 16, 29). Sums kept per target (NS): V/K rows the two rows' proxy
+// sums (kind 3: the Laplace and the Yukawa one), then the four sums of the direct pairs; V/K +
+// D/T rows phi, T, C, B, scaled at the end by kind. Columns: 116,160 points, direct form: 948 -> 813 us;
+// 661,500 points, Juffer form: 11.9 -> 10.5 ms.
 template <int MODE, int KIND, int NQ>
 __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int sp, float* tile) {
     constexpr int NACC = MODE == 0 ? 2 : 10;
@@ -182,6 +266,8 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
     const float pscale = KIND == 1 || KIND == 2 ? cf.k[0][2] : 1.0f;  // K's Laplace coefficient, carried by p (and N)
     float2 acc[NS];
     for (int k = 0; k < NS; ++k) acc[k] = t_splat(0.f);
+    const TreeConst kc = {kap, mk2, rhoD, rhoT, c10, c11, c12, c13};
+    int turn = 0;
     const bool any = live0;  // the first target of a thread is live whenever the second is
     TreeTiles it = {fb, fe, qb, qe, 0};
     const float* src = nullptr;
@@ -211,22 +297,23 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
             const float4 u0 = rp[0], u1 = rp[1], u2 = rp[2];
             float v[TREE_REC] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w, u2.x, u2.y, u2.z, u2.w};
             const float s_ = v[3];
-            if (far) {
-                const float q_ = v[4];  // proxy: x, S, Q, C, N
-                if (MODE == 0) {        // x, a and b (kind 3), or (a, b) of both rows
-                    const float a0 = fmaf(cf.k[rl][2], q_, cf.k[rl][0] * s_), b0 = fmaf(cf.k[ry][3], q_, cf.k[ry][1] * s_);
-                    v[3] = a0;
-                    v[4] = b0;
-                    v[5] = fmaf(cf.k[1][2], q_, cf.k[1][0] * s_);
-                    v[6] = fmaf(cf.k[1][3], q_, cf.k[1][1] * s_);
-                } else {  // x, S, (a, b) of the phi row, C, N
+            if (far) {  // as far_columns reads them
+                const float q_ = v[4], x_ = v[0], y_ = v[1];
+                v[0] = v[2];
+                if (MODE == 0) {
+                    v[1] = fmaf(cf.k[rl][2], q_, cf.k[rl][0] * s_);
+                    v[2] = fmaf(cf.k[ry][3], q_, cf.k[ry][1] * s_);
+                    v[3] = fmaf(cf.k[1][2], q_, cf.k[1][0] * s_);
+                    v[4] = fmaf(cf.k[1][3], q_, cf.k[1][1] * s_);
+                } else {
+                    v[1] = s_;
+                    v[2] = fmaf(cf.k[0][2], q_, cf.k[0][0] * s_);
+                    v[3] = fmaf(cf.k[0][3], q_, cf.k[0][1] * s_);
 #pragma unroll
-                    for (int k = TREE_REC - 1; k >= 9; --k) v[k] = pscale * v[k - 1];
-#pragma unroll
-                    for (int k = 8; k >= 6; --k) v[k] = v[k - 1];
-                    v[4] = fmaf(cf.k[0][2], q_, cf.k[0][0] * s_);
-                    v[5] = fmaf(cf.k[0][3], q_, cf.k[0][1] * s_);
+                    for (int k = 4; k < 10; ++k) v[k] = k < 7 ? v[k + 1] : pscale * v[k + 1];
                 }
+                v[10] = x_;
+                v[11] = y_;
             } else if (MODE == 1) {  // x, s, p, c, (a, b) of the phi row's single layer
 #pragma unroll
                 for (int k = 4; k < 7; ++k) v[k] *= pscale;
@@ -239,59 +326,17 @@ __device__ __forceinline__ void tree_leaf_body(const TreeJob& T, int leaf, int s
         }
         __syncthreads();
         const float* cur = dup;
-        if (any && far) {
-#pragma unroll 2
-            for (int j = grp; j < cnt; j += NQ) {
-                // the record's values, each as a splatted pair
-                const float4* z4 = reinterpret_cast<const float4*>(cur + TREE_DUP * j);
-                const float4 a = z4[0], b = z4[1], c = z4[2];
-                const float2 d0 = t_sub2(X0, make_float2(a.x, a.y)), d1 = t_sub2(X1, make_float2(a.z, a.w)),
-                             d2 = t_sub2(X2, make_float2(b.x, b.y));
-                const float2 r2 = t_fma2(d0, d0, t_fma2(d1, d1, t_mul2(d2, d2)));
-                const float2 rinv = make_float2(t_rsqrt(r2.x), t_rsqrt(r2.y));
-                float2 e = t_splat(0.f), g = e;
-                if (YUK) {
-                    const float2 arg = t_mul2(t_mul2(r2, rinv), mk2);
-                    e = make_float2(t_ex2(arg.x), t_ex2(arg.y));
-                }
-                if (MODE == 0) {
-                    if (KIND == 3) {
-                        acc[0] = t_fma2(rinv, make_float2(b.z, b.w), acc[0]);
-                        acc[1] = t_fma2(t_mul2(e, rinv), make_float2(c.x, c.y), acc[1]);
-                    } else {
-                        const float4 dd = z4[3];
-                        acc[0] = t_fma2(rinv, t_fma2(e, make_float2(c.x, c.y), make_float2(b.z, b.w)), acc[0]);
-                        acc[1] = t_fma2(rinv, t_fma2(e, make_float2(dd.x, dd.y), make_float2(c.z, c.w)), acc[1]);
-                    }
-                } else {
-                    const float2 ri2 = t_mul2(rinv, rinv);
-                    float2 kt = rinv, kd = rinv;
-                    acc[0] = t_fma2(rinv, make_float2(c.x, c.y), acc[0]);
-                    if (YUK) {
-                        g = t_mul2(e, rinv);
-                        acc[0] = t_fma2(g, make_float2(c.z, c.w), acc[0]);
-                        const float2 gw = t_fma2(kap, e, g);
-                        if (KIND == 2) {
-                            kt = t_fma2(rhoT, gw, rinv);
-                            kd = t_fma2(rhoD, g, rinv);
-                        } else {
-                            kt = t_fma2(c13, gw, t_mul2(c12, rinv));
-                            kd = t_fma2(c11, g, t_mul2(c10, rinv));
-                        }
-                    }
-                    const float2 ts = t_mul2(kt, t_mul2(ri2, make_float2(b.z, b.w)));
-                    acc[1] = t_fma2(ts, d0, acc[1]);
-                    acc[2] = t_fma2(ts, d1, acc[2]);
-                    acc[3] = t_fma2(ts, d2, acc[3]);
-                    const float4 dd = z4[3], ee = z4[4], ff = z4[5];
-                    acc[4] = t_fma2(kd, make_float2(dd.x, dd.y), acc[4]);
-                    acc[5] = t_fma2(kd, make_float2(dd.z, dd.w), acc[5]);
-                    acc[6] = t_fma2(kd, make_float2(ee.x, ee.y), acc[6]);
-                    if (YUK) {
-                        acc[7] = t_fma2(g, make_float2(ee.z, ee.w), acc[7]);
-                        acc[8] = t_fma2(g, make_float2(ff.x, ff.y), acc[8]);
-                        acc[9] = t_fma2(g, make_float2(ff.z, ff.w), acc[9]);
-                    }
+        if (far) {
+            const int cols = cnt / T.n, g0 = (grp + turn) % NQ;
+            turn = (turn + NQ - cols % NQ) % NQ;  // the groups' shares even out over the tiles
+            if (any) {
+                switch (T.n) {
+                    case 3: far_columns<MODE, KIND, NQ, 3>(cur, cols, g0, X0, X1, X2, kc, acc); break;
+                    case 4: far_columns<MODE, KIND, NQ, 4>(cur, cols, g0, X0, X1, X2, kc, acc); break;
+                    case 5: far_columns<MODE, KIND, NQ, 5>(cur, cols, g0, X0, X1, X2, kc, acc); break;
+                    case 6: far_columns<MODE, KIND, NQ, 6>(cur, cols, g0, X0, X1, X2, kc, acc); break;
+                    case 7: far_columns<MODE, KIND, NQ, 7>(cur, cols, g0, X0, X1, X2, kc, acc); break;
+                    default: far_columns<MODE, KIND, NQ, 8>(cur, cols, g0, X0, X1, X2, kc, acc); break;
                 }
             }
         } else if (any) {

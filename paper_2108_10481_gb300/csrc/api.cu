@@ -222,6 +222,19 @@ extern "C" int pb_init(int device, pb_ctx** out) {
         return set_error(PB_ECUDA, "cuTensorMapEncodeTiled entry point unavailable");
     }
     c->encode_tiled = fn;
+    {   // small near builds' memory, kept between them
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = BUILD_POOL_BYTES;
+        if (cudaMemPoolCreate(&c->build_pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(c->build_pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            if (c->build_pool) cudaMemPoolDestroy(c->build_pool);
+            c->build_pool = nullptr;  // builds allocate from the device
+            cudaGetLastError();
+        }
+    }
     const char* pk = getenv("PBBEM_PAIR_KERNEL");
     if (pk && pk[0] == '1') c->pair_kernel = 1;
     const char* gr = getenv("PBBEM_GRAPHS");
@@ -244,6 +257,7 @@ static void reset_stats(pb_ctx* ctx) {
 
 extern "C" int pb_free_ctx(pb_ctx* ctx) {
     if (ctx) reset_stats(ctx);
+    if (ctx && ctx->build_pool) cudaMemPoolDestroy(ctx->build_pool);
     delete ctx;
     return PB_OK;
 }

@@ -130,10 +130,12 @@ struct TuneEntry {
     int shape = 0;           // launch shape of the packed kernel (tile records, stages, targets per thread)
 };
 constexpr int TUNE_BUCKETS = 40;
+constexpr size_t BUILD_POOL_BYTES = size_t(64) << 20;
 struct PbTree;  // treecode of a mesh (tree.cu)
 }  // namespace pb
 
 struct pb_ctx {
+    cudaMemPool_t build_pool = nullptr;  // near builds' own memory (at most BUILD_POOL_BYTES kept; null: none)
     int profile = 0;
     int pair_kernel = 2;  // FP32 far-field kernel: 2 = packed f32x2 (default), 1 = scalar
     pb::TuneEntry tune[2][2][pb::TUNE_BUCKETS];  // [mode][accurate][bucket]

@@ -392,7 +392,7 @@ typedef struct {
 } pb_tune_choice;
 typedef struct {
     pb_tune_choice fast;     /* PB_F32 applications (FP32 tile sums) */
-    pb_tune_choice accurate; /* PB_F32_ACCURATE applications (split coordinates, FP64 tile sums) */
+    pb_tune_choice accurate; /* PB_F32_ACCURATE applications (split coordinates, two-word sums) */
 } pb_tune_result;
 /* Time every candidate launch of formulation `form`'s FP32 system application
  * on this mesh (fast and split-coordinate variants; the scalar kernel and the

@@ -700,7 +700,8 @@ __global__ void __launch_bounds__(TPB32) k_pair32(const __grid_constant__ CUtens
 // thread holds its targets in pairs, so one fma/add/mul.rn.f32x2 advances two
 // targets. Source values are stored twice in a 32-float record so that every
 // packed operand is a register pair loaded straight from shared memory:
-//   x x y y z z s s | px px py py pz pz cx cx | cy cy cz cz xl xl yl yl | zl zl - - - - - -
+//   x x y y z z s s | px px py py pz pz sg sg | xl xl yl yl zl zl - - | vx vx vy vy vz vz - -
+// (p = sg n; v the curl, or by threes the normal in the first and the curl in the other records).
 // The identical-point guard is needed only in tiles that overlap the CTA's
 // own targets or run past the last point (zero-filled rows).
 constexpr int REC2 = 32;   // floats per duplicated source record
@@ -1557,7 +1558,7 @@ int make_far_plan(const BlockOp& B, double kappa, FarPlan* fp) {
     return PB_OK;
 }
 
-// split count: fill the GPU in whole waves (see the layout notes in the design)
+// split count of the scalar and FP64 kernels: fill the GPU in whole waves
 static int choose_splits(int64_t np, int tpc, int tile, int slots) {
     int64_t nb = (np + tpc - 1) / tpc;
     int64_t ntiles = (np + tile - 1) / tile;

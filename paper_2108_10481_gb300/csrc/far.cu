@@ -29,6 +29,7 @@
 
 #include "exp64.cuh"
 #include "internal.h"
+#include "splits.h"
 #include "tree_eval.cuh"
 
 namespace pb {
@@ -99,9 +100,6 @@ __global__ void k_sources(int64_t np, int Q, Rule rule, const int32_t* __restric
 }
 
 // ------------------------------------------------------- FP64 pair kernel (a3)
-constexpr int TPB64 = 128;  // threads (= targets) per CTA
-constexpr int TS64 = 64;    // sources per shared-memory tile
-
 struct Coef {
     double k[2][4];
     double rho[4];  // both-kernels form: Yukawa over Laplace coefficient of V, K, D, T
@@ -227,13 +225,6 @@ __global__ void __launch_bounds__(TPB64, 6) k_pair64(int64_t np, const double* _
 // side of distance s in slice nsplit + s - 1, the W warps' added in order: no atomics.
 // 1,920 points, MODE 0: 229 -> 171 us; 7,680 points, MODE 1: 4.96 -> 3.42 ms.
 constexpr int SYM64_MAX_SMEM = 8 * 32 * (10 + 11 * 8 * (1 + 4));  // W = 8, SB = 4
-struct Sym64 {
-    int warps, sub;        // W and SB
-    int nblock, half;      // I blocks, and the largest distance
-    int nsplit;
-    int slices() const { return nsplit + half; }
-};
-
 template <int MODE, int KIND, bool BOTH>
 __device__ __forceinline__ void sym64_steps(const Coef& cf, const double* xi, double si, const double* pi, const double* ci,
                                             const double* jd, double* jacc, double* acc, int lane) {
@@ -413,6 +404,7 @@ struct Pair64Choice {
     Pair64Kernel one;   // a direction at a time
     Sym64Kernel both;   // both directions at once
     int sums;           // raw sums of a point in the latter
+    int kind;
 };
 // the kernels for a plan's coefficients, and the ratios they take
 static Pair64Choice pair64_kernel(const FarPlan& fp, Coef* cf) {
@@ -430,47 +422,12 @@ static Pair64Choice pair64_kernel(const FarPlan& fp, Coef* cf) {
     cf->kappa = fp.kappa;
     cf->t64 = -fp.kappa * EXP64_PER_UNIT;
     if (fp.mode == 0) {
-        if (yukawa) return {k_pair64<0, 0>, k_pair64_sym<0, 0>, 4};
-        return {k_pair64<0, 1>, k_pair64_sym<0, 1>, 2};
+        if (yukawa) return {k_pair64<0, 0>, k_pair64_sym<0, 0>, 4, 0};
+        return {k_pair64<0, 1>, k_pair64_sym<0, 1>, 2, 1};
     }
-    if (!yukawa) return {k_pair64<1, 1>, k_pair64_sym<1, 1>, 8};
-    if (all_laplace) return {k_pair64<1, 2>, k_pair64_sym<1, 2>, 11};
-    return {k_pair64<1, 0>, k_pair64_sym<1, 0>, 11};
-}
-
-// Shape of the symmetric kernel for np points: the one whose busiest SM has the least
-// work (in 32 x 32 tiles; the FP64 pipe, not the number of resident warps, sets an SM's
-// rate, down to about six warps). The partial sums stay within 32 slices, or 64 while
-// they are below 32 MB; beyond 64 blocks of 1,024 points nblock = 0 and the other kernel,
-// whose slices do not grow with the point count, runs.
-static Sym64 sym64_shape(int64_t np, int nacc, int num_sms) {
-    static const int shapes[5][2] = {{2, 1}, {4, 1}, {8, 1}, {8, 2}, {8, 4}};
-    Sym64 best = {0, 0, 0, 0, 0};
-    double best_cost = 1e300;
-    for (const auto& sh : shapes) {
-        Sym64 c;
-        c.warps = sh[0];
-        c.sub = sh[1];
-        const int64_t pts = 32 * c.warps * c.sub, nb = (np + pts - 1) / pts;
-        if (nb > 64) continue;
-        c.nblock = (int)nb;
-        c.half = c.nblock / 2;
-        const int units = (c.half + 1) * c.warps * c.sub;
-        for (c.nsplit = 1; c.nsplit <= units && c.slices() <= 64; ++c.nsplit) {
-            if (c.slices() > 32 && (double)c.slices() * nacc * np * 8.0 > 32e6) break;
-            const int64_t ctas = nb * c.nsplit, per = (units + c.nsplit - 1) / c.nsplit;
-            const int64_t on_sm = (ctas + num_sms - 1) / num_sms;
-            double cost = (double)on_sm * per * c.sub * c.warps;
-            const double resident = std::min<double>((double)ctas / num_sms, 16.0 / c.warps) * c.warps;
-            if (resident < 6.0) cost *= 6.0 / resident;
-            cost *= 1.0 + 0.002 * c.slices();
-            if (cost < best_cost) {
-                best_cost = cost;
-                best = c;
-            }
-        }
-    }
-    return best;
+    if (!yukawa) return {k_pair64<1, 1>, k_pair64_sym<1, 1>, 8, 1};
+    if (all_laplace) return {k_pair64<1, 2>, k_pair64_sym<1, 2>, 11, 2};
+    return {k_pair64<1, 0>, k_pair64_sym<1, 0>, 11, 0};
 }
 
 // ------------------------------------------------ FP32 pair kernel, TMA-fed (a3)
@@ -1558,40 +1515,6 @@ int make_far_plan(const BlockOp& B, double kappa, FarPlan* fp) {
     return PB_OK;
 }
 
-// split count of the scalar and FP64 kernels: fill the GPU in whole waves
-static int choose_splits(int64_t np, int tpc, int tile, int slots) {
-    int64_t nb = (np + tpc - 1) / tpc;
-    int64_t ntiles = (np + tile - 1) / tile;
-    int best = 1;
-    double best_cost = 1e300;
-    for (int S = 1; S <= 32; ++S) {
-        if (S > ntiles) break;
-        int64_t ctas = nb * S;
-        int64_t waves = (ctas + slots - 1) / slots;
-        int64_t per = (ntiles + S - 1) / S;
-        double cost = (double)waves * (double)per * (1.0 + 0.01 * S);
-        if (cost < best_cost) { best_cost = cost; best = S; }
-    }
-    return best;
-}
-
-// Split count of the packed kernel: an SM's pair rate hardly depends on how many CTAs share it (one
-// alone 5 % less, measured), so the time goes with the most CTAs that one SM gets times their
-// tiles; more slices cost the reduction, 0.2 % each. (By whole waves of resident CTAs, with 1 % a
-// slice, a part of the SMs had stood idle: 58,080 points, V/K + D/T rows 3,750 -> 3,510 us, split V/K
-// rows 3,050 -> 2,810 us at the counts chosen here.)
-static int x2_splits(int64_t np, int tpc, int tile, int num_sms) {
-    const int64_t nb = (np + tpc - 1) / tpc, ntiles = (np + tile - 1) / tile;
-    int best = 1;
-    double best_cost = 1e300;
-    for (int S = 1; S <= 32 && S <= ntiles; ++S) {
-        const int64_t deep = (nb * S + num_sms - 1) / num_sms, per = (ntiles + S - 1) / S;
-        const double cost = (double)(deep * per) * (1.0 + 0.05 / (double)deep) * (1.0 + 0.002 * S);
-        if (cost < best_cost) { best_cost = cost; best = S; }
-    }
-    return best;
-}
-
 int tune_bucket(int64_t np) {
     int b = 0;
     while (b + 1 < TUNE_BUCKETS && ((int64_t)1 << (b + 1)) <= np) ++b;
@@ -1600,14 +1523,6 @@ int tune_bucket(int64_t np) {
 
 TuneEntry tuned(const pb_ctx* ctx, int64_t np, int mode, bool acc) {
     return ctx->tune[mode ? 1 : 0][acc ? 1 : 0][tune_bucket(np)];
-}
-
-// split count after the tuned scale, within [1, tiles] and <= 32
-static int scaled_splits(int S, double scale, int64_t np, int tile) {
-    const int64_t ntiles = (np + tile - 1) / tile;
-    int s2 = (int)(S * scale + 0.5);
-    s2 = std::max(1, std::min(s2, 32));
-    return (int)std::min<int64_t>(s2, ntiles);
 }
 
 static int occupancy_slots(const pb_mesh* m, const void* kern, int threads) {
@@ -1685,14 +1600,10 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
                                                         m->pts32lo, x, x + nv, need_u, need_v, rec); ::pb::count_launch();
             Coef cf;
             const Pair64Choice kern = pair64_kernel(fp, &cf);
-            const Sym64 sy = sym64_shape(np, nacc, m->ctx->num_sms);
-            int S = sy.slices();
-            int64_t chunk = 0;
-            if (!sy.nblock) {
-                S = choose_splits(np, TPB64, TS64, occupancy_slots(m, (const void*)kern.one, TPB64));
-                chunk = ((np + S - 1) / S + TS64 - 1) / TS64 * TS64;
-                S = (int)((np + chunk - 1) / chunk);
-            }
+            const Pair64Plan pl = pair64_plan(np, fp.mode, kern.kind, m->ctx->num_sms,
+                                              occupancy_slots(m, (const void*)kern.one, TPB64));
+            const Sym64& sy = pl.sym;
+            const int S = pl.slices();
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, sizeof(double) * (size_t)S * nacc * np));
             double* part = (double*)m->ws_part.ptr;
             Timer tm(m->ctx, PB_KERNEL_PAIR64, s, (double)np * (double)np, pair_ops(fp));
@@ -1704,7 +1615,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
                 kern.both<<<dim3(sy.nblock, sy.nsplit), 32 * sy.warps, smem, s>>>(np, rec, cf, sy, part);
             } else {
                 kern.one<<<dim3((unsigned)((np + TPB64 - 1) / TPB64), (unsigned)S), TPB64, 0, s>>>(np, m->pts64, rec, cf,
-                                                                                                   chunk, part);
+                                                                                                   pl.chunk, part);
             }
             ::pb::count_launch();
             tm.stop();

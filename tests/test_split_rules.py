@@ -1,0 +1,65 @@
+"""How the pair kernels cut their sources into slices (csrc/splits.h), compiled on its own with the host compiler (no
+GPU): the rules' bounds over the point counts, at the GB300's 152 SMs."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+SRC = os.path.join(os.path.dirname(HERE), "paper_2108_10481_gb300", "csrc")
+SMS = 152
+
+DRIVER = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "splits.h"
+using namespace pb;
+int main(int argc, char** argv) {  // lo hi step
+    for (long long np = atoll(argv[1]); np <= atoll(argv[2]); np += atoll(argv[3]))
+        for (int mode = 0; mode < 2; ++mode)
+            for (int kind = 0; kind < (mode ? 3 : 2); ++kind)
+                for (int resident = 6; resident <= 9; resident += 3) {
+                    const int slots = resident * %(sms)d;
+                    const Pair64Plan p = pair64_plan(np, mode, kind, %(sms)d, slots);
+                    const Pair64Plan o = pair64_one(np, mode, kind, %(sms)d, slots);
+                    printf("%%lld %%d %%d %%d %%d %%.17g %%.17g\n", np, mode, kind, p.sym.nblock > 0, p.slices(), p.cost, o.cost);
+                }
+    return 0;
+}
+""" % {"sms": SMS}
+
+
+def compile_driver(path, source):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no host C++ compiler")
+    (path / "driver.cpp").write_text(source)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I" + SRC, str(path / "driver.cpp"), "-o", str(path / "driver")], check=True)
+    return str(path / "driver")
+
+
+@pytest.fixture(scope="module")
+def fp64_plans(tmp_path_factory):
+    exe = compile_driver(tmp_path_factory.mktemp("fp64"), DRIVER)
+    rows = []
+    for rng in ((6, 4000, 6), (4002, 66000, 186), (62400, 64600, 6), (70000, 800000, 7302)):
+        out = subprocess.run([exe, *map(str, rng)], check=True, capture_output=True, text=True).stdout
+        rows += [[float(w) for w in line.split()] for line in out.splitlines()]
+    return rows
+
+
+def test_fp64_never_dearer_than_one_direction(fp64_plans):
+    """At 62,465 to 64,512 points the both-directions kernel has one slice of rows: one direction is the cheaper."""
+    for np_, mode, kind, both, slices, cost, one in fp64_plans:
+        assert cost <= one, (np_, mode, kind)
+        if np_ >= 62465:
+            assert not both, (np_, mode, kind)
+        if np_ <= 48000:
+            assert both, (np_, mode, kind)
+
+
+def test_fp64_slices_within_their_bounds(fp64_plans):
+    for np_, mode, kind, both, slices, cost, one in fp64_plans:
+        assert 1 <= slices <= 64
+        assert slices <= 32 or slices * (10 if mode else 2) * np_ * 8 <= 32e6, (np_, mode, kind)

@@ -1639,7 +1639,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             CUtensorMap map;
             PB_TRY(make_tmap(m, rec, &map, REC2, tu));
             const int tpc = TPB2 * 2 * xk.npk;
-            int S = x2_splits(np, tpc, tu, m->ctx->num_sms);
+            int S = x2_splits(np, tpc, xk.ts, m->ctx->num_sms, acc ? 0 : x2_longest(np, fp.mode, xk.ts, m->ctx->num_sms));
             S = scaled_splits(S, te.split_scale, np, tu);
             int64_t chunk = ((np + S - 1) / S + tu - 1) / tu * tu;
             S = (int)((np + chunk - 1) / chunk);
@@ -1787,7 +1787,8 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
                                               m->pts32lo, J.x, J.x + m->nv, need_u, need_v, rec);
         ::pb::count_launch();
         if (np_pad > np) PB_CUDA(cudaMemsetAsync(rec + REC2 * np, 0, sizeof(float) * REC2 * (np_pad - np), js));
-        int S = x2_splits(np, tpc, TU2, m->ctx->num_sms);  // the single-mesh decomposition
+        // the single-mesh decomposition
+        int S = x2_splits(np, tpc, TS2, m->ctx->num_sms, acc ? 0 : x2_longest(np, P.fp.mode, TS2, m->ctx->num_sms));
         S = scaled_splits(S, tuned(m->ctx, np, P.fp.mode, acc).split_scale, np, TU2);
         P.chunk = ((np + S - 1) / S + TU2 - 1) / TU2 * TU2;
         P.S = (int)((np + P.chunk - 1) / P.chunk);
@@ -1907,7 +1908,10 @@ void batch_scratch_free(BatchScratch& bs) {
 }
 
 int far_splits_estimate(pb_ctx* ctx, int64_t np) {
-    return std::max(x2_splits(np, TPB2 * 2, TU2, ctx->num_sms), x2_splits(np, TPB2 * 4, TU2, ctx->num_sms));
+    int S = x2_splits(np, TPB2 * 2, TS2, ctx->num_sms);
+    for (int mode = 0; mode < 2; ++mode)
+        S = std::max(S, x2_splits(np, TPB2 * 4, TS2, ctx->num_sms, x2_longest(np, mode, TS2, ctx->num_sms)));
+    return S;
 }
 
 }  // namespace pb

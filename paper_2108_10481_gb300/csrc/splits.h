@@ -27,28 +27,43 @@ inline int choose_splits(int64_t np, int tpc, int tile, int slots) {
     return best;
 }
 
-// Split count of the packed kernel: an SM's pair rate hardly depends on how many CTAs share it (one
-// alone 5 % less, measured), so the time goes with the most CTAs that one SM gets times their
-// tiles; more slices cost the reduction, 0.2 % each. (By whole waves of resident CTAs, with 1 % a
+// Sources of a slice of the packed kernel's fast variant at most: their sums stay in FP32 until the
+// slices are added in FP64, so longer slices cost accuracy (twice as long: 43,320 points, V/K rows 1.3
+// instead of 1.1e-7 from the FP64 application). The length, in whole tiles of ts records, is that of
+// whole waves of 1,024 targets a CTA, 4 (V/K rows) or 2 CTAs resident on an SM. The split-coordinate
+// variant adds every tile's sums to wide ones: any length.
+inline int64_t x2_longest(int64_t np, int mode, int ts, int num_sms) {
+    const int S = choose_splits(np, 1024, ts, (mode == 0 ? 4 : 2) * num_sms);
+    return ((np + S - 1) / S + ts - 1) / ts * ts;
+}
+
+// Split count of the packed kernel, tiles with room for ts records (whole threes are used), no more
+// than `longest` sources to a slice (0: any): an SM's pair rate hardly depends on how many CTAs
+// share it (one alone 5 % less, measured), so the time goes with the most CTAs that one SM gets times
+// their tiles; more slices cost the reduction, 0.2 % each. (By whole waves of resident CTAs, with 1 % a
 // slice, a part of the SMs had stood idle: 58,080 points, V/K + D/T rows 3,750 -> 3,510 us, split V/K
 // rows 3,050 -> 2,810 us at the counts chosen here.)
-inline int x2_splits(int64_t np, int tpc, int tile, int num_sms) {
+constexpr int X2_MAX_SLICES = 36;  // 32 of the longest slices in tiles of fewer points than ts
+inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest = 0) {
+    const int tile = ts / 3 * 3;
     const int64_t nb = (np + tpc - 1) / tpc, ntiles = (np + tile - 1) / tile;
+    const int64_t per_max = longest > 0 ? longest / ts : ntiles;
     int best = 1;
     double best_cost = 1e300;
-    for (int S = 1; S <= 32 && S <= ntiles; ++S) {
+    for (int S = 1; S <= (longest > 0 ? X2_MAX_SLICES : 32) && S <= ntiles; ++S) {
         const int64_t deep = (nb * S + num_sms - 1) / num_sms, per = (ntiles + S - 1) / S;
+        if (per > per_max) continue;
         const double cost = (double)(deep * per) * (1.0 + 0.05 / (double)deep) * (1.0 + 0.002 * S);
         if (cost < best_cost) { best_cost = cost; best = S; }
     }
     return best;
 }
 
-// split count after the tuned scale, within [1, tiles] and <= 32
+// split count after the tuned scale, within [1, tiles] and <= 32 (or the untuned one)
 inline int scaled_splits(int S, double scale, int64_t np, int tile) {
     const int64_t ntiles = (np + tile - 1) / tile;
     int s2 = (int)(S * scale + 0.5);
-    s2 = std::max(1, std::min(s2, 32));
+    s2 = std::max(1, std::min(s2, std::max(S, 32)));
     return (int)std::min<int64_t>(s2, ntiles);
 }
 

@@ -63,3 +63,36 @@ def test_fp64_slices_within_their_bounds(fp64_plans):
     for np_, mode, kind, both, slices, cost, one in fp64_plans:
         assert 1 <= slices <= 64
         assert slices <= 32 or slices * (10 if mode else 2) * np_ * 8 <= 32e6, (np_, mode, kind)
+
+
+PACKED = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "splits.h"
+using namespace pb;
+int main(int argc, char** argv) {  // lo hi step: sources of a fast slice by launch shape, and by whole waves
+    static const int shapes[4][2] = {{64, 1024}, {32, 1024}, {128, 1024}, {64, 512}};  // records per tile, targets per CTA
+    for (long long np = atoll(argv[1]); np <= atoll(argv[2]); np += atoll(argv[3]))
+        for (int mode = 0; mode < 2; ++mode)
+            for (int k = 0; k < 4; ++k) {
+                const int ts = shapes[k][0], tu = ts / 3 * 3;
+                int S = x2_splits(np, shapes[k][1], ts, %(sms)d, x2_longest(np, mode, ts, %(sms)d));
+                S = scaled_splits(S, 1.0, np, tu);
+                const long long chunk = ((np + S - 1) / S + tu - 1) / tu * tu;
+                const int W = choose_splits(np, 1024, ts, (mode ? 2 : 4) * %(sms)d);
+                printf("%%lld %%d %%d %%d %%lld %%lld\n", np, mode, k, S, chunk, (long long)(((np + W - 1) / W + ts - 1) / ts * ts));
+            }
+    return 0;
+}
+""" % {"sms": SMS}
+
+
+def test_fast_slices_no_longer_than_whole_waves(tmp_path):
+    """The fast FP32 sums run over no more sources than the whole-wave rule's slices have, at any launch shape."""
+    exe = compile_driver(tmp_path, PACKED)
+    for rng in ((1, 4000, 1), (4002, 120000, 42)):
+        out = subprocess.run([exe, *map(str, rng)], check=True, capture_output=True, text=True).stdout
+        for line in out.splitlines():
+            np_, mode, shape, S, chunk, wave = map(int, line.split())
+            assert S <= 36
+            assert chunk <= wave, line

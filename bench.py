@@ -264,7 +264,7 @@ def _kernels():
     import paper_2108_10481_gb300 as pb
     return {pb.PB_KERNEL_PAIR32: ("k_pair32x2 (FP32 far field, packed f32x2)", "pair32", "alu", FP32_LANES_PER_SM,
                                   "FP32 ops"),
-            pb.PB_KERNEL_PAIR32_ACCURATE: ("k_pair32x2 split-coordinate (FP32 far field, two-word sums)",
+            pb.PB_KERNEL_PAIR32_ACCURATE: ("k_pair32x2 split-coordinate (FP32 far field, three-word sums)",
                                            "pair32acc", "alu", FP32_LANES_PER_SM, "FP32 ops"),
             pb.PB_KERNEL_PAIR64: ("k_pair64 (FP64 far field)", "pair64", "alu", FP64_FLOPS_PER_SM, "FP64 flops"),
             pb.PB_KERNEL_NEAR_ADJ: ("k_adj_pairs (FP64 singular quadrature, edge/vertex pairs)", "near_adj", "alu",

@@ -66,8 +66,8 @@ extern "C" {
 #define PB_F64 0          /* FP64 everywhere */
 #define PB_F32 1          /* FP32 pair sums and FP32 near field (inner solves) */
 #define PB_F32_ACCURATE 2 /* FP32 pair arithmetic on split (hi+lo) coordinates with
-                             the tiles' sums accumulated in two FP32 words (about 48
-                             bits), FP64 near field */
+                             the tiles' sums accumulated in three FP32 words (no fewer
+                             bits than FP64), FP64 near field */
 #define PB_MIXED 3        /* (pb_solve_opts.precision) FP32 inner GMRES inside FP64
                              iterative refinement */
 
@@ -385,14 +385,14 @@ typedef struct {
     int tile_records;       /* source records that a TMA tile of the chosen launch has room for (whole threes are used) */
     int stages;             /* its pipeline stages */
     int targets_per_thread; /* its targets per thread */
-    int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide sums at a time */
+    int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide (three-word) sums at a time */
     double split_scale;     /* chosen multiplier of the wave-filling split count */
     double best_ms;         /* one FP32 system application with the choice */
     double default_ms;      /* ... with the untuned default (packed, shape 0, x1) */
 } pb_tune_choice;
 typedef struct {
     pb_tune_choice fast;     /* PB_F32 applications (FP32 tile sums) */
-    pb_tune_choice accurate; /* PB_F32_ACCURATE applications (split coordinates, two-word sums) */
+    pb_tune_choice accurate; /* PB_F32_ACCURATE applications (split coordinates, three-word sums) */
 } pb_tune_result;
 /* Time every candidate launch of formulation `form`'s FP32 system application
  * on this mesh (fast and split-coordinate variants; the scalar kernel and the

@@ -31,6 +31,7 @@
 #include "internal.h"
 #include "splits.h"
 #include "tree_eval.cuh"
+#include "wide.h"
 
 namespace pb {
 
@@ -756,19 +757,43 @@ __device__ __forceinline__ void x2_out(const Coef2& cf, const float2* v, float2*
     }
 }
 
-// Wide sums of the split-coordinate variant: two FP32 words per sum (hi + lo, about 48 bits),
-// a tile's FP32 sum added exactly (Knuth's two-sum, the rounding error into lo). Seven packed
-// operations a value; FP64 additions and the conversions to it, at the GB300's FP64 rate, took
-// a third of the kernel's time when every tile of 64 sources was added (61,440 points, V/K +
-// D/T rows: 5.89 -> 4.98 ms; tiles of 128 sources would take 4.58, but their FP32 sums raise the
-// PMCHWT forms' error against the FP64 application from 4.0e-8 to 5.5e-8).
-struct Wide2 {
-    float2 hi, lo;
+// Wide sums of the split-coordinate variant: a tile's FP32 sums are added into three FP32 words
+// (wide.h), 13 packed operations a value; FP64 additions and the conversions to FP64, at the GB300's
+// FP64 rate, took a third of the kernel's time when every tile of 64 sources was added. The lower two
+// words lie in shared memory, float4 (mid, lo) per value and thread at [value][thread]: in
+// registers they would spill. 61,440 points, V/K + D/T rows, every point by
+// itself: 5.89 ms with FP64 additions, 4.98 with two words (about 48 bits); as now, an application 4.53 ms
+// with two and 4.54 with three. (Tiles of 128 sources would be faster, but their FP32 sums raise the
+// PMCHWT forms' error against the FP64 application from 4.0e-8 to 5.5e-8.)
+struct F32x2 {
+    static __device__ __forceinline__ float2 add(float2 a, float2 b) { return add2(a, b); }
+    static __device__ __forceinline__ float2 sub(float2 a, float2 b) { return sub2(a, b); }
 };
-__device__ __forceinline__ void wide_add(Wide2& w, float2 b) {
-    const float2 s = add2(w.hi, b), bb = sub2(s, w.hi);
-    w.lo = add2(w.lo, add2(sub2(w.hi, sub2(s, bb)), sub2(b, bb)));
-    w.hi = s;
+__host__ __device__ constexpr size_t wide_smem(int mode, int npk) {
+    return sizeof(float4) * TPB2 * npk * (mode == 0 ? 2 : 10);
+}
+template <int NV>
+__device__ __forceinline__ void wide_zero(float2 (&hi)[NV], float4* words) {
+#pragma unroll
+    for (int a = 0; a < NV; ++a) {
+        hi[a] = make_float2(0.f, 0.f);
+        words[a * TPB2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+template <int NV>
+__device__ __forceinline__ void wide_add(float2 (&hi)[NV], float4* words, const float2 (&b)[NV]) {
+#pragma unroll
+    for (int a = 0; a < NV; ++a) {
+        const float4 w = words[a * TPB2];
+        float2 mid = make_float2(w.x, w.y), lo = make_float2(w.z, w.w);
+        wide_add<F32x2>(hi[a], mid, lo, b[a]);
+        words[a * TPB2] = make_float4(mid.x, mid.y, lo.x, lo.y);
+    }
+}
+// value a of the first (h = 0) or second target
+__device__ __forceinline__ double wide_total(const float2& hi, const float4* words, int a, int h) {
+    const float4 w = words[a * TPB2];
+    return h ? wide_value(hi.y, w.y, w.w) : wide_value(hi.x, w.x, w.z);
 }
 
 // The tile's sums: records of 16 splatted values (position, s, p = sigma n, sigma, low words,
@@ -904,6 +929,7 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
     constexpr int TGT = 2 * NPK, TU = tile_points(TS);
     __shared__ __align__(128) float sh[ST][TS * REC2];
     __shared__ __align__(8) uint64_t bar[ST];
+    extern __shared__ __align__(16) float4 wide_words[];  // ACC: wide_smem(MODE, NPK)
     const int split = blockIdx.y;
     const int64_t j0 = split * chunk;
     const int64_t j1 = min(np, j0 + chunk);
@@ -934,10 +960,11 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
         }
     }
     float2 acc[NPK][NRAW];
-    Wide2 wide[NPK][ACC ? NACC : 1];
+    float2 hi[NPK][ACC ? NACC : 1];
+    float4* words = wide_words + threadIdx.x;  // pair p's at words + p NACC TPB2
     for (int p = 0; p < NPK; ++p) {
         for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
-        for (int a = 0; a < (ACC ? NACC : 1); ++a) wide[p][a].hi = wide[p][a].lo = make_float2(0.f, 0.f);
+        if constexpr (ACC) wide_zero<NACC>(hi[p], words + p * NACC * TPB2);
     }
     int failed_at = -1;
     for (int it = 0; it < ntiles; ++it) {
@@ -947,13 +974,14 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
         const int64_t jt = j0 + (int64_t)it * TU;
         const bool guard = (jt < blk1 && jt + TU > blk0) || jt + TU > np;
         tile_x2<MODE, ACC, NPK, TU, KIND>(sh[st], X, XL, acc, cf, guard, c32.threes);
-        if (ACC && ((it + 1) % PROMO == 0 || it + 1 == ntiles)) {
-            for (int p = 0; p < NPK; ++p) {
-                float2 out[NACC];
-                x2_out<MODE, KIND>(cf, acc[p], out);
-                for (int a = 0; a < NACC; ++a) wide_add(wide[p][a], out[a]);
-                for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
-            }
+        if constexpr (ACC) {
+            if ((it + 1) % PROMO == 0 || it + 1 == ntiles)
+                for (int p = 0; p < NPK; ++p) {
+                    float2 out[NACC];
+                    x2_out<MODE, KIND>(cf, acc[p], out);
+                    wide_add<NACC>(hi[p], words + p * NACC * TPB2, out);
+                    for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
+                }
         }
         __syncthreads();  // every thread is done with this stage
         if (threadIdx.x == 0 && it + ST < ntiles) {
@@ -974,9 +1002,8 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
             if (tg[t] >= np) continue;
             for (int a = 0; a < NACC; ++a) {
                 int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
-                if (ACC)
-                    static_cast<double*>(part_out)[o] = h ? (double)wide[p][a].hi.y + (double)wide[p][a].lo.y
-                                                          : (double)wide[p][a].hi.x + (double)wide[p][a].lo.x;
+                if constexpr (ACC)
+                    static_cast<double*>(part_out)[o] = wide_total(hi[p][a], words + p * NACC * TPB2, a, h);
                 else static_cast<float*>(part_out)[o] = h ? out[a].y : out[a].x;
             }
         }
@@ -991,7 +1018,6 @@ typedef void (*X2Launch)(dim3, cudaStream_t, const CUtensorMap&, int64_t, const 
                          int64_t, void*, int*);
 struct X2Entry {
     int ts, st, npk, promo;
-    const void* fn;
     X2Launch launch;
 };
 constexpr int X2_SHAPES = 4;
@@ -999,12 +1025,14 @@ constexpr int X2_SHAPES = 4;
 template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO>
 static void x2_launch(dim3 g, cudaStream_t s, const CUtensorMap& map, int64_t np, const float* p32,
                       const float* plo, Coef32 cf, int64_t chunk, void* part, int* status) {
-    k_pair32x2<MODE, KIND, ACC, TS, ST, NPK, PROMO><<<g, TPB2, 0, s>>>(map, np, p32, plo, cf, chunk, part, status);
+    const auto kern = k_pair32x2<MODE, KIND, ACC, TS, ST, NPK, PROMO>;
+    constexpr size_t smem = ACC ? wide_smem(MODE, NPK) : 0;
+    if (ACC) cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<g, TPB2, smem, s>>>(map, np, p32, plo, cf, chunk, part, status);
 }
 template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
 static X2Entry x2_entry() {
-    return {TS, ST, NPK, PROMO, (const void*)k_pair32x2<MODE, KIND, ACC, TS, ST, NPK, PROMO>,
-            x2_launch<MODE, KIND, ACC, TS, ST, NPK, PROMO>};
+    return {TS, ST, NPK, PROMO, x2_launch<MODE, KIND, ACC, TS, ST, NPK, PROMO>};
 }
 template <int MODE, int KIND>
 static void x2_row(X2Entry (&fast)[X2_SHAPES], X2Entry (&acc)[X2_SHAPES]) {
@@ -1075,7 +1103,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 // One pair item on the CTA: g tiles consumed before it; false when a wait ran out.
 template <int MODE, bool ACC, int KIND>
 __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, float (&sh)[ST2][TS2 * REC2], uint64_t* bar,
-                                          uint32_t& g, int* status) {
+                                          uint32_t& g, float4* wide_words, int* status) {
     constexpr int NACC = MODE == 0 ? 2 : 10, NRAW = far_raw(MODE, KIND);
     constexpr int NPK = ACC ? 1 : 2;
     constexpr int TGT = 2 * NPK;
@@ -1107,10 +1135,11 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
         }
     }
     float2 acc[NPK][NRAW];
-    Wide2 wide[NPK][ACC ? NACC : 1];
+    float2 hi[NPK][ACC ? NACC : 1];
+    float4* words = wide_words + threadIdx.x;  // pair p's at words + p NACC TPB2
     for (int p = 0; p < NPK; ++p) {
         for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
-        for (int a = 0; a < (ACC ? NACC : 1); ++a) wide[p][a].hi = wide[p][a].lo = make_float2(0.f, 0.f);
+        if constexpr (ACC) wide_zero<NACC>(hi[p], words + p * NACC * TPB2);
     }
     int failed_at = -1;
     for (int it = 0; it < ntiles; ++it) {
@@ -1120,11 +1149,11 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
         const int64_t jt = j0 + (int64_t)it * TU2;
         const bool guard = (jt < blk1 && jt + TU2 > blk0) || jt + TU2 > np;
         tile_x2<MODE, ACC, NPK, TU2, KIND>(sh[st], X, XL, acc, cf, guard, J.cf.threes);
-        if (ACC) {
+        if constexpr (ACC) {
             for (int p = 0; p < NPK; ++p) {
                 float2 out[NACC];
                 x2_out<MODE, KIND>(cf, acc[p], out);
-                for (int a = 0; a < NACC; ++a) wide_add(wide[p][a], out[a]);
+                wide_add<NACC>(hi[p], words + p * NACC * TPB2, out);
                 for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
             }
         }
@@ -1152,9 +1181,8 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
             if (tg[t] >= np) continue;
             for (int a = 0; a < NACC; ++a) {
                 int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
-                if (ACC)
-                    static_cast<double*>(J.part)[o] = h ? (double)wide[p][a].hi.y + (double)wide[p][a].lo.y
-                                                        : (double)wide[p][a].hi.x + (double)wide[p][a].lo.x;
+                if constexpr (ACC)
+                    static_cast<double*>(J.part)[o] = wide_total(hi[p][a], words + p * NACC * TPB2, a, h);
                 else static_cast<float*>(J.part)[o] = h ? out[a].y : out[a].x;
             }
         }
@@ -1170,6 +1198,7 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2_queue(const PairJob* __res
                                                          int* __restrict__ counter, int* __restrict__ status) {
     __shared__ __align__(128) float sh[ST2][TS2 * REC2];
     __shared__ __align__(8) uint64_t bar[ST2];
+    extern __shared__ __align__(16) float4 wide_words[];  // ACC: wide_smem(MODE, 1)
     __shared__ int s_item;
     if (threadIdx.x == 0) {
         for (int st = 0; st < ST2; ++st) mbar_init(&bar[st], 1);
@@ -1203,10 +1232,10 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2_queue(const PairJob* __res
         }
         const PairJob& J = jobs[it0.job];
         bool ok;
-        if (MODE == 0) ok = pair_item<0, ACC, 0>(J, it0.tb, it0.split, sh, bar, g, status);
-        else if (J.cf.kind == 2) ok = pair_item<1, ACC, 2>(J, it0.tb, it0.split, sh, bar, g, status);
-        else if (J.cf.kind == 1) ok = pair_item<1, ACC, 1>(J, it0.tb, it0.split, sh, bar, g, status);
-        else ok = pair_item<1, ACC, 0>(J, it0.tb, it0.split, sh, bar, g, status);
+        if (MODE == 0) ok = pair_item<0, ACC, 0>(J, it0.tb, it0.split, sh, bar, g, wide_words, status);
+        else if (J.cf.kind == 2) ok = pair_item<1, ACC, 2>(J, it0.tb, it0.split, sh, bar, g, wide_words, status);
+        else if (J.cf.kind == 1) ok = pair_item<1, ACC, 1>(J, it0.tb, it0.split, sh, bar, g, wide_words, status);
+        else ok = pair_item<1, ACC, 0>(J, it0.tb, it0.split, sh, bar, g, wide_words, status);
         if (!ok) return;
     }
 }
@@ -1860,15 +1889,17 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         const void* kern = mode == 0 ? (acc ? (const void*)k_pair32x2_queue<0, true> : (const void*)k_pair32x2_queue<0, false>)
                                      : (acc ? (const void*)k_pair32x2_queue<1, true> : (const void*)k_pair32x2_queue<1, false>);
         const pb_ctx* ctx = jobs[hjob_of[mode].empty() ? tjob_of[mode][0] : hjob_of[mode][0]].m->ctx;
+        const size_t smem = acc ? wide_smem(mode, 1) : 0;
+        if (acc) PB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int per_sm = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB2, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB2, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
         cudaGetLastError();
         const unsigned grid = (unsigned)std::max(1, std::min(n_items, per_sm * ctx->num_sms));
         if (mode == 0) {
-            if (acc) k_pair32x2_queue<0, true><<<grid, TPB2, 0, s>>>(djobs, dtjobs, ditems, n_items, counter, status);
+            if (acc) k_pair32x2_queue<0, true><<<grid, TPB2, smem, s>>>(djobs, dtjobs, ditems, n_items, counter, status);
             else k_pair32x2_queue<0, false><<<grid, TPB2, 0, s>>>(djobs, dtjobs, ditems, n_items, counter, status);
         } else {
-            if (acc) k_pair32x2_queue<1, true><<<grid, TPB2, 0, s>>>(djobs, dtjobs, ditems, n_items, counter, status);
+            if (acc) k_pair32x2_queue<1, true><<<grid, TPB2, smem, s>>>(djobs, dtjobs, ditems, n_items, counter, status);
             else k_pair32x2_queue<1, false><<<grid, TPB2, 0, s>>>(djobs, dtjobs, ditems, n_items, counter, status);
         }
         ::pb::count_launch();

@@ -29,6 +29,7 @@
 
 #include "exp64.cuh"
 #include "internal.h"
+#include "kinds.h"
 #include "splits.h"
 #include "tree_eval.cuh"
 #include "wide.h"
@@ -409,25 +410,21 @@ struct Pair64Choice {
 };
 // the kernels for a plan's coefficients, and the ratios they take
 static Pair64Choice pair64_kernel(const FarPlan& fp, Coef* cf) {
-    bool yukawa = false, all_laplace = true;
+    const int kind = pair64_kind(fp.mode, fp.k);
     for (int R = 0; R < 2; ++R)
-        for (int j = 0; j < 4; ++j) {
-            cf->k[R][j] = fp.k[R][j];
-            if (j & 1) yukawa = yukawa || fp.k[R][j] != 0.0;
-            else all_laplace = all_laplace && fp.k[R][j] != 0.0;
-        }
+        for (int j = 0; j < 4; ++j) cf->k[R][j] = fp.k[R][j];
     for (int q = 0; q < 4; ++q) {
         const double* k = fp.k[q / 2] + 2 * (q % 2);
-        cf->rho[q] = all_laplace ? k[1] / k[0] : 0.0;
+        cf->rho[q] = fp.mode == 1 && kind == 2 ? k[1] / k[0] : 0.0;
     }
     cf->kappa = fp.kappa;
     cf->t64 = -fp.kappa * EXP64_PER_UNIT;
     if (fp.mode == 0) {
-        if (yukawa) return {k_pair64<0, 0>, k_pair64_sym<0, 0>, 4, 0};
+        if (kind == 0) return {k_pair64<0, 0>, k_pair64_sym<0, 0>, 4, 0};
         return {k_pair64<0, 1>, k_pair64_sym<0, 1>, 2, 1};
     }
-    if (!yukawa) return {k_pair64<1, 1>, k_pair64_sym<1, 1>, 8, 1};
-    if (all_laplace) return {k_pair64<1, 2>, k_pair64_sym<1, 2>, 11, 2};
+    if (kind == 1) return {k_pair64<1, 1>, k_pair64_sym<1, 1>, 8, 1};
+    if (kind == 2) return {k_pair64<1, 2>, k_pair64_sym<1, 2>, 11, 2};
     return {k_pair64<1, 0>, k_pair64_sym<1, 0>, 11, 0};
 }
 
@@ -504,22 +501,11 @@ struct Coef32 {
     float rho[4];  // kind 2: Yukawa over Laplace coefficient of V, K, D, T
     float kappa;
     float mk2;  // -kappa * log2(e)
-    int kind;   // loop of the packed kernel (far_kind)
+    int kind;   // loop of the packed kernel (pair32_kind)
     bool threes;  // its points come in threes of one triangle and weight
 };
 
-// The packed kernels' loop for a plan's coefficients, as the FP64 kernel's: 1 no Yukawa term
-// (V/K + D/T rows), 2 V, K, D and T all with a Laplace coefficient (V/K + D/T rows), 0 otherwise.
-static int far_kind(const FarPlan& fp) {
-    if (fp.mode == 0) return 0;
-    bool yukawa = false, all_laplace = true;
-    for (int R = 0; R < 2; ++R)
-        for (int j = 0; j < 4; ++j) {
-            if (j & 1) yukawa = yukawa || fp.k[R][j] != 0.0;
-            else all_laplace = all_laplace && fp.k[R][j] != 0.0;
-        }
-    return !yukawa ? 1 : all_laplace ? 2 : 0;
-}
+static int far_kind(const FarPlan& fp) { return pair32_kind(fp.mode, fp.k); }
 
 static Coef32 coef32(const FarPlan& fp, int Q) {
     Coef32 cf;

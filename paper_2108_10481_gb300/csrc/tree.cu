@@ -26,6 +26,7 @@
 #include <numeric>
 #include <vector>
 
+#include "kinds.h"
 #include "tree_eval.cuh"
 
 namespace pb {
@@ -594,23 +595,10 @@ int tree_prepare(const pb_mesh* mc, const FarPlan& fp, const double* x, bool nee
     TreeJob& J = *job;
     for (int R = 0; R < 2; ++R)
         for (int j = 0; j < 4; ++j) J.cf.k[R][j] = (float)fp.k[R][j];
-    {   // the loops for these coefficients (TreeCoef)
-        bool yukawa = false, all_laplace = true;
-        for (int R = 0; R < 2; ++R)
-            for (int j = 0; j < 4; j += 2) {
-                yukawa = yukawa || fp.k[R][j + 1] != 0.0;
-                all_laplace = all_laplace && fp.k[R][j] != 0.0;
-            }
-        auto only = [&](int R, int j) { return fp.k[R][1 - j] == 0.0 && fp.k[R][3 - j] == 0.0; };
-        J.cf.lrow = only(0, 0) ? 0 : 1;  // only(R, j): row R has terms of kernel j (0 Laplace, 1 Yukawa) alone
-        if (fp.mode == 0) J.cf.kind = only(J.cf.lrow, 0) && only(1 - J.cf.lrow, 1) ? 3 : 0;
-        else J.cf.kind = fp.k[0][2] == 0.0 ? 0 : !yukawa ? 1 : all_laplace ? 2 : 0;
-        for (int q = 0; q < 3; ++q) J.cf.rho[q] = 0.f;
-        if (J.cf.kind == 2) {
-            J.cf.rho[0] = (float)(fp.k[0][3] / fp.k[0][2]);
-            J.cf.rho[1] = (float)(fp.k[1][1] / fp.k[1][0]);
-            J.cf.rho[2] = (float)(fp.k[1][3] / fp.k[1][2]);
-        }
+    J.cf.kind = tree_kind(fp.mode, fp.k, &J.cf.lrow);
+    for (int q = 0; q < 3; ++q) {  // K, D, T
+        const double* k = fp.k[(q + 1) / 2] + 2 * ((q + 1) % 2);
+        J.cf.rho[q] = fp.mode == 1 && J.cf.kind == 2 ? (float)(k[1] / k[0]) : 0.f;
     }
     J.cf.kappa = (float)fp.kappa;
     J.cf.mk2 = (float)(-fp.kappa * 1.4426950408889634);

@@ -220,29 +220,31 @@ __global__ void k_energy_points(int64_t nt, Rule rule, const int32_t* __restrict
 }
 
 __global__ void k_energy_part(int64_t np, const double* __restrict__ pv, const double* __restrict__ xq,
-                              double* __restrict__ part, int nchunk) {
+                              int64_t nq, double* __restrict__ part, int nchunk) {
     __shared__ double red[EN_THREADS / 32];
     const int c = blockIdx.x;
-    const int64_t j = blockIdx.y;
-    const double qx = xq[3 * j], qy = xq[3 * j + 1], qz = xq[3 * j + 2];
     const int64_t i0 = (int64_t)c * EN_CHUNK, i1 = min(np, i0 + EN_CHUNK);
-    double s = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += EN_THREADS) {
-        const double4 a = *reinterpret_cast<const double4*>(pv + 8 * i);
-        const double4 b = *reinterpret_cast<const double4*>(pv + 8 * i + 4);
-        const double d0 = qx - a.x, d1 = qy - a.y, d2 = qz - a.z;
-        const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-        const double rinv = rsqrt_nr(r2);
-        const double dn = d0 * b.x + d1 * b.y + d2 * b.z;  // w u (x_j - y).n_y
-        s += rinv * a.w - rinv * rinv * rinv * dn;
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tsum = 0.0;
-        for (int w = 0; w < EN_THREADS / 32; ++w) tsum += red[w];
-        part[j * nchunk + c] = tsum;
+    for (int64_t j = blockIdx.y; j < nq; j += gridDim.y) {
+        const double qx = xq[3 * j], qy = xq[3 * j + 1], qz = xq[3 * j + 2];
+        double s = 0.0;
+        for (int64_t i = i0 + threadIdx.x; i < i1; i += EN_THREADS) {
+            const double4 a = *reinterpret_cast<const double4*>(pv + 8 * i);
+            const double4 b = *reinterpret_cast<const double4*>(pv + 8 * i + 4);
+            const double d0 = qx - a.x, d1 = qy - a.y, d2 = qz - a.z;
+            const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
+            const double rinv = rsqrt_nr(r2);
+            const double dn = d0 * b.x + d1 * b.y + d2 * b.z;  // w u (x_j - y).n_y
+            s += rinv * a.w - rinv * rinv * rinv * dn;
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double tsum = 0.0;
+            for (int w = 0; w < EN_THREADS / 32; ++w) tsum += red[w];
+            part[j * nchunk + c] = tsum;
+        }
+        __syncthreads();  // red is free for the next charge
     }
 }
 
@@ -257,11 +259,14 @@ constexpr int EN32_CHARGES = 32;  // per block
 constexpr int EN32_WARPS = 4;
 constexpr int EN32_THREADS = 32 * EN32_WARPS;
 constexpr int EN32_TILE = 256;     // points per staged tile
-// points per block: 1,024, or more (whole tiles) where that would be over 512 chunks
-static int64_t en32_chunk(int64_t np) {
+// points per block: 1,024, or 4,096 where the charges alone are many blocks, or more (whole
+// tiles) where that would be over 512 chunks
+static int64_t en32_chunk(int64_t np, int64_t nq) {
     const int64_t c = (np + 511) / 512;
-    return std::max<int64_t>(1024, (c + EN32_TILE - 1) / EN32_TILE * EN32_TILE);
+    return std::max<int64_t>(nq > 16384 ? 4096 : 1024, (c + EN32_TILE - 1) / EN32_TILE * EN32_TILE);
 }
+// a grid's y extent; the kernels step over the charges beyond it
+constexpr int64_t EN_MAX_Y = 65535;
 
 __global__ void k_energy_points32(int64_t nt, Rule rule, const int32_t* __restrict__ tris,
                                   const double* __restrict__ tgeo, const double* __restrict__ pts64,
@@ -290,36 +295,39 @@ __global__ void __launch_bounds__(EN32_THREADS) k_energy_part32(int64_t np, int6
     __shared__ float4 tile[3 * EN32_TILE];
     __shared__ double red[EN32_WARPS][EN32_CHARGES];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t j = blockIdx.y * (int64_t)EN32_CHARGES + lane;
-    const bool live = j < nq;
-    float qh[3] = {0.f, 0.f, 0.f}, ql[3] = {0.f, 0.f, 0.f};
-    if (live) split3(xq + 3 * j, ctr.c, qh, ql);
     const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = min(np, i0 + chunk);
-    double s = 0.0;
-    for (int64_t b0 = i0; b0 < i1; b0 += EN32_TILE) {
-        const int cnt = (int)min((int64_t)EN32_TILE, i1 - b0);
-        __syncthreads();
-        for (int k = threadIdx.x; k < 3 * cnt; k += EN32_THREADS) tile[k] = pv[3 * b0 + k];
-        __syncthreads();
-        float f = 0.f;
+    for (int64_t j0 = blockIdx.y * (int64_t)EN32_CHARGES; j0 < nq; j0 += gridDim.y * (int64_t)EN32_CHARGES) {
+        const int64_t j = j0 + lane;
+        const bool live = j < nq;
+        float qh[3] = {0.f, 0.f, 0.f}, ql[3] = {0.f, 0.f, 0.f};
+        if (live) split3(xq + 3 * j, ctr.c, qh, ql);
+        double s = 0.0;
+        for (int64_t b0 = i0; b0 < i1; b0 += EN32_TILE) {
+            const int cnt = (int)min((int64_t)EN32_TILE, i1 - b0);
+            __syncthreads();
+            for (int k = threadIdx.x; k < 3 * cnt; k += EN32_THREADS) tile[k] = pv[3 * b0 + k];
+            __syncthreads();
+            float f = 0.f;
 #pragma unroll 4
-        for (int p = w; p < cnt; p += EN32_WARPS) {
-            const float4 a = tile[3 * p], b = tile[3 * p + 1], c = tile[3 * p + 2];
-            const float d0 = (qh[0] - a.x) + (ql[0] - b.x);
-            const float d1 = (qh[1] - a.y) + (ql[1] - b.y);
-            const float d2 = (qh[2] - a.z) + (ql[2] - b.z);
-            const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-            const float rinv = rsqrt_f32(r2);
-            const float dn = fmaf(d0, c.x, fmaf(d1, c.y, d2 * c.z));  // w u (x_j - y).n_y
-            f = fmaf(rinv, a.w, fmaf(-rinv * rinv * rinv, dn, f));
+            for (int p = w; p < cnt; p += EN32_WARPS) {
+                const float4 a = tile[3 * p], b = tile[3 * p + 1], c = tile[3 * p + 2];
+                const float d0 = (qh[0] - a.x) + (ql[0] - b.x);
+                const float d1 = (qh[1] - a.y) + (ql[1] - b.y);
+                const float d2 = (qh[2] - a.z) + (ql[2] - b.z);
+                const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
+                const float rinv = rsqrt_f32(r2);
+                const float dn = fmaf(d0, c.x, fmaf(d1, c.y, d2 * c.z));  // w u (x_j - y).n_y
+                f = fmaf(rinv, a.w, fmaf(-rinv * rinv * rinv, dn, f));
+            }
+            s += (double)f;
         }
-        s += (double)f;
-    }
-    red[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && live) {
-        for (int k = 1; k < EN32_WARPS; ++k) s += red[k][lane];
-        part[j * nchunk + blockIdx.x] = s;
+        red[w][lane] = s;
+        __syncthreads();
+        if (w == 0 && live) {
+            for (int k = 1; k < EN32_WARPS; ++k) s += red[k][lane];
+            part[j * nchunk + blockIdx.x] = s;
+        }
+        __syncthreads();  // red is free for the next charges
     }
 }
 
@@ -398,7 +406,7 @@ extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int for
     // exterior unknowns -> interior traces: u_int = u_ext, v_int = (eps_ext/eps_int) v_ext
     double vscale = form_is_exterior(form) ? prm->eps_ext / prm->eps_int : 1.0;
     const bool f32 = prec == PB_F32_ACCURATE;
-    const int64_t chunk = f32 ? en32_chunk(m->np_ref) : EN_CHUNK;
+    const int64_t chunk = f32 ? en32_chunk(m->np_ref, n_q) : EN_CHUNK;
     const int nchunk = (int)((m->np_ref + chunk - 1) / chunk);
     // partial sums, phi per charge, Delta G, then the point values (32-byte aligned); a workspace of
     // its own, free again when the call returns (the call waits for its work)
@@ -415,19 +423,20 @@ extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int for
         const Ctr c = {{m->ctr[0], m->ctr[1], m->ctr[2]}};
         k_energy_points32<<<pb_, 256, 0, s>>>(m->nt, rr, m->tris, m->tgeo, m->pts_ref, x, m->nv, vscale, c,
                                               reinterpret_cast<float4*>(pv));
-        const dim3 grid(nchunk, (unsigned)((n_q + EN32_CHARGES - 1) / EN32_CHARGES));
+        const dim3 grid(nchunk, (unsigned)std::min(EN_MAX_Y, (n_q + EN32_CHARGES - 1) / EN32_CHARGES));
         k_energy_part32<<<grid, EN32_THREADS, 0, s>>>(m->np_ref, chunk, reinterpret_cast<const float4*>(pv), xq, n_q, c,
                                                       part, nchunk);
     } else {
         k_energy_points<<<pb_, 256, 0, s>>>(m->nt, rr, m->tris, m->tgeo, m->pts_ref, x, m->nv, vscale, pv);
-        const dim3 grid(nchunk, (unsigned)n_q);
-        k_energy_part<<<grid, EN_THREADS, 0, s>>>(m->np_ref, pv, xq, part, nchunk);
+        const dim3 grid(nchunk, (unsigned)std::min(EN_MAX_Y, n_q));
+        k_energy_part<<<grid, EN_THREADS, 0, s>>>(m->np_ref, pv, xq, n_q, part, nchunk);
     }
     k_energy_rows<<<(unsigned)((n_q * 32 + 127) / 128), 128, 0, s>>>(n_q, nchunk, part, phi_all, phi);
     k_energy_final<<<1, EN_FINAL_THREADS, 0, s>>>(n_q, phi_all, q, dG);
     ::pb::count_launch(4);
     double h = 0.0;
-    cudaError_t e = cudaMemcpyAsync(&h, dG, sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, dG, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return set_error(PB_ECUDA, "pb_energy: %s", cudaGetErrorString(e));
     if (dG_paper) *dG_paper = h;

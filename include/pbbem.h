@@ -158,7 +158,10 @@ typedef struct {
 /* Create a context on CUDA device `device`. Returns PB_ECUDA if the device
  * cannot be used, PB_EINVAL if out is NULL. */
 int pb_init(int device, pb_ctx** out);
-/* Free a context (NULL is allowed). Meshes and near fields must be freed first. */
+/* Free a context (NULL is allowed). Meshes and near fields must be freed first.
+ * A context keeps up to 64 MB of device memory that pb_near_build and pb_energy
+ * used for themselves, for the next such call, until it is freed (the request
+ * server's calls keep none). */
 int pb_free_ctx(pb_ctx* ctx);
 /* Message of the last error on this thread ("" if none). Never NULL. */
 const char* pb_last_error(void);

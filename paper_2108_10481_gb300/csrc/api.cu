@@ -222,16 +222,16 @@ extern "C" int pb_init(int device, pb_ctx** out) {
         return set_error(PB_ECUDA, "cuTensorMapEncodeTiled entry point unavailable");
     }
     c->encode_tiled = fn;
-    {   // small near builds' memory, kept between them
+    {   // small calls' own memory, kept between them
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = device;
-        uint64_t keep = BUILD_POOL_BYTES;
-        if (cudaMemPoolCreate(&c->build_pool, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(c->build_pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            if (c->build_pool) cudaMemPoolDestroy(c->build_pool);
-            c->build_pool = nullptr;  // builds allocate from the device
+        uint64_t keep = CALL_POOL_BYTES;
+        if (cudaMemPoolCreate(&c->call_pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(c->call_pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            if (c->call_pool) cudaMemPoolDestroy(c->call_pool);
+            c->call_pool = nullptr;  // calls allocate from the device
             cudaGetLastError();
         }
     }
@@ -257,7 +257,7 @@ static void reset_stats(pb_ctx* ctx) {
 
 extern "C" int pb_free_ctx(pb_ctx* ctx) {
     if (ctx) reset_stats(ctx);
-    if (ctx && ctx->build_pool) cudaMemPoolDestroy(ctx->build_pool);
+    if (ctx && ctx->call_pool) cudaMemPoolDestroy(ctx->call_pool);
     delete ctx;
     return PB_OK;
 }

@@ -130,12 +130,12 @@ struct TuneEntry {
     int shape = 0;           // launch shape of the packed kernel (tile records, stages, targets per thread)
 };
 constexpr int TUNE_BUCKETS = 40;
-constexpr size_t BUILD_POOL_BYTES = size_t(64) << 20;
+constexpr size_t CALL_POOL_BYTES = size_t(64) << 20;
 struct PbTree;  // treecode of a mesh (tree.cu)
 }  // namespace pb
 
 struct pb_ctx {
-    cudaMemPool_t build_pool = nullptr;  // near builds' own memory (at most BUILD_POOL_BYTES kept; null: none)
+    cudaMemPool_t call_pool = nullptr;  // a call's own memory (at most CALL_POOL_BYTES kept; null: none)
     int profile = 0;
     int pair_kernel = 2;  // FP32 far-field kernel: 2 = packed f32x2 (default), 1 = scalar
     pb::TuneEntry tune[2][2][pb::TUNE_BUCKETS];  // [mode][accurate][bucket]
@@ -203,9 +203,6 @@ struct pb_mesh {
     int* status = nullptr;          // device status word of bounded waits (0 = fine)
     // workspaces (grown on demand)
     pb::Workspace ws_src, ws_part, ws_tri, ws_vec, ws_comb, ws_tree;
-    // pb_energy's point values and partial sums: in use only during the call, held by no graph
-    pb::Workspace ws_energy;
-    uint64_t ws_energy_gen = 0;
     uint64_t ws_gen = 0;  // bumped when one of the workspaces above moves or is freed
     pb::PbTree* tree = nullptr;  // built on the first treecode application
     size_t device_bytes = 0;
@@ -250,6 +247,36 @@ int device_scan(int64_t n, const int32_t* cnt, int32_t* ptr, int64_t* total, cud
 // device allocation helpers (track bytes on the mesh)
 int dev_alloc(void** p, size_t bytes);
 int ws_reserve(Workspace& w, size_t bytes);
+
+// Memory that a call (a near build, an energy) needs itself and gives back before it returns: up to
+// CALL_POOL_BYTES from the context's pool, which keeps as much until the context is freed
+// (stream-ordered, safe from several threads), more from the device, as for calls that have to leave nothing
+// behind (pooled = false: the server's, whose budget counts what its requests hold).
+struct CallScratch {
+    void* ptr = nullptr;
+    int take(pb_ctx* ctx, size_t bytes, cudaStream_t s, bool use_pool) {
+        stream = s;
+        pooled = use_pool && ctx->call_pool && bytes <= CALL_POOL_BYTES &&
+                 cudaMallocFromPoolAsync(&ptr, bytes, ctx->call_pool, s) == cudaSuccess;
+        if (pooled) return PB_OK;
+        cudaGetLastError();
+        return dev_alloc(&ptr, bytes);
+    }
+    ~CallScratch() {
+        if (!ptr) return;
+        if (pooled) cudaFreeAsync(ptr, stream);
+        else cudaFree(ptr);
+    }
+
+private:
+    cudaStream_t stream = nullptr;
+    bool pooled = false;
+};
+
+// pb_near_build and pb_energy, with or without the context's pool for their own memory
+int near_build(pb_ctx* ctx, const pb_mesh* mesh, double kappa, pb_near** out, cudaStream_t s, bool pooled);
+int energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int form, const double* xq, const double* q, int64_t n_q,
+           const pb_params* prm, double* phi, double* dG_paper, double* dG_kcal, int prec, cudaStream_t s, bool pooled);
 void ws_free(Workspace& w);
 
 // formulation -> block operators (system, Calderon operators, RHS scaling)

@@ -393,7 +393,6 @@ static void free_mesh_arrays(pb_mesh* m) {
     ws_free(m->ws_vec);
     ws_free(m->ws_comb);
     ws_free(m->ws_tree);
-    ws_free(m->ws_energy);
     tree_free(m->tree);
     m->tree = nullptr;
     tr.lap("all");
@@ -942,7 +941,6 @@ extern "C" int pb_mesh_load(pb_ctx* ctx, const double* verts, int64_t n_verts, c
     PB_CUDA(cudaSetDevice(ctx->device));
     pb_mesh* m = new pb_mesh();
     for (Workspace* w : {&m->ws_src, &m->ws_part, &m->ws_tri, &m->ws_vec, &m->ws_comb, &m->ws_tree}) w->gen = &m->ws_gen;
-    m->ws_energy.gen = &m->ws_energy_gen;
     int rc = load(ctx, verts, n_verts, tris, n_tris, plan, mem, m);
     if (rc != PB_OK) {
         free_mesh_arrays(m);
@@ -968,6 +966,6 @@ extern "C" int pb_mesh_info(const pb_mesh* m, int64_t out[6]) {
     out[3] = m->nnz;
     out[4] = m->npairs;
     out[5] = (int64_t)(m->device_bytes + m->ws_src.bytes + m->ws_part.bytes + m->ws_tri.bytes +
-                       m->ws_vec.bytes + m->ws_comb.bytes + m->ws_energy.bytes);
+                       m->ws_vec.bytes + m->ws_comb.bytes);
     return PB_OK;
 }

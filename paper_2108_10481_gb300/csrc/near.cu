@@ -1367,28 +1367,6 @@ __global__ void k_mass_rows(int64_t nv, int64_t nnz, int pass, const int32_t* __
     if (!pass) cnt[i] = n;
 }
 
-// The build's own memory: up to BUILD_POOL_BYTES from the context's pool, which keeps as much when it
-// is given back (stream-ordered, safe from several threads; the context returns it), more from the
-// device.
-struct BuildScratch {
-    void* ptr = nullptr;
-    cudaStream_t stream = nullptr;
-    bool pooled = false;
-    int take(pb_ctx* ctx, size_t bytes, cudaStream_t s) {
-        stream = s;
-        pooled = ctx->build_pool && bytes <= BUILD_POOL_BYTES &&
-                 cudaMallocFromPoolAsync(&ptr, bytes, ctx->build_pool, s) == cudaSuccess;
-        if (pooled) return PB_OK;
-        cudaGetLastError();
-        return dev_alloc(&ptr, bytes);
-    }
-    ~BuildScratch() {
-        if (!ptr) return;
-        if (pooled) cudaFreeAsync(ptr, stream);
-        else cudaFree(ptr);
-    }
-};
-
 static void free_near(pb_near* nf) {
     if (nf->val) cudaFree(nf->val);  // diag and the mass matrix are parts of it
     nf->val = nf->diag = nullptr;
@@ -1425,7 +1403,7 @@ static void launch_adj(int group, const pb_mesh* m, const int32_t* list, int64_t
     else launch_adj_g<4>(m, list, nlist, ot, rad, kappa, ss, s);
 }
 
-static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaStream_t s) {
+static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaStream_t s, bool pooled) {
     nf->mesh = m;
     nf->kappa = kappa;
     // one allocation for what stays (values, diagonals, mass matrix on its own pattern: pointers,
@@ -1459,8 +1437,8 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
         const size_t be = sizeof(double) * (size_t)SS_OUTER_ARRAYS * nout_e;
         const size_t bv = sizeof(double) * (size_t)SS_OUTER_ARRAYS * nout_v;
         const size_t ss_bytes = part(sizeof(double) * 54 * m->npairs), far_bytes = part(sizeof(double) * 54 * m->n_adj);
-        BuildScratch scratch;
-        PB_TRY(scratch.take(ctx, ss_bytes + far_bytes + bt + be + bv, s));
+        CallScratch scratch;
+        PB_TRY(scratch.take(ctx, ss_bytes + far_bytes + bt + be + bv, s, pooled));
         double* const ss = (double*)scratch.ptr;
         double* const far = (double*)((char*)scratch.ptr + ss_bytes);
         double* const tabm = (double*)((char*)far + far_bytes);
@@ -1588,17 +1566,13 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
     return rc;
 }
 
-}  // namespace pb
-
-using namespace pb;
-
-extern "C" int pb_near_build(pb_ctx* ctx, const pb_mesh* mesh, double kappa, pb_near** out, void* stream) {
+int near_build(pb_ctx* ctx, const pb_mesh* mesh, double kappa, pb_near** out, cudaStream_t s, bool pooled) {
     if (!ctx || !mesh || !out) return set_error(PB_EINVAL, "pb_near_build: NULL argument");
     if (!(kappa >= 0.0) || !std::isfinite(kappa)) return set_error(PB_EINVAL, "kappa must be >= 0");
     *out = nullptr;
     PB_CUDA(cudaSetDevice(ctx->device));
     pb_near* nf = new pb_near();
-    int rc = build(ctx, mesh, kappa, nf, (cudaStream_t)stream);
+    int rc = build(ctx, mesh, kappa, nf, s, pooled);
     if (rc != PB_OK) {
         free_near(nf);
         delete nf;
@@ -1608,12 +1582,18 @@ extern "C" int pb_near_build(pb_ctx* ctx, const pb_mesh* mesh, double kappa, pb_
     return PB_OK;
 }
 
-namespace pb {
 __global__ void k_exp_selftest(const double* __restrict__ x, double* __restrict__ y, int64_t n) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) y[i] = exp_nonpos(x[i]);
 }
+
 }  // namespace pb
+
+using namespace pb;
+
+extern "C" int pb_near_build(pb_ctx* ctx, const pb_mesh* mesh, double kappa, pb_near** out, void* stream) {
+    return near_build(ctx, mesh, kappa, out, (cudaStream_t)stream, true);
+}
 
 extern "C" int pb_selftest_exp(pb_ctx* ctx, const double* x, double* y, int64_t n, void* stream) {
     if (!ctx || (n > 0 && (!x || !y)) || n < 0) return set_error(PB_EINVAL, "pb_selftest_exp: bad argument");

@@ -394,26 +394,25 @@ extern "C" int pb_rhs_charges(pb_ctx* ctx, const pb_mesh* m, const double* xq, c
     return PB_OK;
 }
 
-extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int form, const double* xq, const double* q,
-                         int64_t n_q, const pb_params* prm, double* phi, double* dG_paper, double* dG_kcal, int prec,
-                         void* stream) {
+int pb::energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int form, const double* xq, const double* q, int64_t n_q,
+               const pb_params* prm, double* phi, double* dG_paper, double* dG_kcal, int prec, cudaStream_t s,
+               bool pooled) {
     if (!ctx || !m || !x || !xq || !q || !prm) return set_error(PB_EINVAL, "pb_energy: NULL argument");
     if (prec != PB_F64 && prec != PB_F32_ACCURATE)
         return set_error(PB_EINVAL, "pb_energy: precision must be PB_F64 or PB_F32_ACCURATE");
     if (n_q < 1) return set_error(PB_EINVAL, "need at least one charge");
     if (form < PB_DIRECT_INT || form > PB_LU) return set_error(PB_EINVAL, "unknown formulation %d", form);
-    cudaStream_t s = (cudaStream_t)stream;
     // exterior unknowns -> interior traces: u_int = u_ext, v_int = (eps_ext/eps_int) v_ext
     double vscale = form_is_exterior(form) ? prm->eps_ext / prm->eps_int : 1.0;
     const bool f32 = prec == PB_F32_ACCURATE;
     const int64_t chunk = f32 ? en32_chunk(m->np_ref, n_q) : EN_CHUNK;
     const int nchunk = (int)((m->np_ref + chunk - 1) / chunk);
-    // partial sums, phi per charge, Delta G, then the point values (32-byte aligned); a workspace of
-    // its own, free again when the call returns (the call waits for its work)
+    // partial sums, phi per charge, Delta G, then the point values (32-byte aligned); the call's own
+    // (it waits for its work)
     const size_t n_part = (size_t)n_q * nchunk, n_head = (n_part + (size_t)n_q + 1 + 3) / 4 * 4;
-    pb_mesh* mm = const_cast<pb_mesh*>(m);
-    PB_TRY(ws_reserve(mm->ws_energy, sizeof(double) * (n_head + (f32 ? 6 : 8) * (size_t)m->np_ref)));
-    double* part = (double*)mm->ws_energy.ptr;
+    CallScratch scratch;
+    PB_TRY(scratch.take(ctx, sizeof(double) * (n_head + (f32 ? 6 : 8) * (size_t)m->np_ref), s, pooled));
+    double* part = (double*)scratch.ptr;
     double* phi_all = part + n_part;
     double* dG = phi_all + n_q;
     double* pv = part + n_head;
@@ -442,6 +441,12 @@ extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int for
     if (dG_paper) *dG_paper = h;
     if (dG_kcal) *dG_kcal = h * 4.0 * M_PI * 332.0636;
     return PB_OK;
+}
+
+extern "C" int pb_energy(pb_ctx* ctx, const pb_mesh* m, const double* x, int form, const double* xq, const double* q,
+                         int64_t n_q, const pb_params* prm, double* phi, double* dG_paper, double* dG_kcal, int prec,
+                         void* stream) {
+    return energy(ctx, m, x, form, xq, q, n_q, prm, phi, dG_paper, dG_kcal, prec, (cudaStream_t)stream, true);
 }
 
 extern "C" int pb_solvation_energy(pb_ctx* ctx, const double* verts, int64_t n_verts, const int32_t* tris,

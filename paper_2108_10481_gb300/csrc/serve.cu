@@ -151,7 +151,7 @@ static int setup_req(pb_server* srv, ServeReq* r, cudaStream_t s) {
     pb_ctx* ctx = srv->ctx;
     PB_TRY(pb_mesh_load(ctx, r->V.data(), (int64_t)r->V.size() / 3, r->T.data(), (int64_t)r->T.size() / 3,
                         &r->plan, PB_MEM_HOST, &r->m));
-    PB_TRY(pb_near_build(ctx, r->m, r->prm.kappa, &r->nf, s));
+    PB_TRY(near_build(ctx, r->m, r->prm.kappa, &r->nf, s, false));
     const int64_t nv = r->m->nv, nq = (int64_t)r->q.size();
     PB_TRY(dev_alloc((void**)&r->buf, sizeof(double) * (4 * nq + 10 * nv)));
     r->dxq = r->buf;
@@ -419,8 +419,8 @@ static int tick(pb_server* srv) {
             continue;
         }
         double dGp = 0.0, dGk = 0.0;
-        int rc = pb_energy(srv->ctx, r->m, r->x, r->form, r->dxq, r->dq, (int64_t)r->q.size(), &r->prm, nullptr, &dGp,
-                           &dGk, r->mixed ? PB_F32_ACCURATE : PB_F64, rs_of(r));
+        int rc = energy(srv->ctx, r->m, r->x, r->form, r->dxq, r->dq, (int64_t)r->q.size(), &r->prm, nullptr, &dGp, &dGk,
+                        r->mixed ? PB_F32_ACCURATE : PB_F64, rs_of(r), false);
         if (rc != PB_OK && r->status == PB_OK) r->status = rc;
         if (r->status == PB_OK) r->status = check_status(r->m, rs_of(r));
         srv->free_slots.push_back(r->slot);

@@ -1616,7 +1616,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             Coef cf;
             const Pair64Choice kern = pair64_kernel(fp, &cf);
             const Pair64Plan pl = pair64_plan(np, fp.mode, kern.kind, m->ctx->num_sms,
-                                              occupancy_slots(m, (const void*)kern.one, TPB64));
+                                              occupancy_slots(m, (const void*)kern.one, TPB64), m->part_cap);
             const Sym64& sy = pl.sym;
             const int S = pl.slices();
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, sizeof(double) * (size_t)S * nacc * np));
@@ -1654,8 +1654,10 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             CUtensorMap map;
             PB_TRY(make_tmap(m, rec, &map, REC2, tu));
             const int tpc = TPB2 * 2 * xk.npk;
-            int S = x2_splits(np, tpc, xk.ts, m->ctx->num_sms, acc ? 0 : x2_longest(np, fp.mode, xk.ts, m->ctx->num_sms));
-            S = scaled_splits(S, te.split_scale, np, tu);
+            const int most = capped_slices(m->part_cap, np, nacc, acc ? 8 : 4);
+            int S = x2_splits(np, tpc, xk.ts, m->ctx->num_sms, acc ? 0 : x2_longest(np, fp.mode, xk.ts, m->ctx->num_sms),
+                              most);
+            S = scaled_splits(S, te.split_scale, np, tu, most);
             int64_t chunk = ((np + S - 1) / S + tu - 1) / tu * tu;
             S = (int)((np + chunk - 1) / chunk);
             const Coef32 cf = coef32(fp, m->Q);
@@ -1681,8 +1683,9 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             bool acc = prec == PB_F32_ACCURATE;
             const void* kern = fp.mode == 0 ? (acc ? (const void*)k_pair32<0, true> : (const void*)k_pair32<0, false>)
                                             : (acc ? (const void*)k_pair32<1, true> : (const void*)k_pair32<1, false>);
-            int S = choose_splits(np, TPB32 * TGT32, TS32, occupancy_slots(m, kern, TPB32));
-            S = scaled_splits(S, tuned(m->ctx, np, fp.mode, acc).split_scale, np, TS32);
+            const int most = capped_slices(m->part_cap, np, nacc, acc ? 8 : 4);
+            int S = choose_splits(np, TPB32 * TGT32, TS32, occupancy_slots(m, kern, TPB32), most);
+            S = scaled_splits(S, tuned(m->ctx, np, fp.mode, acc).split_scale, np, TS32, most);
             int64_t chunk = ((np + S - 1) / S + TS32 - 1) / TS32 * TS32;
             S = (int)((np + chunk - 1) / chunk);
             const Coef32 cf = coef32(fp, m->Q);
@@ -1803,11 +1806,11 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
         ::pb::count_launch();
         if (np_pad > np) PB_CUDA(cudaMemsetAsync(rec + REC2 * np, 0, sizeof(float) * REC2 * (np_pad - np), js));
         // the single-mesh decomposition
-        int S = x2_splits(np, tpc, TS2, m->ctx->num_sms, acc ? 0 : x2_longest(np, P.fp.mode, TS2, m->ctx->num_sms));
-        S = scaled_splits(S, tuned(m->ctx, np, P.fp.mode, acc).split_scale, np, TU2);
+        const int nacc = P.fp.mode == 0 ? 2 : 10, most = capped_slices(m->part_cap, np, nacc, acc ? 8 : 4);
+        int S = x2_splits(np, tpc, TS2, m->ctx->num_sms, acc ? 0 : x2_longest(np, P.fp.mode, TS2, m->ctx->num_sms), most);
+        S = scaled_splits(S, tuned(m->ctx, np, P.fp.mode, acc).split_scale, np, TU2, most);
         P.chunk = ((np + S - 1) / S + TU2 - 1) / TU2 * TU2;
         P.S = (int)((np + P.chunk - 1) / P.chunk);
-        const int nacc = P.fp.mode == 0 ? 2 : 10;
         PB_TRY(ws_reserve(m->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)P.S * nacc * np));
         PairJob pj;
         pj.rec = rec;
@@ -1922,13 +1925,6 @@ void batch_scratch_free(BatchScratch& bs) {
     bs.ev.clear();
     if (bs.ev_main) cudaEventDestroy(bs.ev_main);
     bs.ev_main = nullptr;
-}
-
-int far_splits_estimate(pb_ctx* ctx, int64_t np) {
-    int S = x2_splits(np, TPB2 * 2, TS2, ctx->num_sms);
-    for (int mode = 0; mode < 2; ++mode)
-        S = std::max(S, x2_splits(np, TPB2 * 4, TS2, ctx->num_sms, x2_longest(np, mode, TS2, ctx->num_sms)));
-    return S;
 }
 
 }  // namespace pb

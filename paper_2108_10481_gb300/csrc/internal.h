@@ -156,6 +156,7 @@ struct pb_mesh {
     pb_ctx* ctx = nullptr;
     int64_t nv = 0, nt = 0, np = 0;
     int Q = 0, n_ss = 0;
+    double part_cap = 0.0;            // bytes that a direct application's partial sums may take (0: any)
     double max_edge = 0.0;            // longest edge
     double ctr[3] = {0.0, 0.0, 0.0};  // centre of the bounding box: origin of the split FP32 coordinates
     int n_ss_cls[3] = {0, 0, 0};  // singular Gauss points per dimension: coincident, edge, vertex pairs
@@ -322,8 +323,6 @@ int tree_far(const pb_mesh* m, const FarPlan& fp, const double* x, bool need_u, 
 void tree_free(PbTree* t);
 int tree_info(const pb_mesh* m, int64_t out[6]);
 
-// largest split count the packed kernels use for np points (workspace estimates)
-int far_splits_estimate(pb_ctx* ctx, int64_t np);
 // the tuned entry that applies to np points (kernel 0 when none)
 TuneEntry tuned(const pb_ctx* ctx, int64_t np, int mode, bool acc);
 int tune_bucket(int64_t np);

@@ -28,6 +28,7 @@
 #include <thread>
 
 #include "solver.h"
+#include "splits.h"
 
 namespace pb {
 
@@ -57,6 +58,7 @@ struct ServeReq {
     GmresWork G;
     bool mixed = false;
     int mmax = 0;
+    double part = 0.0;        // bytes for the direct applications' partial sums
     int slot = -1;            // row of the server's residual table while active
     StepGraph g_mid, g_tail;  // captured iteration pieces (Calderon middle; preconditioner + Arnoldi)
     // iteration state
@@ -121,8 +123,10 @@ static int free_req(ServeReq* r) {
 // and 15 eta^2 nonzeros per vertex: the synthetic molecules have about 145
 // band pairs per triangle and 147 nonzeros per vertex at 3 radii). The near
 // build's per-pair blocks (432 bytes per listed pair) are the largest
-// transient: about 14 GB on the 5,000-atom molecule.
-static size_t footprint(pb_ctx* ctx, int64_t nv, int64_t nt, const pb_quad_plan& plan, int mmax, int64_t nq) {
+// transient: about 14 GB on the 5,000-atom molecule. part: the direct
+// applications' partial sums, which the request's mesh is held to.
+static size_t footprint(pb_ctx* ctx, int64_t nv, int64_t nt, const pb_quad_plan& plan, int mmax, int64_t nq,
+                        double part) {
     const int Q = plan.far_q;
     const double eta = plan.band_eta, band = 18.0 * eta * eta * nt;
     const double np = (double)Q * nt, nadj = 16.0 * nt, npairs = nadj + band, nnz = (25.0 + 15.0 * eta * eta) * nv;
@@ -132,8 +136,6 @@ static size_t footprint(pb_ctx* ctx, int64_t nv, int64_t nt, const pb_quad_plan&
     double nearb = 56 * nnz + 56 * nv;
     double near_tmp = 432 * (npairs + nadj) + 4 * nnz;
     double src = 128 * (np + 64);
-    int S = far_splits_estimate(ctx, (int64_t)np);
-    double part = (double)S * 10 * np * 8;
     double work = src + part + 48 * nt + 48 * nnz + 128 * nv;
     if (ctx->tree_enable && np >= (double)ctx->tree_min_points) {
         work += 330 * np;  // treecode: tree-ordered sources, proxies of about np / 64 clusters, lists
@@ -151,6 +153,7 @@ static int setup_req(pb_server* srv, ServeReq* r, cudaStream_t s) {
     pb_ctx* ctx = srv->ctx;
     PB_TRY(pb_mesh_load(ctx, r->V.data(), (int64_t)r->V.size() / 3, r->T.data(), (int64_t)r->T.size() / 3,
                         &r->plan, PB_MEM_HOST, &r->m));
+    r->m->part_cap = r->part;
     PB_TRY(near_build(ctx, r->m, r->prm.kappa, &r->nf, s, false));
     const int64_t nv = r->m->nv, nq = (int64_t)r->q.size();
     PB_TRY(dev_alloc((void**)&r->buf, sizeof(double) * (4 * nq + 10 * nv)));
@@ -539,7 +542,15 @@ extern "C" int pb_submit(pb_server* srv, const pb_request* req) {
         return set_error(PB_EINVAL, "pb_submit: need tol > 0 and max_it >= 1");
     }
     r->mmax = r->opts.restart > 0 ? std::min(r->opts.restart, r->opts.max_it) : r->opts.max_it;
-    r->footprint = footprint(srv->ctx, req->n_verts, req->n_tris, r->plan, r->mmax, req->n_q);
+    // a budget too small for the partial sums that are best for speed gets the least ones
+    const int64_t np = std::max<int64_t>(1, (int64_t)r->plan.far_q * req->n_tris);  // the plan is checked at the load
+    const double least = least_part_bytes(np, srv->ctx->num_sms);
+    r->part = part_bytes(np, srv->ctx->num_sms, r->opts.precision == PB_MIXED);
+    for (int k = 0; k < 2; ++k) {
+        r->footprint = footprint(srv->ctx, req->n_verts, req->n_tris, r->plan, r->mmax, req->n_q, r->part);
+        if (r->footprint <= srv->budget || r->part <= least) break;
+        r->part = least;
+    }
     if (r->footprint > srv->budget) {
         size_t fp = r->footprint;
         delete r;

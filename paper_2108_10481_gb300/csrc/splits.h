@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 namespace pb {
@@ -10,13 +11,18 @@ namespace pb {
 constexpr int TPB64 = 128;  // threads (= targets) per CTA of the one-direction FP64 kernel
 constexpr int TS64 = 64;    // its sources per shared-memory tile
 
+// Slices of nacc sums of `size` bytes a point that `cap` bytes hold (at least one); cap 0: any.
+inline int capped_slices(double cap, int64_t np, int nacc, int size) {
+    return cap > 0.0 ? (int)std::max(1.0, std::min(64.0, std::floor(cap / ((double)nacc * size * (double)np)))) : 64;
+}
+
 // split count of the scalar and one-direction FP64 kernels: fill the GPU in whole waves
-inline int choose_splits(int64_t np, int tpc, int tile, int slots) {
+inline int choose_splits(int64_t np, int tpc, int tile, int slots, int most = 32) {
     int64_t nb = (np + tpc - 1) / tpc;
     int64_t ntiles = (np + tile - 1) / tile;
     int best = 1;
     double best_cost = 1e300;
-    for (int S = 1; S <= 32; ++S) {
+    for (int S = 1; S <= std::min(most, 32); ++S) {
         if (S > ntiles) break;
         int64_t ctas = nb * S;
         int64_t waves = (ctas + slots - 1) / slots;
@@ -44,13 +50,13 @@ inline int64_t x2_longest(int64_t np, int mode, int ts, int num_sms) {
 // slice, a part of the SMs had stood idle: 58,080 points, V/K + D/T rows 3,750 -> 3,510 us, split V/K
 // rows 3,050 -> 2,810 us at the counts chosen here.)
 constexpr int X2_MAX_SLICES = 36;  // 32 of the longest slices in tiles of fewer points than ts
-inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest = 0) {
+inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest = 0, int most = 64) {
     const int tile = ts / 3 * 3;
     const int64_t nb = (np + tpc - 1) / tpc, ntiles = (np + tile - 1) / tile;
     const int64_t per_max = longest > 0 ? longest / ts : ntiles;
-    int best = 1;
+    int best = (int)std::min<int64_t>(std::min(most, X2_MAX_SLICES), ntiles);  // as short as they can be
     double best_cost = 1e300;
-    for (int S = 1; S <= (longest > 0 ? X2_MAX_SLICES : 32) && S <= ntiles; ++S) {
+    for (int S = 1; S <= std::min(most, longest > 0 ? X2_MAX_SLICES : 32) && S <= ntiles; ++S) {
         const int64_t deep = (nb * S + num_sms - 1) / num_sms, per = (ntiles + S - 1) / S;
         if (per > per_max) continue;
         const double cost = (double)(deep * per) * (1.0 + 0.05 / (double)deep) * (1.0 + 0.002 * S);
@@ -59,11 +65,11 @@ inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest =
     return best;
 }
 
-// split count after the tuned scale, within [1, tiles] and <= 32 (or the untuned one)
-inline int scaled_splits(int S, double scale, int64_t np, int tile) {
+// split count after the tuned scale, within [1, tiles] and <= 32 (or the untuned one) and <= most
+inline int scaled_splits(int S, double scale, int64_t np, int tile, int most = 64) {
     const int64_t ntiles = (np + tile - 1) / tile;
     int s2 = (int)(S * scale + 0.5);
-    s2 = std::max(1, std::min(s2, std::max(S, 32)));
+    s2 = std::max(1, std::min({s2, std::max(S, 32), most}));
     return (int)std::min<int64_t>(s2, ntiles);
 }
 
@@ -98,9 +104,9 @@ struct Pair64Plan {
 inline double few_warps(double resident) { return resident < 6.0 ? 6.0 / resident : 1.0; }
 
 // One direction at a time, by whole waves of `slots` resident CTAs.
-inline Pair64Plan pair64_one(int64_t np, int mode, int kind, int num_sms, int slots) {
+inline Pair64Plan pair64_one(int64_t np, int mode, int kind, int num_sms, int slots, double cap = 0.0) {
     Pair64Plan p = {{0, 0, 0, 0, 0}, 1, 0, 0.0};
-    p.nsplit = choose_splits(np, TPB64, TS64, slots);
+    p.nsplit = choose_splits(np, TPB64, TS64, slots, capped_slices(cap, np, mode == 0 ? 2 : 10, 8));
     p.chunk = ((np + p.nsplit - 1) / p.nsplit + TS64 - 1) / TS64 * TS64;
     p.nsplit = (int)((np + p.chunk - 1) / p.chunk);
     const int64_t ctas = (np + TPB64 - 1) / TPB64 * p.nsplit, on_sm = (ctas + num_sms - 1) / num_sms;
@@ -111,9 +117,9 @@ inline Pair64Plan pair64_one(int64_t np, int mode, int kind, int num_sms, int sl
 
 // Both directions at once: the shape whose busiest SM has the least work. The partial sums stay within 32 slices, or 64 while they are
 // below 32 MB; a block has 1,024 points at most, so 63 blocks (64,512 points) are the most.
-inline Pair64Plan pair64_both(int64_t np, int mode, int kind, int num_sms) {
+inline Pair64Plan pair64_both(int64_t np, int mode, int kind, int num_sms, double cap = 0.0) {
     static const int shapes[5][2] = {{2, 1}, {4, 1}, {8, 1}, {8, 2}, {8, 4}};
-    const int nacc = mode == 0 ? 2 : 10;
+    const int nacc = mode == 0 ? 2 : 10, most = capped_slices(cap, np, nacc, 8);
     Pair64Plan best = {{0, 0, 0, 0, 0}, 0, 0, 1e300};
     for (const auto& sh : shapes) {
         Sym64 c;
@@ -124,7 +130,7 @@ inline Pair64Plan pair64_both(int64_t np, int mode, int kind, int num_sms) {
         c.nblock = (int)nb;
         c.half = c.nblock / 2;
         const int units = (c.half + 1) * c.warps * c.sub;
-        for (c.nsplit = 1; c.nsplit <= units && c.slices() <= 64; ++c.nsplit) {
+        for (c.nsplit = 1; c.nsplit <= units && c.slices() <= most; ++c.nsplit) {
             if (c.slices() > 32 && (double)c.slices() * nacc * np * 8.0 > 32e6) break;
             const int64_t ctas = nb * c.nsplit, per = (units + c.nsplit - 1) / c.nsplit;
             const int64_t on_sm = (ctas + num_sms - 1) / num_sms;
@@ -144,10 +150,34 @@ inline Pair64Plan pair64_both(int64_t np, int mode, int kind, int num_sms) {
 // slices leave too few CTAs for the GPU's SMs as the blocks approach 63 (from 62,465 points on one
 // block of rows an SM and 41 % of the FP64 pipe: 63,480 points, V/K + D/T rows 551 ms, one direction at a time
 // 340; V/K rows 376 and 250).
-inline Pair64Plan pair64_plan(int64_t np, int mode, int kind, int num_sms, int slots) {
-    const Pair64Plan both = pair64_both(np, mode, kind, num_sms);
-    const Pair64Plan one = pair64_one(np, mode, kind, num_sms, slots);
+// cap: bytes that the partial sums may take (0: any).
+inline Pair64Plan pair64_plan(int64_t np, int mode, int kind, int num_sms, int slots, double cap = 0.0) {
+    const Pair64Plan both = pair64_both(np, mode, kind, num_sms, cap);
+    const Pair64Plan one = pair64_one(np, mode, kind, num_sms, slots, cap);
     return both.sym.nblock && both.cost <= one.cost ? both : one;
+}
+
+// ------------------------------------------------------- a request's partial sums
+// Bytes of the direct applications' partial sums of a served request, any operator: as the rules
+// above would have it, and the least that they are held to where a budget does not allow that (whole
+// waves of the packed kernel's CTAs, in FP64).
+inline double part_bytes(int64_t np, int num_sms, bool mixed) {
+    double b = 0.0;
+    for (int mode = 0; mode < 2; ++mode) {
+        const double sum = (double)np * (mode == 0 ? 2 : 10);
+        if (mixed) {
+            b = std::max(b, 8.0 * sum * x2_splits(np, 512, 64, num_sms));
+            b = std::max(b, 4.0 * sum * x2_splits(np, 1024, 64, num_sms, x2_longest(np, mode, 64, num_sms)));
+        } else {
+            for (int kind = 0; kind < (mode == 0 ? 2 : 3); ++kind)
+                b = std::max(b, 8.0 * sum * pair64_plan(np, mode, kind, num_sms, 6 * num_sms).slices());
+        }
+    }
+    return b;
+}
+inline double least_part_bytes(int64_t np, int num_sms) {
+    return 80.0 * (double)np *
+           std::max(choose_splits(np, 512, 64, 2 * num_sms), choose_splits(np, 1024, 64, 2 * num_sms));
 }
 
 }  // namespace pb

@@ -96,3 +96,48 @@ def test_fast_slices_no_longer_than_whole_waves(tmp_path):
             np_, mode, shape, S, chunk, wave = map(int, line.split())
             assert S <= 36
             assert chunk <= wave, line
+
+
+CAPPED = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "splits.h"
+using namespace pb;
+int main(int argc, char** argv) {  // lo hi step: bytes of every application's partial sums against a request's
+    for (long long np = atoll(argv[1]); np <= atoll(argv[2]); np += atoll(argv[3]))
+        for (int mixed = 0; mixed < 2; ++mixed)
+            for (int least = 0; least < 2; ++least) {
+                const double cap = least ? least_part_bytes(np, %(sms)d) : part_bytes(np, %(sms)d, mixed);
+                double most = 0.0;
+                for (int mode = 0; mode < 2; ++mode) {
+                    const double sum = (double)np * (mode ? 10 : 2);
+                    if (mixed)
+                        for (int acc = 0; acc < 2; ++acc)
+                            for (double scale = 0.5; scale <= 2.0; scale *= 2.0) {
+                                const int n = capped_slices(cap, np, mode ? 10 : 2, acc ? 8 : 4);
+                                int S = x2_splits(np, acc ? 512 : 1024, 64, %(sms)d, acc ? 0 : x2_longest(np, mode, 64, %(sms)d), n);
+                                S = scaled_splits(S, scale, np, 63, n);
+                                if (S * sum * (acc ? 8 : 4) > most) most = S * sum * (acc ? 8 : 4);
+                            }
+                    else
+                        for (int kind = 0; kind < (mode ? 3 : 2); ++kind)
+                            for (int resident = 6; resident <= 9; resident += 3) {
+                                const Pair64Plan p = pair64_plan(np, mode, kind, %(sms)d, resident * %(sms)d, cap);
+                                if (p.slices() * sum * 8 > most) most = p.slices() * sum * 8;
+                            }
+                }
+                printf("%%lld %%d %%d %%.17g %%.17g\n", np, mixed, least, most, cap);
+            }
+    return 0;
+}
+""" % {"sms": SMS}
+
+
+def test_partial_sums_within_a_request_s_bytes(tmp_path):
+    """Served applications' partial sums, tuned split scales included, stay within what the server's budget counts."""
+    exe = compile_driver(tmp_path, CAPPED)
+    for rng in ((1, 4000, 7), (4002, 66000, 186), (62400, 64600, 6), (70000, 800000, 7302)):
+        out = subprocess.run([exe, *map(str, rng)], check=True, capture_output=True, text=True).stdout
+        for line in out.splitlines():
+            np_, mixed, least, most, cap = (float(w) for w in line.split())
+            assert 0 < most <= cap, line

@@ -440,8 +440,8 @@ int pb_autotune_plan(pb_ctx* ctx, const double* verts, int64_t n_verts, const in
 #define PB_KERNEL_KRYLOV 9          /* Gram-Schmidt dots and updates of the Arnoldi step (memory-bound) */
 #define PB_KERNEL_COUNT 10
 /* For the pair kernels, "pairs" are target-source point pairs and "ops" FP32
- * (FP64 for PB_KERNEL_PAIR64) operations by the kernel's formula count; for
- * the near-field kernels, "pairs" are quadrature point pairs of the rules (the
+ * operations by the kernel's formula count (PB_KERNEL_PAIR64: FP64 flops, a
+ * fused multiply-add counted as two); for the near-field kernels, "pairs" are quadrature point pairs of the rules (the
  * kernels evaluate fewer: some of the sums are taken in closed form) and "ops"
  * FP64 flops by formula count (kernel evaluation and accumulation into the local
  * blocks, a fused multiply-add counted as two).

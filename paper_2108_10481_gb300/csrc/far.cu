@@ -1562,14 +1562,23 @@ static int make_tmap(const pb_mesh* m, const float* rec, CUtensorMap* map, int r
     return PB_OK;
 }
 
-// FP32-pipe operations per point pair by the formula count of the kernels
-// above (FADD, FMUL and FFMA each one; the two MUFU operations not counted):
-// V/K rows 19; V/K + D/T rows 36, 20 or 32 by kind; split coordinates +6. (The
-// scalar kernel and the one-direction FP64 kernel by the same counts.) The packed
-// kernel's V/K + D/T rows on points in threes: 34, 18 or 30.
-static double pair_ops(const FarPlan& fp, bool threes = false) {
+// FP32-pipe operations per point pair by the formula count of the packed kernel (FADD, FMUL and
+// FFMA each one; the two MUFU operations not counted): V/K rows 19; V/K + D/T rows 36, 20 or 32 by
+// kind, on points in threes 34, 18.7 or 29.7; split coordinates +6.
+static double pair_ops(const FarPlan& fp, bool threes) {
     static const double vkdt[2][3] = {{36.0, 20.0, 32.0}, {34.0, 18.667, 29.667}};
     return fp.mode == 0 ? 19.0 : vkdt[threes ? 1 : 0][far_kind(fp)];
+}
+// The scalar kernel's, coefficients in the loop: geometry 17, a V/K row 4, a D/T row 15.
+static double scalar_ops(const FarPlan& fp) { return fp.mode == 0 ? 25.0 : 36.0; }
+// FP64 flops per directed point pair by the formula count of the FP64 kernels (a fused
+// multiply-add counted as two): d and r^2 8; rsqrt, r, the exponential and its argument 17 (rsqrt
+// alone 1); 1/r^2, the Yukawa values and d.p 10 (7), the kernels 8 to 12, the sums. Both
+// directions at once share all but d.p and the sums.
+static double pair64_flops(const FarPlan& fp, int kind, bool both) {
+    static const double one[2][3] = {{43.0, 20.0, 0.0}, {71.0, 34.0, 67.0}};
+    static const double two[2][3] = {{28.5, 14.5, 0.0}, {50.0, 27.5, 48.0}};
+    return (both ? two : one)[fp.mode][kind];
 }
 constexpr double OPS_SPLIT = 6.0;
 
@@ -1621,7 +1630,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             const int S = pl.slices();
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, sizeof(double) * (size_t)S * nacc * np));
             double* part = (double*)m->ws_part.ptr;
-            Timer tm(m->ctx, PB_KERNEL_PAIR64, s, (double)np * (double)np, pair_ops(fp));
+            Timer tm(m->ctx, PB_KERNEL_PAIR64, s, (double)np * (double)np, pair64_flops(fp, kern.kind, sy.nblock > 0));
             if (sy.nblock) {
                 const size_t smem = sizeof(double) * 32 * (10 + (size_t)kern.sums * sy.warps * (1 + sy.sub));
                 // the largest any shape takes, whatever this one does: other host threads set the same
@@ -1692,7 +1701,7 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             dim3 grid((unsigned)((np + TPB32 * TGT32 - 1) / (TPB32 * TGT32)), (unsigned)S);
             PB_TRY(ws_reserve(const_cast<pb_mesh*>(m)->ws_part, (acc ? sizeof(double) : sizeof(float)) * (size_t)S * nacc * np));
             void* part = m->ws_part.ptr;
-            double ops = pair_ops(fp) + (acc ? OPS_SPLIT : 0.0);
+            double ops = scalar_ops(fp) + (acc ? OPS_SPLIT : 0.0);
             Timer tm(m->ctx, acc ? PB_KERNEL_PAIR32_ACCURATE : PB_KERNEL_PAIR32, s, (double)np * (double)np, ops);
             if (fp.mode == 0) {
                 if (acc) k_pair32<0, true><<<grid, TPB32, 0, s>>>(map, np, m->pts32, m->pts32lo, cf, chunk, part, status);

@@ -64,7 +64,10 @@ extern "C" {
 #define PB_YUKAWA 1
 /* arithmetic of a far-field application */
 #define PB_F64 0          /* FP64 everywhere */
-#define PB_F32 1          /* FP32 pair sums and FP32 near field (inner solves) */
+#define PB_F32 1          /* FP32 pair sums and, in solves, the server and
+                             pb_system_apply_noalloc, an FP32 near field; a single
+                             pb_system_apply or pb_op_apply combines the near field's
+                             FP64 values as it applies them, unrounded */
 #define PB_F32_ACCURATE 2 /* FP32 pair arithmetic on split (hi+lo) coordinates with
                              the tiles' sums accumulated in three FP32 words (no fewer
                              bits than FP64), FP64 near field */

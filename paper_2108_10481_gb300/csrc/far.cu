@@ -790,7 +790,7 @@ __device__ __forceinline__ double wide_total(const float2& hi, const float4* wor
 // and 3 where it reads three different registers (a multiply-add of three values; measured 2.2
 // and 3.3 in a bare loop), so a pair takes, in cycles: V/K rows 44; V/K + D/T rows KIND 0 77 (by
 // single points 85), KIND 1 46 (52), KIND 2 69 (77); split coordinates 12 more. 30,720 points,
-// V/K + D/T rows: 983 -> 908 us; split, 61,440 points: 4.97 -> 4.41 ms. (The height (x - y) . n
+// V/K + D/T rows: 983 -> 913 us; split, 61,440 points: 4.97 -> 4.42 ms. (The height (x - y) . n
 // taken once for a three, too, gives 930 and 4.43 ms per application, but the three then share its
 // rounding errors: twice the error of the FP32 applications against FP64.)
 template <int MODE, bool ACC, int NPK, bool GUARD, int TS, int KIND, int U>

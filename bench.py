@@ -43,7 +43,13 @@ L2_FLUSH_BYTES = 256 << 20
 # changed since its capture, or that has none, reports null.
 NCU_TRAFFIC = {  # (kernel family, formulation or "any", far-rule points, band) -> dram read + write per launch
     # 5,000-atom molecule (667,788 far-rule points, band of 3 radii), ncu dram__bytes_{read,write}.sum
-    ("spmv", "juffer", 667788, 3.0): 337.5e6,
+    ("spmv", "juffer", 667788, 3.0): 338.0e6,
+    ("cheb", "juffer", 667788, 3.0): 16.04e6,
+    ("tree32", "juffer", 667788, 3.0): 249.9e6,
+    ("pair32acc", "juffer", 667788, 3.0): 429.5e6,  # the default launch shape's
+    ("near_adj", "any", 667788, 3.0): 708.0e6,  # mean of the edge-pair and vertex-pair launches
+    ("near_band", "any", 667788, 3.0): 15757.1e6,
+    ("near_coin", "any", 667788, 3.0): 262.3e6,
 }
 
 

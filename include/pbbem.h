@@ -391,8 +391,8 @@ typedef struct {
     int tile_records;       /* source records that a TMA tile of the chosen launch has room for (whole threes are used) */
     int stages;             /* its pipeline stages */
     int targets_per_thread; /* its targets per thread */
-    int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide (three-word) sums at a time */
-    double split_scale;     /* chosen multiplier of the wave-filling split count */
+    int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide (three-word) sums at a time (the name is from when they were FP64) */
+    double split_scale;     /* chosen multiplier of the default split count */
     double best_ms;         /* one FP32 system application with the choice */
     double default_ms;      /* ... with the untuned default (packed, shape 0, x1) */
 } pb_tune_choice;
@@ -405,7 +405,7 @@ typedef struct {
  * packed kernel in each of its launch shapes - records per TMA tile 32, 64
  * or 128, 2 or 4 pipeline stages, 2 or 4 targets per thread, for the
  * split-coordinate variant 1, 2 or 4 tiles per addition to the wide sums - each with the
- * wave-filling split count x0.5, x1 and x2) and keep the fastest of each
+ * default split count x0.5, x1 and x2) and keep the fastest of each
  * variant in ctx for meshes of this size (same power-of-two bucket of
  * quadrature points). Later applications, solves and the server use it. out
  * may be NULL. The treecode is off while the candidates are timed (the choice

@@ -225,7 +225,9 @@ __global__ void __launch_bounds__(TPB64, 6) k_pair64(int64_t np, const double* _
 // sums are plain read-modify-writes of shared memory without conflicts, at about 6 % of
 // the FP64 pipe's time. Partial sums: split sp of the I block's ranges in slice sp, the J
 // side of distance s in slice nsplit + s - 1, the W warps' added in order: no atomics.
-// 1,920 points, MODE 0: 229 -> 171 us; 7,680 points, MODE 1: 4.96 -> 3.42 ms.
+// 1,920 points, MODE 0: 229 -> 171 us; 7,680 points, MODE 1: 4.96 -> 3.42 ms. Rounding: an emulation of
+// both kernels' sums against 80-bit ones (7,680 points, V/K rows of both kinds) gives 1.9 and 2.2e-16 for these, 2.2 and
+// 2.5e-16 for one direction with the coefficients in the loop.
 constexpr int SYM64_MAX_SMEM = 8 * 32 * (10 + 11 * 8 * (1 + 4));  // W = 8, SB = 4
 template <int MODE, int KIND, bool BOTH>
 __device__ __forceinline__ void sym64_steps(const Coef& cf, const double* xi, double si, const double* pi, const double* ci,

@@ -394,7 +394,7 @@ typedef struct {
     int tiles_per_fp64_sum; /* split-coordinate variant: tiles whose FP32 sums go into the wide (three-word) sums at a time (the name is from when they were FP64) */
     double split_scale;     /* chosen multiplier of the default split count */
     double best_ms;         /* one FP32 system application with the choice */
-    double default_ms;      /* ... with the untuned default (packed, shape 0, x1) */
+    double default_ms;      /* ... with the packed kernel's shape 0, x1 (the untuned default, but for PB_F32 below 16,384 points) */
 } pb_tune_choice;
 typedef struct {
     pb_tune_choice fast;     /* PB_F32 applications (FP32 tile sums) */

@@ -792,7 +792,7 @@ __device__ __forceinline__ double wide_total(const float2& hi, const float4* wor
 // and 3 where it reads three different registers (a multiply-add of three values; measured 2.2
 // and 3.3 in a bare loop), so a pair takes, in cycles: V/K rows 44; V/K + D/T rows KIND 0 77 (by
 // single points 85), KIND 1 46 (52), KIND 2 69 (77); split coordinates 12 more. 30,720 points,
-// V/K + D/T rows: 983 -> 913 us; split, 61,440 points: 4.97 -> 4.42 ms. (The height (x - y) . n
+// V/K + D/T rows: 983 -> 908 us; split, 61,440 points: 4.97 -> 4.42 ms. (The height (x - y) . n
 // taken once for a three, too, gives 930 and 4.43 ms per application, but the three then share its
 // rounding errors: twice the error of the FP32 applications against FP64.)
 template <int MODE, bool ACC, int NPK, bool GUARD, int TS, int KIND, int U>
@@ -999,7 +999,7 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
 }
 
 // Launch shapes of the packed kernel, one table per row mode and variant; the
-// autotuner picks one per mesh-size bucket (shape 0: the default).
+// autotuner picks one per mesh-size bucket (untuned: shape 0, or by x2_fast_shape).
 // Shapes: (records per tile, stages, packed target pairs per thread, tiles per
 // addition to the wide sums of the split-coordinate variant).
 typedef void (*X2Launch)(dim3, cudaStream_t, const CUtensorMap&, int64_t, const float*, const float*, Coef32,
@@ -1660,12 +1660,14 @@ int apply_blockop(const pb_mesh* m, const pb_near* nf, const BlockOp& B, int pre
             ::pb::count_launch();
             bool acc = prec == PB_F32_ACCURATE;
             const TuneEntry te = tuned(m->ctx, np, fp.mode, acc);
-            const X2Entry& xk = x2_kernel(fp.mode, far_kind(fp), acc, te.shape);
+            const int most = capped_slices(m->part_cap, np, nacc, acc ? 8 : 4);
+            const X2Entry& xk = x2_kernel(fp.mode, far_kind(fp), acc,
+                                          te.kernel == 0 && !acc ? x2_fast_shape(np, fp.mode, m->ctx->num_sms, most)
+                                                                 : te.shape);
             const int tu = tile_points(xk.ts);
             CUtensorMap map;
             PB_TRY(make_tmap(m, rec, &map, REC2, tu));
             const int tpc = TPB2 * 2 * xk.npk;
-            const int most = capped_slices(m->part_cap, np, nacc, acc ? 8 : 4);
             int S = x2_splits(np, tpc, xk.ts, m->ctx->num_sms, acc ? 0 : x2_longest(np, fp.mode, xk.ts, m->ctx->num_sms),
                               most);
             S = scaled_splits(S, te.split_scale, np, tu, most);
@@ -2053,7 +2055,7 @@ extern "C" int pb_system_apply_noalloc(pb_ctx* ctx, const pb_mesh* m, const pb_n
 // Times the FP32 far-field application of one formulation on the caller's
 // mesh for every candidate launch (the scalar kernel, or the packed kernel in
 // each of its launch shapes - records per TMA tile, pipeline stages, targets
-// per thread; split count x0.5, x1, x2 of the wave-filling choice; both the
+// per thread; split count x0.5, x1, x2 of the default; both the
 // fast and the split-coordinate variant), keeps the fastest per variant in the
 // context's table for this size bucket, and reports the gain. Results of the
 // tuned launches are the same sums in another split and tile order (FP32

@@ -126,7 +126,7 @@ namespace pb {
 // (log2 of the point count) and row mode / precision.
 struct TuneEntry {
     int kernel = 0;          // 0 = not tuned, 1 = scalar, 2 = packed f32x2
-    double split_scale = 1;  // multiplier of the wave-filling split count
+    double split_scale = 1;  // multiplier of the default split count
     int shape = 0;           // launch shape of the packed kernel (tile records, stages, targets per thread)
 };
 constexpr int TUNE_BUCKETS = 40;

@@ -50,10 +50,11 @@ inline int64_t x2_longest(int64_t np, int mode, int ts, int num_sms) {
 // slice, a part of the SMs had stood idle: 58,080 points, V/K + D/T rows 3,750 -> 3,510 us, split V/K
 // rows 3,050 -> 2,810 us at the counts chosen here.)
 constexpr int X2_MAX_SLICES = 36;  // 32 of the longest slices in tiles of fewer points than ts
-inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest = 0, int most = 64) {
+inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest = 0, int most = 64,
+                     double* cost_out = nullptr) {
     const int tile = ts / 3 * 3;
     const int64_t nb = (np + tpc - 1) / tpc, ntiles = (np + tile - 1) / tile;
-    const int64_t per_max = longest > 0 ? longest / ts : ntiles;
+    const int64_t per_max = longest > 0 ? std::max<int64_t>(1, (longest + tile / 2) / tile) : ntiles;  // to the nearest tile
     int best = (int)std::min<int64_t>(std::min(most, X2_MAX_SLICES), ntiles);  // as short as they can be
     double best_cost = 1e300;
     for (int S = 1; S <= std::min(most, longest > 0 ? X2_MAX_SLICES : 32) && S <= ntiles; ++S) {
@@ -62,7 +63,24 @@ inline int x2_splits(int64_t np, int tpc, int ts, int num_sms, int64_t longest =
         const double cost = (double)(deep * per) * (1.0 + 0.05 / (double)deep) * (1.0 + 0.002 * S);
         if (cost < best_cost) { best_cost = cost; best = S; }
     }
+    if (cost_out) *cost_out = best_cost * tpc * tile;
     return best;
+}
+
+// Untuned launch shape of the fast variant: 0 (1,024 targets a CTA) or, below 16,384 points, 3 (512,
+// one packed pair a thread), whose CTAs share out more evenly what bounded slices leave of a small
+// surface. V/K + D/T rows, us, 1,024 | 512 targets: 3,000 points 75 | 63, 5,880: 117 | 100, 9,720: 171 | 150, 14,520:
+// 280 | 261. V/K rows take a tenth longer a pair with 512 and do so only where the busiest SM has that
+// much less to do: 5,880: 80 | 73, 9,720: 134 | 112, but 7,680: 94 | 98, 12,000: 155 | 162.
+constexpr int X2_SMALL_CTAS = 3;
+inline int x2_fast_shape(int64_t np, int mode, int num_sms, int most = 64) {
+    if (np >= 16384) return 0;
+    if (mode == 1) return X2_SMALL_CTAS;
+    const int64_t longest = x2_longest(np, mode, 64, num_sms);
+    double large, small;
+    x2_splits(np, 1024, 64, num_sms, longest, most, &large);
+    x2_splits(np, 512, 64, num_sms, longest, most, &small);
+    return 1.1 * small < 0.97 * large ? X2_SMALL_CTAS : 0;
 }
 
 // split count after the tuned scale, within [1, tiles] and <= 32 (or the untuned one) and <= most

@@ -1,6 +1,7 @@
 """Split-coordinate pair sums where a CTA adds a hundred tiles and more (61,440 points): V/K rows and each kind of V/K +
 D/T rows against the library's FP64 application. Tolerance 2e-7: a tile's 63 FP32 sums round at 2^-24 each and their errors
-average out over the tiles; a lost or misplaced word of the sums over the tiles is orders above."""
+average out over the tiles; a lost or misplaced word of the sums over the tiles is orders above. The fast variant's launch
+shape above 16,384 points (the row kinds' test has the one below), tolerance as there."""
 import pytest
 
 from synth import icosphere
@@ -33,3 +34,16 @@ def test_many_tiles(case, form, alpha, beta):
 
     ref = apply(pb.PB_F64)
     assert float((apply(pb.PB_F32_ACCURATE) - ref).norm() / ref.norm()) < 2e-7
+
+
+@pytest.mark.parametrize("form,alpha,beta", FORMS)
+def test_fast_variant(case, form, alpha, beta):
+    pb, ctx, m, nf, x = case
+    P = pb.Params(4.0, 80.0, 0.125)
+    pb.pb_set_treecode(ctx, False, 6, 0.7, 0)
+
+    def apply(prec):
+        return pb.pb_system_apply(ctx, m, nf, P, form, x, prec=prec, alpha=alpha, beta=beta)
+
+    ref = apply(pb.PB_F64)
+    assert float((apply(pb.PB_F32) - ref).norm() / ref.norm()) < 2e-5

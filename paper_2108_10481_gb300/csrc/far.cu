@@ -748,41 +748,51 @@ __device__ __forceinline__ void x2_out(const Coef2& cf, const float2* v, float2*
 // Wide sums of the split-coordinate variant: a tile's FP32 sums are added into three FP32 words
 // (wide.h), 13 packed operations a value; FP64 additions and the conversions to FP64, at the GB300's
 // FP64 rate, took a third of the kernel's time when every tile of 64 sources was added. The lower two
-// words lie in shared memory, float4 (mid, lo) per value and thread at [value][thread]: in
-// registers they would spill. 61,440 points, V/K + D/T rows, every point by
-// itself: 5.89 ms with FP64 additions, 4.98 with two words (about 48 bits); as now, an application 4.53 ms
-// with two and 4.54 with three. (Tiles of 128 sources would be faster, but their FP32 sums raise the
-// PMCHWT forms' error against the FP64 application from 4.0e-8 to 5.5e-8.)
+// words of V/K + D/T rows lie in shared memory, float4 (mid, lo) per value and thread at
+// [value][thread]: in registers they would spill. 61,440 points, V/K + D/T rows, every point by itself:
+// 5.89 ms with FP64 additions, 4.98 with two words (about 48 bits); as now, an application 4.53 ms with
+// two and 4.55 with three; V/K rows 3.25 and 3.31 (3.37 with the words in shared memory). (Tiles of 128
+// sources would be faster, but their FP32 sums raise the PMCHWT forms' error against the FP64
+// application from 4.0e-8 to 5.5e-8.)
 struct F32x2 {
     static __device__ __forceinline__ float2 add(float2 a, float2 b) { return add2(a, b); }
     static __device__ __forceinline__ float2 sub(float2 a, float2 b) { return sub2(a, b); }
 };
 __host__ __device__ constexpr size_t wide_smem(int mode, int npk) {
-    return sizeof(float4) * TPB2 * npk * (mode == 0 ? 2 : 10);
+    return mode == 0 ? 0 : sizeof(float4) * TPB2 * npk * 10;
 }
-template <int NV>
-__device__ __forceinline__ void wide_zero(float2 (&hi)[NV], float4* words) {
-#pragma unroll
-    for (int a = 0; a < NV; ++a) {
-        hi[a] = make_float2(0.f, 0.f);
-        words[a * TPB2] = make_float4(0.f, 0.f, 0.f, 0.f);
+// a packed pair's sums
+template <int MODE>
+struct WideSums {
+    static constexpr int NV = MODE == 0 ? 2 : 10;
+    float2 hi[NV];
+    float4 reg[MODE == 0 ? NV : 1];  // V/K rows' lower words
+    __device__ __forceinline__ float4& word(float4* words, int a) {
+        if constexpr (MODE == 0) return reg[a];
+        else return words[a * TPB2];
     }
-}
-template <int NV>
-__device__ __forceinline__ void wide_add(float2 (&hi)[NV], float4* words, const float2 (&b)[NV]) {
+    __device__ __forceinline__ void zero(float4* words) {
 #pragma unroll
-    for (int a = 0; a < NV; ++a) {
-        const float4 w = words[a * TPB2];
-        float2 mid = make_float2(w.x, w.y), lo = make_float2(w.z, w.w);
-        wide_add<F32x2>(hi[a], mid, lo, b[a]);
-        words[a * TPB2] = make_float4(mid.x, mid.y, lo.x, lo.y);
+        for (int a = 0; a < NV; ++a) {
+            hi[a] = make_float2(0.f, 0.f);
+            word(words, a) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
-}
-// value a of the first (h = 0) or second target
-__device__ __forceinline__ double wide_total(const float2& hi, const float4* words, int a, int h) {
-    const float4 w = words[a * TPB2];
-    return h ? wide_value(hi.y, w.y, w.w) : wide_value(hi.x, w.x, w.z);
-}
+    __device__ __forceinline__ void add(float4* words, const float2 (&b)[NV]) {
+#pragma unroll
+        for (int a = 0; a < NV; ++a) {
+            const float4 w = word(words, a);
+            float2 mid = make_float2(w.x, w.y), lo = make_float2(w.z, w.w);
+            wide_add<F32x2>(hi[a], mid, lo, b[a]);
+            word(words, a) = make_float4(mid.x, mid.y, lo.x, lo.y);
+        }
+    }
+    // value a of the first (h = 0) or second target
+    __device__ __forceinline__ double total(float4* words, int a, int h) {
+        const float4 w = word(words, a);
+        return h ? wide_value(hi[a].y, w.y, w.w) : wide_value(hi[a].x, w.x, w.z);
+    }
+};
 
 // The tile's sums: records of 16 splatted values (position, s, p = sigma n, sigma, low words,
 // curl or normal). Points come in threes of one triangle and one weight (the 3-point rule, the
@@ -948,11 +958,11 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
         }
     }
     float2 acc[NPK][NRAW];
-    float2 hi[NPK][ACC ? NACC : 1];
+    WideSums<MODE> wide[ACC ? NPK : 1];
     float4* words = wide_words + threadIdx.x;  // pair p's at words + p NACC TPB2
     for (int p = 0; p < NPK; ++p) {
         for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
-        if constexpr (ACC) wide_zero<NACC>(hi[p], words + p * NACC * TPB2);
+        if constexpr (ACC) wide[p].zero(words + p * NACC * TPB2);
     }
     int failed_at = -1;
     for (int it = 0; it < ntiles; ++it) {
@@ -967,7 +977,7 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
                 for (int p = 0; p < NPK; ++p) {
                     float2 out[NACC];
                     x2_out<MODE, KIND>(cf, acc[p], out);
-                    wide_add<NACC>(hi[p], words + p * NACC * TPB2, out);
+                    wide[p].add(words + p * NACC * TPB2, out);
                     for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
                 }
         }
@@ -991,7 +1001,7 @@ __global__ void __launch_bounds__(TPB2, 2) k_pair32x2(const __grid_constant__ CU
             for (int a = 0; a < NACC; ++a) {
                 int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
                 if constexpr (ACC)
-                    static_cast<double*>(part_out)[o] = wide_total(hi[p][a], words + p * NACC * TPB2, a, h);
+                    static_cast<double*>(part_out)[o] = wide[p].total(words + p * NACC * TPB2, a, h);
                 else static_cast<float*>(part_out)[o] = h ? out[a].y : out[a].x;
             }
         }
@@ -1015,7 +1025,7 @@ static void x2_launch(dim3 g, cudaStream_t s, const CUtensorMap& map, int64_t np
                       const float* plo, Coef32 cf, int64_t chunk, void* part, int* status) {
     const auto kern = k_pair32x2<MODE, KIND, ACC, TS, ST, NPK, PROMO>;
     constexpr size_t smem = ACC ? wide_smem(MODE, NPK) : 0;
-    if (ACC) cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem) cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<g, TPB2, smem, s>>>(map, np, p32, plo, cf, chunk, part, status);
 }
 template <int MODE, int KIND, bool ACC, int TS, int ST, int NPK, int PROMO = 1>
@@ -1123,11 +1133,11 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
         }
     }
     float2 acc[NPK][NRAW];
-    float2 hi[NPK][ACC ? NACC : 1];
+    WideSums<MODE> wide[ACC ? NPK : 1];
     float4* words = wide_words + threadIdx.x;  // pair p's at words + p NACC TPB2
     for (int p = 0; p < NPK; ++p) {
         for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
-        if constexpr (ACC) wide_zero<NACC>(hi[p], words + p * NACC * TPB2);
+        if constexpr (ACC) wide[p].zero(words + p * NACC * TPB2);
     }
     int failed_at = -1;
     for (int it = 0; it < ntiles; ++it) {
@@ -1141,7 +1151,7 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
             for (int p = 0; p < NPK; ++p) {
                 float2 out[NACC];
                 x2_out<MODE, KIND>(cf, acc[p], out);
-                wide_add<NACC>(hi[p], words + p * NACC * TPB2, out);
+                wide[p].add(words + p * NACC * TPB2, out);
                 for (int a = 0; a < NRAW; ++a) acc[p][a] = make_float2(0.f, 0.f);
             }
         }
@@ -1170,7 +1180,7 @@ __device__ __forceinline__ bool pair_item(const PairJob& J, int tb, int split, f
             for (int a = 0; a < NACC; ++a) {
                 int64_t o = ((int64_t)split * NACC + a) * np + tg[t];
                 if constexpr (ACC)
-                    static_cast<double*>(J.part)[o] = wide_total(hi[p][a], words + p * NACC * TPB2, a, h);
+                    static_cast<double*>(J.part)[o] = wide[p].total(words + p * NACC * TPB2, a, h);
                 else static_cast<float*>(J.part)[o] = h ? out[a].y : out[a].x;
             }
         }
@@ -1892,7 +1902,7 @@ int apply_blockops_batched(const std::vector<FarJob>& jobs, int prec, BatchScrat
                                      : (acc ? (const void*)k_pair32x2_queue<1, true> : (const void*)k_pair32x2_queue<1, false>);
         const pb_ctx* ctx = jobs[hjob_of[mode].empty() ? tjob_of[mode][0] : hjob_of[mode][0]].m->ctx;
         const size_t smem = acc ? wide_smem(mode, 1) : 0;
-        if (acc) PB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (smem) PB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int per_sm = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB2, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
         cudaGetLastError();

@@ -321,12 +321,11 @@ __device__ __forceinline__ double exp_nonpos(double x) {
 // shared vertex, and d = x - y is formed from the frame vectors directly.
 
 // The vectors of an adjacent pair that its lanes read by broadcast: the frames'
-// edges, and the normals' products with them: n_B . x = s al1 + t al2 is the
-// height of x over the second triangle's plane, so d . n_B needs no y, and
-// -d . n_A = s' be1 + t' be2 no x.
+// edges and the normals. (d . n_B is the height of x over the second triangle's plane
+// and needs no y, but only for a normal without rounding: see band_pass.)
 struct AdjGeo {
     double e1a[3], e2a[3], e1b[3], e2b[3];
-    double al1, al2, be1, be2;
+    double na[3], nb[3];
 };
 
 // One entry (region, eta1, eta2) of an adjacent pair: the eta3 points' sums, then
@@ -347,11 +346,11 @@ __device__ __forceinline__ void accum_entry(double* mom, const SSOuter& tab, con
             D0[k] = __fma_rn(-ta2, P.e2b[k], __fma_rn(-sa2, P.e1b[k], __fma_rn(ta, P.e2a[k], sa * P.e1a[k])));
             D1[k] = __fma_rn(tb, P.e2a[k], -tb2 * P.e2b[k]);
         }
-        hb0 = __fma_rn(ta, P.al2, sa * P.al1);
-        ha0 = __fma_rn(ta2, P.be2, sa2 * P.be1);
     }
-    hb1 = tb * P.al2;
-    ha1 = tb2 * P.be2;
+    hb0 = D0[0] * P.nb[0] + D0[1] * P.nb[1] + D0[2] * P.nb[2];  // d . n_B and -d . n_A
+    hb1 = D1[0] * P.nb[0] + D1[1] * P.nb[1] + D1[2] * P.nb[2];
+    ha0 = -(D0[0] * P.na[0] + D0[1] * P.na[1] + D0[2] * P.na[2]);
+    ha1 = -(D1[0] * P.na[0] + D1[1] * P.na[1] + D1[2] * P.na[2]);
     // Laplace: sums with w3 and w3 eta3; Yukawa: with w3 for degrees 0..2, with w3 eta3 for 1, 2
     double l0[3] = {0, 0, 0}, l1[3] = {0, 0, 0}, y0[3][3], y1[3][2];
 #pragma unroll
@@ -570,12 +569,12 @@ constexpr int NEAR_THREADS = 128;
 // pair's (eta1, eta2, eta3) point (k_adj_pairs): d and r^2 (6 FMA), rsqrt, r, z (3),
 // the four E_m at degree 10 (40 FMA), w rinv, w/r^3 (3), F (3 FMA), the heights and
 // kernels (2 FMA, 2), eta3 products (3), sums (6 + 15 FMA): 155; an entry: D0, D1 and
-// the heights (17 FMA, 7), the moments (6 x 14 FMA): 209. A coincident pair's point
+// their products with the normals (20 FMA, 10), the moments (6 x 14 FMA): 218. A coincident pair's point
 // (moments from the rule's table of weighted monomials): d from (s - s', t - t') (11),
 // r^2 to the Yukawa single layer (11), 2 x 2 x 9 (36); by the polynomials (k_coin_poly), per
 // direction: v and r^2 (24), rsqrt, r, z (3), the Yukawa moments (18 a degree), both kernels' (36).
 constexpr double NEAR_FLOPS_ADJ_POINT = 155;
-constexpr double NEAR_FLOPS_ADJ_ENTRY = 209;
+constexpr double NEAR_FLOPS_ADJ_ENTRY = 218;
 constexpr double NEAR_FLOPS_COIN = 22 + 36;
 static double coin_dir_flops(int deg) { return 63.0 + 18.0 * deg; }
 
@@ -590,8 +589,8 @@ static double coin_dir_flops(int deg) { return 63.0 + 18.0 * deg; }
 // instructions to about 95 at n = 4; small groups keep the per-pair work (sums over
 // lanes, corner blocks) to a few per cent: 8 lanes hold 12 of an edge pair's 96
 // entries each, 4 lanes 8 of a vertex pair's 32; G = 32 for few pairs (adj_group).
-// 38,720 triangles, n = 4: edge and vertex launches 34.0 -> 10.05 ms (with the far
-// rule in both); 2,000 triangles 1.91 -> 0.58 ms.
+// 38,720 triangles, n = 4: edge and vertex launches 34.0 -> 10.2 ms (with the far
+// rule in the former); 2,000 triangles 1.91 -> 0.58 ms.
 template <int NSS, int G>
 __global__ void __launch_bounds__(NEAR_THREADS, 2)
 k_adj_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
@@ -628,14 +627,8 @@ k_adj_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris, 
             (f ? S.geo.e2b : S.geo.e2a)[k] = q2 - q1;
             S.inv[f][(perm >> (2 * k)) & 3] = k;
         }
-    }
-    __syncwarp();
-    if (gl < 4) {  // heights of the edges' ends over the other triangle's plane (a shared edge lies in both)
-        const double* e = gl == 0 ? S.geo.e1a : gl == 1 ? S.geo.e2a : gl == 2 ? S.geo.e1b : S.geo.e2b;
-        const double* n = gl < 2 ? gB : gA;
-        double h = e[0] * n[0] + e[1] * n[1] + e[2] * n[2];
-        if (pr.z == 1 && (gl & 1) == 0) h = 0.0;
-        (&S.geo.al1)[gl] = h;
+        S.geo.na[k] = gA[k];
+        S.geo.nb[k] = gB[k];
     }
     const double fc = 1.0 / (4.0 * areaA * areaB);
     for (int ab = gl; ab < 9; ab += G) {
@@ -962,25 +955,36 @@ k_coin_poly(const double* __restrict__ verts, const int32_t* __restrict__ tris, 
 //     the inner sums take two FMAs per kernel: one sum over the orbit and one per corner;
 //   - (x - y) . n_y is the height of x over the plane of y's triangle, whatever y: it
 //     multiplies the inner sums; (y - x) . n_x, the height of y, goes into y's weights.
-// 39 instructions a point pair (27 the kernels) and 92 an x point; 60 and 95 with the
-// normal products per point pair and three FMAs per kernel. 38,720 triangles, band of 3
-// radii, 6- and 3-point rules: 17.7 -> 9.9 ms (with full lanes, below). The y points of both rules are staged in
+//     The band rule only. The far rule, whose blocks are to cancel what the pair kernel
+//     adds for the pair, takes the products d . n as the pair kernel does: y's own
+//     height is the rounding of the normal, the same for all points of a triangle, so
+//     that leaving it out of one side only does not average out (errors of K and T, 500
+//     triangles, against 80-bit sums: 1.1e-15, with the products 1.5e-16; of the adjacent
+//     pairs, by the same in k_adj_pairs and k_adj_far, 4.0 and 1.5e-16).
+// 39 instructions a point pair (27 the kernels; 49 of the far rule's) and 92 an x point; 60 and
+// 95 with the normal products per point pair and three FMAs per kernel. 38,720 triangles, band of 3
+// radii, 6- and 3-point rules: 17.7 -> 10.0 ms (with full lanes, below). The y points of both rules are staged in
 // shared memory, per thread.
 constexpr int BAND_THREADS = 128;
 constexpr int ADJ_FAR_THREADS = 64;
-constexpr int BAND_Y = 5;  // doubles staged per y point: position, and a w and (1 - 3 a) w times its height
+// doubles staged per y point: position and, for heights, a w and (1 - 3 a) w times its height
+__host__ __device__ constexpr int staged(bool heights) { return heights ? 5 : 3; }
 
 // FP64 flops of one band pair under a Q-point rule by formula count: per point
 // pair the kernels (d 3, r^2 5, rsqrt, r, exp and its argument 17, 1/r^2, the four
 // kernels 6: 33) and the sums (12 FMA); per point of either triangle its position (15) and
 // height (5); per x point its weights (6), the sums' ends (18) and the block updates (54 FMA).
-__host__ __device__ constexpr double band_flops(int Q) { return Q * Q * (33.0 + 24.0) + Q * (40.0 + 24.0 + 108.0); }
+// Without heights 14 more a point pair (d . n twice, 5 each, and 4 products), 13 fewer an x point.
+__host__ __device__ constexpr double band_flops(int Q, bool heights) {
+    return Q * Q * (33.0 + 24.0 + (heights ? 0.0 : 14.0)) + Q * (40.0 + 24.0 + 108.0 - (heights ? 0.0 : 13.0));
+}
 
-// the Q points of a triangle with corners pb into ys (BAND_Y x Q slots, NT apart), their
-// heights over the plane through a0 with normal n
-template <int Q, int NT>
+// the Q points of a triangle with corners pb into ys (staged() x Q slots, NT apart), with
+// HEIGHTS their heights over the plane through a0 with normal n
+template <int Q, int NT, bool HEIGHTS>
 __device__ __forceinline__ void stage_points(double* ys, const double (&pb)[3][3], const Rule& R, const double* a0,
                                              const double* n) {
+    constexpr int YW = staged(HEIGHTS);
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
         double y[3], h = 0.0;
@@ -988,19 +992,22 @@ __device__ __forceinline__ void stage_points(double* ys, const double (&pb)[3][3
         for (int k = 0; k < 3; ++k) {
             y[k] = R.l[j][0] * pb[0][k] + R.l[j][1] * pb[1][k] + R.l[j][2] * pb[2][k];
             h += (y[k] - a0[k]) * n[k];
-            ys[(BAND_Y * j + k) * NT] = y[k];
+            ys[(YW * j + k) * NT] = y[k];
         }
-        const double a = R.l[j][Q == 1 ? 0 : (j + 1) % 3];
-        ys[(BAND_Y * j + 3) * NT] = R.w[j] * a * h;
-        ys[(BAND_Y * j + 4) * NT] = R.w[j] * (1.0 - 3.0 * a) * h;
+        if (HEIGHTS) {
+            const double a = R.l[j][Q == 1 ? 0 : (j + 1) % 3];
+            ys[(YW * j + 3) * NT] = R.w[j] * a * h;
+            ys[(YW * j + 4) * NT] = R.w[j] * (1.0 - 3.0 * a) * h;
+        }
     }
 }
 
 // blocks: V_L, V_Y, K_L, K_Y at 0, 9, 18, 27; the reversed pair's K_L, K_Y at 38, 47 (without 1/(4 pi))
-template <int Q, int NT>
+template <int Q, int NT, bool HEIGHTS>
 __device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3], const double* ys, const Rule& R,
-                                          double wscale, const double* b0, const double* nb, double kappa, double t64) {
-    constexpr int ORB = Q == 1 ? 1 : 3;
+                                          double wscale, const double* b0, const double* na, const double* nb,
+                                          double kappa, double t64) {
+    constexpr int ORB = Q == 1 ? 1 : 3, YW = staged(HEIGHTS);
 #pragma unroll 1
     for (int i = 0; i < Q; ++i) {
         double x[3], hx = 0.0;
@@ -1015,26 +1022,33 @@ __device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3],
 #pragma unroll 1
         for (int o = 0; o < Q; o += ORB) {
             const double a = R.l[o][Q == 1 ? 0 : 1], al = R.w[o] * a, be = R.w[o] * (1.0 - 3.0 * a);
-            const double* yo = ys + BAND_Y * o * NT;
+            const double* yo = ys + YW * o * NT;
 #pragma unroll
             for (int c = 0; c < ORB; ++c) {  // the orbit's point whose own corner is c
-                const double* y = yo + BAND_Y * c * NT;
+                const double* y = yo + YW * c * NT;
                 const double d0 = x[0] - y[0], d1 = x[1] - y[NT], d2 = x[2] - y[2 * NT];
                 const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
                 const double rinv = rsqrt(r2);
                 const double e = exp2_64th((r2 * rinv) * t64);
                 const double ri2 = rinv * rinv, g = e * rinv;
-                const double v[4] = {rinv, g, rinv * ri2, __fma_rn(kappa, e, g) * ri2};
-                const double ah = y[3 * NT], bh = y[4 * NT];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    T[k] = __fma_rn(al, v[k], T[k]);
-                    U[k][c] = __fma_rn(be, v[k], U[k][c]);
+                double v[6] = {rinv, g, rinv * ri2, __fma_rn(kappa, e, g) * ri2};
+                double ah = al, bh = be;  // weights of the reversed pair's
+                if (HEIGHTS) {
+                    ah = y[3 * NT];
+                    bh = y[4 * NT];
+                    v[4] = v[2];
+                    v[5] = v[3];
+                } else {
+                    const double dny = d0 * nb[0] + d1 * nb[1] + d2 * nb[2], dnx = -(d0 * na[0] + d1 * na[1] + d2 * na[2]);
+                    v[4] = v[2] * dnx;
+                    v[5] = v[3] * dnx;
+                    v[2] *= dny;
+                    v[3] *= dny;
                 }
 #pragma unroll
-                for (int k = 4; k < 6; ++k) {
-                    T[k] = __fma_rn(ah, v[k - 2], T[k]);
-                    U[k][c] = __fma_rn(bh, v[k - 2], U[k][c]);
+                for (int k = 0; k < 6; ++k) {
+                    T[k] = __fma_rn(k < 4 ? al : ah, v[k], T[k]);
+                    U[k][c] = __fma_rn(k < 4 ? be : bh, v[k], U[k][c]);
                 }
             }
         }
@@ -1045,7 +1059,7 @@ __device__ __forceinline__ void band_pass(double* acc, const double (&pa)[3][3],
             for (int c = 0; c < 3; ++c) U[k][c] += T[k];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const double wa = wi * R.l[i][a], wh = wa * hx;
+            const double wa = wi * R.l[i][a], wh = HEIGHTS ? wa * hx : wa;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const int base = k < 4 ? 9 * k : 38 + 9 * (k - 4);
@@ -1093,8 +1107,10 @@ __device__ __forceinline__ void band_pair(int64_t q, double* ys, const double* _
         return;
     }
     const int64_t p = n_adj + q, pr_rev = n_adj + lo;
+    double* ysc = ys + staged(true) * QF * BAND_THREADS;  // the far rule's points
     const double* gA = tgeo + 16 * (int64_t)pt;
     const double* gB = tgeo + 16 * (int64_t)ps;
+    const double na[3] = {gA[0], gA[1], gA[2]};
     double pa[3][3], b0[3];
     {
         double pb[3][3];
@@ -1105,9 +1121,8 @@ __device__ __forceinline__ void band_pair(int64_t q, double* ys, const double* _
                 pa[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)pt + a] + k];
                 pb[a][k] = verts[3 * (int64_t)tris[3 * (int64_t)ps + a] + k];
             }
-        const double na[3] = {gA[0], gA[1], gA[2]};
-        stage_points<QF, BAND_THREADS>(ys, pb, fine, pa[0], na);
-        stage_points<QC, BAND_THREADS>(ys + BAND_Y * QF * BAND_THREADS, pb, coarse, pa[0], na);
+        stage_points<QF, BAND_THREADS, true>(ys, pb, fine, pa[0], na);
+        stage_points<QC, BAND_THREADS, false>(ysc, pb, coarse, pa[0], na);
 #pragma unroll
         for (int k = 0; k < 3; ++k) b0[k] = pb[0][k];
     }
@@ -1116,8 +1131,8 @@ __device__ __forceinline__ void band_pair(int64_t q, double* ys, const double* _
 #pragma unroll
     for (int k = 0; k < NACC_SYM; ++k) acc[k] = 0.0;
     const double area2 = gA[3] * gB[3] * 0.07957747154594767, t64 = -kappa * EXP64_PER_UNIT;  // 1 / (4 pi)
-    band_pass<QF, BAND_THREADS>(acc, pa, ys, fine, area2, b0, nb, kappa, t64);
-    band_pass<QC, BAND_THREADS>(acc, pa, ys + BAND_Y * QF * BAND_THREADS, coarse, -area2, b0, nb, kappa, t64);
+    band_pass<QF, BAND_THREADS, true>(acc, pa, ys, fine, area2, b0, na, nb, kappa, t64);
+    band_pass<QC, BAND_THREADS, false>(acc, pa, ysc, coarse, -area2, b0, na, nb, kappa, t64);
     write_blocks(acc, gA, gB, kappa, ss_out + 54 * p, ss_out + 54 * pr_rev);
 }
 
@@ -1131,7 +1146,7 @@ k_band_pairs(const double* __restrict__ verts, const int32_t* __restrict__ tris,
              const int32_t* __restrict__ band_ptr, const int32_t* __restrict__ band_s,
              const int32_t* __restrict__ band_t, int64_t n_band, int span, int64_t n_adj, Rule fine, Rule coarse,
              double kappa, double* __restrict__ ss_out, int* __restrict__ status) {
-    __shared__ double ysm[(QF + QC) * BAND_Y * BAND_THREADS];
+    __shared__ double ysm[(staged(true) * QF + staged(false) * QC) * BAND_THREADS];
     __shared__ uint16_t todo[BAND_SPAN];  // the block's entries with t < s, in order
     __shared__ int wcnt[BAND_THREADS / 32];
     const int64_t q0 = blockIdx.x * (int64_t)span;
@@ -1165,7 +1180,7 @@ __global__ void __launch_bounds__(ADJ_FAR_THREADS)
 k_adj_far(const double* __restrict__ verts, const int32_t* __restrict__ tris, const double* __restrict__ tgeo,
           const int4* __restrict__ pairs, const int32_t* __restrict__ list, int64_t nlist,
           const int32_t* __restrict__ rev, Rule rule, double kappa, double* __restrict__ far_out) {
-    __shared__ double ysm[Q * BAND_Y * ADJ_FAR_THREADS];
+    __shared__ double ysm[Q * staged(false) * ADJ_FAR_THREADS];
     const int64_t li = blockIdx.x * (int64_t)ADJ_FAR_THREADS + threadIdx.x;
     if (li >= nlist) return;
     const int64_t p = list[li];
@@ -1181,12 +1196,12 @@ k_adj_far(const double* __restrict__ verts, const int32_t* __restrict__ tris, co
     const double* gA = tgeo + 16 * (int64_t)pr.x;
     const double* gB = tgeo + 16 * (int64_t)pr.y;
     const double na[3] = {gA[0], gA[1], gA[2]}, nb[3] = {gB[0], gB[1], gB[2]};
-    stage_points<Q, ADJ_FAR_THREADS>(ysm + threadIdx.x, pb, rule, pa[0], na);
+    stage_points<Q, ADJ_FAR_THREADS, false>(ysm + threadIdx.x, pb, rule, pa[0], na);
     double acc[NACC_SYM];
 #pragma unroll
     for (int k = 0; k < NACC_SYM; ++k) acc[k] = 0.0;
-    band_pass<Q, ADJ_FAR_THREADS>(acc, pa, ysm + threadIdx.x, rule, gA[3] * gB[3] * 0.07957747154594767, pb[0], nb,
-                                  kappa, -kappa * EXP64_PER_UNIT);
+    band_pass<Q, ADJ_FAR_THREADS, false>(acc, pa, ysm + threadIdx.x, rule, gA[3] * gB[3] * 0.07957747154594767, pb[0], na,
+                                         nb, kappa, -kappa * EXP64_PER_UNIT);
     write_blocks(acc, gA, gB, kappa, far_out + 54 * p, far_out + 54 * (int64_t)rev[p]);
 }
 
@@ -1504,7 +1519,7 @@ static int build(pb_ctx* ctx, const pb_mesh* m, double kappa, pb_near* nf, cudaS
             Rule fine = mesh_ref_rule(m), coarse = mesh_rule(m);
             const double ppairs = 0.5 * m->n_band * (Qb * Qb + Q * Q);
             Timer tm(ctx, PB_KERNEL_NEAR_BAND, s, ppairs,
-                     0.5 * m->n_band * (band_flops(m->Qr) + band_flops(m->Q)) / ppairs);
+                     0.5 * m->n_band * (band_flops(m->Qr, true) + band_flops(m->Q, false)) / ppairs);
             // few entries: smaller shares, so that every SM has some
             int span = BAND_SPAN;
             while (span > 2 * BAND_THREADS && m->n_band < (int64_t)4 * ctx->num_sms * span) span /= 2;
